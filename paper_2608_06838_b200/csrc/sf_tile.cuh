@@ -1,0 +1,185 @@
+// Register-tiled float32 products on CUDA cores, shared by the float32 / small-head kernels and the chunkwise forms of the
+// extension operators.
+//
+// Operands live in shared memory as row-major float32 tiles whose 16-byte units are XOR-swizzled with the row's index over
+// four: unit u of row r sits at position u ^ ((r >> 2) & 7).  A product C[m][n] += sum_k A(m,k) B(k,n) reads an operand
+// either along k (rows are m or n: one LDS.128 gives four k of one row) or across k (rows are k: one LDS.128 gives four
+// neighbouring m or n).  A thread owns groups of four consecutive m and n, so in the first form the lanes of a warp read
+// rows four apart, which the swizzle spreads over all banks, and in the second they read neighbouring units of one row:
+// both are free of conflicts from the same storage, and no tile is ever stored twice or transposed.
+#pragma once
+#include "sf_common.cuh"
+
+namespace sf {
+namespace tile {
+
+// Word offset of element (row, col) of a tile with rows of LD floats (LD a multiple of 32).
+template <int LD>
+__device__ __forceinline__ int at(int row, int col) {
+    return row * LD + ((((col >> 2) ^ ((row >> 2) & 7)) << 2) | (col & 3));
+}
+__device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
+__device__ __forceinline__ void st4(float* p, float4 v) { *reinterpret_cast<float4*>(p) = v; }
+
+// How NT threads share an M x N product: TM x TN outputs per thread (4 or 8), TYN x TXN threads take part (whole warps; a
+// warp covers 4 x 8 of them).  Thread (ty, tx) owns m in {4 ty .. 4 ty + 3} (+ M/2 for the second group) and n likewise.
+template <int M, int N, int NT>
+struct Map {
+    static constexpr int PER = M * N / 16 <= NT ? 16 : (M * N / 32 <= NT ? 32 : 64);
+    static constexpr int TM = PER == 64 ? 8 : (PER == 32 && M > N ? 8 : 4);
+    static constexpr int TN = PER / TM;
+    static constexpr int TYN = M / TM, TXN = N / TN;
+    static constexpr int ACTIVE = TYN * TXN;
+    static_assert(ACTIVE <= NT && TYN % 4 == 0 && TXN % 8 == 0, "shape does not map onto whole warps");
+    static constexpr int GM = TM / 4, GN = TN / 4;
+    int ty, tx;
+    bool on;
+    __device__ __forceinline__ Map() {
+        const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+        constexpr int WX = TXN / 8;
+        ty = (w / WX) * 4 + (l >> 3);
+        tx = (w % WX) * 8 + (l & 7);
+        on = (int)threadIdx.x < ACTIVE;
+    }
+    __device__ __forceinline__ int m(int i) const { return (i >> 2) * (M / GM) + 4 * ty + (i & 3); }
+    __device__ __forceinline__ int n4(int g) const { return g * (N / GN) + 4 * tx; }      // first of the g-th group of four
+    // rows covered by this warp's first / last thread group: limits of triangular products (TM == 4 only)
+    __device__ __forceinline__ int warp_m0() const { return 4 * (ty & ~3); }
+};
+
+// acc += A B over k in [k0, k1), both multiples of 4.  AK: A is stored [m][k], else [k][m]; BK: B is stored [n][k], else [k][n].
+template <class Mp, bool AK, bool BK, int LDA, int LDB>
+__device__ __forceinline__ void product(float (&acc)[Mp::TM][Mp::TN], const float* __restrict__ A, const float* __restrict__ B, int k0, int k1,
+                                        const Mp& mp) {
+#pragma unroll 2
+    for (int k = k0; k < k1; k += 4) {
+        const int u = k >> 2;
+        float b[4][Mp::TN];                                      // [kk][n]
+        if constexpr (BK) {
+            const int off = (u ^ (mp.tx & 7)) << 2;              // row n: (n >> 2) & 7 == tx & 7, also for the second group (N/2 is a multiple of 32)
+#pragma unroll
+            for (int g = 0; g < Mp::GN; ++g)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const float4 v = ld4(B + (mp.n4(g) + j) * LDB + off);
+                    b[0][4 * g + j] = v.x; b[1][4 * g + j] = v.y; b[2][4 * g + j] = v.z; b[3][4 * g + j] = v.w;
+                }
+        } else {
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk)
+#pragma unroll
+                for (int g = 0; g < Mp::GN; ++g) {
+                    const float4 v = ld4(B + (k + kk) * LDB + (((mp.n4(g) >> 2) ^ (u & 7)) << 2));
+                    b[kk][4 * g] = v.x; b[kk][4 * g + 1] = v.y; b[kk][4 * g + 2] = v.z; b[kk][4 * g + 3] = v.w;
+                }
+        }
+        if constexpr (AK) {
+            const int off = (u ^ (mp.ty & 7)) << 2;
+#pragma unroll
+            for (int i = 0; i < Mp::TM; ++i) {
+                const float4 a = ld4(A + mp.m(i) * LDA + off);
+#pragma unroll
+                for (int j = 0; j < Mp::TN; ++j) {
+                    acc[i][j] = fmaf(a.x, b[0][j], acc[i][j]);
+                    acc[i][j] = fmaf(a.y, b[1][j], acc[i][j]);
+                    acc[i][j] = fmaf(a.z, b[2][j], acc[i][j]);
+                    acc[i][j] = fmaf(a.w, b[3][j], acc[i][j]);
+                }
+            }
+        } else {
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk)
+#pragma unroll
+                for (int g = 0; g < Mp::GM; ++g) {
+                    const float4 a = ld4(A + (k + kk) * LDA + (((mp.m(4 * g) >> 2) ^ (u & 7)) << 2));
+                    const float av[4] = {a.x, a.y, a.z, a.w};
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+#pragma unroll
+                        for (int j = 0; j < Mp::TN; ++j) acc[4 * g + i][j] = fmaf(av[i], b[kk][j], acc[4 * g + i][j]);
+                }
+        }
+    }
+}
+
+template <class Mp>
+__device__ __forceinline__ void zero(float (&acc)[Mp::TM][Mp::TN]) {
+#pragma unroll
+    for (int i = 0; i < Mp::TM; ++i)
+#pragma unroll
+        for (int j = 0; j < Mp::TN; ++j) acc[i][j] = 0.f;
+}
+
+// Four neighbouring elements of a row in global memory (16-byte aligned float32, 8-byte aligned bf16).
+__device__ __forceinline__ float4 load4(const float* p) { return __ldg(reinterpret_cast<const float4*>(p)); }
+__device__ __forceinline__ float4 load4(const __nv_bfloat16* p) {
+    const uint2 v = __ldg(reinterpret_cast<const uint2*>(p));
+    const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&v.x));
+    const float2 b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&v.y));
+    return make_float4(a.x, a.y, b.x, b.y);
+}
+__device__ __forceinline__ void store4(float* p, float4 v) { *reinterpret_cast<float4*>(p) = v; }
+__device__ __forceinline__ void store4(__nv_bfloat16* p, float4 v) {
+    const __nv_bfloat162 a = __floats2bfloat162_rn(v.x, v.y), b = __floats2bfloat162_rn(v.z, v.w);
+    uint2 o;
+    o.x = *reinterpret_cast<const uint32_t*>(&a);
+    o.y = *reinterpret_cast<const uint32_t*>(&b);
+    *reinterpret_cast<uint2*>(p) = o;
+}
+
+// ROWS x D tile from global rows `stride` elements apart; rows at or beyond `valid` become zero.
+template <int ROWS, int D, int NT, typename T>
+__device__ __forceinline__ void load(float* dst, const T* __restrict__ src, long long stride, int valid) {
+    constexpr int U = D / 4, IT = ROWS * U / NT;
+    static_assert(ROWS * U % NT == 0, "tile does not divide among the threads");
+    float4 v[IT < 8 ? IT : 8];
+#pragma unroll
+    for (int i0 = 0; i0 < IT; i0 += 8) {
+#pragma unroll
+        for (int i = 0; i < 8 && i0 + i < IT; ++i) {
+            const int idx = threadIdx.x + (i0 + i) * NT, r = idx / U, c = (idx % U) * 4;
+            v[i] = r < valid ? load4(src + r * stride + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+#pragma unroll
+        for (int i = 0; i < 8 && i0 + i < IT; ++i) {
+            const int idx = threadIdx.x + (i0 + i) * NT, r = idx / U, c = (idx % U) * 4;
+            st4(dst + at<D>(r, c), v[i]);
+        }
+    }
+}
+// The same with a factor per row.
+template <int ROWS, int D, int NT, typename T>
+__device__ __forceinline__ void load_scaled(float* dst, const T* __restrict__ src, long long stride, int valid, const float* w) {
+    constexpr int U = D / 4, IT = ROWS * U / NT;
+    static_assert(ROWS * U % NT == 0, "tile does not divide among the threads");
+#pragma unroll
+    for (int i0 = 0; i0 < IT; i0 += 8) {
+        float4 v[8];
+#pragma unroll
+        for (int i = 0; i < 8 && i0 + i < IT; ++i) {
+            const int idx = threadIdx.x + (i0 + i) * NT, r = idx / U, c = (idx % U) * 4;
+            v[i] = r < valid ? load4(src + r * stride + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+#pragma unroll
+        for (int i = 0; i < 8 && i0 + i < IT; ++i) {
+            const int idx = threadIdx.x + (i0 + i) * NT, r = idx / U, c = (idx % U) * 4;
+            const float f = w[r];
+            st4(dst + at<D>(r, c), make_float4(v[i].x * f, v[i].y * f, v[i].z * f, v[i].w * f));
+        }
+    }
+}
+// Rows of a tile times a factor per row, in place.
+template <int ROWS, int D, int NT>
+__device__ __forceinline__ void scale_rows(float* x, const float* w) {
+    for (int idx = threadIdx.x; idx < ROWS * D / 4; idx += NT) {
+        const int r = idx / (D / 4);
+        float4* p = reinterpret_cast<float4*>(x) + idx;          // the swizzle permutes units inside a row only
+        const float f = w[r];
+        float4 v = *p;
+        v.x *= f; v.y *= f; v.z *= f; v.w *= f;
+        *p = v;
+    }
+}
+
+}  // namespace tile
+}  // namespace sf

@@ -136,11 +136,30 @@ int chain_chunks_per_block(int NC, long long bh) {
     return (int)((NC + nb - 1) / nb);
 }
 
+// Block length of the CUDA-core kernels, which walk a block in tiles of 64 tokens: waves * (tiles per block + what a CTA costs
+// besides its tiles), one wave being all CTAs that fit on the device at once.  A tile is 10-25 us of arithmetic, so unlike
+// on the tensor-core path short blocks cost little; at most 16 tiles, beyond which the block states no longer count.
+// Ties go to the longer block.
+int simt_chunks_per_block(const sf_seg_desc_t* d) {
+    const int tile = sf::simt::CT, cpt = tile / d->chunk;                 // chunks per tile
+    const long long ntile = ((long long)d->seg_len + tile - 1) / tile, bh = (long long)d->B * d->H;
+    const long long slots = (long long)sm_count() * (d->d_k == 128 ? 1 : (d->d_k == 64 ? 2 : 3));
+    long long best_cost = -1;
+    int best = 1;
+    for (int r = 1; r <= 16; ++r) {
+        const long long nb = (ntile + r - 1) / r, waves = (nb * bh + slots - 1) / slots, cost = waves * (10 * r + 6);
+        if (best_cost < 0 || cost <= best_cost) { best_cost = cost; best = r; }
+        if (r >= ntile) break;
+    }
+    return best * cpt;
+}
+bool on_tensor_cores(const sf_seg_desc_t* d) { return d->dtype == SF_BF16 && d->d_k == 128 && d->d_v == 128; }
+
 // Descriptor of segment i of a chain: the caller's block length if given, else the chain model above.
 sf_seg_desc_t chain_segment_desc(const sf_seg_desc_t* desc, int32_t seg_len, int32_t n_seg) {
     sf_seg_desc_t t = *desc;
     t.seg_len = seg_len;
-    if (t.chunks_per_block == 0 && n_seg > 1 && t.chunk > 0)
+    if (t.chunks_per_block == 0 && n_seg > 1 && t.chunk > 0 && on_tensor_cores(desc))
         t.chunks_per_block = chain_chunks_per_block((seg_len + t.chunk - 1) / t.chunk, (long long)t.B * t.H);
     return t;
 }
@@ -150,7 +169,7 @@ SegParams make_params(const sf_seg_desc_t* d, int cpb_override = 0) {
     p.B = d->B; p.H = d->H; p.L = d->seg_len; p.C = d->chunk;
     p.NC = (d->seg_len + d->chunk - 1) / d->chunk;      // the last chunk may be partial
     int r = cpb_override > 0 ? cpb_override : d->chunks_per_block;
-    p.R = r > 0 ? r : auto_chunks_per_block(p.NC, (long long)d->B * d->H);
+    p.R = r > 0 ? r : (on_tensor_cores(d) ? auto_chunks_per_block(p.NC, (long long)d->B * d->H) : simt_chunks_per_block(d));
     p.NB = (p.NC + p.R - 1) / p.R;
     p.tqk = d->tok_stride_qk; p.tv = d->tok_stride_v; p.tg = d->tok_stride_g;
     p.bqk = d->batch_stride_qk; p.bv = d->batch_stride_v; p.bg = d->batch_stride_g;
@@ -225,11 +244,11 @@ struct RoleArgs {
 template <typename T, int DK, int DV>
 sf_status_t launch_simt(Role role, const SegParams& p, const RoleArgs& a, cudaStream_t st) {
     using namespace sf::simt;
-    dim3 grid(p.NB, p.H, p.B), block(NT);
+    dim3 grid(p.NB, p.H, p.B), block(kThreads<DK>);
     switch (role) {
         case Role::Aggregate: {
             auto kern = block_aggregate_kernel<T, DK, DV>;
-            constexpr size_t sm = smem_aggregate<DK, DV>();
+            constexpr size_t sm = sizeof(AggSmem<DK, DV>);
             SF_TRY(set_smem(kern, sm));
             const T* X = static_cast<const T*>(a.mode == 0 ? a.k : a.q);
             const T* Y = static_cast<const T*>(a.mode == 0 ? a.v : a.dO);
@@ -238,7 +257,7 @@ sf_status_t launch_simt(Role role, const SegParams& p, const RoleArgs& a, cudaSt
         }
         case Role::FwdOut: {
             auto kern = fwd_out_kernel<T, DK, DV>;
-            constexpr size_t sm = smem_fwd_out<DK, DV>();
+            constexpr size_t sm = sizeof(FwdSmem<DK, DV>);
             SF_TRY(set_smem(kern, sm));
             kern<<<grid, block, sm, st>>>(p, static_cast<const T*>(a.q), static_cast<const T*>(a.k),
                                           static_cast<const T*>(a.v), a.g, a.states, static_cast<T*>(a.o));
@@ -246,7 +265,7 @@ sf_status_t launch_simt(Role role, const SegParams& p, const RoleArgs& a, cudaSt
         }
         case Role::BwdDq: {
             auto kern = bwd_dq_kernel<T, DK, DV>;
-            constexpr size_t sm = smem_bwd_dq<DK, DV>();
+            constexpr size_t sm = sizeof(DqSmem<DK, DV>);
             SF_TRY(set_smem(kern, sm));
             kern<<<grid, block, sm, st>>>(p, static_cast<const T*>(a.q), static_cast<const T*>(a.k),
                                           static_cast<const T*>(a.v), a.g, static_cast<const T*>(a.dO), a.states,
@@ -255,7 +274,7 @@ sf_status_t launch_simt(Role role, const SegParams& p, const RoleArgs& a, cudaSt
         }
         case Role::BwdDkDv: {
             auto kern = bwd_dkdv_kernel<T, DK, DV>;
-            constexpr size_t sm = smem_bwd_dkdv<DK, DV>();
+            constexpr size_t sm = sizeof(DkdvSmem<DK, DV>);
             SF_TRY(set_smem(kern, sm));
             kern<<<grid, block, sm, st>>>(p, static_cast<const T*>(a.q), static_cast<const T*>(a.k),
                                           static_cast<const T*>(a.v), a.g, static_cast<const T*>(a.dO), a.states,
@@ -523,13 +542,13 @@ bool merged_desc(const sf_seg_desc_t* desc, const int32_t* seg_lens, int32_t n_s
     }
     int R = desc->chunks_per_block;
     if (R == 0) {
-        // the longest block length (at most 64 chunks) that divides the chunk count of every segment but the last
-        for (R = 64; R >= 1; --R) {
+        // the longest block length up to the library's choice that divides the chunk count of every segment but the last
+        for (R = simt_chunks_per_block(&t); R >= 1; --R) {
             bool ok = true;
             for (int i = 0; i + 1 < n_seg && ok; ++i) ok = (seg_lens[i] / C) % R == 0;
             if (ok) break;
         }
-        if (R < 4) return false;
+        if (R * C < sf::simt::CT) return false;
     } else {
         for (int i = 0; i + 1 < n_seg; ++i)
             if ((seg_lens[i] / C) % R) return false;
@@ -705,7 +724,11 @@ sf_status_t sf_segment_fwd_static(const sf_seg_desc_t* desc, const void* q, cons
     const Path path = classify(desc);
     if (path == Path::Invalid) return SF_ERR_INVALID_ARG;
     if (path == Path::Unsupported) return SF_ERR_UNSUPPORTED;
-    if (sf_workspace_bytes(desc, 0) > SF_STATIC_SCRATCH_BYTES) return SF_ERR_WORKSPACE;
+    // The scratch array bounds the number of blocks: where the library's choice has more than fit, the longest that fit.
+    sf_seg_desc_t d = *desc;
+    if (d.chunks_per_block == 0)
+        for (int r = make_params(&d).R; sf_workspace_bytes(&d, 0) > SF_STATIC_SCRATCH_BYTES && r < sf::simt::MAXR;) d.chunks_per_block = ++r;
+    if (sf_workspace_bytes(&d, 0) > SF_STATIC_SCRATCH_BYTES) return SF_ERR_WORKSPACE;
     // device address of the scratch array, looked up once per device with that device current
     constexpr int kMaxDevices = 64;
     static void* scratch_of_device[kMaxDevices] = {};
@@ -722,7 +745,7 @@ sf_status_t sf_segment_fwd_static(const sf_seg_desc_t* desc, const void* q, cons
         }
         scratch = scratch_of_device[dev];
     }
-    return sf_segment_fwd(desc, q, k, v, g, S_in, o, S_out, scratch, SF_STATIC_SCRATCH_BYTES, stream);
+    return sf_segment_fwd(&d, q, k, v, g, S_in, o, S_out, scratch, SF_STATIC_SCRATCH_BYTES, stream);
 }
 
 sf_status_t sf_state_scan(const sf_seg_desc_t* desc, int32_t chunks_per_block, int32_t reverse, const float* log_decay,
