@@ -20,7 +20,7 @@
 // at d = 64, against 2.8 / 1.4 KB of memory traffic; 35 T multiply-adds/s were measured from registers alone).  A thread
 // therefore owns 16 to 64 outputs of a product and feeds four multiply-adds per operand word read from shared memory.  Chains
 // forward + backward, before (one output and one scalar inner product at a time) and now: float32 d = 128, 8144 tokens x 16
-// heads 11.4 -> 1.64 ms (16 T multiply-adds/s); bf16 d = 64, 16384 tokens x 16 heads 6.05 -> 1.09 ms (17 T).
+// heads 11.4 -> 1.58 ms (17 T multiply-adds/s); bf16 d = 64, 16384 tokens x 16 heads 5.92 -> 0.99 ms (18 T).
 #pragma once
 #include "sf_common.cuh"
 #include "sf_tile.cuh"
@@ -151,10 +151,8 @@ __device__ __forceinline__ void row_dots(const float (&acc)[Mp::TM][Mp::TN], con
             s = fmaf(acc[i][4 * gq], v.x, s); s = fmaf(acc[i][4 * gq + 1], v.y, s);
             s = fmaf(acc[i][4 * gq + 2], v.z, s); s = fmaf(acc[i][4 * gq + 3], v.w, s);
         }
-        s += __shfl_xor_sync(0xffffffffu, s, 1);
-        s += __shfl_xor_sync(0xffffffffu, s, 2);
-        s += __shfl_xor_sync(0xffffffffu, s, 4);
-        if ((threadIdx.x & 7) == 0) red[mp.m(i) * WX + (mp.tx >> 3)] = s;
+        s = tile::sum_x(s);
+        if ((mp.tx & 7) == 0) red[mp.m(i) * WX + (mp.tx >> 3)] = s;
     }
 }
 template <int WX>
