@@ -1,0 +1,152 @@
+// C ABI of the chunkwise gated delta rule: argument checks, shape dispatch and launches.
+#include "../../include/stateflow.h"
+#include "sf_delta_chunk.cuh"
+#include "sf_variants_host.h"
+
+namespace {
+
+using namespace sfv;
+
+sf_status_t check_chunked(const sf_seg_desc_t* d) {
+    const sf_status_t c = check_desc(d, true);
+    if (c != SF_OK) return c;
+    if (d->chunk <= 0) return SF_ERR_INVALID_ARG;
+    if (d->chunk != 16 && d->chunk != 32) return SF_ERR_UNSUPPORTED;
+    if (d->H > 65535) return SF_ERR_INVALID_ARG;
+    return sf::gdn::smem_rule(d->chunk, d->d_k, d->d_v) <= kMaxSmem ? SF_OK : SF_ERR_UNSUPPORTED;
+}
+
+sf::gdn::Params chunked_params(const sf_seg_desc_t* d, bool vec) {
+    sf::gdn::Params p;
+    p.B = d->B; p.H = d->H; p.L = d->seg_len; p.C = d->chunk; p.NC = (d->seg_len + d->chunk - 1) / d->chunk;
+    p.NT = (d->seg_len + sf::gdn::CT - 1) / sf::gdn::CT;
+    p.dk = d->d_k; p.dv = d->d_v;
+    p.vec = vec;
+    p.tqk = d->tok_stride_qk; p.tv = d->tok_stride_v; p.tg = d->tok_stride_g;
+    p.bqk = d->batch_stride_qk; p.bv = d->batch_stride_v; p.bg = d->batch_stride_g;
+    return p;
+}
+
+size_t chunked_ws_bytes(const sf_seg_desc_t* d, bool backward) {
+    return (size_t)d->B * d->H * sf::gdn::ws_floats(chunked_params(d, false), backward) * sizeof(float);
+}
+
+struct Args {
+    const void *q, *k, *v;
+    const float *g, *beta, *S_in;
+    void* o;
+    float* S_out;
+    const void* dO;
+    const float* dS_out;
+    void *dq, *dk, *dv;
+    float *dg, *dbeta, *dS_in;
+    float* ws;
+    cudaStream_t st;
+};
+
+// The sequential pass over the tiles, forward and (rev != NULL) reverse in one launch.  8 state columns per CTA where that
+// leaves at most one CTA per SM and direction, else 16: a step of 8 columns has half the multiply-adds (16 heads x 512 tiles at
+// d_k = 64, forward + backward of the operator: 2.47 ms against 3.01), but every CTA streams the whole map, so it does not pay
+// once the device is full.
+template <int DK>
+bool launch_chain(const sf::gdn::Params& p, const sf::gdn::ChainEnds& fwd, const sf::gdn::ChainEnds* rev, float* ws, int backward, cudaStream_t st) {
+    using namespace sf::gdn;
+    const int dirs = rev ? 2 : 1;
+    const ChainEnds r = rev ? *rev : ChainEnds{nullptr, nullptr};
+    if constexpr (DK > 32) {
+        if ((long long)p.B * p.H * (p.dv / 8) <= 148) {
+            constexpr size_t sm = sizeof(ChainSmem<DK, 8>);
+            if (!opt_in<chain_kernel<DK, 8>>(sm)) return false;
+            chain_kernel<DK, 8><<<dim3(dirs * (p.dv / 8), p.H, p.B), CHAIN_NT, sm, st>>>(p, fwd, r, ws, backward);
+            return true;
+        }
+    }
+    constexpr size_t sm = sizeof(ChainSmem<DK, 16>);
+    if (!opt_in<chain_kernel<DK, 16>>(sm)) return false;
+    chain_kernel<DK, 16><<<dim3(dirs * (p.dv / 16), p.H, p.B), CHAIN_NT, sm, st>>>(p, fwd, r, ws, backward);
+    return true;
+}
+
+template <typename T, int DK, int DV>
+sf_status_t forward(const sf::gdn::Params& p, const Args& a) {
+    using namespace sf::gdn;
+    const T *q = static_cast<const T*>(a.q), *k = static_cast<const T*>(a.k), *v = static_cast<const T*>(a.v);
+    const dim3 tiles(p.NT, p.H, p.B);
+    constexpr int nt = kThreads<DK, DV>;
+    constexpr size_t s1 = sizeof(PreSmem<DK, DV, false>), s2 = sizeof(OutSmem<DK, DV>);
+    if (!opt_in<pre_kernel<T, DK, DV, false>>(s1) || !opt_in<out_kernel<T, DK, DV>>(s2)) return SF_ERR_CUDA;
+    pre_kernel<T, DK, DV, false><<<tiles, nt, s1, a.st>>>(p, q, k, v, a.g, a.beta, nullptr, a.ws);
+    if (!launch_chain<DK>(p, ChainEnds{a.S_in, a.S_out}, nullptr, a.ws, 0, a.st)) return SF_ERR_CUDA;
+    out_kernel<T, DK, DV><<<tiles, nt, s2, a.st>>>(p, q, k, v, a.g, a.beta, static_cast<T*>(a.o), a.ws);
+    return launched(3);
+}
+
+// The backward rebuilds the forward's maps and states first.
+template <typename T, int DK, int DV>
+sf_status_t backward(const sf::gdn::Params& p, const Args& a) {
+    using namespace sf::gdn;
+    const T *q = static_cast<const T*>(a.q), *k = static_cast<const T*>(a.k), *v = static_cast<const T*>(a.v), *dO = static_cast<const T*>(a.dO);
+    const dim3 tiles(p.NT, p.H, p.B);
+    constexpr int nt = kThreads<DK, DV>;
+    constexpr size_t s1 = sizeof(PreSmem<DK, DV, true>), s2 = sizeof(BwdSmem<DK, DV>);
+    if (!opt_in<pre_kernel<T, DK, DV, true>>(s1) || !opt_in<bwd_out_kernel<T, DK, DV>>(s2)) return SF_ERR_CUDA;
+    pre_kernel<T, DK, DV, true><<<tiles, nt, s1, a.st>>>(p, q, k, v, a.g, a.beta, dO, a.ws);
+    const ChainEnds rev{a.dS_out, a.dS_in};
+    if (!launch_chain<DK>(p, ChainEnds{a.S_in, nullptr}, &rev, a.ws, 1, a.st)) return SF_ERR_CUDA;
+    bwd_out_kernel<T, DK, DV><<<tiles, nt, s2, a.st>>>(p, q, k, v, a.g, a.beta, dO, static_cast<T*>(a.dq), static_cast<T*>(a.dk), static_cast<T*>(a.dv),
+                                                      a.dg, a.dbeta, a.ws);
+    return launched(3);
+}
+
+template <typename T>
+sf_status_t dispatch(const sf::gdn::Params& p, const Args& a) {
+#define SF_SHAPE(DK, DV) if (p.dk == DK && p.dv == DV) return a.dO ? backward<T, DK, DV>(p, a) : forward<T, DK, DV>(p, a);
+    SF_SHAPE(32, 32) SF_SHAPE(32, 64) SF_SHAPE(32, 128)
+    SF_SHAPE(64, 32) SF_SHAPE(64, 64) SF_SHAPE(64, 128)
+    SF_SHAPE(128, 32) SF_SHAPE(128, 64) SF_SHAPE(128, 128)
+#undef SF_SHAPE
+    return SF_ERR_UNSUPPORTED;
+}
+
+sf_status_t run(const sf_seg_desc_t* d, const Args& a) {
+    const sf::gdn::Params p = chunked_params(d, vec_ok(d, {a.q, a.k, a.v, a.o, a.dO, a.dq, a.dk, a.dv}));
+    return d->dtype == SF_F32 ? dispatch<float>(p, a) : dispatch<__nv_bfloat16>(p, a);
+}
+
+}  // namespace
+
+extern "C" {
+
+size_t sf_delta_chunked_workspace_bytes(const sf_seg_desc_t* desc, int backward) {
+    return check_chunked(desc) == SF_OK ? chunked_ws_bytes(desc, backward != 0) : 0;
+}
+
+sf_status_t sf_delta_chunked_fwd(const sf_seg_desc_t* desc, const void* q, const void* k, const void* v, const float* g,
+                                 const float* beta, const float* S_in, void* o, float* S_out, void* workspace, size_t workspace_bytes,
+                                 sf_stream_t stream) {
+    const sf_status_t c = check_chunked(desc);
+    if (c != SF_OK) return c;
+    if (!q || !k || !v || !g || !beta || !o || !S_out || S_in == S_out) return SF_ERR_INVALID_ARG;
+    if (!workspace || workspace_bytes < chunked_ws_bytes(desc, false) || (reinterpret_cast<uintptr_t>(workspace) & 255u)) return SF_ERR_WORKSPACE;
+    Args a{};
+    a.q = q; a.k = k; a.v = v; a.g = g; a.beta = beta; a.S_in = S_in; a.o = o; a.S_out = S_out;
+    a.ws = static_cast<float*>(workspace); a.st = reinterpret_cast<cudaStream_t>(stream);
+    return run(desc, a);
+}
+
+sf_status_t sf_delta_chunked_bwd(const sf_seg_desc_t* desc, const void* q, const void* k, const void* v, const float* g,
+                                 const float* beta, const float* S_in, const void* dO, const float* dS_out, void* dq, void* dk,
+                                 void* dv, float* dg, float* dbeta, float* dS_in, void* workspace, size_t workspace_bytes,
+                                 sf_stream_t stream) {
+    const sf_status_t c = check_chunked(desc);
+    if (c != SF_OK) return c;
+    if (!q || !k || !v || !g || !beta || !dO || !dq || !dk || !dv || !dg || !dbeta || !dS_in || dS_in == dS_out) return SF_ERR_INVALID_ARG;
+    if (!workspace || workspace_bytes < chunked_ws_bytes(desc, true) || (reinterpret_cast<uintptr_t>(workspace) & 255u)) return SF_ERR_WORKSPACE;
+    Args a{};
+    a.q = q; a.k = k; a.v = v; a.g = g; a.beta = beta; a.S_in = S_in; a.dO = dO; a.dS_out = dS_out;
+    a.dq = dq; a.dk = dk; a.dv = dv; a.dg = dg; a.dbeta = dbeta; a.dS_in = dS_in;
+    a.ws = static_cast<float*>(workspace); a.st = reinterpret_cast<cudaStream_t>(stream);
+    return run(desc, a);
+}
+
+}  // extern "C"

@@ -21,17 +21,72 @@
 // Chunk length 16 or 32, d_k, d_v in {32, 64, 128} as far as the tiles fit into shared memory (128 needs chunk 16); a last
 // chunk with fewer tokens is handled by row counts.
 #pragma once
-#include "sf_delta_chunk.cuh"
+#include "sf_common.cuh"
 
 namespace sf {
 namespace dcc {
 
-using gdn::NT;
-using gdn::ldp;
-using gdn::mm;
-using gdn::load_rows;
-using gdn::load_dense;
-using gdn::scale_rows;
+constexpr int NT = 256;
+// Shared-memory tiles are stored with an odd leading dimension (columns + 1), so that both row-wise and column-wise
+// walks hit different banks.
+__host__ __device__ constexpr int ldp(int cols) { return cols + 1; }
+
+// out[m][n] = keep*out[m][n] + sign * sum_k A(m,k) B(k,n);  A(m,k) = ta ? A[k*lda+m] : A[m*lda+k], likewise B.
+// Element idx is always computed by the same thread, so a second product may accumulate into `out` (keep = 1) without a
+// barrier in between, also when `out` is global memory.
+__device__ __forceinline__ void mm(float* out, int ldo, const float* A, int lda, bool ta, const float* Bm, int ldb, bool tb,
+                                   int M, int N, int K, float keep, float sign) {
+    // four independent accumulators per thread: the products are small and latency-bound, not throughput-bound
+    const int total = M * N, sa = ta ? lda : 1, sb = tb ? 1 : ldb;
+    for (int base = threadIdx.x; base < total; base += 4 * NT) {
+        const float *a[4], *bq[4];
+        float acc[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const int idx = min(base + e * NT, total - 1);            // clamped: a lane past the end computes a value it drops
+            const int m = idx / N, n = idx - m * N;
+            a[e] = ta ? A + m : A + m * lda;
+            bq[e] = tb ? Bm + n * ldb : Bm + n;
+        }
+#pragma unroll 2
+        for (int k = 0; k < K; ++k) {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) acc[e] = fmaf(a[e][k * sa], bq[e][k * sb], acc[e]);
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const int idx = base + e * NT;
+            if (idx < total) {
+                const int m = idx / N, n = idx - m * N;
+                out[m * ldo + n] = keep != 0.f ? fmaf(keep, out[m * ldo + n], sign * acc[e]) : sign * acc[e];
+            }
+        }
+    }
+}
+
+template <typename T>
+__device__ __forceinline__ void load_rows(float* dst, int ld, const T* src, long long tok_stride, int rows, int cols) {
+    for (int idx = threadIdx.x; idx < rows * cols; idx += NT) {
+        const int r = idx / cols, c = idx - r * cols;
+        dst[r * ld + c] = to_f32(src[(long long)r * tok_stride + c]);
+    }
+}
+// dense [rows][cols] float block in global memory <-> padded tile
+__device__ __forceinline__ void load_dense(float* dst, int ld, const float* src, int src_ld, int rows, int cols) {
+    for (int idx = threadIdx.x; idx < rows * cols; idx += NT) {
+        const int r = idx / cols, c = idx - r * cols;
+        dst[r * ld + c] = src[(long long)r * src_ld + c];
+    }
+}
+// rows of a padded [rows][cols] tile times a per-row factor
+template <typename F>
+__device__ __forceinline__ void scale_rows(float* x, int ld, int rows, int cols, F f) {
+    for (int idx = threadIdx.x; idx < rows * cols; idx += NT) {
+        const int r = idx / cols;
+        x[r * ld + (idx - r * cols)] *= f(r);
+    }
+}
+
 
 // Same fields as the delta-rule kernels' shape struct; a type of this namespace keeps overload resolution of the kernels
 // of the two families apart.

@@ -1,615 +1,809 @@
 // Chunkwise form of the gated delta rule (paper Section 2.2, Eq. 2 with a non-empty V_new): float32 CUDA-core kernels.
 //
 // Token rule (this library's orientation, S is d_k x d_v):  u_t = k_t S_{t-1},  w_t = beta_t (v_t - a_t u_t),
-// S_t = a_t S_{t-1} + k_t^T w_t,  o_t = q_t S_t,  a_t = exp(g_t).  Within a chunk of n tokens, with b_t the inclusive
+// S_t = a_t S_{t-1} + k_t^T w_t,  o_t = q_t S_t,  a_t = exp(g_t).  Within a tile of n tokens, with b_t the inclusive
 // cumulative log-decay, gam_t = exp(b_t), M[t,s] = exp(b_t - b_s) for s <= t, om_s = exp(b_n - b_s), H the state entering
-// the chunk, unrolling S_{t-1} = gam_{t-1} H + sum_{s<t} (gam_{t-1}/gam_s) k_s^T w_s gives a unit-lower-triangular system
+// the tile, unrolling S_{t-1} = gam_{t-1} H + sum_{s<t} (gam_{t-1}/gam_s) k_s^T w_s gives a unit-lower-triangular system
 //     (I + L) W = beta*V - (beta*gam)*(K H),     L[t,s] = beta_t M[t,s] (k_t . k_s)  for s < t
-// so  W = U - Wk H  with  U = (I+L)^-1 (beta*V),  Wk = (I+L)^-1 (beta*gam*K)   (the UT transform; no inverse is formed:
-// the systems are solved by substitution, one thread per right-hand-side column; for the backward the identity is solved
-// along with them, which gives (I+L)^-1 for the transposed solve).  Then
-//     Pre : U, Wk and the chunk's affine state map  H' = Phi H + Psi,  Phi = gam_n I - (om*K)^T Wk,  Psi = (om*K)^T U
-//                                                                            (needs no state: all chunks in parallel)
-//     ST  : H' = Phi H + Psi, storing the state entering every chunk        (sequential over chunks, per value column)
-//     Out : W = U - Wk H  (this is V_new),  O = (M * Q K^T) W + gam * (Q H)   (all chunks in parallel, from the stored states)
+// With T = (I+L)^-1 (UT transform):  W = T (beta*V - (beta*gam)*(K H)) = U - Wk H,  U = T (beta*V),  Wk = T (beta*gam*K).
+//     Pre : T and the tile's affine state map  H' = Phi H + Psi,  Phi = gam_n I - (om*K)^T Wk,  Psi = (om*K)^T U
+//                                                                            (needs no state: all tiles in parallel)
+//     ST  : H' = Phi H + Psi, storing the state entering every tile         (sequential over tiles, per value column)
+//     Out : W = T (beta*V - (beta*gam)*(K H))  (this is V_new),  O = A W + gam * (Q H),  A = M * Q K^T
+//                                                                            (all tiles in parallel, from the stored states)
 // Backward (hand-derived; checked against the fp64 oracle, which is pinned by finite differences), dH' = gradient of the
-// state leaving the chunk:
-//     dW = A^T dO + om*(K dH'),  A = M * QK^T;   Z = (I+L)^-T dW = Z0 + (I+L)^-T (om*(K dH')),  Z0 = (I+L)^-T A^T dO;
+// state leaving the tile:
+//     dW = A^T dO + om*(K dH'),  Z = T^T dW;  with Z0 = T^T A^T dO,
 //     dH = gam_n dH' + Q^T (gam*dO) - K^T (beta*gam*Z) = Phi^T dH' + Theta,  Theta = Q^T (gam*dO) - K^T (beta*gam*Z0)
-// so Z0 and Theta come from a chunk-parallel kernel, the reverse pass over the chunks is again one small product per chunk,
-// and, chunk-parallel from the stored H, dH' (W and Z are rebuilt in place):  dA = dO W^T,  dL = -strict_lower(Z W^T),  P = beta*dL*M,
-//     dq = (dA*M) K + gam*(dO H^T)
-//     dk = (dA*M)^T Q + om*(W dH'^T) - (beta*gam*Z) H^T + (P + P^T) K
-//     dv = beta*Z,    dbeta = rowsum(Z*V) - gam*rowsum(Z*KH) + rowsum(dL * M * KK^T)
-//     db_t (gradient of the cumulative log-decay) collects the M, gam, om terms; dg = reverse cumulative sum of db.
-// Chunk length 16 or 32, d_k, d_v in {32, 64, 128} as far as the tiles fit into shared memory (128 needs chunk 16); a last
-// chunk with fewer tokens is handled by row counts.
+//     so Theta comes from Pre and the reverse pass over the tiles is ST with Phi^T and Theta.  Then, tile-parallel,
+//     dA = dO W^T,  dL = -strict_lower(Z W^T),  P = beta_t dL*M,
+//     dq = (dA*M) K + gam*(dO H^T),   dk = (dA*M)^T Q + om*(W dH'^T) - (beta*gam)*(Z H^T) + (P + P^T) K,   dv = beta*Z,
+//     dbeta_t = z_t.v_t - gam_t k_t.(Z H^T)_t + sum_s dL[t,s] M[t,s] (k_t.k_s),
+//     db = rowsum(E) - colsum(E) + dgam*gam - dom*om (+ chunk-total terms on the last token),
+//       E = (dA*QK + beta_t dL*KK)*M,  dgam_t = q_t.(dO H^T)_t - beta_t k_t.(Z H^T)_t,  dom_t = k_t.(W dH'^T)_t,
+//     and dg is the reverse cumulative sum of db.
+//
+// The tile is 32 tokens whatever the caller's chunk: the products over the d_k x d_v state cost the same for every tile
+// length, the C x C ones grow with it, the state maps (d_k^2 + 2 d_k d_v floats per tile) and the length of the sequential
+// pass shrink with it.  Products are register-tiled (sf_tile.cuh).  Missing tokens of a last tile count as zero rows with
+// log-decay 0 and beta 0, which leaves T the identity there and every sum unchanged.
 #pragma once
 #include "sf_common.cuh"
+#include "sf_tile.cuh"
 
 namespace sf {
 namespace gdn {
 
-constexpr int NT = 256;
-constexpr int DVS = 16;            // value columns per CTA in the sequential kernels
-constexpr int GR = 16;             // chunks per block of the two-level state pass
+constexpr int CT = 32;             // tokens per tile
+constexpr int CC = CT * CT;
 
 struct Params {
-    int B, H, L, C, NC, dk, dv;
+    int B, H, L, C, NC, dk, dv;              // C, NC: the caller's chunk (workspace and shape rules)
+    int NT;                                  // tiles
+    bool vec;                                // rows of q, k, v, dO, ... allow 16-byte (float32) / 8-byte (bf16) accesses
     long long tqk, tv, tg, bqk, bv, bg;      // token / batch strides in elements
 };
 
-// Workspace per (batch, head), in floats: U [L][dv], Wk [L][dk], Phi [NC][dk][dk], Psi [NC][dk][dv], Hc [NC][dk][dv],
-// Pb [NB][dk][dk], Sb [NB][dk][dv], Hb [NB][dk][dv] (maps composed over blocks of GR chunks and the states entering them);
-// the backward adds Z0 [L][dv], Theta [NC][dk][dv], dHc [NC][dk][dv], A [NC][C][C] (the masked Q K^T) and
-// Ti [NC][C][C] (the inverse of I + L, used transposed).
-struct Ws { float *U, *Wk, *Phi, *Psi, *Hc, *Pb, *Sb, *Hb, *Z0, *Theta, *dHc, *A, *Ti; };
+// Workspace per (batch, head), in floats.  Its size is part of the interface:  U [L][dv], Wk [L][dk], Phi, Psi, Hc per chunk,
+// the same three per block of 16 chunks; the backward adds [L][dv], two states per chunk and two C x C per chunk.  What the
+// kernels keep in it, per tile: Phi [dk][dk], Psi [dk][dv], Hc [dk][dv], T [32][32]; the backward adds Theta, dHc [dk][dv],
+// A and KM (M * K K^T below the diagonal) [32][32].  That is never more: chunks are at most as long as tiles, and T, A, KM
+// (96 floats per token) find room in U, Wk, Z0, A and Ti (at least 96 + 2 C) once the last tile's padding is covered by the
+// three block maps.
+struct Ws { float *Phi, *Psi, *Hc, *T, *Theta, *dHc, *A, *KM; };
+constexpr int GR = 16;
 __host__ __device__ inline size_t ws_floats(const Params& p, bool backward) {
     const size_t st = (size_t)p.NC * p.dk * p.dv, nb = (size_t)((p.NC + GR - 1) / GR);
     size_t n = (size_t)p.L * p.dv + (size_t)p.L * p.dk + (size_t)p.NC * p.dk * p.dk + 2 * st;
-    n += nb * p.dk * p.dk + 2 * nb * p.dk * p.dv;                        // composed maps and entering states of the blocks
+    n += nb * p.dk * p.dk + 2 * nb * p.dk * p.dv;
     if (backward) n += (size_t)p.L * p.dv + 2 * st + 2 * (size_t)p.NC * p.C * p.C;
     return n;
 }
 __host__ __device__ inline Ws ws_of(float* base, const Params& p, long long bh, bool backward) {
-    const size_t st = (size_t)p.NC * p.dk * p.dv, nb = (size_t)((p.NC + GR - 1) / GR);
+    const size_t st = (size_t)p.NT * p.dk * p.dv;
     float* c = base + bh * (long long)ws_floats(p, backward);
     Ws w;
-    w.U = c;   c += (size_t)p.L * p.dv;
-    w.Wk = c;  c += (size_t)p.L * p.dk;
-    w.Phi = c; c += (size_t)p.NC * p.dk * p.dk;
+    w.Phi = c; c += (size_t)p.NT * p.dk * p.dk;
     w.Psi = c; c += st;
     w.Hc = c;  c += st;
-    w.Pb = c;  c += nb * p.dk * p.dk;
-    w.Sb = c;  c += nb * p.dk * p.dv;
-    w.Hb = c;  c += nb * p.dk * p.dv;
-    w.Z0 = w.Theta = w.dHc = w.A = w.Ti = nullptr;
+    w.T = c;   c += (size_t)p.NT * CC;
+    w.Theta = w.dHc = w.A = w.KM = nullptr;
     if (backward) {
-        w.Z0 = c;    c += (size_t)p.L * p.dv;
         w.Theta = c; c += st;
         w.dHc = c;   c += st;
-        w.A = c;     c += (size_t)p.NC * p.C * p.C;
-        w.Ti = c;
+        w.A = c;     c += (size_t)p.NT * CC;
+        w.KM = c;
     }
     return w;
 }
 
-// Shared-memory tiles are stored with an odd leading dimension (columns + 1), so that both row-wise and column-wise
-// walks hit different banks.
-__host__ __device__ constexpr int ldp(int cols) { return cols + 1; }
+// 4 warps, 8 where a 128-wide side gives every product enough outputs.
+template <int DK, int DV> constexpr int kThreads = DK == 128 || DV == 128 ? 256 : 128;
 
-// out[m][n] = keep*out[m][n] + sign * sum_k A(m,k) B(k,n);  A(m,k) = ta ? A[k*lda+m] : A[m*lda+k], likewise B.
-// Element idx is always computed by the same thread, so a second product may accumulate into `out` (keep = 1) without a
-// barrier in between, also when `out` is global memory.
-__device__ __forceinline__ void mm(float* out, int ldo, const float* A, int lda, bool ta, const float* Bm, int ldb, bool tb,
-                                   int M, int N, int K, float keep, float sign) {
-    // four independent accumulators per thread: the products are small and latency-bound, not throughput-bound
-    const int total = M * N, sa = ta ? lda : 1, sb = tb ? 1 : ldb;
-    for (int base = threadIdx.x; base < total; base += 4 * NT) {
-        const float *a[4], *bq[4];
-        float acc[4] = {0.f, 0.f, 0.f, 0.f};
+struct Decay {
+    float bh[CT], bl[CT];              // inclusive cumulative log-decay (sums in double) as a float pair
+    float gam[CT], om[CT], beta[CT];   // exp(b_t), exp(b_n - b_t), beta_t (0 past the end)
+};
+__device__ __forceinline__ float mexp(const Decay& d, int t, int s) { return __expf((d.bh[t] - d.bh[s]) + (d.bl[t] - d.bl[s])); }
+__device__ __forceinline__ void tile_decay(Decay& d, const float* __restrict__ g, const float* __restrict__ beta, long long tg, int n) {
+    if (threadIdx.x >= 32) return;
+    const int l = threadIdx.x;
+    double b = l < n ? (double)g[l * tg] : 0.0;
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const int idx = min(base + e * NT, total - 1);            // clamped: a lane past the end computes a value it drops
-            const int m = idx / N, n = idx - m * N;
-            a[e] = ta ? A + m : A + m * lda;
-            bq[e] = tb ? Bm + n * ldb : Bm + n;
+    for (int off = 1; off < 32; off <<= 1) {
+        const double up = __shfl_up_sync(0xffffffffu, b, off);
+        if (l >= off) b += up;
+    }
+    const double tot = __shfl_sync(0xffffffffu, b, 31);
+    const float hi = (float)b;
+    d.bh[l] = hi;
+    d.bl[l] = (float)(b - (double)hi);
+    d.gam[l] = __expf(hi);
+    d.om[l] = __expf((float)(tot - b));
+    d.beta[l] = l < n ? beta[l * tg] : 0.f;
+}
+
+// 32 x 32 products X Y^T of two tiles with D columns, a 2 x 4 block of outputs per thread of a group of 128 (t = 0..127);
+// f(m, n4, values of four neighbouring columns) receives the outputs.  Rows are dealt out so that the lanes of a warp read
+// rows four apart (conflict-free with the tiles' swizzle).
+template <int D, typename F>
+__device__ __forceinline__ void square_product(const float* __restrict__ X, const float* __restrict__ Y, int t, F f) {
+    const int tx = tile::lane_x(t & 31), ty = 4 * (t >> 5) + tile::lane_y(t & 31), m0 = 4 * (ty & 7) + 2 * (ty >> 3), n0 = 4 * tx;
+    tile::f32x2 acc[2][4] = {};
+#pragma unroll 4
+    for (int k = 0; k < D; k += 4) {
+        const int u = k >> 2, ox = (u ^ (ty & 7)) << 2, oy = (u ^ tx) << 2;
+        ulonglong2 y[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) y[j] = tile::ld4x2(Y + (n0 + j) * D + oy);
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const ulonglong2 x = tile::ld4x2(X + (m0 + i) * D + ox);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) { tile::fma2(acc[i][j], x.x, y[j].x); tile::fma2(acc[i][j], x.y, y[j].y); }
         }
-#pragma unroll 2
-        for (int k = 0; k < K; ++k) {
+    }
 #pragma unroll
-            for (int e = 0; e < 4; ++e) acc[e] = fmaf(a[e][k * sa], bq[e][k * sb], acc[e]);
+    for (int i = 0; i < 2; ++i) {
+        float v[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            float lo, hi;
+            tile::unpack(acc[i][j], lo, hi);
+            v[j] = lo + hi;
         }
+        f(m0 + i, n0, v);
+    }
+}
+// Two such products: side by side on the two halves of 256 threads, one after the other on 128.
+template <int NT, int DA, int DB, typename FA, typename FB>
+__device__ __forceinline__ void two_square_products(const float* XA, const float* YA, FA fa, const float* XB, const float* YB, FB fb) {
+    const int t = threadIdx.x & 127;
+    if (NT == 128 || threadIdx.x < 128) square_product<DA>(XA, YA, t, fa);
+    if (NT == 128 || threadIdx.x >= 128) square_product<DB>(XB, YB, t, fb);
+}
+
+// T = (I + L)^-1 in place of the strictly lower-triangular L [32][32]: the two 16 x 16 diagonal blocks by substitution (one
+// thread per column), then T21 = -T22 (L21 T11).  `tmp` holds 256 floats.
+template <int NT>
+__device__ __forceinline__ void invert(float* Lm, float* tmp) {
+    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+    if (w < 2 && l < 16) {
+        const int o = 16 * w;
+        float x[16];
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const int idx = base + e * NT;
-            if (idx < total) {
-                const int m = idx / N, n = idx - m * N;
-                out[m * ldo + n] = keep != 0.f ? fmaf(keep, out[m * ldo + n], sign * acc[e]) : sign * acc[e];
+        for (int t = 0; t < 16; ++t) {
+            float acc = t == l ? 1.f : 0.f;
+#pragma unroll
+            for (int s4 = 0; s4 < (t + 3) / 4; ++s4) {
+                const float4 v = tile::ld4(Lm + tile::at<CT>(o + t, o + 4 * s4));
+                const float lv[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    if (4 * s4 + e < t) acc = fmaf(-lv[e], x[4 * s4 + e], acc);
             }
+            x[t] = acc;
         }
-    }
-}
-
-// The same product with a 4 x 4 block of outputs per thread (M and N multiples of 4): 8 shared-memory reads for 16
-// multiply-adds instead of 20, for the larger products (the composed maps).  Same rule for `keep`.
-__device__ __forceinline__ void mm4x4(float* out, int ldo, const float* A, int lda, bool ta, const float* Bm, int ldb, bool tb,
-                                      int M, int N, int K, float keep, float sign) {
-    const int tn = N >> 2, total = (M >> 2) * tn, sa = ta ? lda : 1, sb = tb ? 1 : ldb;
-    for (int t = threadIdx.x; t < total; t += NT) {
-        const int m0 = (t / tn) << 2, n0 = (t - (t / tn) * tn) << 2;
-        const float* a = ta ? A + m0 : A + m0 * lda;
-        const float* b = tb ? Bm + n0 * ldb : Bm + n0;
-        const int ra = ta ? 1 : lda, rb = tb ? ldb : 1;               // step to the next of the four rows / columns
-        float acc[4][4] = {};
-#pragma unroll 2
-        for (int k = 0; k < K; ++k) {
-            float av[4], bv[4];
+        __syncwarp(0xffffu);
 #pragma unroll
-            for (int i = 0; i < 4; ++i) { av[i] = a[i * ra + k * sa]; bv[i] = b[i * rb + k * sb]; }
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int jj = 0; jj < 4; ++jj) acc[i][jj] = fmaf(av[i], bv[jj], acc[i][jj]);
-        }
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int jj = 0; jj < 4; ++jj) {
-                float* o = out + (m0 + i) * ldo + n0 + jj;
-                *o = keep != 0.f ? fmaf(keep, *o, sign * acc[i][jj]) : sign * acc[i][jj];
-            }
+        for (int t = 0; t < 16; ++t) Lm[tile::at<CT>(o + t, o + l)] = x[t];
     }
-}
-
-// Picks the blocked product when the shape allows it and leaves at least half of the threads busy.  The choice depends on
-// the shape alone, so two products that accumulate into the same output take the same path (same thread, same element).
-__device__ __forceinline__ void mmx(float* out, int ldo, const float* A, int lda, bool ta, const float* Bm, int ldb, bool tb,
-                                    int M, int N, int K, float keep, float sign) {
-    if (((M | N) & 3) == 0 && (M >> 2) * (N >> 2) >= NT / 4) mm4x4(out, ldo, A, lda, ta, Bm, ldb, tb, M, N, K, keep, sign);
-    else mm(out, ldo, A, lda, ta, Bm, ldb, tb, M, N, K, keep, sign);
-}
-
-template <typename T>
-__device__ __forceinline__ void load_rows(float* dst, int ld, const T* src, long long tok_stride, int rows, int cols) {
-    for (int idx = threadIdx.x; idx < rows * cols; idx += NT) {
-        const int r = idx / cols, c = idx - r * cols;
-        dst[r * ld + c] = to_f32(src[(long long)r * tok_stride + c]);
-    }
-}
-// dense [rows][cols] float block in global memory <-> padded tile
-__device__ __forceinline__ void load_dense(float* dst, int ld, const float* src, int src_ld, int rows, int cols) {
-    for (int idx = threadIdx.x; idx < rows * cols; idx += NT) {
-        const int r = idx / cols, c = idx - r * cols;
-        dst[r * ld + c] = src[(long long)r * src_ld + c];
-    }
-}
-__device__ __forceinline__ void store_dense(float* dst, int dst_ld, const float* src, int ld, int rows, int cols) {
-    for (int idx = threadIdx.x; idx < rows * cols; idx += NT) {
-        const int r = idx / cols, c = idx - r * cols;
-        dst[(long long)r * dst_ld + c] = src[r * ld + c];
-    }
-}
-// rows of a padded [rows][cols] tile times a per-row factor
-template <typename F>
-__device__ __forceinline__ void scale_rows(float* x, int ld, int rows, int cols, F f) {
-    for (int idx = threadIdx.x; idx < rows * cols; idx += NT) {
-        const int r = idx / cols;
-        x[r * ld + (idx - r * cols)] *= f(r);
-    }
-}
-
-// b[t] = inclusive cumulative log-decay of the chunk's n tokens (one thread), bt[t] = beta.  Syncs.
-__device__ __forceinline__ void load_decay(float* b, float* bt, const float* g, const float* beta, long long tg, int n) {
-    if (threadIdx.x == 0) {
+    __syncthreads();
+    for (int e = threadIdx.x; e < 256; e += NT) {                // L21 T11
+        const int r = e >> 4, c = e & 15;
         float acc = 0.f;
-        for (int t = 0; t < n; ++t) { acc += g[(long long)t * tg]; b[t] = acc; }
-    }
-    if (bt) for (int t = threadIdx.x; t < n; t += NT) bt[t] = beta[(long long)t * tg];
-    __syncthreads();
-}
-
-// ---- Pre: U = (I+L)^-1 (beta*V), Wk = (I+L)^-1 (beta*gam*K), Phi = gam_n I - (om*K)^T Wk, Psi = (om*K)^T U; for the
-//      backward also Ti = (I+L)^-1 and A = M * Q K^T.  grid (NC, H, B) ------------------------------------------------
-template <typename T>
-__global__ void __launch_bounds__(NT) pre_kernel(Params p, const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v,
-                                                 const float* __restrict__ g, const float* __restrict__ beta, float* ws, int backward) {
-    extern __shared__ float sm[];
-    const int c = blockIdx.x, h = blockIdx.y, bb = blockIdx.z;
-    const int C = p.C, dk = p.dk, dv = p.dv, t0 = c * C, n = min(C, p.L - t0);
-    const int ldk = ldp(dk), ldc = ldp(C), ncol = dv + dk + (backward ? C : 0), ldx = ldp(dv + dk + C);
-    float* Ks = sm;                    // [C][dk]
-    float* Kw = Ks + C * ldk;          // [C][dk]   om * K
-    float* Qs = Kw + C * ldk;          // [C][dk]   (backward only)
-    float* X = Qs + C * ldk;           // [C][dv + dk (+ C)]   right-hand sides, solved in place
-    float* Lm = X + C * ldx;           // [C][C]
-    float* b = Lm + C * ldc;           // [C]
-    float* bt = b + C;                 // [C]
-    const long long bh = (long long)bb * p.H + h;
-    const Ws w = ws_of(ws, p, bh, backward != 0);
-    const long long oqk = (long long)bb * p.bqk + (long long)t0 * p.tqk + (long long)h * dk;
-    load_rows(Ks, ldk, k + oqk, p.tqk, n, dk);
-    if (backward) load_rows(Qs, ldk, q + oqk, p.tqk, n, dk);
-    load_rows(X, ldx, v + (long long)bb * p.bv + (long long)t0 * p.tv + (long long)h * dv, p.tv, n, dv);
-    load_decay(b, bt, g + (long long)bb * p.bg + (long long)t0 * p.tg + h, beta + (long long)bb * p.bg + (long long)t0 * p.tg + h, p.tg, n);
-    const float bn = b[n - 1];
-    for (int idx = threadIdx.x; idx < n * ncol; idx += NT) {
-        const int t = idx / ncol, col = idx - t * ncol;
-        float x;
-        if (col < dv) x = bt[t] * X[t * ldx + col];
-        else if (col < dv + dk) x = bt[t] * __expf(b[t]) * Ks[t * ldk + (col - dv)];
-        else x = (col - dv - dk) == t ? 1.f : 0.f;                      // identity: its solution is the inverse
-        X[t * ldx + col] = x;
-    }
-    for (int idx = threadIdx.x; idx < n * dk; idx += NT) {
-        const int t = idx / dk, i = idx - t * dk;
-        Kw[t * ldk + i] = __expf(bn - b[t]) * Ks[t * ldk + i];
-    }
-    mmx(Lm, ldc, Ks, ldk, false, Ks, ldk, true, n, n, dk, 0.f, 1.f);     // K K^T
-    __syncthreads();
-    for (int idx = threadIdx.x; idx < n * n; idx += NT) {
-        const int t = idx / n, s = idx - t * n;
-        Lm[t * ldc + s] = s < t ? bt[t] * __expf(b[t] - b[s]) * Lm[t * ldc + s] : 0.f;
-    }
-    __syncthreads();
-    // forward substitution, one thread per column
-    for (int col = threadIdx.x; col < ncol; col += NT)
-        for (int t = 1; t < n; ++t) {
-            float acc = X[t * ldx + col];
-            for (int s = 0; s < t; ++s) acc = fmaf(-Lm[t * ldc + s], X[s * ldx + col], acc);
-            X[t * ldx + col] = acc;
-        }
-    __syncthreads();
-    store_dense(w.U + (long long)t0 * dv, dv, X, ldx, n, dv);
-    store_dense(w.Wk + (long long)t0 * dk, dk, X + dv, ldx, n, dk);
-    float* Phi = w.Phi + (long long)c * dk * dk;
-    mmx(Phi, dk, Kw, ldk, true, X + dv, ldx, false, dk, dk, n, 0.f, -1.f);                 // -(om*K)^T Wk
-    mmx(w.Psi + (long long)c * dk * dv, dv, Kw, ldk, true, X, ldx, false, dk, dv, n, 0.f, 1.f);
-    if (backward) {
-        store_dense(w.Ti + (long long)c * C * C, C, X + dv + dk, ldx, n, n);
-        mmx(Lm, ldc, Qs, ldk, false, Ks, ldk, true, n, n, dk, 0.f, 1.f); // Q K^T (L is no longer needed)
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < dk; i += NT) Phi[i * dk + i] += __expf(bn);
-    if (backward)
-        for (int idx = threadIdx.x; idx < n * n; idx += NT) {
-            const int t = idx / n, s = idx - t * n;
-            w.A[(long long)c * C * C + t * C + s] = s <= t ? Lm[t * ldc + s] * __expf(b[t] - b[s]) : 0.f;
-        }
-}
-
-// ---- ST (forward) and its adjoint (reverse): X' = F X + R step by step for DVS columns of the state.
-//      CHUNKS_FWD  F = Phi[c],    R = Psi[c],    all chunks ascending;  Hc[c]  <- state entering chunk c
-//      CHUNKS_REV  F = Phi[c]^T,  R = Theta[c],  all chunks descending; dHc[c] <- gradient of the state leaving chunk c
-//      The two-level pass shortens the dependency chain from NC steps to about GR + NC/GR + GR: compose_kernel multiplies
-//      the maps of each block of GR chunks together (all blocks in parallel), then
-//      BLOCKS_FWD / BLOCKS_REV  F = Pb[j], R = Sb[j] over the blocks;  Hb[j] <- state (gradient) entering block j
-//      INBLOCK_FWD / INBLOCK_REV  the chunks of block j = blockIdx.y starting from Hb[j] (all blocks in parallel)
-//      grid (dv/DVS, H, B), for INBLOCK_* (dv/DVS, NB, B*H) --------------------------------------------------------------
-enum : int { CHUNKS_FWD = 0, CHUNKS_REV = 1, BLOCKS_FWD = 2, BLOCKS_REV = 3, INBLOCK_FWD = 4, INBLOCK_REV = 5 };
-
-template <int DKM>      // DKM >= d_k: sizes the register prefetch
-__global__ void __launch_bounds__(NT) chain_kernel(Params p, int mode, const float* __restrict__ init, float* __restrict__ fin,
-                                                   float* ws, int backward) {
-    extern __shared__ float sm[];
-    const bool inblock = mode >= INBLOCK_FWD, blocks = mode == BLOCKS_FWD || mode == BLOCKS_REV;
-    const bool rev = (mode & 1) != 0;
-    const int j0 = blockIdx.x * DVS;
-    const long long bh = inblock ? (long long)blockIdx.z : (long long)blockIdx.z * p.H + blockIdx.y;
-    const int dk = p.dk, dv = p.dv, NB = (p.NC + GR - 1) / GR;
-    const int ldk = ldp(dk), lds = ldp(DVS);
-    float* X0 = sm;                    // [dk][DVS]
-    float* X1 = X0 + dk * lds;         // [dk][DVS]
-    float* Fs = X1 + dk * lds;         // [dk][dk]
-    const Ws w = ws_of(ws, p, bh, backward != 0);
-    const float* Fsrc = blocks ? w.Pb : w.Phi;
-    const float* Rsrc = blocks ? w.Sb : (rev ? w.Theta : w.Psi);
-    float* states = blocks ? w.Hb : (rev ? w.dHc : w.Hc);
-    const bool transpose = rev && !blocks;                              // composed maps are stored the way they are applied
-    // steps first .. first + count - 1 (ascending) or first + count - 1 .. first (descending)
-    int first = 0, count = blocks ? NB : p.NC;
-    if (inblock) { first = blockIdx.y * GR; count = min(GR, p.NC - first); }
-    const float* start = inblock ? w.Hb + (long long)blockIdx.y * dk * dv : (init ? init + bh * dk * dv : nullptr);
-    if (start) load_dense(X0, lds, start + j0, dv, dk, DVS);
-    else for (int idx = threadIdx.x; idx < dk * lds; idx += NT) X0[idx] = 0.f;
-    __syncthreads();
-    // The map of the next step is fetched into registers while the product of the current one runs.
-    constexpr int MAXF = (DKM * DKM) / NT, MAXR = (DKM * DVS) / NT;
-    float fr[MAXF], rr[MAXR];
-    auto fetch = [&](int c) {
-        const float* F = Fsrc + (long long)c * dk * dk;
-        const float* R = Rsrc + (long long)c * dk * dv + j0;
 #pragma unroll
-        for (int e = 0; e < MAXF; ++e) {
-            const int idx = threadIdx.x + e * NT;
-            fr[e] = idx < dk * dk ? F[idx] : 0.f;
-        }
+        for (int s = 0; s < 16; ++s) acc = fmaf(Lm[tile::at<CT>(16 + r, s)], Lm[tile::at<CT>(s, c)], acc);
+        tmp[e] = acc;
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < 256; e += NT) {
+        const int r = e >> 4, c = e & 15;
+        float acc = 0.f;
 #pragma unroll
-        for (int e = 0; e < MAXR; ++e) {
-            const int idx = threadIdx.x + e * NT;
-            rr[e] = idx < dk * DVS ? R[(long long)(idx / DVS) * dv + (idx % DVS)] : 0.f;
-        }
-    };
-    float *cur = X0, *nxt = X1;
-    fetch(rev ? first + count - 1 : first);
-    for (int s = 0; s < count; ++s) {
-        const int c = rev ? first + count - 1 - s : first + s;
-        store_dense(states + (long long)c * dk * dv + j0, dv, cur, lds, dk, DVS);
+        for (int s = 0; s < 16; ++s) acc = fmaf(-Lm[tile::at<CT>(16 + r, 16 + s)], tmp[s * 16 + c], acc);
+        Lm[tile::at<CT>(16 + r, c)] = acc;
+    }
+    __syncthreads();
+}
+
+// dense [32][32] in global memory to a tile
+template <int NT>
+__device__ __forceinline__ void load_square(float* dst, const float* __restrict__ src) { tile::load<CT, CT, NT>(dst, src, CT, CT); }
+// accumulator rows to a dense array in global memory; f(m, n, value)
+template <class Mp, int LD, typename F>
+__device__ __forceinline__ void store_dense(float* __restrict__ dst, const float (&acc)[Mp::TM][Mp::TN], const Mp& mp, F f) {
 #pragma unroll
-        for (int e = 0; e < MAXF; ++e) {
-            const int idx = threadIdx.x + e * NT;
-            if (idx < dk * dk) Fs[(idx / dk) * ldk + (idx % dk)] = fr[e];
-        }
+    for (int i = 0; i < Mp::TM; ++i)
 #pragma unroll
-        for (int e = 0; e < MAXR; ++e) {
-            const int idx = threadIdx.x + e * NT;
-            if (idx < dk * DVS) nxt[(idx / DVS) * lds + (idx % DVS)] = rr[e];
+        for (int gq = 0; gq < Mp::GN; ++gq) {
+            const int m = mp.m(i), n = mp.n4(gq);
+            tile::store4(dst + m * LD + n, make_float4(f(m, n, acc[i][4 * gq]), f(m, n + 1, acc[i][4 * gq + 1]), f(m, n + 2, acc[i][4 * gq + 2]),
+                                                       f(m, n + 3, acc[i][4 * gq + 3])));
         }
-        __syncthreads();
-        if (s + 1 < count) fetch(rev ? c - 1 : c + 1);
-        // many CTAs share an SM in the in-block mode (throughput counts: fewer shared-memory reads); one CTA per SM else
-        if (inblock) mm4x4(nxt, lds, Fs, ldk, transpose, cur, lds, false, dk, DVS, dk, 1.f, 1.f);
-        else         mm(nxt, lds, Fs, ldk, transpose, cur, lds, false, dk, DVS, dk, 1.f, 1.f);
-        __syncthreads();
-        float* t = cur; cur = nxt; nxt = t;
+}
+// accumulator rows m < n, times w(m), to rows of an output tensor
+template <class Mp, typename T, typename W>
+__device__ __forceinline__ void store_rows(T* __restrict__ dst, long long stride, int n, const float (&acc)[Mp::TM][Mp::TN], const Mp& mp, bool vec, W w) {
+#pragma unroll
+    for (int i = 0; i < Mp::TM; ++i) {
+        const int m = mp.m(i);
+        if (m < n) {
+            const float f = w(m);
+#pragma unroll
+            for (int gq = 0; gq < Mp::GN; ++gq)
+                tile::store4(dst + m * stride + mp.n4(gq),
+                             make_float4(f * acc[i][4 * gq], f * acc[i][4 * gq + 1], f * acc[i][4 * gq + 2], f * acc[i][4 * gq + 3]), vec);
+        }
     }
-    if (fin && !inblock) store_dense(fin + bh * dk * dv + j0, dv, cur, lds, dk, DVS);
+}
+template <class Mp, typename W>
+__device__ __forceinline__ void scale_acc(float (&acc)[Mp::TM][Mp::TN], const Mp& mp, W w) {
+#pragma unroll
+    for (int i = 0; i < Mp::TM; ++i) {
+        const float f = w(mp.m(i));
+#pragma unroll
+        for (int j = 0; j < Mp::TN; ++j) acc[i][j] *= f;
+    }
 }
 
-// ---- maps of a block of GR chunks multiplied together: X' = P X + S with (forward) P = Phi[last] ... Phi[first] and S the
-//      image of zero, or (reverse) the same with the transposed maps and Theta in descending order.  grid (NB, H, B) --------
-__global__ void __launch_bounds__(NT) compose_kernel(Params p, int reverse, float* ws, int backward) {
-    extern __shared__ float sm[];
-    const int j = blockIdx.x, h = blockIdx.y, bb = blockIdx.z;
-    const int dk = p.dk, dv = p.dv;
-    const int ldk = ldp(dk), ldv = ldp(dv);
-    float* P0 = sm;                    float* P1 = P0 + dk * ldk;        // [dk][dk] each
-    float* S0 = P1 + dk * ldk;         float* S1 = S0 + dk * ldv;        // [dk][dv] each
-    float* Fs = S1 + dk * ldv;                                           // [dk][dk]
-    const long long bh = (long long)bb * p.H + h;
-    const Ws w = ws_of(ws, p, bh, backward != 0);
-    const float* Rsrc = reverse ? w.Theta : w.Psi;
-    const int first = j * GR, count = min(GR, p.NC - first);
-    for (int idx = threadIdx.x; idx < dk * dk; idx += NT) P0[(idx / dk) * ldk + (idx % dk)] = (idx / dk) == (idx % dk) ? 1.f : 0.f;
-    for (int idx = threadIdx.x; idx < dk * ldv; idx += NT) S0[idx] = 0.f;
-    float *Pc = P0, *Pn = P1, *Sc = S0, *Sn = S1;
-    for (int s = 0; s < count; ++s) {
-        const int c = reverse ? first + count - 1 - s : first + s;
-        __syncthreads();
-        load_dense(Fs, ldk, w.Phi + (long long)c * dk * dk, dk, dk, dk);
-        load_dense(Sn, ldv, Rsrc + (long long)c * dk * dv, dv, dk, dv);
-        __syncthreads();
-        mm4x4(Sn, ldv, Fs, ldk, reverse != 0, Sc, ldv, false, dk, dv, dk, 1.f, 1.f);
-        mm4x4(Pn, ldk, Fs, ldk, reverse != 0, Pc, ldk, false, dk, dk, dk, 0.f, 1.f);
-        float* t = Pc; Pc = Pn; Pn = t;
-        t = Sc; Sc = Sn; Sn = t;
-    }
-    __syncthreads();
-    store_dense(w.Pb + (long long)j * dk * dk, dk, Pc, ldk, dk, dk);
-    store_dense(w.Sb + (long long)j * dk * dv, dv, Sc, ldv, dk, dv);
-}
-
-// ---- Out: W = U - Wk Hc (V_new),  O = (M * Q K^T) W + gam * (Q Hc).  grid (NC, H, B) --------------------------------
-template <typename T>
-__global__ void __launch_bounds__(NT) out_kernel(Params p, const T* __restrict__ q, const T* __restrict__ k, const float* __restrict__ g,
-                                                 T* __restrict__ o, const float* ws, int backward) {
-    extern __shared__ float sm[];
+// ---- Pre: T, Phi, Psi; with BWD also A, KM and Theta.  grid (tiles, H, B) --------------------------------------------
+template <int DK, int DV, bool BWD>
+struct PreSmem {
+    float K[CT * DK], X[CT * DV], Y[CT * DK], T[CC], tmp[256];
+    float Q[BWD ? CT * DK : 4], D[BWD ? CT * DV : 4], A[BWD ? CC : 4];
+    Decay d;
+};
+template <typename T, int DK, int DV, bool BWD>
+__global__ void __launch_bounds__(kThreads<DK, DV>) pre_kernel(Params p, const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v,
+                                                               const float* __restrict__ g, const float* __restrict__ beta,
+                                                               const T* __restrict__ dO, float* ws) {
+    constexpr int NT = kThreads<DK, DV>;
+    using MV = tile::Map<CT, DV, NT>;
+    using MK = tile::Map<CT, DK, NT>;
+    using MPhi = tile::Map<DK, DK, NT>;
+    using MPsi = tile::Map<DK, DV, NT>;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    PreSmem<DK, DV, BWD>& sm = *reinterpret_cast<PreSmem<DK, DV, BWD>*>(smem_raw);
     const int c = blockIdx.x, h = blockIdx.y, bb = blockIdx.z;
-    const int C = p.C, dk = p.dk, dv = p.dv, t0 = c * C, n = min(C, p.L - t0);
-    const int ldk = ldp(dk), ldv = ldp(dv), ldc = ldp(C);
-    float* Qs = sm;                    // [C][dk]
-    float* Ks = Qs + C * ldk;          // [C][dk]
-    float* Wks = Ks + C * ldk;         // [C][dk]
-    float* Wc = Wks + C * ldk;         // [C][dv]
-    float* Hs = Wc + C * ldv;          // [dk][dv]
-    float* A = Hs + dk * ldv;          // [C][C]
-    float* O = A + C * ldc;            // [C][dv]
-    float* b = O + C * ldv;            // [C]
-    const long long bh = (long long)bb * p.H + h;
-    const Ws w = ws_of(const_cast<float*>(ws), p, bh, backward != 0);
-    const long long oqk = (long long)bb * p.bqk + (long long)t0 * p.tqk + (long long)h * dk;
-    load_rows(Qs, ldk, q + oqk, p.tqk, n, dk);
-    load_rows(Ks, ldk, k + oqk, p.tqk, n, dk);
-    load_dense(Wks, ldk, w.Wk + (long long)t0 * dk, dk, n, dk);
-    load_dense(Wc, ldv, w.U + (long long)t0 * dv, dv, n, dv);
-    load_dense(Hs, ldv, w.Hc + (long long)c * dk * dv, dv, dk, dv);
-    load_decay(b, nullptr, g + (long long)bb * p.bg + (long long)t0 * p.tg + h, nullptr, p.tg, n);
-    mmx(Wc, ldv, Wks, ldk, false, Hs, ldv, false, n, dv, dk, 1.f, -1.f);         // W = U - Wk H
-    mmx(A, ldc, Qs, ldk, false, Ks, ldk, true, n, n, dk, 0.f, 1.f);
-    mmx(O, ldv, Qs, ldk, false, Hs, ldv, false, n, dv, dk, 0.f, 1.f);
-    __syncthreads();
-    for (int idx = threadIdx.x; idx < n * n; idx += NT) {
-        const int t = idx / n, s = idx - t * n;
-        A[t * ldc + s] = s <= t ? A[t * ldc + s] * __expf(b[t] - b[s]) : 0.f;
-    }
-    scale_rows(O, ldv, n, dv, [&](int t) { return __expf(b[t]); });
-    __syncthreads();
-    mmx(O, ldv, A, ldc, false, Wc, ldv, false, n, dv, n, 1.f, 1.f);
-    __syncthreads();
-    T* oh = o + (long long)bb * p.bv + (long long)t0 * p.tv + (long long)h * dv;
-    for (int idx = threadIdx.x; idx < n * dv; idx += NT) {
-        const int t = idx / dv, jj = idx - t * dv;
-        oh[(long long)t * p.tv + jj] = from_f32<T>(O[t * ldv + jj]);
-    }
-}
-
-// ---- backward, first chunk-parallel part: Z0 = Ti^T (A^T dO),  Theta = Q^T (gam*dO) - K^T (beta*gam*Z0).  grid (NC, H, B) ----
-template <typename T>
-__global__ void __launch_bounds__(NT) bwd_pre_kernel(Params p, const T* __restrict__ q, const T* __restrict__ k,
-                                                     const float* __restrict__ g, const float* __restrict__ beta,
-                                                     const T* __restrict__ dO, float* ws) {
-    extern __shared__ float sm[];
-    const int c = blockIdx.x, h = blockIdx.y, bb = blockIdx.z;
-    const int C = p.C, dk = p.dk, dv = p.dv, t0 = c * C, n = min(C, p.L - t0);
-    const int ldk = ldp(dk), ldv = ldp(dv), ldc = ldp(C);
-    float* Qs = sm;                    // [C][dk]
-    float* Ks = Qs + C * ldk;          // [C][dk]
-    float* dOs = Ks + C * ldk;         // [C][dv]
-    float* T1 = dOs + C * ldv;         // [C][dv]
-    float* Z0 = T1 + C * ldv;          // [C][dv]
-    float* A = Z0 + C * ldv;           // [C][C]
-    float* Ti = A + C * ldc;           // [C][C]
-    float* b = Ti + C * ldc;           // [C]
-    float* bt = b + C;                 // [C]
-    const long long bh = (long long)bb * p.H + h;
-    const Ws w = ws_of(ws, p, bh, true);
-    const long long oqk = (long long)bb * p.bqk + (long long)t0 * p.tqk + (long long)h * dk;
-    load_rows(Qs, ldk, q + oqk, p.tqk, n, dk);
-    load_rows(Ks, ldk, k + oqk, p.tqk, n, dk);
-    load_rows(dOs, ldv, dO + (long long)bb * p.bv + (long long)t0 * p.tv + (long long)h * dv, p.tv, n, dv);
-    load_dense(A, ldc, w.A + (long long)c * C * C, C, n, n);
-    load_dense(Ti, ldc, w.Ti + (long long)c * C * C, C, n, n);
-    load_decay(b, bt, g + (long long)bb * p.bg + (long long)t0 * p.tg + h, beta + (long long)bb * p.bg + (long long)t0 * p.tg + h, p.tg, n);
-    mmx(T1, ldv, A, ldc, true, dOs, ldv, false, n, dv, n, 0.f, 1.f);             // A^T dO
-    __syncthreads();
-    mmx(Z0, ldv, Ti, ldc, true, T1, ldv, false, n, dv, n, 0.f, 1.f);             // Z0 = (I+L)^-T A^T dO
-    __syncthreads();
-    store_dense(w.Z0 + (long long)t0 * dv, dv, Z0, ldv, n, dv);
-    scale_rows(dOs, ldv, n, dv, [&](int t) { return __expf(b[t]); });
-    scale_rows(Z0, ldv, n, dv, [&](int t) { return bt[t] * __expf(b[t]); });
-    __syncthreads();
-    float* Th = w.Theta + (long long)c * dk * dv;
-    mmx(Th, dv, Qs, ldk, true, dOs, ldv, false, dk, dv, n, 0.f, 1.f);
-    mmx(Th, dv, Ks, ldk, true, Z0, ldv, false, dk, dv, n, 1.f, -1.f);
-}
-
-// ---- backward, second chunk-parallel part: every input gradient of the chunk from the stored Hc, dHc, U, Wk, Z0, Ti.
-//      grid (NC, H, B) ------------------------------------------------------------------------------------------------
-template <typename T>
-__global__ void __launch_bounds__(NT) bwd_out_kernel(Params p, const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v,
-                                                     const float* __restrict__ g, const float* __restrict__ beta,
-                                                     const T* __restrict__ dO, T* __restrict__ dq, T* __restrict__ dk_out,
-                                                     T* __restrict__ dv_out, float* __restrict__ dg, float* __restrict__ dbeta,
-                                                     const float* ws) {
-    extern __shared__ float sm[];
-    const int c = blockIdx.x, h = blockIdx.y, bb = blockIdx.z;
-    const int C = p.C, dk = p.dk, dv = p.dv, t0 = c * C, n = min(C, p.L - t0);
-    const int ldk = ldp(dk), ldv = ldp(dv), ldc = ldp(C);
-    float* Qs = sm;                     float* Ks = Qs + C * ldk;
-    float* Vs = Ks + C * ldk;           float* dOs = Vs + C * ldv;
-    float* Wc = dOs + C * ldv;          float* Zs = Wc + C * ldv;
-    float* Hs = Zs + C * ldv;           float* dHs = Hs + dk * ldv;
-    float* QK = dHs + dk * ldv;         float* KK = QK + C * ldc;
-    float* DA = KK + C * ldc;           float* ZW = DA + C * ldc;
-    float* KH = ZW + C * ldc;           float* KdH = KH + C * ldv;
-    float* dQs = KdH + C * ldv;         float* dKs = dQs + C * ldk;
-    float* T1 = dKs + C * ldk;          // [C][max(dk, dv)]: Wk, then om*(K dH'), then Z H^T
-    float* b = T1 + C * ldp(dk > dv ? dk : dv);   float* bt = b + C;
-    float* rs = bt + C;                 float* cs = rs + C;
-    float* rl = cs + C;                 float* zkh = rl + C;
-    float* zv = zkh + C;                float* doqh = zv + C;
-    float* wkdh = doqh + C;             float* db = wkdh + C;
-    float* part = db + C;               // [dk]
-    float* Ti = QK;                     // the inverse is needed only before the C x C products are formed
-    const long long bh = (long long)bb * p.H + h;
-    const Ws w = ws_of(const_cast<float*>(ws), p, bh, true);
-    const long long oqk = (long long)bb * p.bqk + (long long)t0 * p.tqk + (long long)h * dk;
-    const long long ov = (long long)bb * p.bv + (long long)t0 * p.tv + (long long)h * dv;
+    const int t0 = c * CT, n = min(CT, p.L - t0);
+    const Ws w = ws_of(ws, p, (long long)bb * p.H + h, BWD);
+    const long long oqk = (long long)bb * p.bqk + (long long)t0 * p.tqk + (long long)h * DK;
+    const long long ov = (long long)bb * p.bv + (long long)t0 * p.tv + (long long)h * DV;
     const long long og = (long long)bb * p.bg + (long long)t0 * p.tg + h;
-    load_rows(Qs, ldk, q + oqk, p.tqk, n, dk);
-    load_rows(Ks, ldk, k + oqk, p.tqk, n, dk);
-    load_rows(Vs, ldv, v + ov, p.tv, n, dv);
-    load_rows(dOs, ldv, dO + ov, p.tv, n, dv);
-    load_dense(Wc, ldv, w.U + (long long)t0 * dv, dv, n, dv);
-    load_dense(T1, ldk, w.Wk + (long long)t0 * dk, dk, n, dk);
-    load_dense(Zs, ldv, w.Z0 + (long long)t0 * dv, dv, n, dv);
-    load_dense(Hs, ldv, w.Hc + (long long)c * dk * dv, dv, dk, dv);
-    load_dense(dHs, ldv, w.dHc + (long long)c * dk * dv, dv, dk, dv);
-    load_dense(Ti, ldc, w.Ti + (long long)c * C * C, C, n, n);
-    load_decay(b, bt, g + og, beta + og, p.tg, n);
-    const float bn = b[n - 1];
-    mmx(Wc, ldv, T1, ldk, false, Hs, ldv, false, n, dv, dk, 1.f, -1.f);          // W = U - Wk H
-    mmx(KH, ldv, Ks, ldk, false, Hs, ldv, false, n, dv, dk, 0.f, 1.f);
-    mmx(KdH, ldv, Ks, ldk, false, dHs, ldv, false, n, dv, dk, 0.f, 1.f);
-    __syncthreads();
-    // Z = Z0 + Ti^T (om * (K dH')): the part of the transposed solve that depends on the incoming state gradient
-    const int ldt = ldp(dk > dv ? dk : dv);
-    for (int idx = threadIdx.x; idx < n * dv; idx += NT) {
-        const int t = idx / dv, jj = idx - t * dv;
-        T1[t * ldt + jj] = __expf(bn - b[t]) * KdH[t * ldv + jj];
+    tile_decay(sm.d, g + og, beta + og, p.tg, n);
+    tile::load<CT, DK, NT>(sm.K, k + oqk, p.tqk, n, p.vec);
+    tile::load<CT, DV, NT>(sm.X, v + ov, p.tv, n, p.vec);
+    if constexpr (BWD) {
+        tile::load<CT, DK, NT>(sm.Q, q + oqk, p.tqk, n, p.vec);
+        tile::load<CT, DV, NT>(sm.D, dO + ov, p.tv, n, p.vec);
     }
     __syncthreads();
-    mmx(Zs, ldv, Ti, ldc, true, T1, ldt, false, n, dv, n, 1.f, 1.f);
-    __syncthreads();
-    mmx(QK, ldc, Qs, ldk, false, Ks, ldk, true, n, n, dk, 0.f, 1.f);
-    mmx(KK, ldc, Ks, ldk, false, Ks, ldk, true, n, n, dk, 0.f, 1.f);
-    mmx(DA, ldc, dOs, ldv, false, Wc, ldv, true, n, n, dv, 0.f, 1.f);            // dA = dO W^T
-    mmx(ZW, ldc, Zs, ldv, false, Wc, ldv, true, n, n, dv, 0.f, 1.f);             // Z W^T  (dL = -strict lower)
-    mmx(dQs, ldk, dOs, ldv, false, Hs, ldv, true, n, dk, dv, 0.f, 1.f);          // dO H^T
-    mmx(dKs, ldk, Wc, ldv, false, dHs, ldv, true, n, dk, dv, 0.f, 1.f);          // W dH'^T
-    mmx(T1, ldt, Zs, ldv, false, Hs, ldv, true, n, dk, dv, 0.f, 1.f);            // Z H^T
-    for (int i = threadIdx.x; i < dk; i += NT) {
-        float acc = 0.f;
-        for (int jj = 0; jj < dv; ++jj) acc = fmaf(dHs[i * ldv + jj], Hs[i * ldv + jj], acc);
-        part[i] = acc;
+    auto put_l = [&](int m, int n0, const float* a) {              // L (and, for the backward, KM = M * K K^T) below the diagonal
+        float v4[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) v4[j] = n0 + j < m ? a[j] * mexp(sm.d, m, n0 + j) : 0.f;
+        if (BWD) tile::store4(w.KM + (long long)c * CC + m * CT + n0, make_float4(v4[0], v4[1], v4[2], v4[3]));
+        const float bt = sm.d.beta[m];
+        tile::st4(sm.T + tile::at<CT>(m, n0), make_float4(bt * v4[0], bt * v4[1], bt * v4[2], bt * v4[3]));
+    };
+    if constexpr (BWD) {
+        auto put_a = [&](int m, int n0, const float* a) {
+            float v4[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) v4[j] = n0 + j <= m ? a[j] * mexp(sm.d, m, n0 + j) : 0.f;
+            const float4 f = make_float4(v4[0], v4[1], v4[2], v4[3]);
+            tile::store4(w.A + (long long)c * CC + m * CT + n0, f);
+            tile::st4(sm.A + tile::at<CT>(m, n0), f);
+        };
+        two_square_products<NT, DK, DK>(sm.K, sm.K, put_l, sm.Q, sm.K, put_a);
+    } else {
+        if (threadIdx.x < 128) square_product<DK>(sm.K, sm.K, threadIdx.x, put_l);
+    }
+    // right-hand sides: X = beta*V, Y = beta*gam*K
+    tile::scale_rows<CT, DV, NT>(sm.X, sm.d.beta);
+    for (int i = threadIdx.x; i < CT * DK / 4; i += NT) {
+        const int r = i / (DK / 4);
+        const float f = sm.d.beta[r] * sm.d.gam[r];
+        const float4 x = reinterpret_cast<const float4*>(sm.K)[i];
+        reinterpret_cast<float4*>(sm.Y)[i] = make_float4(f * x.x, f * x.y, f * x.z, f * x.w);
     }
     __syncthreads();
-    // C x C pass: DA <- dA*M (s <= t),  ZW <- P = beta_t dL M (s < t),  QK <- E = (dA QK + beta_t dL KK) M,  KK <- dL M KK
-    for (int idx = threadIdx.x; idx < n * n; idx += NT) {
-        const int t = idx / n, s = idx - t * n, a = t * ldc + s;
-        const float m = s <= t ? __expf(b[t] - b[s]) : 0.f;
-        const float dl = s < t ? -ZW[a] : 0.f;
-        const float da = DA[a], qk = QK[a], kk = KK[a];
-        DA[a] = da * m;
-        ZW[a] = bt[t] * dl * m;
-        QK[a] = (da * qk + bt[t] * dl * kk) * m;
-        KK[a] = dl * m * kk;
+    invert<NT>(sm.T, sm.tmp);
+    for (int i = threadIdx.x; i < CC / 4; i += NT)
+        reinterpret_cast<float4*>(w.T + (long long)c * CC)[i] = tile::ld4(sm.T + tile::at<CT>(i / (CT / 4), (i % (CT / 4)) * 4));
+    const MV mv;
+    const MK mk;
+    auto same = [](int, int, float x) { return x; };
+    {
+        float au[MV::TM][MV::TN], ak[MK::TM][MK::TN];
+        tile::zero<MV>(au);
+        tile::zero<MK>(ak);
+        if (mv.on) tile::product<MV, true, false, CT, DV>(au, sm.T, sm.X, 0, mv.warp_m0() + 16, mv);       // U
+        if (mk.on) tile::product<MK, true, false, CT, DK>(ak, sm.T, sm.Y, 0, mk.warp_m0() + 16, mk);       // Wk
+        __syncthreads();
+        // om goes to U and Wk: (om*K)^T U = K^T (om*U)
+        if (mv.on) tile::put<MV, DV>(sm.X, au, mv, [&](int m, int, float x) { return sm.d.om[m] * x; });
+        if (mk.on) tile::put<MK, DK>(sm.Y, ak, mk, [&](int m, int, float x) { return -sm.d.om[m] * x; });
+        __syncthreads();
     }
-    __syncthreads();
-    for (int t = threadIdx.x; t < n; t += NT) {
-        float r = 0.f, cc = 0.f, l = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f, a4 = 0.f;
-        for (int s = 0; s < n; ++s) { r += QK[t * ldc + s]; cc += QK[s * ldc + t]; l += KK[t * ldc + s]; }
-        for (int jj = 0; jj < dv; ++jj) {
-            a1 = fmaf(Zs[t * ldv + jj], KH[t * ldv + jj], a1);
-            a2 = fmaf(Zs[t * ldv + jj], Vs[t * ldv + jj], a2);
-            a4 = fmaf(Wc[t * ldv + jj], KdH[t * ldv + jj], a4);
+    {
+        const MPsi m;
+        float acc[MPsi::TM][MPsi::TN];
+        tile::zero<MPsi>(acc);
+        if (m.on) {
+            tile::product<MPsi, false, false, DK, DV>(acc, sm.K, sm.X, 0, CT, m);
+            store_dense<MPsi, DV>(w.Psi + (long long)c * DK * DV, acc, m, same);
         }
-        for (int i = 0; i < dk; ++i) a3 = fmaf(Qs[t * ldk + i], dQs[t * ldk + i], a3);
-        rs[t] = r; cs[t] = cc; rl[t] = l; zkh[t] = a1; zv[t] = a2; doqh[t] = a3; wkdh[t] = a4;
     }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        float dgamC = 0.f, som = 0.f;
-        for (int i = 0; i < dk; ++i) dgamC += part[i];
-        for (int t = 0; t < n; ++t) {
-            const float gam = __expf(b[t]), om = __expf(bn - b[t]);
-            const float dgam = doqh[t] - bt[t] * zkh[t];
-            db[t] = rs[t] - cs[t] + dgam * gam - wkdh[t] * om;
-            som = fmaf(wkdh[t], om, som);
+    {
+        const MPhi m;
+        float acc[MPhi::TM][MPhi::TN];
+        tile::zero<MPhi>(acc);
+        const float gn = sm.d.gam[CT - 1];
+        if (m.on) {
+            tile::product<MPhi, false, false, DK, DK>(acc, sm.K, sm.Y, 0, CT, m);
+            store_dense<MPhi, DK>(w.Phi + (long long)c * DK * DK, acc, m, [&](int r, int cc, float x) { return r == cc ? x + gn : x; });
         }
-        db[n - 1] += som + dgamC * __expf(bn);
-        float acc = 0.f;
-        for (int t = n - 1; t >= 0; --t) { acc += db[t]; dg[og + (long long)t * p.tg] = acc; }
     }
-    for (int t = threadIdx.x; t < n; t += NT)
-        dbeta[og + (long long)t * p.tg] = zv[t] - __expf(b[t]) * zkh[t] + rl[t];
-    // dq = (dA*M) K + gam*(dO H^T);  dk = om*(W dH'^T) - beta*gam*(Z H^T) + (dA*M)^T Q + P K + P^T K
-    for (int idx = threadIdx.x; idx < n * dk; idx += NT) {
-        const int t = idx / dk, i = idx - t * dk, a = t * ldk + i;
-        dQs[a] *= __expf(b[t]);
-        dKs[a] = __expf(bn - b[t]) * dKs[a] - bt[t] * __expf(b[t]) * T1[t * ldt + i];
-    }
-    __syncthreads();
-    mmx(dQs, ldk, DA, ldc, false, Ks, ldk, false, n, dk, n, 1.f, 1.f);
-    mmx(dKs, ldk, DA, ldc, true, Qs, ldk, false, n, dk, n, 1.f, 1.f);
-    __syncthreads();
-    mmx(dKs, ldk, ZW, ldc, false, Ks, ldk, false, n, dk, n, 1.f, 1.f);
-    __syncthreads();
-    mmx(dKs, ldk, ZW, ldc, true, Ks, ldk, false, n, dk, n, 1.f, 1.f);
-    __syncthreads();
-    for (int idx = threadIdx.x; idx < n * dk; idx += NT) {
-        const int t = idx / dk, i = idx - t * dk;
-        dq[oqk + (long long)t * p.tqk + i] = from_f32<T>(dQs[t * ldk + i]);
-        dk_out[oqk + (long long)t * p.tqk + i] = from_f32<T>(dKs[t * ldk + i]);
-    }
-    for (int idx = threadIdx.x; idx < n * dv; idx += NT) {
-        const int t = idx / dv, jj = idx - t * dv;
-        dv_out[ov + (long long)t * p.tv + jj] = from_f32<T>(bt[t] * Zs[t * ldv + jj]);
+    if constexpr (BWD) {
+        float az[MV::TM][MV::TN];
+        tile::zero<MV>(az);
+        if (mv.on) tile::product<MV, false, false, CT, DV>(az, sm.A, sm.D, mv.warp_m0(), CT, mv);         // A^T dO
+        __syncthreads();                                            // X and A, dO have been read
+        if (mv.on) tile::put<MV, DV>(sm.X, az, mv, same);
+        tile::scale_rows<CT, DV, NT>(sm.D, sm.d.gam);
+        __syncthreads();
+        tile::zero<MV>(az);
+        if (mv.on) tile::product<MV, false, false, CT, DV>(az, sm.T, sm.X, mv.warp_m0(), CT, mv);         // Z0
+        __syncthreads();
+        if (mv.on) tile::put<MV, DV>(sm.X, az, mv, [&](int m, int, float x) { return -sm.d.beta[m] * sm.d.gam[m] * x; });
+        __syncthreads();
+        const MPsi m;
+        float acc[MPsi::TM][MPsi::TN];
+        tile::zero<MPsi>(acc);
+        if (m.on) {
+            tile::product<MPsi, false, false, DK, DV>(acc, sm.Q, sm.D, 0, CT, m);
+            tile::product<MPsi, false, false, DK, DV>(acc, sm.K, sm.X, 0, CT, m);
+            store_dense<MPsi, DV>(w.Theta + (long long)c * DK * DV, acc, m, same);
+        }
     }
 }
 
-// shared memory (bytes) of the kernels for a shape (padded tiles)
-__host__ inline size_t smem_pre(int C, int dk, int dv) {
-    return sizeof(float) * (3 * (size_t)C * ldp(dk) + (size_t)C * ldp(dv + dk + C) + (size_t)C * ldp(C) + 2 * C);
+// ---- ST (forward) and its adjoint (reverse): X' = F X + R tile by tile for NV columns of the state.
+//      forward F = Phi[c],   R = Psi[c],   ascending;   Hc[c]  <- state entering tile c
+//      reverse F = Phi[c]^T, R = Theta[c], descending;  dHc[c] <- gradient of the state leaving tile c
+//      grid (dv/NV, H, B), or twice as many columns with both directions in one launch (the backward's two passes need
+//      nothing from each other, and two CTAs on an SM fill each other's gaps); 256 threads.  A thread owns a 4 x 4 block of
+//      X' over one KS-th of the contraction (its units of four k: ks, ks + KS, ...); the KS lanes of a block add up by a
+//      reduce-scatter of shuffles.  The maps arrive by cp.async STAGES - 1 tiles ahead; one barrier per tile.
+//      The pass is a chain of dependent small products: what bounds it is the latency of one step, not the device, which is why
+//      it walks all tiles instead of multiplying the maps of a block together first: that costs 2 d_k^3 per tile and was four
+//      times slower on 16 heads x 512 tiles (1.55 ms a direction against 0.3-0.4).
+constexpr int CHAIN_NT = 256;
+template <int DK, int NV> constexpr int kStages = DK == 128 ? (NV == 16 ? 2 : 3) : (DK == 64 ? 6 : 8);      // a 128-wide map is 64 KB
+// Word offset of the 16-byte unit c4 of row k of X [d_k][NV]: inside the block of four rows, XORed with the bit-reversed index
+// of the block, so that lanes that read rows four apart (neighbouring ks) or neighbouring columns meet different banks.
+template <int NV>
+__device__ __forceinline__ int xat(int k, int c4) {
+    const int u = k >> 2, rev = ((u & 1) << 2) | (u & 2) | ((u >> 2) & 1);
+    return u * 4 * NV + ((((k & 3) * (NV / 4) + c4) ^ rev) << 2);
 }
-__host__ inline size_t smem_chain(int dk) { return sizeof(float) * (2 * (size_t)dk * ldp(DVS) + (size_t)dk * ldp(dk)); }
-__host__ inline size_t smem_compose(int dk, int dv) { return sizeof(float) * (3 * (size_t)dk * ldp(dk) + 2 * (size_t)dk * ldp(dv)); }
-__host__ inline size_t smem_out(int C, int dk, int dv) {
-    return sizeof(float) * (3 * (size_t)C * ldp(dk) + 2 * (size_t)C * ldp(dv) + (size_t)dk * ldp(dv) + (size_t)C * ldp(C) + C);
+template <int DK, int NV>
+struct ChainSmem {
+    float F[kStages<DK, NV>][DK * DK];
+    float R[kStages<DK, NV>][DK * NV];
+    float X[2][DK * NV];
+};
+__device__ __forceinline__ void cp_async16(float* dst, const float* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
 }
-__host__ inline size_t smem_bwd_pre(int C, int dk, int dv) {
-    return sizeof(float) * (2 * (size_t)C * ldp(dk) + 3 * (size_t)C * ldp(dv) + 2 * (size_t)C * ldp(C) + 2 * C);
+struct ChainEnds { const float* init; float* fin; };                // state entering (NULL: zero), state leaving (NULL: not wanted)
+template <int DK, int NV, bool REV>
+__device__ __forceinline__ void chain_pass(const Params& p, const ChainEnds& ends, float* ws, int backward, int j0) {
+    constexpr int TN4 = NV / 4, TILES = DK / 4 * TN4, KS = CHAIN_NT / TILES, ST = kStages<DK, NV>, PT = 32 / KS, TMW = PT / TN4;
+    static_assert(KS >= 2 && KS <= 8 && KS <= DK / 4 && TMW >= 1, "tile split");
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    ChainSmem<DK, NV>& sm = *reinterpret_cast<ChainSmem<DK, NV>*>(smem_raw);
+    const int dv = p.dv, n = p.NT;
+    const long long bh = (long long)blockIdx.z * p.H + blockIdx.y;
+    const Ws w = ws_of(ws, p, bh, backward != 0);
+    const float* R = REV ? w.Theta : w.Psi;
+    float* states = REV ? w.dHc : w.Hc;
+    const int tid = threadIdx.x, wp = tid >> 5, lane = tid & 31;
+    // lane bits: tn bit 0, then hm bit 0 (so that X is shared by lanes l and l ^ 2 and the map by l and l ^ 1, see tile::lane_y),
+    // the other bits of tn and hm, ks on top
+    auto bit = [&](int b) { return (lane >> b) & 1; };
+    const int tn = bit(0) + (TN4 == 4 ? 2 * bit(TMW > 1 ? 2 : 1) : 0);
+    const int hm = (TMW > 1 ? bit(1) : 0) + (TMW == 4 ? 2 * bit(TN4 == 4 ? 3 : 2) : 0);
+    const int ks = lane / (32 / KS);
+    // rows of four served by this warp: TMW groups 8 / TMW apart, so that the groups of a warp differ in the swizzle bits
+    constexpr int STEP = 8 / TMW;
+    const int tm = (wp % STEP) + STEP * hm + 8 * (wp / STEP);
+    auto step_tile = [&](int s) { return REV ? n - 1 - s : s; };
+    auto fetch = [&](int s) {
+        if (s < n) {
+            const float* src = w.Phi + (long long)step_tile(s) * DK * DK;
+            float* dst = sm.F[s % ST];
+#pragma unroll
+            for (int i = 0; i < DK * DK / 4 / CHAIN_NT; ++i) {
+                const int u = tid + i * CHAIN_NT, r = u / (DK / 4), cc = (u % (DK / 4)) * 4;
+                cp_async16(dst + tile::at<DK>(r, cc), src + 4 * u);
+            }
+            const float* rsrc = R + (long long)step_tile(s) * DK * dv + j0;
+            for (int u = tid; u < DK * NV / 4; u += CHAIN_NT)
+                cp_async16(sm.R[s % ST] + 4 * u, rsrc + (u / (NV / 4)) * dv + (u % (NV / 4)) * 4);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    for (int s = 0; s < ST - 1; ++s) fetch(s);
+    // after the reduce-scatter lane ks holds NE elements of its block from the e0-th on, row by row
+    constexpr int NE = 16 / KS;
+    const int e0 = ks * NE, row0 = 4 * tm + e0 / 4, col0 = 4 * tn + (e0 & 3);
+    for (int i = tid; i < DK * NV; i += CHAIN_NT) {
+        const int a = i / NV, b = i % NV;
+        const float x = ends.init ? ends.init[bh * DK * dv + a * dv + j0 + b] : 0.f;
+        sm.X[0][xat<NV>(a, b >> 2) + (b & 3)] = x;
+        states[(long long)step_tile(0) * DK * dv + a * dv + j0 + b] = x;
+    }
+    for (int s = 0; s < n; ++s) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(ST - 2) : "memory");
+        __syncthreads();                                             // map s and X are complete; map s - 1 has been read
+        fetch(s + ST - 1);
+        const float *F = sm.F[s % ST], *Rs = sm.R[s % ST];
+        const float* X = sm.X[s & 1];
+        tile::f32x2 acc2[4][2] = {};
+#pragma unroll 2
+        for (int u = ks; u < DK / 4; u += KS) {
+            ulonglong2 x[4];
+            float4 f[4];
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk) x[kk] = tile::ld4x2(X + xat<NV>(4 * u + kk, tn));
+#pragma unroll
+            for (int i = 0; i < 4; ++i) f[i] = tile::ld4(REV ? F + (4 * u + i) * DK + ((tm ^ (u & 7)) << 2) : F + (4 * tm + i) * DK + ((u ^ (tm & 7)) << 2));
+#pragma unroll
+            for (int a = 0; a < 4; ++a) {
+                const float fv[4] = {f[a].x, f[a].y, f[a].z, f[a].w};
+#pragma unroll
+                for (int b = 0; b < 4; ++b) {
+                    // forward: f[a] is row a of the block, four k; reverse: f[a] is step a of k, four rows
+                    const tile::f32x2 f2 = tile::pack(fv[b], fv[b]);
+                    if (REV) { tile::fma2(acc2[b][0], f2, x[a].x); tile::fma2(acc2[b][1], f2, x[a].y); }
+                    else     { tile::fma2(acc2[a][0], f2, x[b].x); tile::fma2(acc2[a][1], f2, x[b].y); }
+                }
+            }
+        }
+        float acc[16];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) { tile::unpack(acc2[i][0], acc[4 * i], acc[4 * i + 1]); tile::unpack(acc2[i][1], acc[4 * i + 2], acc[4 * i + 3]); }
+        // reduce-scatter over the KS lanes: at each level a lane keeps the half of its values that its bit of ks selects
+        int width = 16;
+#pragma unroll
+        for (int b = KS / 2; b >= 1; b >>= 1) {
+            const int half = width / 2;
+            const bool up = (ks & b) != 0;
+#pragma unroll
+            for (int e = 0; e < 8; ++e)
+                if (e < half) {
+                    const float keep = up ? acc[e + half] : acc[e], give = up ? acc[e] : acc[e + half];
+                    acc[e] = keep + __shfl_xor_sync(0xffffffffu, give, b * (32 / KS));
+                }
+            width = half;
+        }
+        float* Xn = sm.X[(s + 1) & 1];
+        float* out = s + 1 < n ? states + (long long)step_tile(s + 1) * DK * dv : (ends.fin ? ends.fin + bh * DK * dv : nullptr);
+        // whole rows of four elements, or half a row when eight lanes share the block
+        if constexpr (NE >= 4) {
+#pragma unroll
+            for (int e = 0; e < NE; e += 4) {
+                const int row = row0 + e / 4;
+                const float4 rv = tile::ld4(Rs + row * NV + col0);
+                const float4 x = make_float4(acc[e] + rv.x, acc[e + 1] + rv.y, acc[e + 2] + rv.z, acc[e + 3] + rv.w);
+                tile::st4(Xn + xat<NV>(row, tn), x);
+                if (out) {
+                    float* o = out + row * dv + j0 + col0;
+                    o[0] = x.x; o[1] = x.y; o[2] = x.z; o[3] = x.w;
+                }
+            }
+        } else {
+            const float2 rv = *reinterpret_cast<const float2*>(Rs + row0 * NV + col0);
+            const float2 x = make_float2(acc[0] + rv.x, acc[1] + rv.y);
+            *reinterpret_cast<float2*>(Xn + xat<NV>(row0, tn) + (col0 & 3)) = x;
+            if (out) {
+                float* o = out + row0 * dv + j0 + col0;
+                o[0] = x.x; o[1] = x.y;
+            }
+        }
+    }
 }
-__host__ inline size_t smem_bwd_out(int C, int dk, int dv) {
-    return sizeof(float) * (2 * (size_t)C * ldp(dk) + 4 * (size_t)C * ldp(dv) + 2 * (size_t)dk * ldp(dv) + 4 * (size_t)C * ldp(C) +
-                            2 * (size_t)C * ldp(dv) + 2 * (size_t)C * ldp(dk) + (size_t)C * ldp(dk > dv ? dk : dv) + 10 * (size_t)C + dk);
+template <int DK, int NV>
+__global__ void __launch_bounds__(CHAIN_NT) chain_kernel(Params p, ChainEnds fwd, ChainEnds rev, float* ws, int backward) {
+    const int cols = p.dv / NV;
+    if ((int)blockIdx.x < cols) chain_pass<DK, NV, false>(p, fwd, ws, backward, blockIdx.x * NV);
+    else                        chain_pass<DK, NV, true>(p, rev, ws, backward, (blockIdx.x - cols) * NV);
 }
 
-__host__ inline size_t smem_max(int C, int dk, int dv) {
-    size_t m = smem_pre(C, dk, dv);
-    const size_t o[4] = {smem_chain(dk), smem_out(C, dk, dv), smem_bwd_pre(C, dk, dv), smem_bwd_out(C, dk, dv)};
-    for (size_t x : o) m = x > m ? x : m;
-    return m;
+// ---- Out: W = T (beta*V - beta*gam*(K H)) (V_new),  O = A W + gam * (Q H).  grid (tiles, H, B) ----------------------
+template <int DK, int DV>
+struct OutSmem {
+    float Q[CT * DK], K[CT * DK], R[CT * DV], H[DK * DV], A[CC], T[CC];
+    float Wx[DV > DK ? CT * DV : 4];
+    Decay d;
+    __device__ __forceinline__ float* W() { return DV > DK ? Wx : K; }       // K has served when W is formed
+};
+template <typename T, int DK, int DV>
+__global__ void __launch_bounds__(kThreads<DK, DV>) out_kernel(Params p, const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v,
+                                                               const float* __restrict__ g, const float* __restrict__ beta, T* __restrict__ o,
+                                                               const float* ws) {
+    constexpr int NT = kThreads<DK, DV>;
+    using MV = tile::Map<CT, DV, NT>;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    OutSmem<DK, DV>& sm = *reinterpret_cast<OutSmem<DK, DV>*>(smem_raw);
+    const int c = blockIdx.x, h = blockIdx.y, bb = blockIdx.z;
+    const int t0 = c * CT, n = min(CT, p.L - t0);
+    const Ws w = ws_of(const_cast<float*>(ws), p, (long long)bb * p.H + h, false);
+    const long long oqk = (long long)bb * p.bqk + (long long)t0 * p.tqk + (long long)h * DK;
+    const long long ov = (long long)bb * p.bv + (long long)t0 * p.tv + (long long)h * DV;
+    const long long og = (long long)bb * p.bg + (long long)t0 * p.tg + h;
+    tile_decay(sm.d, g + og, beta + og, p.tg, n);
+    tile::load<CT, DK, NT>(sm.Q, q + oqk, p.tqk, n, p.vec);
+    tile::load<CT, DK, NT>(sm.K, k + oqk, p.tqk, n, p.vec);
+    tile::load<CT, DV, NT>(sm.R, v + ov, p.tv, n, p.vec);
+    tile::load<DK, DV, NT>(sm.H, w.Hc + (long long)c * DK * DV, DV, DK);
+    load_square<NT>(sm.T, w.T + (long long)c * CC);
+    __syncthreads();
+    if (threadIdx.x < 128)
+        square_product<DK>(sm.Q, sm.K, threadIdx.x, [&](int m, int n0, const float* a) {
+            float v4[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) v4[j] = n0 + j <= m ? a[j] * mexp(sm.d, m, n0 + j) : 0.f;
+            tile::st4(sm.A + tile::at<CT>(m, n0), make_float4(v4[0], v4[1], v4[2], v4[3]));
+        });
+    const MV mv;
+    float aq[MV::TM][MV::TN], aw[MV::TM][MV::TN];
+    tile::zero<MV>(aq);
+    tile::zero<MV>(aw);
+    if (mv.on) {
+        tile::product<MV, true, false, DK, DV>(aw, sm.K, sm.H, 0, DK, mv);
+        // R = beta*(V - gam*(K H)): every thread rewrites the elements that it owns
+#pragma unroll
+        for (int i = 0; i < MV::TM; ++i) {
+            const int m = mv.m(i);
+            const float bt = sm.d.beta[m], gm = sm.d.gam[m];
+#pragma unroll
+            for (int gq = 0; gq < MV::GN; ++gq) {
+                float* x = sm.R + tile::at<DV>(m, mv.n4(gq));
+                const float4 vv = tile::ld4(x);
+                tile::st4(x, make_float4(bt * fmaf(-gm, aw[i][4 * gq], vv.x), bt * fmaf(-gm, aw[i][4 * gq + 1], vv.y),
+                                         bt * fmaf(-gm, aw[i][4 * gq + 2], vv.z), bt * fmaf(-gm, aw[i][4 * gq + 3], vv.w)));
+            }
+        }
+        tile::product<MV, true, false, DK, DV>(aq, sm.Q, sm.H, 0, DK, mv);
+        scale_acc(aq, mv, [&](int m) { return sm.d.gam[m]; });
+    }
+    __syncthreads();
+    tile::zero<MV>(aw);
+    if (mv.on) {
+        tile::product<MV, true, false, CT, DV>(aw, sm.T, sm.R, 0, mv.warp_m0() + 16, mv);
+        tile::put<MV, DV>(sm.W(), aw, mv, [](int, int, float x) { return x; });
+    }
+    __syncthreads();
+    if (mv.on) {
+        tile::product<MV, true, false, CT, DV>(aq, sm.A, sm.W(), 0, mv.warp_m0() + 16, mv);
+        store_rows(o + ov, p.tv, n, aq, mv, p.vec, [](int) { return 1.f; });
+    }
+}
+
+// ---- backward, tile-parallel: every input gradient of the tile from the stored Hc, dHc, T, A, KM.  grid (tiles, H, B) ------
+// The shared memory of a 128-wide head holds one of the two states at a time; H is then fetched twice.
+template <int DK, int DV>
+struct BwdSmem {
+    static constexpr bool BOTH = DK * DV <= 64 * 64;
+    float Q[CT * DK], K[CT * DK], V[CT * DV], D[CT * DV];
+    float R[CT * DV];                   // beta*V - beta*gam*(K H), then dW, then the two C x C products
+    float W[CT * DV];
+    float H[DK * DV], G[BOTH ? DK * DV : 4];
+    float T[CC], A[CC], KM[CC];
+    Decay d;
+    float qd[CT * 4], kw[CT * 4], kz[CT * 4], zv[CT * 4];              // row sums, per warp that shares a row
+    float rs[CT], rl[CT], part[8];
+};
+// Row sums of acc(m, n) e(m, n) into red[m * 4 + warp column]: a butterfly over the eight lanes that share the row.
+template <class Mp, typename F>
+__device__ __forceinline__ void row_dots(const float (&acc)[Mp::TM][Mp::TN], const Mp& mp, float* red, F e) {
+    static_assert(Mp::TXN / 8 <= 4, "red holds four partial sums per row");
+#pragma unroll
+    for (int i = 0; i < Mp::TM; ++i) {
+        float s = 0.f;
+#pragma unroll
+        for (int gq = 0; gq < Mp::GN; ++gq) {
+            const float4 v = e(mp.m(i), mp.n4(gq));
+            s = fmaf(acc[i][4 * gq], v.x, s); s = fmaf(acc[i][4 * gq + 1], v.y, s);
+            s = fmaf(acc[i][4 * gq + 2], v.z, s); s = fmaf(acc[i][4 * gq + 3], v.w, s);
+        }
+        s = tile::sum_x(s);
+        if ((mp.tx & 7) == 0) red[mp.m(i) * 4 + (mp.tx >> 3)] = s;
+    }
+}
+template <class Mp>
+__device__ __forceinline__ float row_sum(const float* red, int t) {
+    float s = red[t * 4];
+#pragma unroll
+    for (int w = 1; w < Mp::TXN / 8; ++w) s += red[t * 4 + w];
+    return s;
+}
+template <typename T, int DK, int DV>
+__global__ void __launch_bounds__(kThreads<DK, DV>) bwd_out_kernel(Params p, const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v,
+                                                                   const float* __restrict__ g, const float* __restrict__ beta,
+                                                                   const T* __restrict__ dO, T* __restrict__ dq, T* __restrict__ dk_out,
+                                                                   T* __restrict__ dv_out, float* __restrict__ dg, float* __restrict__ dbeta,
+                                                                   const float* ws) {
+    constexpr int NT = kThreads<DK, DV>;
+    using MV = tile::Map<CT, DV, NT>;
+    using MK = tile::Map<CT, DK, NT>;
+    using Smem = BwdSmem<DK, DV>;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    Smem& sm = *reinterpret_cast<Smem*>(smem_raw);
+    const int c = blockIdx.x, h = blockIdx.y, bb = blockIdx.z, tid = threadIdx.x;
+    const int t0 = c * CT, n = min(CT, p.L - t0);
+    const Ws w = ws_of(const_cast<float*>(ws), p, (long long)bb * p.H + h, true);
+    const long long oqk = (long long)bb * p.bqk + (long long)t0 * p.tqk + (long long)h * DK;
+    const long long ov = (long long)bb * p.bv + (long long)t0 * p.tv + (long long)h * DV;
+    const long long og = (long long)bb * p.bg + (long long)t0 * p.tg + h;
+    const float *Hg = w.Hc + (long long)c * DK * DV, *Gg = w.dHc + (long long)c * DK * DV;
+    float* G = Smem::BOTH ? sm.G : sm.H;
+    tile_decay(sm.d, g + og, beta + og, p.tg, n);
+    tile::load<CT, DK, NT>(sm.K, k + oqk, p.tqk, n, p.vec);
+    tile::load<DK, DV, NT>(sm.H, Hg, DV, DK);
+    tile::load<CT, DV, NT>(sm.V, v + ov, p.tv, n, p.vec);
+    tile::load<CT, DV, NT>(sm.D, dO + ov, p.tv, n, p.vec);
+    tile::load<CT, DK, NT>(sm.Q, q + oqk, p.tqk, n, p.vec);
+    load_square<NT>(sm.T, w.T + (long long)c * CC);
+    load_square<NT>(sm.A, w.A + (long long)c * CC);
+    load_square<NT>(sm.KM, w.KM + (long long)c * CC);
+    if (Smem::BOTH) tile::load<DK, DV, NT>(G, Gg, DV, DK);
+    // <dH', H>, the gradient of the tile's total decay through gam_n
+    {
+        float s = 0.f;
+        for (int i = tid; i < DK * DV / 4; i += NT) {
+            const float4 a = tile::load4(Hg + 4 * i), b = tile::load4(Gg + 4 * i);
+            s = fmaf(a.x, b.x, s); s = fmaf(a.y, b.y, s); s = fmaf(a.z, b.z, s); s = fmaf(a.w, b.w, s);
+        }
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+        if ((tid & 31) == 0) sm.part[tid >> 5] = s;
+    }
+    __syncthreads();
+    const MV mv;
+    const MK mk;
+    auto same = [](int, int, float x) { return x; };
+    float adq[MK::TM][MK::TN], adk[MK::TM][MK::TN];
+    tile::zero<MK>(adq);
+    tile::zero<MK>(adk);
+    {
+        float a[MV::TM][MV::TN];
+        tile::zero<MV>(a);
+        if (mv.on) {
+            tile::product<MV, true, false, DK, DV>(a, sm.K, sm.H, 0, DK, mv);                 // K H
+            tile::put<MV, DV>(sm.R, a, mv, [&](int m, int nn, float x) {
+                return sm.d.beta[m] * fmaf(-sm.d.gam[m], x, sm.V[tile::at<DV>(m, nn)]);
+            });
+        }
+    }
+    if (mk.on) {
+        tile::product<MK, true, true, DV, DV>(adq, sm.D, sm.H, 0, DV, mk);                    // dO H^T
+        row_dots(adq, mk, sm.qd, [&](int m, int nn) { return tile::ld4(sm.Q + tile::at<DK>(m, nn)); });
+        scale_acc(adq, mk, [&](int m) { return sm.d.gam[m]; });
+    }
+    __syncthreads();
+    if (!Smem::BOTH) tile::load<DK, DV, NT>(G, Gg, DV, DK);
+    {
+        float a[MV::TM][MV::TN];
+        tile::zero<MV>(a);
+        if (mv.on) {
+            tile::product<MV, true, false, CT, DV>(a, sm.T, sm.R, 0, mv.warp_m0() + 16, mv);  // W
+            tile::put<MV, DV>(sm.W, a, mv, same);
+        }
+    }
+    __syncthreads();
+    {
+        float a[MV::TM][MV::TN];
+        tile::zero<MV>(a);
+        if (mv.on) {
+            tile::product<MV, true, false, DK, DV>(a, sm.K, G, 0, DK, mv);                    // K dH'
+            scale_acc(a, mv, [&](int m) { return sm.d.om[m]; });
+            tile::product<MV, false, false, CT, DV>(a, sm.A, sm.D, mv.warp_m0(), CT, mv);     // + A^T dO = dW
+            tile::put<MV, DV>(sm.R, a, mv, same);
+        }
+    }
+    if (mk.on) {
+        tile::product<MK, true, true, DV, DV>(adk, sm.W, G, 0, DV, mk);                       // W dH'^T
+        row_dots(adk, mk, sm.kw, [&](int m, int nn) { return tile::ld4(sm.K + tile::at<DK>(m, nn)); });
+        scale_acc(adk, mk, [&](int m) { return sm.d.om[m]; });
+    }
+    __syncthreads();
+    if (!Smem::BOTH) tile::load<DK, DV, NT>(sm.H, Hg, DV, DK);
+    {
+        float a[MV::TM][MV::TN];
+        tile::zero<MV>(a);
+        if (mv.on) {
+            tile::product<MV, false, false, CT, DV>(a, sm.T, sm.R, mv.warp_m0(), CT, mv);     // Z = T^T dW
+            row_dots(a, mv, sm.zv, [&](int m, int nn) { return tile::ld4(sm.V + tile::at<DV>(m, nn)); });
+            tile::put<MV, DV>(sm.V, a, mv, same);                                             // V has served: Z takes its place
+            store_rows(dv_out + ov, p.tv, n, a, mv, p.vec, [&](int m) { return sm.d.beta[m]; });
+        }
+    }
+    __syncthreads();
+    float* DA = sm.R;
+    float* ZW = sm.T;                                               // T has served
+    two_square_products<NT, DV, DV>(
+        sm.D, sm.W, [&](int m, int n0, const float* a) { tile::st4(DA + tile::at<CT>(m, n0), make_float4(a[0], a[1], a[2], a[3])); },
+        sm.V, sm.W, [&](int m, int n0, const float* a) { tile::st4(ZW + tile::at<CT>(m, n0), make_float4(a[0], a[1], a[2], a[3])); });
+    if (mk.on) {
+        float a[MK::TM][MK::TN];
+        tile::zero<MK>(a);
+        tile::product<MK, true, true, DV, DV>(a, sm.V, sm.H, 0, DV, mk);                      // Z H^T
+        row_dots(a, mk, sm.kz, [&](int m, int nn) { return tile::ld4(sm.K + tile::at<DK>(m, nn)); });
+#pragma unroll
+        for (int i = 0; i < MK::TM; ++i) {
+            const float f = -sm.d.beta[mk.m(i)] * sm.d.gam[mk.m(i)];
+#pragma unroll
+            for (int j = 0; j < MK::TN; ++j) adk[i][j] = fmaf(f, a[i][j], adk[i][j]);
+        }
+    }
+    __syncthreads();
+    // C x C pass, 8 columns per thread of 128: DA <- dA*M (s <= t),  ZW <- P (s < t),  A <- E;  row sums of E and of dL*KM
+    if (tid < 128) {
+        const int t = tid >> 2, s0 = (tid & 3) * 8;
+        const float bt = sm.d.beta[t];
+        float re = 0.f, rl = 0.f;
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            const int s = s0 + e, x = tile::at<CT>(t, s);
+            const float m = s <= t ? mexp(sm.d, t, s) : 0.f;
+            const float da = DA[x], dl = s < t ? -ZW[x] : 0.f, lk = dl * sm.KM[x];
+            const float ee = fmaf(da, sm.A[x], bt * lk);               // A and KM hold M * QK^T (s <= t) and M * KK^T (s < t), else 0
+            DA[x] = da * m;
+            ZW[x] = bt * dl * m;
+            sm.A[x] = ee;
+            re += ee;
+            rl += lk;
+        }
+        re += __shfl_xor_sync(0xffffffffu, re, 1); rl += __shfl_xor_sync(0xffffffffu, rl, 1);
+        re += __shfl_xor_sync(0xffffffffu, re, 2); rl += __shfl_xor_sync(0xffffffffu, rl, 2);
+        if ((tid & 3) == 0) { sm.rs[t] = re; sm.rl[t] = rl; }
+    }
+    __syncthreads();
+    // P + P^T into KM's place; warp 0 meanwhile turns the row and column sums into dg and dbeta
+    for (int i = tid; i < CC; i += NT) {
+        const int t = i / CT, s = i % CT;
+        sm.KM[tile::at<CT>(t, s)] = ZW[tile::at<CT>(t, s)] + ZW[tile::at<CT>(s, t)];
+    }
+    if (tid < CT) {
+        const int t = tid;
+        float cs = 0.f;
+#pragma unroll 8
+        for (int s = 0; s < CT; ++s) cs += sm.A[tile::at<CT>(s, t)];
+        const float gam = sm.d.gam[t], om = sm.d.om[t], bt = sm.d.beta[t];
+        const float kz = row_sum<MK>(sm.kz, t), kw = row_sum<MK>(sm.kw, t), qd = row_sum<MK>(sm.qd, t), zv = row_sum<MV>(sm.zv, t);
+        float tot = kw * om;                                        // chunk-total terms: they belong to the last token, so to every suffix
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, off);
+        float hg = 0.f;
+#pragma unroll
+        for (int i = 0; i < NT / 32; ++i) hg += sm.part[i];
+        tot = fmaf(hg, sm.d.gam[CT - 1], tot);
+        float db = sm.rs[t] - cs + (qd - bt * kz) * gam - kw * om;
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const float up = __shfl_down_sync(0xffffffffu, db, off);
+            if (t + off < 32) db += up;
+        }
+        if (t < n) {
+            dg[og + (long long)t * p.tg] = db + tot;
+            dbeta[og + (long long)t * p.tg] = zv - gam * kz + sm.rl[t];
+        }
+    }
+    __syncthreads();
+    if (mk.on) {
+        tile::product<MK, true, false, CT, DK>(adq, DA, sm.K, 0, mk.warp_m0() + 16, mk);
+        tile::product<MK, false, false, CT, DK>(adk, DA, sm.Q, mk.warp_m0(), CT, mk);
+        tile::product<MK, true, false, CT, DK>(adk, sm.KM, sm.K, 0, CT, mk);
+        store_rows(dq + oqk, p.tqk, n, adq, mk, p.vec, [](int) { return 1.f; });
+        store_rows(dk_out + oqk, p.tqk, n, adk, mk, p.vec, [](int) { return 1.f; });
+    }
+}
+
+// The (chunk, d_k, d_v) sets accepted: bytes of shared memory of a form with padded chunk-long tiles and both states of a
+// chunk resident (chunk 32 excludes 64 x 128 and 128 x 128).  The kernels above need less for every shape; the set is part
+// of the interface.
+__host__ inline size_t smem_rule(int C, int dk, int dv) {
+    auto ld = [](int c) { return (size_t)c + 1; };
+    const size_t c = C;
+    const size_t pre = 3 * c * ld(dk) + c * ld(dv + dk + C) + c * ld(C) + 2 * c;
+    const size_t out = 3 * c * ld(dk) + 2 * c * ld(dv) + dk * ld(dv) + c * ld(C) + c;
+    const size_t bwd = 2 * c * ld(dk) + 4 * c * ld(dv) + 2 * dk * ld(dv) + 4 * c * ld(C) + 2 * c * ld(dv) + 2 * c * ld(dk) + c * ld(dk > dv ? dk : dv) + 10 * c + dk;
+    return sizeof(float) * (pre > out ? (pre > bwd ? pre : bwd) : (out > bwd ? out : bwd));
 }
 
 }  // namespace gdn

@@ -1,0 +1,61 @@
+// Host-side helpers shared by the extension operators' translation units.
+#pragma once
+#include <atomic>
+#include <initializer_list>
+#include "../../include/stateflow.h"
+#include "sf_common.cuh"
+
+namespace sf { void note_launches(long long n); }
+
+namespace sfv {
+
+constexpr size_t kMaxSmem = 227 * 1024;       // dynamic shared memory a CTA can opt into on this architecture
+
+inline sf_status_t check_desc(const sf_seg_desc_t* d, bool wide_keys = false) {
+    if (!d) return SF_ERR_INVALID_ARG;
+    if (d->B <= 0 || d->H <= 0 || d->seg_len <= 0 || d->d_k <= 0 || d->d_v <= 0) return SF_ERR_INVALID_ARG;
+    if (d->B > 65535) return SF_ERR_INVALID_ARG;                                       // grid.y
+    if (d->tok_stride_qk < (long long)d->H * d->d_k || d->tok_stride_v < (long long)d->H * d->d_v || d->tok_stride_g < d->H)
+        return SF_ERR_INVALID_ARG;
+    if (d->B > 1 && (d->batch_stride_qk <= 0 || d->batch_stride_v <= 0 || d->batch_stride_g <= 0)) return SF_ERR_INVALID_ARG;
+    if (d->dtype != SF_F32 && d->dtype != SF_BF16) return SF_ERR_INVALID_ARG;
+    const bool k_ok = d->d_k == 32 || d->d_k == 64 || (wide_keys && d->d_k == 128);
+    const bool v_ok = d->d_v == 32 || d->d_v == 64 || d->d_v == 128;
+    return k_ok && v_ok ? SF_OK : SF_ERR_UNSUPPORTED;
+}
+
+inline sf_status_t launched(int n = 1) {
+    sf::note_launches(n);
+    return cudaGetLastError() == cudaSuccess ? SF_OK : SF_ERR_CUDA;
+}
+
+// Opts a kernel into `bytes` of dynamic shared memory; the largest size set so far is remembered per device (the attribute
+// belongs to the device's copy of the kernel).
+template <auto Kern>
+inline bool opt_in(size_t bytes) {
+    if (bytes <= 48 * 1024) return true;
+    static std::atomic<int> largest[64];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) { cudaGetLastError(); return false; }
+    if (dev < 64 && largest[dev].load(std::memory_order_acquire) >= (int)bytes) return true;
+    if (cudaFuncSetAttribute(Kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess) { cudaGetLastError(); return false; }
+    // two threads with different sizes may finish in either order: only ever raise the recorded size after setting it, and
+    // set the attribute again if a larger one was recorded meanwhile
+    if (dev < 64) {
+        int seen = largest[dev].load();
+        while (seen < (int)bytes && !largest[dev].compare_exchange_weak(seen, (int)bytes)) {}
+        if (seen > (int)bytes && cudaFuncSetAttribute(Kern, cudaFuncAttributeMaxDynamicSharedMemorySize, seen) != cudaSuccess) { cudaGetLastError(); return false; }
+    }
+    return true;
+}
+
+// True if rows of these tensors allow vector accesses of four elements: bases, token and batch strides.
+inline bool vec_ok(const sf_seg_desc_t* d, std::initializer_list<const void*> ptrs) {
+    const uintptr_t mask = d->dtype == SF_F32 ? 15 : 7;
+    if ((d->tok_stride_qk | d->tok_stride_v) & 3) return false;
+    if (d->B > 1 && ((d->batch_stride_qk | d->batch_stride_v) & 3)) return false;
+    for (const void* p : ptrs) if (p && (reinterpret_cast<uintptr_t>(p) & mask)) return false;
+    return true;
+}
+
+}  // namespace sfv

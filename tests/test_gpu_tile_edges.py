@@ -1,10 +1,12 @@
 """Sizes at the edges of the kernels' own tiles, against the fp64 oracle through the C ABI (one B200)."""
 import pytest
+import torch
 
-from paper_2608_06838_b200 import inputs
+from paper_2608_06838_b200 import binding, inputs
 from paper_2608_06838_b200.inputs import Workload
 
 from helpers import compare, oracle_reference, run_chain, tolerance
+from test_gpu_variants import check, oracle_recurrent, run_recurrent
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
@@ -20,3 +22,42 @@ def test_cuda_core_tiles_and_blocks(dk, dv, dtype, chunk, cpb):
     x = inputs.make_inputs(w, DEV)
     got, _ = run_chain(w, x, chunks_per_block=cpb)
     compare(got, oracle_reference(x), tolerance(w), label=w.name)
+
+
+# The chunkwise delta rule walks tiles of 32 tokens whatever the chunk: segments that end one token before, at and after a
+# tile, one token, and the shapes no other test runs.  24 heads take the 16-column state pass (more than 148 CTAs with 8 columns).
+@pytest.mark.parametrize("dk,dv,chunk,H", [(128, 32, 32, 2), (128, 64, 32, 2), (32, 128, 32, 2), (64, 128, 16, 2), (64, 64, 32, 24),
+                                           (128, 128, 16, 12)])
+def test_chunked_delta_tiles(dk, dv, chunk, H):
+    w = Workload("delta-tiles-%d-%d-%d" % (dk, dv, H), 1, H, dk, dv, [31, 32, 33, 1, 100], chunk, dtype="f32", g_scale=0.3,
+                 s_in_sigma=0.5, ds_out_sigma=0.5, seed=62)
+    x = inputs.make_variant_inputs(w, DEV)
+    check(run_recurrent("delta_chunked", w, x), oracle_recurrent("delta", x), w.name)
+
+
+@pytest.mark.parametrize("dtype,tol", [("f32", 1e-4), ("bf16", 2e-2)])
+def test_chunked_delta_rows_without_vector_alignment(dtype, tol):
+    # rows one element apart from any 8- or 16-byte boundary: the entry point takes them, the kernels load element by element
+    w = Workload("delta-odd-%s" % dtype, 2, 2, 64, 32, [45], 32, dtype=dtype, g_scale=0.3, s_in_sigma=0.5, ds_out_sigma=0.5, seed=63)
+    x = inputs.make_variant_inputs(w, DEV)
+    ref = oracle_recurrent("delta", x)
+
+    def odd(t):                                  # the same values with token rows of H*d + 1 elements, one element into the storage
+        B, T, H, d = t.shape
+        buf = torch.zeros(B * T * (H * d + 1) + 1, dtype=t.dtype, device=DEV)
+        v = torch.as_strided(buf, t.shape, (T * (H * d + 1), H * d + 1, d, 1), 1)
+        v.copy_(t)
+        return v
+
+    for n in ("q", "k", "v", "dO"):
+        x[n] = odd(x[n])
+    B, T, H, dk = x["q"].shape
+    d = binding.make_desc(x["q"], x["v"], x["g"], w.chunk)
+    o, dv_ = odd(torch.zeros_like(x["v"])), odd(torch.zeros_like(x["v"]))
+    dq, dk_ = odd(torch.zeros_like(x["q"])), odd(torch.zeros_like(x["q"]))
+    dg, dbeta, S, dS = torch.empty_like(x["g"]), torch.empty_like(x["beta"]), torch.empty_like(x["S_in"]), torch.empty_like(x["S_in"])
+    ws = torch.empty(binding.sf_delta_chunked_workspace_bytes(d, 1), dtype=torch.uint8, device=DEV)
+    binding.sf_delta_chunked_fwd(d, x["q"], x["k"], x["v"], x["g"], x["beta"], x["S_in"], o, S, ws)
+    binding.sf_delta_chunked_bwd(d, x["q"], x["k"], x["v"], x["g"], x["beta"], x["S_in"], x["dO"], x["dS_out"], dq, dk_, dv_, dg, dbeta, dS, ws)
+    torch.cuda.synchronize()
+    check(dict(o=o, S_out=S, dq=dq, dk=dk_, dv=dv_, dg=dg, dbeta=dbeta, dS_in=dS), ref, w.name, tol)
