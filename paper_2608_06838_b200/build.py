@@ -10,7 +10,7 @@ _HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(_HERE, "csrc")
 LIB = os.path.join(_HERE, "libstateflow.so")
 
-SOURCES = ["stateflow.cu", "variants.cu", "delta_chunked.cu"]
+SOURCES = ["stateflow.cu", "variants.cu", "delta_chunked.cu", "channel_chunked.cu"]
 
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC"]

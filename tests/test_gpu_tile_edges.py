@@ -24,23 +24,35 @@ def test_cuda_core_tiles_and_blocks(dk, dv, dtype, chunk, cpb):
     compare(got, oracle_reference(x), tolerance(w), label=w.name)
 
 
-# The chunkwise delta rule walks tiles of 32 tokens whatever the chunk: segments that end one token before, at and after a
-# tile, one token, and the shapes no other test runs.  24 heads take the 16-column state pass (more than 148 CTAs with 8 columns).
+# The chunkwise operators walk tiles of 32 tokens whatever the chunk: segments that end one token before, at and after a
+# tile, inside its first four-token block, one token, and the shapes no other test runs.  24 heads take the delta rule's
+# 16-column state pass (more than 148 CTAs with 8 columns).
+@pytest.mark.parametrize("kind", ["delta", "channel"])
 @pytest.mark.parametrize("dk,dv,chunk,H", [(128, 32, 32, 2), (128, 64, 32, 2), (32, 128, 32, 2), (64, 128, 16, 2), (64, 64, 32, 24),
                                            (128, 128, 16, 12)])
-def test_chunked_delta_tiles(dk, dv, chunk, H):
-    w = Workload("delta-tiles-%d-%d-%d" % (dk, dv, H), 1, H, dk, dv, [31, 32, 33, 1, 100], chunk, dtype="f32", g_scale=0.3,
+def test_chunked_operator_tiles(kind, dk, dv, chunk, H):
+    w = Workload("%s-tiles-%d-%d-%d" % (kind, dk, dv, H), 1, H, dk, dv, [31, 32, 33, 3, 1, 100], chunk, dtype="f32", g_scale=0.3,
                  s_in_sigma=0.5, ds_out_sigma=0.5, seed=62)
     x = inputs.make_variant_inputs(w, DEV)
-    check(run_recurrent("delta_chunked", w, x), oracle_recurrent("delta", x), w.name)
+    check(run_recurrent(kind + "_chunked", w, x), oracle_recurrent(kind, x), w.name)
 
 
-@pytest.mark.parametrize("dtype,tol", [("f32", 1e-4), ("bf16", 2e-2)])
-def test_chunked_delta_rows_without_vector_alignment(dtype, tol):
-    # rows one element apart from any 8- or 16-byte boundary: the entry point takes them, the kernels load element by element
-    w = Workload("delta-odd-%s" % dtype, 2, 2, 64, 32, [45], 32, dtype=dtype, g_scale=0.3, s_in_sigma=0.5, ds_out_sigma=0.5, seed=63)
+def test_chunked_diagonal_decay_with_wiped_channels():
+    # channels that forget everything at some tokens: exponents down to -3000 inside a tile, every factor must stay finite
+    w = Workload("channel-wipe", 1, 2, 64, 64, [100, 64], 32, dtype="f32", g_scale=0.05, s_in_sigma=0.5, ds_out_sigma=0.5, seed=64)
     x = inputs.make_variant_inputs(w, DEV)
-    ref = oracle_recurrent("delta", x)
+    x["g_channel"][:, 37, :, ::3] = -100.0
+    x["g_channel"][:, 40:70, :, 1] = -100.0
+    check(run_recurrent("channel_chunked", w, x), oracle_recurrent("channel", x), w.name)
+
+
+@pytest.mark.parametrize("kind", ["delta", "channel"])
+@pytest.mark.parametrize("dtype,tol", [("f32", 1e-4), ("bf16", 2e-2)])
+def test_chunked_operator_rows_without_vector_alignment(kind, dtype, tol):
+    # rows one element apart from any 8- or 16-byte boundary: the entry points take them, the kernels load element by element
+    w = Workload("%s-odd-%s" % (kind, dtype), 2, 2, 64, 32, [45], 32, dtype=dtype, g_scale=0.3, s_in_sigma=0.5, ds_out_sigma=0.5, seed=63)
+    x = inputs.make_variant_inputs(w, DEV)
+    ref = oracle_recurrent(kind, x)
 
     def odd(t):                                  # the same values with token rows of H*d + 1 elements, one element into the storage
         B, T, H, d = t.shape
@@ -49,15 +61,21 @@ def test_chunked_delta_rows_without_vector_alignment(dtype, tol):
         v.copy_(t)
         return v
 
-    for n in ("q", "k", "v", "dO"):
+    for n in ("q", "k", "v", "dO", "g_channel"):
         x[n] = odd(x[n])
-    B, T, H, dk = x["q"].shape
-    d = binding.make_desc(x["q"], x["v"], x["g"], w.chunk)
-    o, dv_ = odd(torch.zeros_like(x["v"])), odd(torch.zeros_like(x["v"]))
-    dq, dk_ = odd(torch.zeros_like(x["q"])), odd(torch.zeros_like(x["q"]))
-    dg, dbeta, S, dS = torch.empty_like(x["g"]), torch.empty_like(x["beta"]), torch.empty_like(x["S_in"]), torch.empty_like(x["S_in"])
-    ws = torch.empty(binding.sf_delta_chunked_workspace_bytes(d, 1), dtype=torch.uint8, device=DEV)
-    binding.sf_delta_chunked_fwd(d, x["q"], x["k"], x["v"], x["g"], x["beta"], x["S_in"], o, S, ws)
-    binding.sf_delta_chunked_bwd(d, x["q"], x["k"], x["v"], x["g"], x["beta"], x["S_in"], x["dO"], x["dS_out"], dq, dk_, dv_, dg, dbeta, dS, ws)
+    q, k, v, dO, S_in, dS_out = (x[n] for n in ("q", "k", "v", "dO", "S_in", "dS_out"))
+    d = binding.make_desc(q, v, x["g"], w.chunk)
+    o, dv_, dq, dk_ = (odd(torch.zeros_like(t)) for t in (v, v, q, k))
+    dbeta, S, dS = torch.empty_like(x["beta"]), torch.empty_like(S_in), torch.empty_like(S_in)
+    if kind == "delta":
+        dg = torch.empty_like(x["g"])
+        ws = torch.empty(binding.sf_delta_chunked_workspace_bytes(d, 1), dtype=torch.uint8, device=DEV)
+        binding.sf_delta_chunked_fwd(d, q, k, v, x["g"], x["beta"], S_in, o, S, ws)
+        binding.sf_delta_chunked_bwd(d, q, k, v, x["g"], x["beta"], S_in, dO, dS_out, dq, dk_, dv_, dg, dbeta, dS, ws)
+    else:
+        dg = odd(torch.zeros_like(x["g_channel"]))
+        ws = torch.empty(binding.sf_channel_chunked_workspace_bytes(d, 1), dtype=torch.uint8, device=DEV)
+        binding.sf_channel_chunked_fwd(d, q, k, v, x["g_channel"], S_in, o, S, ws)
+        binding.sf_channel_chunked_bwd(d, q, k, v, x["g_channel"], S_in, dO, dS_out, dq, dk_, dv_, dg, dS, ws)
     torch.cuda.synchronize()
     check(dict(o=o, S_out=S, dq=dq, dk=dk_, dv=dv_, dg=dg, dbeta=dbeta, dS_in=dS), ref, w.name, tol)
