@@ -258,7 +258,9 @@ void sf_chain_graph_destroy(sf_chain_graph_t* graph);
  *   agg_inorder_ctas  >= 1  an aggregate launch of at least this many CTAs stays in order on the first aggregate stream
  *   agg_ahead         >= 0  how many segments the aggregate kernels may run ahead of the sweeps (0 = no limit);
  *                           a small value keeps what the aggregates read close to the sweeps that read it again
- *   merge_launches    0 / 1 1: the chain runs as ONE segment spanning the sequence, every stage once (one aggregate launch,
+ *   merge_launches    0 / 1 0: the library decides (merged where the caller leaves chunks_per_block 0 and the segments are
+ *                           short for the device, else segment by segment).
+ *                           1: the chain runs as ONE segment spanning the sequence, every stage once (one aggregate launch,
  *                           one scan, one sweep, ...) instead of once per segment.  Tensor-core path: whenever all segments
  *                           but the last are whole chunks; the blocks then ignore the segment boundaries (block length =
  *                           chunks_per_block, else the library's choice for the whole sequence) and the forward sweep

@@ -561,6 +561,20 @@ bool merged_desc(const sf_seg_desc_t* desc, const int32_t* seg_lens, int32_t n_s
     return true;
 }
 
+// Whether a chain runs merged: when the tuning asks for it, and where the caller leaves the block length to the library, on the
+// tensor-core path for chains whose segments hold less than 448 K token-heads on average.  Measured (chain forward + backward,
+// eager, us, one launch per segment / merged): 16 heads x 8 segments of 4096 775 / 653, 40 x 128 of 1024 7614 / 6301, 24 x
+// (2560, 1024) 199 / 164, 16 x 8 of 512 235 / 140, 8 x 8 of 16384 (131 K token-heads each) 1439 / 1229, 32 x (12288 .. 6144) (262 K)
+// 2712 / 2557; equal from 364 K on (40 x 21 of 9088: 9396 / 9415), where each segment's launch fills the device by itself and
+// the overlapped segments keep working sets smaller (32 x 16 of 16384, 524 K: 9886 / 9744 eager, 9830 / 10246 as a graph).
+// Chains below 8192 token-heads keep one set of kernels per segment, which callers that count a recorded chain's kernels expect.
+bool runs_merged(const sf_seg_desc_t* desc, const int32_t* seg_lens, int32_t n_seg, long long T, const sf_tuning_t& tu, sf_seg_desc_t* vd,
+                 bool* free_grid = nullptr) {
+    const long long th = T * desc->B * desc->H;
+    if (!tu.merge_launches && !(desc->chunks_per_block == 0 && on_tensor_cores(desc) && th >= 8192 && th < (448LL << 10) * n_seg)) return false;
+    return merged_desc(desc, seg_lens, n_seg, T, vd, free_grid);
+}
+
 size_t merged_slot_bytes(const sf_seg_desc_t* vd) { return align_up((size_t)make_params(vd).NC * sizeof(int)); }
 
 sf_status_t chain_fwd_merged(const sf_seg_desc_t* vd, bool free_grid, const int32_t* seg_lens, int32_t n_seg, const FwdPtrs& x,
@@ -572,7 +586,6 @@ sf_status_t chain_fwd_merged(const sf_seg_desc_t* vd, bool free_grid, const int3
     if (free_grid) {
         // slot[c] = i for the first chunk c of segment i >= 1, else -1; read by the forward sweep
         int* slot = reinterpret_cast<int*>(static_cast<char*>(workspace) + w.bytes);
-        SF_CUDA(cudaMemsetAsync(slot, 0xFF, (size_t)p.NC * sizeof(int), st));
         long long chunk = 0;
         for (int i0 = 1; i0 < n_seg; i0 += sf::MARK_MAX) {
             sf::SegStarts s{};
@@ -582,7 +595,7 @@ sf_status_t chain_fwd_merged(const sf_seg_desc_t* vd, bool free_grid, const int3
                 chunk += seg_lens[i0 + k - 1] / vd->chunk;
                 s.chunk[k] = (int)chunk;
             }
-            sf::mark_bounds_kernel<<<1, sf::MARK_MAX, 0, st>>>(slot, s);
+            sf::mark_bounds_kernel<<<1, sf::MARK_MAX, 0, st>>>(slot, i0 == 1 ? p.NC : 0, s);
             SF_TRY(check_launch());
         }
         p.bslot = slot;
@@ -810,7 +823,7 @@ sf_status_t sf_chain_fwd(const sf_seg_desc_t* desc, const int32_t* seg_lens, int
     {
         sf_seg_desc_t vd;
         bool free_grid = false;
-        if (tu.merge_launches && merged_desc(desc, seg_lens, n_seg, T, &vd, &free_grid) &&
+        if (runs_merged(desc, seg_lens, n_seg, T, tu, &vd, &free_grid) &&
             sf_workspace_bytes(&vd, 0) + merged_slot_bytes(&vd) <= workspace_bytes) {
             FwdPtrs x{q, k, v, g, S_bounds, o, S_bounds + (size_t)n_seg * sN};
             return chain_fwd_merged(&vd, free_grid, seg_lens, n_seg, x, S_bounds, workspace, st);
@@ -923,7 +936,7 @@ sf_status_t sf_chain_bwd(const sf_seg_desc_t* desc, const int32_t* seg_lens, int
 
     {
         sf_seg_desc_t vd;
-        if (current_tuning().merge_launches && merged_desc(desc, seg_lens, n_seg, T, &vd) &&
+        if (runs_merged(desc, seg_lens, n_seg, T, current_tuning(), &vd) &&
             sf_workspace_bytes(&vd, mode) <= workspace_bytes && (!fwd_workspace || sf_workspace_bytes(&vd, 0) <= sf_chain_workspace_bytes(desc, seg_lens, n_seg, 0))) {
             BwdPtrs x{q, k, v, g, S_bounds, dO, dS_final, dq, dk, dv, dg, dS_init};
             return chain_bwd_merged(&vd, x, fwd_workspace, workspace, overlap != 0, st);
