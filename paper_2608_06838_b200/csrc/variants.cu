@@ -1,5 +1,6 @@
 // C ABI of the extension operators: diagonal decay, gated delta rule, short convolution with a carried tail.
 // Argument checks happen before any launch; nothing here allocates, synchronises or falls back to the host.
+#include <algorithm>
 #include <type_traits>
 #include "../../include/stateflow.h"
 #include "sf_recurrent.cuh"
@@ -98,11 +99,10 @@ sf_status_t check_conv(int32_t B, int32_t L, int32_t C, int32_t W) {
     return SF_OK;
 }
 
-// Launch shape of the row-walking convolution kernels over `rows` rows: V channels per thread (4 when the channel
-// count and every pointer allow 16-byte accesses).
-bool conv_vec4(int C, std::initializer_list<const void*> ptrs) {
-    if (C % 4) return false;
-    for (const void* p : ptrs) if (p && (reinterpret_cast<uintptr_t>(p) & 15u)) return false;
+// True if V channels at a time can be accessed at once: the channel count and every pointer allow it.
+bool conv_vec(int V, int C, std::initializer_list<const void*> ptrs) {
+    if (C % V) return false;
+    for (const void* p : ptrs) if (p && (reinterpret_cast<uintptr_t>(p) & (4u * V - 1))) return false;
     return true;
 }
 // Calls f with the convolution width as a compile-time constant (1 .. CONV_MAXW, checked before).
@@ -122,6 +122,43 @@ void conv_width_switch(int W, F&& f) {
 dim3 conv_grid(int B, long long rows, int C, int V) {
     const int groups = (C + V - 1) / V;
     return dim3((unsigned)((groups + 31) / 32), (unsigned)((rows + 8LL * sf::rec::CONV_TS - 1) / (8LL * sf::rec::CONV_TS)), (unsigned)B);
+}
+
+// One cluster per group of channels: 8 CTAs where that fills the device (a portable size), else 16; fewer when there are not
+// enough rows for all of their row slices.
+template <int V, int W>
+bool launch_conv_bwd(int B, int L, int C, const float* x, const float* w, const float* tail_in, const float* dy, const float* dtail_out,
+                     float* dx, float* dw, float* dtail_in, cudaStream_t st) {
+    using namespace sf::rec;
+    constexpr int LN = kConvLanes<V>, SL = CONV_NT / LN;
+    auto kern = conv_bwd_kernel<V, W>;
+    const int groups = (C + LN * V - 1) / (LN * V);
+    const long long units = (long long)B * ((L + W - 1 + CONV_UNIT_MIN - 1) / CONV_UNIT_MIN);
+    int cluster = groups >= 148 / 8 ? 8 : 16;
+    while (cluster > 1 && (long long)(cluster / 2) * SL >= units) cluster /= 2;
+    // unit length: one unit per row slice where a batch has enough rows (every unit begins with W - 1 rows of both windows)
+    const long long rows = (long long)L + W - 1, slices = ((long long)cluster * SL + B - 1) / B;
+    const int unit = (int)std::max<long long>(CONV_UNIT_MIN, (rows + slices - 1) / slices);
+    if (cluster > 8) {
+        static std::atomic<unsigned long long> done{0};          // per device
+        int dev = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess) return false;
+        const unsigned long long bit = dev < 64 ? 1ull << dev : 0;
+        if (!(done.load() & bit)) {
+            if (cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return false;
+            done.fetch_or(bit);
+        }
+    }
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)groups, (unsigned)cluster);
+    cfg.blockDim = dim3(CONV_NT);
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = 1; at[0].val.clusterDim.y = (unsigned)cluster; at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, B, L, C, x, w, tail_in, dy, dtail_out, dx, dw, dtail_in, unit) == cudaSuccess;
 }
 
 }  // namespace
@@ -163,7 +200,7 @@ sf_status_t sf_conv_segment_fwd(int32_t B, int32_t L, int32_t C, int32_t W, cons
     if (c != SF_OK) return c;
     if (!x || !w || !y || (W > 1 && !tail_out) || (tail_in && tail_in == tail_out)) return SF_ERR_INVALID_ARG;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    const bool v4 = conv_vec4(C, {x, w, tail_in, y, tail_out});
+    const bool v4 = conv_vec(4, C, {x, w, tail_in, y, tail_out});
     const dim3 grid = conv_grid(B, L, C, v4 ? 4 : 1), block(32, 8);
     conv_width_switch(W, [&](auto wc) {
         constexpr int Wc = decltype(wc)::value;
@@ -180,20 +217,16 @@ sf_status_t sf_conv_segment_bwd(int32_t B, int32_t L, int32_t C, int32_t W, cons
     if (c != SF_OK) return c;
     if (!x || !w || !dy || !dx || !dw || (W > 1 && !dtail_in) || (dtail_out && dtail_out == dtail_in)) return SF_ERR_INVALID_ARG;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    const long long rows = (long long)L + W - 1;
-    const bool v4 = conv_vec4(C, {w, dy, dtail_out, dx, dtail_in});
-    const dim3 grid = conv_grid(B, rows, C, v4 ? 4 : 1), block(32, 8);
+    const bool v2 = conv_vec(2, C, {x, w, tail_in, dy, dtail_out, dx, dtail_in});
+    bool ok = true;
     conv_width_switch(W, [&](auto wc) {
         constexpr int Wc = decltype(wc)::value;
-        if (v4) sf::rec::conv_bwd_input_kernel<4, Wc><<<grid, block, 0, st>>>(B, L, C, w, dy, dtail_out, dx, dtail_in);
-        else    sf::rec::conv_bwd_input_kernel<1, Wc><<<grid, block, 0, st>>>(B, L, C, w, dy, dtail_out, dx, dtail_in);
+        constexpr int V = Wc <= 6 ? 2 : 1;                       // two channels per thread as far as the windows stay in registers
+        ok = v2 ? launch_conv_bwd<V, Wc>(B, L, C, x, w, tail_in, dy, dtail_out, dx, dw, dtail_in, st)
+                : launch_conv_bwd<1, Wc>(B, L, C, x, w, tail_in, dy, dtail_out, dx, dw, dtail_in, st);
     });
-    if (cudaGetLastError() != cudaSuccess) return SF_ERR_CUDA;
-    conv_width_switch(W, [&](auto wc) {
-        sf::rec::conv_bwd_weight_kernel<decltype(wc)::value><<<dim3((C + sf::rec::CONV_WC - 1) / sf::rec::CONV_WC),
-                                                                 dim3(sf::rec::CONV_WC, sf::rec::CONV_WT), 0, st>>>(B, L, C, x, tail_in, dy, dw);
-    });
-    return launched(2);
+    if (!ok) { cudaGetLastError(); return SF_ERR_CUDA; }
+    return launched();
 }
 
 }  // extern "C"
