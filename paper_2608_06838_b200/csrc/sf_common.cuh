@@ -25,6 +25,12 @@ struct SegParams {
     const int* bslot;
     float* bbase;
     long long bstride;
+    // A segment of one block needs no aggregate and no scan: with `single` set the sweeps start from s_init [B,H,d_k,d_v] (NULL:
+    // zero) instead of the workspace's block states, and store the state (gradient) that leaves the block to s_final and, if
+    // given, the one that entered it to s_copy.
+    int single;
+    const float* s_init;
+    float *s_final, *s_copy;
 };
 
 // Error codes written to the device status word by kernels whose bounded waits run out.

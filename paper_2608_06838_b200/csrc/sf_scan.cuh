@@ -147,12 +147,12 @@ __global__ void __launch_bounds__(DG_NT) dg_epilogue_kernel(SegParams p, int m, 
     const long long bh = (long long)b * p.H + h;
     const int C = p.C;
     const int c0 = j * p.R, nch = min(p.R, p.NC - c0);
-    const float* Hj = Hs + (bh * p.NB + j) * (long long)m;
+    const float* Hj = Hs ? Hs + (bh * p.NB + j) * (long long)m : nullptr;       // NULL: states of zeros
     const float* Gin = (j == 0) ? (dS_in + bh * (long long)m) : (Gs + (bh * p.NB + (j - 1)) * (long long)m);
 
     // anchor: fixed-order tree reduction so that the result is reproducible run to run
     float part = 0.f;
-    for (int e = threadIdx.x * 4; e < m; e += DG_NT * 4) {
+    if (Hj) for (int e = threadIdx.x * 4; e < m; e += DG_NT * 4) {
         const float4 hv = *reinterpret_cast<const float4*>(Hj + e);
         const float4 gv = *reinterpret_cast<const float4*>(Gin + e);
         part = fmaf(hv.x, gv.x, part); part = fmaf(hv.y, gv.y, part);

@@ -231,9 +231,9 @@ __device__ __forceinline__ void mask_pass(uint32_t sc, const float* bch, unsigne
 // accumulator at TMEM columns `acc`; the thread owns lane a = threadIdx.x & 127.  Writes the bf16 copy
 // of the state to `sb` (two boxes of [128 rows x 64 columns], 16 KB apart) and scales the accumulator
 // by `decay`.  If init != nullptr the state is taken from global memory (init[a*128 + i], or
-// init[i*128 + a] when `transposed`) instead of TMEM.
+// init[i*128 + a] when `transposed`) instead of TMEM; `first` without it means a state of zeros.
 template <int NU>
-__device__ __forceinline__ void state_pass(uint32_t acc, unsigned char* sb, float decay, const float* __restrict__ init, bool transposed,
+__device__ __forceinline__ void state_pass(uint32_t acc, unsigned char* sb, float decay, bool first, const float* __restrict__ init, bool transposed,
                                            int u0, float* __restrict__ dump = nullptr) {
     const int a = threadIdx.x & 127, warp = a >> 5;
     const uint32_t taddr = acc + ((uint32_t)(warp * 32) << 16);
@@ -242,7 +242,12 @@ __device__ __forceinline__ void state_pass(uint32_t acc, unsigned char* sb, floa
     for (int k0 = 0; k0 < NU; k0 += 2) {
         const int nk = (NU - k0) < 2 ? (NU - k0) : 2;
         float v[2][16];
-        if (init) {
+        if (first && !init) {
+#pragma unroll
+            for (int k = 0; k < 2; ++k)
+#pragma unroll
+                for (int i = 0; i < 16; ++i) v[k][i] = 0.f;
+        } else if (first) {
 #pragma unroll
             for (int k = 0; k < 2; ++k) {
                 if (k < nk) {
@@ -292,6 +297,23 @@ __device__ __forceinline__ void state_pass(uint32_t acc, unsigned char* sb, floa
         }
     }
     ptx::tmem_st_wait();
+}
+
+// Rows of the [128 x 128] float32 accumulator at TMEM columns `acc` to a dense array: NU units of 16 columns from u0 on, the
+// thread owns lane threadIdx.x & 127.
+template <int NU>
+__device__ __forceinline__ void state_out(uint32_t acc, float* __restrict__ dst, int u0) {
+    const int a = threadIdx.x & 127;
+    const uint32_t taddr = acc + ((uint32_t)((a >> 5) * 32) << 16);
+#pragma unroll
+    for (int k = 0; k < NU; ++k) {
+        float v[16];
+        ptx::tmem_ld16(taddr + (u0 + k) * 16, v);
+        ptx::tmem_ld_wait();
+        float4* o4 = reinterpret_cast<float4*>(dst + a * D + (u0 + k) * 16);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) o4[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+    }
 }
 
 // Weighted copy of one [64 x 64] box: dst = diag(w) src, by the 128 threads of a warpgroup (t = 0..127);
@@ -649,8 +671,9 @@ __device__ __forceinline__ void sweep_body(const CUtensorMap* tmQ, const CUtenso
             }
         }
     } else if (warp < 16) {
-        const float* H0 = Hs + (((long long)b * p.H + h) * p.NB + j) * (long long)(D * D);
-        ptx::prefetch_l2(H0 + tid * 32);                 // the block's initial state (512 lines) is on its way while the tables are built
+        const long long bh = ((long long)b * p.H + h) * (long long)(D * D);
+        const float* H0 = p.single ? (p.s_init ? p.s_init + bh : nullptr) : Hs + bh * p.NB + (long long)j * (D * D);
+        if (H0) ptx::prefetch_l2(H0 + tid * 32);                 // the block's initial state (512 lines) is on its way while the tables are built
         prep_decay(g + (long long)b * p.bg + h, p.tg, t0, nch, p.L, sm.bloc, sm.ctot, 16, &sm.g_issued);
         ptx::named_bar_sync(1, 512);
         const int wg = warp >> 2, t = tid & 127;
@@ -698,7 +721,8 @@ __device__ __forceinline__ void sweep_body(const CUtensorMap* tmQ, const CUtenso
                 const float* bch = sm.bloc + c * C;
                 const float bC = sm.ctot[c];
                 float* dump = nullptr;                   // merged launches: the state entering a segment's first chunk goes out
-                if (!DQ && p.bslot) {
+                if (!DQ && c == 0 && p.single && p.s_copy) dump = p.s_copy + bh;
+                else if (!DQ && p.bslot) {
                     const int slot = __ldg(p.bslot + c0 + c);
                     if (slot >= 0) dump = p.bbase + slot * p.bstride + ((long long)b * p.H + h) * (long long)(D * D);
                 }
@@ -706,8 +730,8 @@ __device__ __forceinline__ void sweep_body(const CUtensorMap* tmQ, const CUtenso
                 if (c > 0) SF_WAIT(&sm.st_done, (c - 1) & 1, DEV_TIMEOUT_MMA);
                 ptx::tc_fence_after_sync();
                 // 16-column units: WG0 0-2, WG1 3-5, WG2 6-7
-                if (wg < 2) state_pass<3>(tmem + T_ST, sm.sb, fast_exp(bC), c == 0 ? H0 : nullptr, DQ, 3 * wg, dump);
-                else        state_pass<2>(tmem + T_ST, sm.sb, fast_exp(bC), c == 0 ? H0 : nullptr, DQ, 6, dump);
+                if (wg < 2) state_pass<3>(tmem + T_ST, sm.sb, fast_exp(bC), c == 0, H0, DQ, 3 * wg, dump);
+                else        state_pass<2>(tmem + T_ST, sm.sb, fast_exp(bC), c == 0, H0, DQ, 6, dump);
                 ptx::fence_proxy_async();
                 ptx::tc_fence_before_sync();
                 ptx::mbar_arrive_warp(&sm.st_ready);
@@ -717,6 +741,12 @@ __device__ __forceinline__ void sweep_body(const CUtensorMap* tmQ, const CUtenso
                     ptx::mbar_arrive_warp(&sm.w_ready);
                 }
                 if (wg == 2 && c + 1 < nch) mask(c + 1);
+            }
+            if (!DQ && p.single) {                       // the state leaving the segment
+                SF_WAIT(&sm.st_done, (nch - 1) & 1, DEV_TIMEOUT_MMA);
+                ptx::tc_fence_after_sync();
+                if (wg < 2) state_out<3>(tmem + T_ST, p.s_final + bh, 3 * wg);
+                else        state_out<2>(tmem + T_ST, p.s_final + bh, 6);
             }
         }
     }
@@ -865,8 +895,9 @@ __device__ __forceinline__ void dkdv_body(const CUtensorMap* tmQ, const CUtensor
             }
         }
     } else if (warp < 16) {
-        const float* G0 = Gs + (((long long)b * p.H + h) * p.NB + j) * (long long)(D * D);
-        ptx::prefetch_l2(G0 + tid * 32);                 // the block's incoming state gradient, on its way while the tables are built
+        const long long bh = ((long long)b * p.H + h) * (long long)(D * D);
+        const float* G0 = p.single ? (p.s_init ? p.s_init + bh : nullptr) : Gs + bh * p.NB + (long long)j * (D * D);
+        if (G0) ptx::prefetch_l2(G0 + tid * 32);                 // the block's incoming state gradient, on its way while the tables are built
         prep_decay(g + (long long)b * p.bg + h, p.tg, t0, nch, p.L, sm.bloc, sm.ctot, 16, &sm.g_issued);
         ptx::named_bar_sync(1, 512);
         const int wg = warp >> 2, t = tid & 127;
@@ -923,13 +954,18 @@ __device__ __forceinline__ void dkdv_body(const CUtensorMap* tmQ, const CUtensor
                 // after every MMA that read them
                 if (i > 0) SF_WAIT(&sm.st_done[(i - 1) & 1], ((i - 1) >> 1) & 1, DEV_TIMEOUT_MMA);
                 ptx::tc_fence_after_sync();
-                state_pass<4>(tmem + T_G, sm.gb, fast_exp(sm.ctot[c]), i == 0 ? G0 : nullptr, false, 4 * wg);
+                state_pass<4>(tmem + T_G, sm.gb, fast_exp(sm.ctot[c]), i == 0, G0, false, 4 * wg);
                 ptx::fence_proxy_async();
                 ptx::tc_fence_before_sync();
                 ptx::mbar_arrive_warp(&sm.st_ready);
                 scale_box(sm.qw + wg * BOX, sm.tiles[s][0] + wg * BOX, t, [&](int row) { return fast_exp(bch[row]); });
                 ptx::fence_proxy_async();
                 ptx::mbar_arrive_warp(&sm.w_ready);
+            }
+            if (p.single) {                              // the gradient of the state entering the segment
+                SF_WAIT(&sm.st_done[(nch - 1) & 1], ((nch - 1) >> 1) & 1, DEV_TIMEOUT_MMA);
+                ptx::tc_fence_after_sync();
+                state_out<4>(tmem + T_G, p.s_final + bh, 4 * wg);
             }
         }
     }

@@ -103,7 +103,8 @@ int sm_count() {
 }
 
 // Block length when the caller leaves it open: one CTA per (batch, head, block) and one CTA per SM, so a
-// kernel takes waves * (chunks per block + a fixed per-CTA cost of about six chunk times).  Pick the
+// kernel takes waves * (chunks per block + a fixed per-CTA cost of about six chunk times); more than one block adds the
+// aggregate and the scan, about four chunk times (a segment of one block needs neither, see one_block()).  Pick the
 // length in [4, 64] that minimises this; ties go to the longer block (fewer block states in HBM).
 int auto_chunks_per_block(int NC, long long bh) {
     const int sms = sm_count();
@@ -113,7 +114,7 @@ int auto_chunks_per_block(int NC, long long bh) {
         const int reff = r < NC ? r : NC;
         const long long nb = (NC + reff - 1) / reff;
         const long long waves = (nb * bh + sms - 1) / sms;
-        const long long cost = waves * (reff + 6);
+        const long long cost = waves * (reff + 6) + (nb > 1 ? 4 : 0);
         if (best_cost < 0 || cost <= best_cost) { best_cost = cost; best = reff; }
         if (r >= NC) break;
     }
@@ -174,6 +175,7 @@ SegParams make_params(const sf_seg_desc_t* d, int cpb_override = 0) {
     p.tqk = d->tok_stride_qk; p.tv = d->tok_stride_v; p.tg = d->tok_stride_g;
     p.bqk = d->batch_stride_qk; p.bv = d->batch_stride_v; p.bg = d->batch_stride_g;
     p.bslot = nullptr; p.bbase = nullptr; p.bstride = 0;
+    p.single = 0; p.s_init = nullptr; p.s_final = p.s_copy = nullptr;
     return p;
 }
 
@@ -401,6 +403,48 @@ sf_status_t bwd_dg(const sf_seg_desc_t* d, const SegParams& p, const BwdPtrs& x,
     dim3 grid(p.NB, p.H, p.B);
     sf::dg_epilogue_kernel<<<grid, sf::DG_NT, 0, st>>>(p, d->d_k * d->d_v, w.xq, w.xk, Hs, w.GU, x.dS_in, x.dg);
     return check_launch();
+}
+
+// A segment of one block on the tensor-core path: the sweeps start from the boundary state itself and store the state that
+// leaves, so the aggregate and the scan (two launches of 4-9 us each way, and their passes over k, v, q, dO) are left out.
+// The forward keeps the entering state in the workspace for the backward, as the scan would.
+// 200 tokens x 16 heads, forward: 27.6 -> 20.5 us.
+bool one_block(Path path, const SegParams& p) { return path == Path::Tc && p.NB == 1; }
+
+sf_status_t segment_fwd(Path path, const sf_seg_desc_t* d, const SegParams& p, const FwdPtrs& x, const FwdWs& w, cudaStream_t st) {
+    if (one_block(path, p)) {
+        SegParams s = p;
+        s.single = 1; s.s_init = x.S_in; s.s_final = x.S_out; s.s_copy = w.UH;
+        return fwd_out(path, d, s, x, w, st);
+    }
+    SF_TRY(fwd_pre(path, d, p, x, w, st));
+    SF_TRY(fwd_scan(d, p, x, w, st));
+    return fwd_out(path, d, p, x, w, st);
+}
+
+// `saved`: the forward's workspace, or NULL to replay the block states into replay (its state-out goes to sfin).
+sf_status_t segment_bwd(Path path, const sf_seg_desc_t* d, const SegParams& p, const BwdPtrs& x, const BwdWs& w, const FwdWs* saved,
+                        const FwdWs& replay, float* sfin, cudaStream_t st) {
+    if (one_block(path, p)) {
+        const float* H = saved ? saved->UH : x.S_in;
+        SegParams s = p;
+        s.single = 1; s.s_init = H;
+        SF_TRY(bwd_dq(path, d, s, x, w, nullptr, st));
+        s.s_init = x.dS_out; s.s_final = x.dS_in;
+        SF_TRY(bwd_dkdv(path, d, s, x, w, st));
+        return bwd_dg(d, p, x, w, H, st);
+    }
+    if (!saved) {
+        FwdPtrs fx{x.q, x.k, x.v, x.g, x.S_in, nullptr, sfin};               // SR: block-entering states from S_in
+        SF_TRY(fwd_pre(path, d, p, fx, replay, st));
+        SF_TRY(fwd_scan(d, p, fx, replay, st));
+        saved = &replay;
+    }
+    SF_TRY(bwd_pre(path, d, p, x, w, nullptr, st));
+    SF_TRY(bwd_scan(d, p, x, w, saved->beta, st));
+    SF_TRY(bwd_dq(path, d, p, x, w, saved->UH, st));
+    SF_TRY(bwd_dkdv(path, d, p, x, w, st));
+    return bwd_dg(d, p, x, w, saved->UH, st);
 }
 
 sf_status_t validate_fwd(const sf_seg_desc_t* d, const FwdPtrs& x, const void* ws, size_t ws_bytes, Path* path) {
@@ -696,11 +740,7 @@ sf_status_t sf_segment_fwd(const sf_seg_desc_t* desc, const void* q, const void*
     SF_TRY(validate_fwd(desc, x, workspace, workspace_bytes, &path));
     const SegParams p = make_params(desc);
     const FwdWs w = fwd_ws(desc, p, workspace);
-    cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    SF_TRY(fwd_pre(path, desc, p, x, w, st));
-    SF_TRY(fwd_scan(desc, p, x, w, st));
-    SF_TRY(fwd_out(path, desc, p, x, w, st));
-    return SF_OK;
+    return segment_fwd(path, desc, p, x, w, reinterpret_cast<cudaStream_t>(stream));
 }
 
 sf_status_t sf_segment_bwd(const sf_seg_desc_t* desc, const void* q, const void* k, const void* v, const float* g,
@@ -712,24 +752,13 @@ sf_status_t sf_segment_bwd(const sf_seg_desc_t* desc, const void* q, const void*
     const SegParams p = make_params(desc);
     const BwdWs w = bwd_ws(desc, p, workspace);
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    FwdWs fw;
     if (fwd_saved) {
-        fw = fwd_ws(desc, p, const_cast<void*>(fwd_saved));
-    } else {
-        // SR: replay the block-entering states from S_in
-        char* base = static_cast<char*>(workspace) + w.bytes;
-        fw = fwd_ws(desc, p, base);
-        float* sfin = reinterpret_cast<float*>(base + fw.bytes);
-        FwdPtrs fx{q, k, v, g, S_in, nullptr, sfin};
-        SF_TRY(fwd_pre(path, desc, p, fx, fw, st));
-        SF_TRY(fwd_scan(desc, p, fx, fw, st));
+        const FwdWs fw = fwd_ws(desc, p, const_cast<void*>(fwd_saved));
+        return segment_bwd(path, desc, p, x, w, &fw, fw, nullptr, st);
     }
-    SF_TRY(bwd_pre(path, desc, p, x, w, nullptr, st));
-    SF_TRY(bwd_scan(desc, p, x, w, fw.beta, st));
-    SF_TRY(bwd_dq(path, desc, p, x, w, fw.UH, st));
-    SF_TRY(bwd_dkdv(path, desc, p, x, w, st));
-    SF_TRY(bwd_dg(desc, p, x, w, fw.UH, st));
-    return SF_OK;
+    char* base = static_cast<char*>(workspace) + w.bytes;
+    const FwdWs fw = fwd_ws(desc, p, base);
+    return segment_bwd(path, desc, p, x, w, nullptr, fw, reinterpret_cast<float*>(base + fw.bytes), st);
 }
 
 sf_status_t sf_segment_fwd_static(const sf_seg_desc_t* desc, const void* q, const void* k, const void* v, const float* g,

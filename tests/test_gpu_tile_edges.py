@@ -79,3 +79,25 @@ def test_chunked_operator_rows_without_vector_alignment(kind, dtype, tol):
         binding.sf_channel_chunked_bwd(d, q, k, v, x["g_channel"], S_in, dO, dS_out, dq, dk_, dv_, dg, dS, ws)
     torch.cuda.synchronize()
     check(dict(o=o, S_out=S, dq=dq, dk=dk_, dv=dv_, dg=dg, dbeta=dbeta, dS_in=dS), ref, w.name, tol)
+
+
+# Tensor-core segments of one block start from the boundary state itself (no aggregate, no scan): one token, one chunk and its
+# neighbours, the longest one-block segment of the library's choice, a longer one by request; boundary states present and absent.
+@pytest.mark.parametrize("L,cpb", [(1, 0), (63, 0), (64, 0), (65, 0), (500, 0), (512, 0), (1100, 18)])
+@pytest.mark.parametrize("states", [True, False])
+@pytest.mark.parametrize("saved", [True, False])
+def test_one_block_segments(L, cpb, states, saved):
+    w = Workload("one-block-%d" % L, 2, 3, 128, 128, [L], 64, g_scale=0.1, s_in_sigma=0.3 if states else None,
+                 ds_out_sigma=0.3 if states else None, seed=65)
+    x = inputs.make_inputs(w, DEV)
+    d = binding.make_desc(x["q"], x["v"], x["g"], 64, cpb)
+    assert binding.sf_num_blocks(d) == 1
+    o, dq, dk, dv, dg = (torch.empty_like(x[n]) for n in ("v", "q", "k", "v", "g"))
+    S, dS = (torch.empty(w.B, w.H, 128, 128, device=DEV) for _ in range(2))
+    ws_f = torch.empty(binding.sf_workspace_bytes(d, 0), dtype=torch.uint8, device=DEV)
+    ws_b = torch.empty(binding.sf_workspace_bytes(d, 1 if saved else 2), dtype=torch.uint8, device=DEV)
+    binding.sf_segment_fwd(d, x["q"], x["k"], x["v"], x["g"], x["S_in"], o, S, ws_f)
+    binding.sf_segment_bwd(d, x["q"], x["k"], x["v"], x["g"], x["S_in"], x["dO"], x["dS_out"], dq, dk, dv, dg, dS, ws_f if saved else None, ws_b)
+    torch.cuda.synchronize()
+    assert binding.sf_device_status() == 0
+    compare(dict(o=o, S_out=S, dq=dq, dk=dk, dv=dv, dg=dg, dS_in=dS), oracle_reference(x), tolerance(w), label=w.name)
