@@ -33,6 +33,26 @@ struct SegParams {
     float *s_final, *s_copy;
 };
 
+// Programmatic dependent launch.  A kernel launched with launch_after() may start while the kernel before it in the stream
+// still runs, once every CTA of that one has called grid_launch_next(); what it does before grid_wait() may only touch its own
+// on-chip state and the caller's inputs (which no kernel of this library's call writes).  grid_wait() returns when the
+// kernel before has completed and its writes are visible; every CTA calls it, so completion carries over a sequence of such
+// launches.  The first kernel of a call is launched the ordinary way and so waits for everything before it.
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <typename... P, typename... A>
+inline bool launch_after(bool early, void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = early ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kern, P(args)...) == cudaSuccess;
+}
+
 // Error codes written to the device status word by kernels whose bounded waits run out.
 enum : int { DEV_OK = 0, DEV_TIMEOUT_TMA = 1, DEV_TIMEOUT_MMA = 2, DEV_TIMEOUT_SELFTEST = 3 };
 

@@ -19,6 +19,8 @@ constexpr int SCAN_UNROLL = 4;
 __global__ void __launch_bounds__(SCAN_NT) state_scan_kernel(int n, int m, int reverse, const float* __restrict__ ld,
                                                              const float* U, const float* __restrict__ init,
                                                              float* states, float* __restrict__ final_state) {
+    grid_launch_next();
+    grid_wait();
     const int bh = blockIdx.y;
     const int e = (blockIdx.x * SCAN_NT + threadIdx.x) * 4;
     if (e >= m) return;
@@ -143,6 +145,8 @@ __global__ void __launch_bounds__(DG_NT) dg_epilogue_kernel(SegParams p, int m, 
     __shared__ float red[DG_NT / 32];
     __shared__ float sx[64], P_next[64];
     __shared__ float suffix[64 * 64];
+    grid_launch_next();
+    grid_wait();
     const int j = blockIdx.x, h = blockIdx.y, b = blockIdx.z;
     const long long bh = (long long)b * p.H + h;
     const int C = p.C;

@@ -464,6 +464,7 @@ struct AggSmem {
     float bloc[MAXR * C];
     float ctot[MAXR];
     float cofs[MAXR];
+    float beta;
     uint64_t full[AGG_STAGES], empty[AGG_STAGES], ready[AGG_STAGES], done, g_issued;
     uint32_t tmem_base;
     int abort_flag;
@@ -482,6 +483,7 @@ tc_aggregate_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_consta
     constexpr int WT = AGG_COMP / 32, WM = WT + 1;
 
     if (tid == 0) {
+        grid_launch_next();
         sm.abort_flag = 0;
         for (int s = 0; s < AGG_STAGES; ++s) { ptx::mbar_init(&sm.full[s], 1); ptx::mbar_init(&sm.empty[s], 1); ptx::mbar_init(&sm.ready[s], AGG_COMP / 32); }
         ptx::mbar_init(&sm.done, 1);
@@ -529,7 +531,7 @@ tc_aggregate_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_consta
             float acc = 0.f;
             if (mode == 0) { for (int c = nch - 1; c >= 0; --c) { sm.cofs[c] = acc; acc += sm.ctot[c]; } }
             else           { for (int c = 0; c < nch; ++c)      { sm.cofs[c] = acc; acc += sm.ctot[c]; } }
-            if (beta_out) beta_out[((long long)b * p.H + h) * p.NB + j] = acc;
+            sm.beta = acc;
         }
         ptx::named_bar_sync(1, AGG_COMP);
         for (int c = 0; c < nch; ++c) {
@@ -544,6 +546,8 @@ tc_aggregate_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_consta
         }
         SF_WAIT(&sm.done, 0, DEV_TIMEOUT_MMA);
         ptx::tc_fence_after_sync();
+        grid_wait();                                       // the workspace may still be in use by the kernels before
+        if (tid == 0 && beta_out) beta_out[((long long)b * p.H + h) * p.NB + j] = sm.beta;
         // 8 warps read the [128 x 128] accumulator: warp w covers lanes 32*(w&3).., column half w>>2
         const int row = tid & 127, half = tid >> 7;
         float* Uo = U + (((long long)b * p.H + h) * p.NB + j) * (long long)(D * D) + (long long)row * D + half * 64;
@@ -599,6 +603,7 @@ __device__ __forceinline__ void sweep_body(const CUtensorMap* tmQ, const CUtenso
     constexpr uint32_t T_ST = 0, T_O = 128, T_SC = 384;
 
     if (tid == 0) {
+        grid_launch_next();
         sm.abort_flag = 0;
         for (int s = 0; s < SW_STAGES; ++s) ptx::mbar_init(&sm.full[s], 1);
         for (int i = 0; i < 2; ++i) {
@@ -712,10 +717,13 @@ __device__ __forceinline__ void sweep_body(const CUtensorMap* tmQ, const CUtenso
             ptx::tc_fence_before_sync();
             ptx::mbar_arrive_warp(&sm.o_free[bf]);
         };
+        // tables, first tiles, scores and mask need only the caller's inputs: they run while the scan finishes
         if (wg == 3) {
+            grid_wait();
             for (int c = 0; c < nch; ++c) epilogue(c);
         } else {
             if (wg == 2) mask(0);
+            grid_wait();
             for (int c = 0; c < nch; ++c) {
                 const int s = c % SW_STAGES;
                 const float* bch = sm.bloc + c * C;
@@ -804,6 +812,7 @@ __device__ __forceinline__ void dkdv_body(const CUtensorMap* tmQ, const CUtensor
     constexpr uint32_t T_G = 0, T_DK = 128, T_DV = 256, T_SC = 384;
 
     if (tid == 0) {
+        grid_launch_next();
         sm.abort_flag = 0;
         for (int i = 0; i < 2; ++i) {
             ptx::mbar_init(&sm.full[i], 1);
@@ -918,6 +927,7 @@ __device__ __forceinline__ void dkdv_body(const CUtensorMap* tmQ, const CUtensor
         };
         if (wg >= 2) {
             if (wg == 2) mask(0);
+            grid_wait();
             for (int i = 0; i < nch; ++i) {
                 const int c = nch - 1 - i;
                 const long long tokA = t0 + c * C + rA, tokB = tokA + 8;
@@ -946,6 +956,7 @@ __device__ __forceinline__ void dkdv_body(const CUtensorMap* tmQ, const CUtensor
                 }
             }
         } else {
+            grid_wait();
             for (int i = 0; i < nch; ++i) {
                 const int c = nch - 1 - i, s = i & 1;
                 const float* bch = sm.bloc + c * C;
@@ -1036,15 +1047,16 @@ inline sf_status_t launch_wait_selftest(long long limit_cycles, cudaStream_t st)
     return cudaGetLastError() == cudaSuccess ? SF_OK : SF_ERR_CUDA;
 }
 
-// role: 0 aggregate, 1 forward output pass, 2 dq pass, 3 dk/dv pass (same order as the host's Role enum)
+// role: 0 aggregate, 1 forward output pass, 2 dq pass, 3 dk/dv pass (same order as the host's Role enum); early: launch_after()
 inline sf_status_t launch(int role, const sf_seg_desc_t* d, const SegParams& p, const void* q, const void* k, const void* v,
                           const void* dO, const float* g, int mode, float* U, float* beta, const float* states, void* o,
-                          void* dq, void* dk, void* dv, float* xq, float* xk, cudaStream_t st, long long* n_launch) {
+                          void* dq, void* dk, void* dv, float* xq, float* xk, bool early, cudaStream_t st, long long* n_launch) {
     DeviceState* ds = device_state();
     if (!ds) return SF_ERR_CUDA;
     int* status = ds->status;
     if (p.R > MAXR) return SF_ERR_UNSUPPORTED;
     dim3 grid(p.H, p.NB, p.B);
+    bool ok = false;
     auto map_qk = [&](CUtensorMap* m, const void* base) { return make_tmap(m, base, p.B, p.L, p.H, p.tqk, p.bqk); };
     auto map_v = [&](CUtensorMap* m, const void* base) { return make_tmap(m, base, p.B, p.L, p.H, p.tv, p.bv); };
     if (role == 0) {
@@ -1052,34 +1064,35 @@ inline sf_status_t launch(int role, const sf_seg_desc_t* d, const SegParams& p, 
         if (!map_qk(&tmX, mode == 0 ? k : q) || !map_v(&tmY, mode == 0 ? v : dO)) return SF_ERR_CUDA;
         constexpr size_t smem = sizeof(AggSmem) + 1024;
         if (!opt_in_smem(ds, K_AGG, tc_aggregate_kernel, smem)) return SF_ERR_CUDA;
-        tc_aggregate_kernel<<<grid, AGG_THREADS, smem, st>>>(tmX, tmY, p, g, mode, U, beta, status);
+        ok = launch_after(early, tc_aggregate_kernel, grid, AGG_THREADS, smem, st, tmX, tmY, p, g, mode, U, beta, status);
     } else if (role == 1) {
         CUtensorMap tq, tk, tv;
         if (!map_qk(&tq, q) || !map_qk(&tk, k) || !map_v(&tv, v)) return SF_ERR_CUDA;
         constexpr size_t smem = sizeof(SweepSmem) + 1024;
         if (!opt_in_smem(ds, K_FWD, tc_sweep_kernel<false>, smem)) return SF_ERR_CUDA;
-        tc_sweep_kernel<false><<<grid, SW_THREADS, smem, st>>>(tq, tk, tv, p, g, states, static_cast<__nv_bfloat16*>(o), p.tv, p.bv,
-                                                               nullptr, nullptr, status);
+        ok = launch_after(early, tc_sweep_kernel<false>, grid, SW_THREADS, smem, st, tq, tk, tv, p, g, states, static_cast<__nv_bfloat16*>(o), p.tv, p.bv,
+                          static_cast<const __nv_bfloat16*>(nullptr), static_cast<float*>(nullptr), status);
     } else if (role == 2) {
         CUtensorMap tk, tv, td;
         if (!map_qk(&tk, k) || !map_v(&tv, v) || !map_v(&td, dO)) return SF_ERR_CUDA;
         constexpr size_t smem = sizeof(SweepSmem) + 1024;
         if (!opt_in_smem(ds, K_DQ, tc_sweep_kernel<true>, smem)) return SF_ERR_CUDA;
         // roles: xq = dO, xk = v, xv = k; q is read from global memory for the row dot products
-        tc_sweep_kernel<true><<<grid, SW_THREADS, smem, st>>>(td, tv, tk, p, g, states, static_cast<__nv_bfloat16*>(dq), p.tqk, p.bqk,
-                                                              static_cast<const __nv_bfloat16*>(q), xq, status);
+        ok = launch_after(early, tc_sweep_kernel<true>, grid, SW_THREADS, smem, st, td, tv, tk, p, g, states, static_cast<__nv_bfloat16*>(dq), p.tqk, p.bqk,
+                          static_cast<const __nv_bfloat16*>(q), xq, status);
     } else if (role == 3) {
         CUtensorMap tq, tk, tv, td;
         if (!map_qk(&tq, q) || !map_qk(&tk, k) || !map_v(&tv, v) || !map_v(&td, dO)) return SF_ERR_CUDA;
         constexpr size_t smem = sizeof(DkdvSmem) + 1024;
         if (!opt_in_smem(ds, K_DKDV, tc_dkdv_kernel, smem)) return SF_ERR_CUDA;
-        tc_dkdv_kernel<<<grid, SW_THREADS, smem, st>>>(tq, tk, tv, td, p, g, states, static_cast<const __nv_bfloat16*>(k),
-                                                       static_cast<__nv_bfloat16*>(dk), static_cast<__nv_bfloat16*>(dv), xk, status);
+        ok = launch_after(early, tc_dkdv_kernel, grid, SW_THREADS, smem, st, tq, tk, tv, td, p, g, states, static_cast<const __nv_bfloat16*>(k),
+                          static_cast<__nv_bfloat16*>(dk), static_cast<__nv_bfloat16*>(dv), xk, status);
     } else {
         return SF_ERR_UNSUPPORTED;
     }
     *n_launch += 1;
-    return cudaGetLastError() == cudaSuccess ? SF_OK : SF_ERR_CUDA;
+    if (!ok) cudaGetLastError();
+    return ok ? SF_OK : SF_ERR_CUDA;
 }
 
 }  // namespace tc

@@ -212,9 +212,9 @@ BwdWs bwd_ws(const sf_seg_desc_t* d, const SegParams& p, void* base) {
 
 size_t state_bytes(const sf_seg_desc_t* d) { return align_up((size_t)d->B * d->H * d->d_k * d->d_v * sizeof(float)); }
 
-inline sf_status_t check_launch() {
+inline sf_status_t check_launch(bool launched = true) {
     g_launches.fetch_add(1, std::memory_order_relaxed);
-    return cudaGetLastError() == cudaSuccess ? SF_OK : SF_ERR_CUDA;
+    return cudaGetLastError() == cudaSuccess && launched ? SF_OK : SF_ERR_CUDA;
 }
 
 #define SF_TRY(expr) do { sf_status_t st__ = (expr); if (st__ != SF_OK) return st__; } while (0)
@@ -298,14 +298,17 @@ sf_status_t launch_simt_d(Role role, const sf_seg_desc_t* d, const SegParams& p,
     return SF_ERR_UNSUPPORTED;
 }
 
-sf_status_t launch_role(Path path, Role role, const sf_seg_desc_t* d, const SegParams& p, const RoleArgs& a, cudaStream_t st) {
+// `early`: the kernel may start while the one before it in the stream finishes (launch_after()); it must then follow a kernel of
+// the same call.  The CUDA-core kernels do not take part.
+sf_status_t launch_role(Path path, Role role, const sf_seg_desc_t* d, const SegParams& p, const RoleArgs& a, cudaStream_t st, bool early) {
     const int stage = role == Role::Aggregate ? (a.mode == 0 ? ST_AGG_KV : ST_AGG_QDO)
                     : role == Role::FwdOut ? ST_FWD_OUT : role == Role::BwdDq ? ST_DQ : ST_DKDV;
     StageTimer timer(stage, st);
+    early = early && !g_timing_on;                             // a timed kernel is bracketed by events
     if (path == Path::Tc) {
         long long n = 0;
         sf_status_t s = sf::tc::launch(static_cast<int>(role), d, p, a.q, a.k, a.v, a.dO, a.g, a.mode, a.U, a.beta, a.states,
-                                       a.o, a.dq, a.dk, a.dv, a.xq, a.xk, st, &n);
+                                       a.o, a.dq, a.dk, a.dv, a.xq, a.xk, early, st, &n);
         g_launches.fetch_add(n, std::memory_order_relaxed);
         return s;
     }
@@ -314,12 +317,12 @@ sf_status_t launch_role(Path path, Role role, const sf_seg_desc_t* d, const SegP
 }
 
 sf_status_t launch_scan(const sf_seg_desc_t* d, const SegParams& p, int reverse, const float* ld, const float* U,
-                        const float* init, float* states, float* fin, cudaStream_t st) {
+                        const float* init, float* states, float* fin, cudaStream_t st, bool early = false) {
     const int m = d->d_k * d->d_v;
     StageTimer timer(ST_SCAN, st);
     dim3 grid((m / 4 + sf::SCAN_NT - 1) / sf::SCAN_NT, p.B * p.H);
-    sf::state_scan_kernel<<<grid, sf::SCAN_NT, 0, st>>>(p.NB, m, reverse, ld, U, init, states, fin);
-    return check_launch();
+    const bool ok = sf::launch_after(early && !g_timing_on, sf::state_scan_kernel, grid, sf::SCAN_NT, 0, st, p.NB, m, reverse, ld, U, init, states, fin);
+    return check_launch(ok);
 }
 
 // Scan of a group of consecutive segments in one launch (the chaining driver's way to shorten the serial chain of
@@ -360,18 +363,18 @@ int scan_group_size(const int32_t* seg_lens, int n_seg, int i, int dir, long lon
 struct FwdPtrs { const void *q, *k, *v; const float* g; const float* S_in; void* o; float* S_out; };
 
 // Stage split used by the chaining driver: `pre` needs no boundary state, `post` does.
-sf_status_t fwd_pre(Path path, const sf_seg_desc_t* d, const SegParams& p, const FwdPtrs& x, const FwdWs& w, cudaStream_t st) {
+sf_status_t fwd_pre(Path path, const sf_seg_desc_t* d, const SegParams& p, const FwdPtrs& x, const FwdWs& w, cudaStream_t st, bool early = false) {
     RoleArgs a{};
     a.k = x.k; a.v = x.v; a.g = x.g; a.mode = 0; a.U = w.UH; a.beta = w.beta;
-    return launch_role(path, Role::Aggregate, d, p, a, st);
+    return launch_role(path, Role::Aggregate, d, p, a, st, early);
 }
-sf_status_t fwd_scan(const sf_seg_desc_t* d, const SegParams& p, const FwdPtrs& x, const FwdWs& w, cudaStream_t st) {
-    return launch_scan(d, p, 0, w.beta, w.UH, x.S_in, w.UH, x.S_out, st);
+sf_status_t fwd_scan(const sf_seg_desc_t* d, const SegParams& p, const FwdPtrs& x, const FwdWs& w, cudaStream_t st, bool early = false) {
+    return launch_scan(d, p, 0, w.beta, w.UH, x.S_in, w.UH, x.S_out, st, early);
 }
-sf_status_t fwd_out(Path path, const sf_seg_desc_t* d, const SegParams& p, const FwdPtrs& x, const FwdWs& w, cudaStream_t st) {
+sf_status_t fwd_out(Path path, const sf_seg_desc_t* d, const SegParams& p, const FwdPtrs& x, const FwdWs& w, cudaStream_t st, bool early = false) {
     RoleArgs a{};
     a.q = x.q; a.k = x.k; a.v = x.v; a.g = x.g; a.states = w.UH; a.o = x.o;
-    return launch_role(path, Role::FwdOut, d, p, a, st);
+    return launch_role(path, Role::FwdOut, d, p, a, st, early);
 }
 
 struct BwdPtrs {
@@ -380,29 +383,29 @@ struct BwdPtrs {
 };
 
 sf_status_t bwd_pre(Path path, const sf_seg_desc_t* d, const SegParams& p, const BwdPtrs& x, const BwdWs& w, float* beta_out,
-                    cudaStream_t st) {
+                    cudaStream_t st, bool early = false) {
     RoleArgs a{};
     a.q = x.q; a.dO = x.dO; a.g = x.g; a.mode = 1; a.U = w.GU; a.beta = beta_out;
-    return launch_role(path, Role::Aggregate, d, p, a, st);
+    return launch_role(path, Role::Aggregate, d, p, a, st, early);
 }
-sf_status_t bwd_scan(const sf_seg_desc_t* d, const SegParams& p, const BwdPtrs& x, const BwdWs& w, const float* beta, cudaStream_t st) {
-    return launch_scan(d, p, 1, beta, w.GU, x.dS_out, w.GU, x.dS_in, st);
+sf_status_t bwd_scan(const sf_seg_desc_t* d, const SegParams& p, const BwdPtrs& x, const BwdWs& w, const float* beta, cudaStream_t st, bool early = false) {
+    return launch_scan(d, p, 1, beta, w.GU, x.dS_out, w.GU, x.dS_in, st, early);
 }
-sf_status_t bwd_dq(Path path, const sf_seg_desc_t* d, const SegParams& p, const BwdPtrs& x, const BwdWs& w, const float* Hs, cudaStream_t st) {
+sf_status_t bwd_dq(Path path, const sf_seg_desc_t* d, const SegParams& p, const BwdPtrs& x, const BwdWs& w, const float* Hs, cudaStream_t st, bool early = false) {
     RoleArgs a{};
     a.q = x.q; a.k = x.k; a.v = x.v; a.dO = x.dO; a.g = x.g; a.states = Hs; a.dq = x.dq; a.xq = w.xq;
-    return launch_role(path, Role::BwdDq, d, p, a, st);
+    return launch_role(path, Role::BwdDq, d, p, a, st, early);
 }
-sf_status_t bwd_dkdv(Path path, const sf_seg_desc_t* d, const SegParams& p, const BwdPtrs& x, const BwdWs& w, cudaStream_t st) {
+sf_status_t bwd_dkdv(Path path, const sf_seg_desc_t* d, const SegParams& p, const BwdPtrs& x, const BwdWs& w, cudaStream_t st, bool early = false) {
     RoleArgs a{};
     a.q = x.q; a.k = x.k; a.v = x.v; a.dO = x.dO; a.g = x.g; a.states = w.GU; a.dk = x.dk; a.dv = x.dv; a.xk = w.xk;
-    return launch_role(path, Role::BwdDkDv, d, p, a, st);
+    return launch_role(path, Role::BwdDkDv, d, p, a, st, early);
 }
-sf_status_t bwd_dg(const sf_seg_desc_t* d, const SegParams& p, const BwdPtrs& x, const BwdWs& w, const float* Hs, cudaStream_t st) {
+sf_status_t bwd_dg(const sf_seg_desc_t* d, const SegParams& p, const BwdPtrs& x, const BwdWs& w, const float* Hs, cudaStream_t st, bool early = false) {
     StageTimer timer(ST_DG, st);
     dim3 grid(p.NB, p.H, p.B);
-    sf::dg_epilogue_kernel<<<grid, sf::DG_NT, 0, st>>>(p, d->d_k * d->d_v, w.xq, w.xk, Hs, w.GU, x.dS_in, x.dg);
-    return check_launch();
+    const bool ok = sf::launch_after(early && !g_timing_on, sf::dg_epilogue_kernel, grid, sf::DG_NT, 0, st, p, d->d_k * d->d_v, w.xq, w.xk, Hs, w.GU, x.dS_in, x.dg);
+    return check_launch(ok);
 }
 
 // A segment of one block on the tensor-core path: the sweeps start from the boundary state itself and store the state that
@@ -418,8 +421,8 @@ sf_status_t segment_fwd(Path path, const sf_seg_desc_t* d, const SegParams& p, c
         return fwd_out(path, d, s, x, w, st);
     }
     SF_TRY(fwd_pre(path, d, p, x, w, st));
-    SF_TRY(fwd_scan(d, p, x, w, st));
-    return fwd_out(path, d, p, x, w, st);
+    SF_TRY(fwd_scan(d, p, x, w, st, true));
+    return fwd_out(path, d, p, x, w, st, true);
 }
 
 // `saved`: the forward's workspace, or NULL to replay the block states into replay (its state-out goes to sfin).
@@ -431,20 +434,21 @@ sf_status_t segment_bwd(Path path, const sf_seg_desc_t* d, const SegParams& p, c
         s.single = 1; s.s_init = H;
         SF_TRY(bwd_dq(path, d, s, x, w, nullptr, st));
         s.s_init = x.dS_out; s.s_final = x.dS_in;
-        SF_TRY(bwd_dkdv(path, d, s, x, w, st));
-        return bwd_dg(d, p, x, w, H, st);
+        SF_TRY(bwd_dkdv(path, d, s, x, w, st, true));
+        return bwd_dg(d, p, x, w, H, st, true);
     }
-    if (!saved) {
+    const bool replayed = !saved;
+    if (replayed) {
         FwdPtrs fx{x.q, x.k, x.v, x.g, x.S_in, nullptr, sfin};               // SR: block-entering states from S_in
         SF_TRY(fwd_pre(path, d, p, fx, replay, st));
-        SF_TRY(fwd_scan(d, p, fx, replay, st));
+        SF_TRY(fwd_scan(d, p, fx, replay, st, true));
         saved = &replay;
     }
-    SF_TRY(bwd_pre(path, d, p, x, w, nullptr, st));
-    SF_TRY(bwd_scan(d, p, x, w, saved->beta, st));
-    SF_TRY(bwd_dq(path, d, p, x, w, saved->UH, st));
-    SF_TRY(bwd_dkdv(path, d, p, x, w, st));
-    return bwd_dg(d, p, x, w, saved->UH, st);
+    SF_TRY(bwd_pre(path, d, p, x, w, nullptr, st, replayed));
+    SF_TRY(bwd_scan(d, p, x, w, saved->beta, st, true));
+    SF_TRY(bwd_dq(path, d, p, x, w, saved->UH, st, true));
+    SF_TRY(bwd_dkdv(path, d, p, x, w, st, true));
+    return bwd_dg(d, p, x, w, saved->UH, st, true);
 }
 
 sf_status_t validate_fwd(const sf_seg_desc_t* d, const FwdPtrs& x, const void* ws, size_t ws_bytes, Path* path) {
@@ -647,7 +651,7 @@ sf_status_t chain_fwd_merged(const sf_seg_desc_t* vd, bool free_grid, const int3
         p.bstride = (long long)sN;
     }
     SF_TRY(fwd_pre(path, vd, p, x, w, st));
-    SF_TRY(fwd_scan(vd, p, x, w, st));
+    SF_TRY(fwd_scan(vd, p, x, w, st, true));
     if (!free_grid) {
         // S_bounds[i] = state entering the first block of segment i (a strided copy: one state per batch x head)
         long long blk = 0;
@@ -657,7 +661,7 @@ sf_status_t chain_fwd_merged(const sf_seg_desc_t* vd, bool free_grid, const int3
                                       m * sizeof(float), (size_t)vd->B * vd->H, cudaMemcpyDeviceToDevice, st));
         }
     }
-    return fwd_out(path, vd, p, x, w, st);
+    return fwd_out(path, vd, p, x, w, st, free_grid);
 }
 
 sf_status_t chain_bwd_merged(const sf_seg_desc_t* vd, const BwdPtrs& x, const void* fwd_workspace, void* workspace, bool overlap,
@@ -687,11 +691,11 @@ sf_status_t chain_bwd_merged(const sf_seg_desc_t* vd, const BwdPtrs& x, const vo
         SF_CUDA(cudaEventRecord(res->ev[6], res->side[1]));
     }
     SF_TRY(bwd_pre(path, vd, p, x, w, nullptr, st));
-    SF_TRY(bwd_scan(vd, p, x, w, fw.beta, st));
-    if (!overlap) SF_TRY(bwd_dq(path, vd, p, x, w, fw.UH, st));
-    SF_TRY(bwd_dkdv(path, vd, p, x, w, st));
+    SF_TRY(bwd_scan(vd, p, x, w, fw.beta, st, true));
+    if (!overlap) SF_TRY(bwd_dq(path, vd, p, x, w, fw.UH, st, true));
+    SF_TRY(bwd_dkdv(path, vd, p, x, w, st, true));
     if (overlap) SF_CUDA(cudaStreamWaitEvent(st, res->ev[6], 0));
-    return bwd_dg(vd, p, x, w, fw.UH, st);
+    return bwd_dg(vd, p, x, w, fw.UH, st, !overlap);
 }
 
 }  // namespace
