@@ -31,13 +31,15 @@ struct SegParams {
     int single;
     const float* s_init;
     float *s_final, *s_copy;
+    int wait_first;          // the first kernel of a call: grid_wait() before any access to global memory
 };
 
 // Programmatic dependent launch.  A kernel launched with launch_after() may start while the kernel before it in the stream
 // still runs, once every CTA of that one has called grid_launch_next(); what it does before grid_wait() may only touch its own
 // on-chip state and the caller's inputs (which no kernel of this library's call writes).  grid_wait() returns when the
 // kernel before has completed and its writes are visible; every CTA calls it, so completion carries over a sequence of such
-// launches.  The first kernel of a call is launched the ordinary way and so waits for everything before it.
+// launches.  The first kernel of a call (SegParams::wait_first) waits before it touches global memory at all: only its barriers
+// and tensor memory are set up early, whatever came before in the stream.
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

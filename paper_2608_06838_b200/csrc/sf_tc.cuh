@@ -495,6 +495,7 @@ tc_aggregate_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_consta
     __syncthreads();
     ptx::tc_fence_after_sync();
     const uint32_t tmem = sm.tmem_base;
+    if (p.wait_first) grid_wait();
 
     if (warp == WT) {
         if (lane == 0) {
@@ -592,10 +593,10 @@ template <bool DQ>
 __device__ __forceinline__ void sweep_body(const CUtensorMap* tmQ, const CUtensorMap* tmK, const CUtensorMap* tmV, const SegParams& p,
                                            const float* __restrict__ g, const float* __restrict__ Hs, __nv_bfloat16* __restrict__ out,
                                            long long out_tok, long long out_bat, const __nv_bfloat16* __restrict__ e_glob,
-                                           float* __restrict__ xout, int* status, int h) {
+                                           float* __restrict__ xout, int* status, int h, int j) {
     extern __shared__ unsigned char smem_raw[];
     SweepSmem& sm = *reinterpret_cast<SweepSmem*>(align1024(smem_raw));
-    const int j = blockIdx.y, b = blockIdx.z;
+    const int b = blockIdx.z;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int c0 = j * p.R, nch = min(p.R, p.NC - c0);
     const long long t0 = (long long)c0 * C;
@@ -621,6 +622,7 @@ __device__ __forceinline__ void sweep_body(const CUtensorMap* tmQ, const CUtenso
     __syncthreads();
     ptx::tc_fence_after_sync();
     const uint32_t tmem = sm.tmem_base;
+    if (p.wait_first) grid_wait();
     // the decay tables are built by the compute warps while the first tiles are already on their way
 
     if (warp == W_TMA) {
@@ -769,7 +771,7 @@ tc_sweep_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
                 SegParams p, const float* __restrict__ g, const float* __restrict__ Hs, __nv_bfloat16* __restrict__ out, long long out_tok,
                 long long out_bat, const __nv_bfloat16* __restrict__ e_glob, float* __restrict__ xout, int* status) {
     // heads fastest: co-resident CTAs read neighbouring 256-byte pieces of the same tokens
-    sweep_body<DQ>(&tmQ, &tmK, &tmV, p, g, Hs, out, out_tok, out_bat, e_glob, xout, status, blockIdx.x);
+    sweep_body<DQ>(&tmQ, &tmK, &tmV, p, g, Hs, out, out_tok, out_bat, e_glob, xout, status, blockIdx.x, blockIdx.y);
 }
 
 // ==================================================================================================
@@ -801,10 +803,10 @@ struct DkdvSmem {
 __device__ __forceinline__ void dkdv_body(const CUtensorMap* tmQ, const CUtensorMap* tmK, const CUtensorMap* tmV, const CUtensorMap* tmD,
                                           const SegParams& p, const float* __restrict__ g, const float* __restrict__ Gs,
                                           const __nv_bfloat16* __restrict__ k_glob, __nv_bfloat16* __restrict__ dk,
-                                          __nv_bfloat16* __restrict__ dv, float* __restrict__ xk, int* status, int h) {
+                                          __nv_bfloat16* __restrict__ dv, float* __restrict__ xk, int* status, int h, int j) {
     extern __shared__ unsigned char smem_raw[];
     DkdvSmem& sm = *reinterpret_cast<DkdvSmem*>(align1024(smem_raw));
-    const int j = blockIdx.y, b = blockIdx.z;
+    const int b = blockIdx.z;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int c0 = j * p.R, nch = min(p.R, p.NC - c0);
     const long long t0 = (long long)c0 * C;
@@ -834,6 +836,7 @@ __device__ __forceinline__ void dkdv_body(const CUtensorMap* tmQ, const CUtensor
     __syncthreads();
     ptx::tc_fence_after_sync();
     const uint32_t tmem = sm.tmem_base;
+    if (p.wait_first) grid_wait();
     // the decay tables are built by the compute warps while the first tiles are already on their way
 
     // iteration i handles chunk c = nch-1-i
@@ -990,7 +993,28 @@ tc_dkdv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                const __grid_constant__ CUtensorMap tmD, SegParams p, const float* __restrict__ g, const float* __restrict__ Gs,
                const __nv_bfloat16* __restrict__ k_glob, __nv_bfloat16* __restrict__ dk, __nv_bfloat16* __restrict__ dv,
                float* __restrict__ xk, int* status) {
-    dkdv_body(&tmQ, &tmK, &tmV, &tmD, p, g, Gs, k_glob, dk, dv, xk, status, blockIdx.x);
+    dkdv_body(&tmQ, &tmK, &tmV, &tmD, p, g, Gs, k_glob, dk, dv, xk, status, blockIdx.x, blockIdx.y);
+}
+
+// Both sweeps of the backward in one launch, for launches that leave at least half of the device idle: they need nothing from
+// each other, so they then take the time of the longer one.  grid (H, 2 NB, B).
+struct PairArgs {
+    const float *Hs, *Gs;
+    const __nv_bfloat16 *q, *k;
+    __nv_bfloat16 *dq, *dk, *dv;
+    float *xq, *xk;
+    const float* g_init;                        // one-block segments: the gradient of the leaving state (SegParams::s_init is the entering state)
+};
+__global__ void __launch_bounds__(SW_THREADS, 1)
+tc_backward_pair_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
+                        const __grid_constant__ CUtensorMap tmD, SegParams p, const float* __restrict__ g, PairArgs a, int* status) {
+    const int j = blockIdx.y;
+    if (j < p.NB) {
+        sweep_body<true>(&tmD, &tmV, &tmK, p, g, a.Hs, a.dq, p.tqk, p.bqk, a.q, a.xq, status, blockIdx.x, j);
+    } else {
+        p.s_init = a.g_init;
+        dkdv_body(&tmQ, &tmK, &tmV, &tmD, p, g, a.Gs, a.k, a.dk, a.dv, a.xk, status, blockIdx.x, j - p.NB);
+    }
 }
 
 // Self-test of the bounded wait: one warp waits on a barrier on which nothing ever arrives, with a short limit given by
@@ -1011,7 +1035,7 @@ __global__ void wait_selftest_kernel(long long limit_cycles, int* status) {
 // Per-device host state: the address of the status word and whether the kernels' shared-memory attribute has been
 // set there (both belong to a device, not to the process).
 constexpr int MAX_DEVICES = 64;
-enum { K_AGG = 0, K_FWD, K_DQ, K_DKDV, K_COUNT };
+enum { K_AGG = 0, K_FWD, K_DQ, K_DKDV, K_PAIR, K_COUNT };
 struct DeviceState {
     int* status = nullptr;
     bool attr_done[K_COUNT] = {};
@@ -1090,6 +1114,24 @@ inline sf_status_t launch(int role, const sf_seg_desc_t* d, const SegParams& p, 
     } else {
         return SF_ERR_UNSUPPORTED;
     }
+    *n_launch += 1;
+    if (!ok) cudaGetLastError();
+    return ok ? SF_OK : SF_ERR_CUDA;
+}
+
+// dq and dk/dv sweeps of a segment in one launch; `a` holds everything but the tensor maps' tensors.
+inline sf_status_t launch_pair(const SegParams& p, const void* q, const void* k, const void* v, const void* dO, const float* g, PairArgs a,
+                               bool early, cudaStream_t st, long long* n_launch) {
+    DeviceState* ds = device_state();
+    if (!ds) return SF_ERR_CUDA;
+    if (p.R > MAXR) return SF_ERR_UNSUPPORTED;
+    CUtensorMap tq, tk, tv, td;
+    if (!make_tmap(&tq, q, p.B, p.L, p.H, p.tqk, p.bqk) || !make_tmap(&tk, k, p.B, p.L, p.H, p.tqk, p.bqk) ||
+        !make_tmap(&tv, v, p.B, p.L, p.H, p.tv, p.bv) || !make_tmap(&td, dO, p.B, p.L, p.H, p.tv, p.bv))
+        return SF_ERR_CUDA;
+    constexpr size_t smem = (sizeof(DkdvSmem) > sizeof(SweepSmem) ? sizeof(DkdvSmem) : sizeof(SweepSmem)) + 1024;
+    if (!opt_in_smem(ds, K_PAIR, tc_backward_pair_kernel, smem)) return SF_ERR_CUDA;
+    const bool ok = launch_after(early, tc_backward_pair_kernel, dim3(p.H, 2 * p.NB, p.B), SW_THREADS, smem, st, tq, tk, tv, td, p, g, a, ds->status);
     *n_launch += 1;
     if (!ok) cudaGetLastError();
     return ok ? SF_OK : SF_ERR_CUDA;

@@ -104,7 +104,10 @@ int sm_count() {
 
 // Block length when the caller leaves it open: one CTA per (batch, head, block) and one CTA per SM, so a
 // kernel takes waves * (chunks per block + a fixed per-CTA cost of about six chunk times); more than one block adds the
-// aggregate and the scan, about four chunk times (a segment of one block needs neither, see one_block()).  Pick the
+// aggregate and the scan, about two chunk times where their launches overlap (a segment of one block needs neither, see
+// one_block(); 16 heads x 500 tokens, forward: one block 24.5 us, two 20.7); so does
+// a launch too large for the backward's two sweeps to share the device (bwd_sweeps(); 64 heads x 500 tokens, forward + backward
+// with replay: one block 84 us, two 96).  Pick the
 // length in [4, 64] that minimises this; ties go to the longer block (fewer block states in HBM).
 int auto_chunks_per_block(int NC, long long bh) {
     const int sms = sm_count();
@@ -114,7 +117,7 @@ int auto_chunks_per_block(int NC, long long bh) {
         const int reff = r < NC ? r : NC;
         const long long nb = (NC + reff - 1) / reff;
         const long long waves = (nb * bh + sms - 1) / sms;
-        const long long cost = waves * (reff + 6) + (nb > 1 ? 4 : 0);
+        const long long cost = waves * (reff + 6) + (nb > 1 ? 2 : 0) + (nb > 1 && 2 * nb * bh > sms ? 2 : 0);
         if (best_cost < 0 || cost <= best_cost) { best_cost = cost; best = reff; }
         if (r >= NC) break;
     }
@@ -176,6 +179,7 @@ SegParams make_params(const sf_seg_desc_t* d, int cpb_override = 0) {
     p.bqk = d->batch_stride_qk; p.bv = d->batch_stride_v; p.bg = d->batch_stride_g;
     p.bslot = nullptr; p.bbase = nullptr; p.bstride = 0;
     p.single = 0; p.s_init = nullptr; p.s_final = p.s_copy = nullptr;
+    p.wait_first = 0;
     return p;
 }
 
@@ -411,18 +415,45 @@ sf_status_t bwd_dg(const sf_seg_desc_t* d, const SegParams& p, const BwdPtrs& x,
 // A segment of one block on the tensor-core path: the sweeps start from the boundary state itself and store the state that
 // leaves, so the aggregate and the scan (two launches of 4-9 us each way, and their passes over k, v, q, dO) are left out.
 // The forward keeps the entering state in the workspace for the backward, as the scan would.
-// 200 tokens x 16 heads, forward: 27.6 -> 20.5 us.
+// 200 tokens x 16 heads, forward: 27.6 -> 18.3 us.
 bool one_block(Path path, const SegParams& p) { return path == Path::Tc && p.NB == 1; }
+
+// The first kernel of a call: launched early like the others, but it waits before it touches global memory.
+SegParams first_kernel(const SegParams& p) {
+    SegParams f = p;
+    f.wait_first = 1;
+    return f;
+}
 
 sf_status_t segment_fwd(Path path, const sf_seg_desc_t* d, const SegParams& p, const FwdPtrs& x, const FwdWs& w, cudaStream_t st) {
     if (one_block(path, p)) {
-        SegParams s = p;
+        SegParams s = first_kernel(p);
         s.single = 1; s.s_init = x.S_in; s.s_final = x.S_out; s.s_copy = w.UH;
-        return fwd_out(path, d, s, x, w, st);
+        return fwd_out(path, d, s, x, w, st, true);
     }
-    SF_TRY(fwd_pre(path, d, p, x, w, st));
+    SF_TRY(fwd_pre(path, d, first_kernel(p), x, w, st, true));
     SF_TRY(fwd_scan(d, p, x, w, st, true));
     return fwd_out(path, d, p, x, w, st, true);
+}
+
+// dq and dk/dv sweeps, in one launch (tc_backward_pair_kernel) where both fit on the device at once.  `s` carries the one-block
+// settings for the dq sweep, g_init the gradient of the leaving state.  A timed run keeps the two launches apart.
+// 200 tokens x 16 heads, forward + backward: 76 us with eight launches, 44 with three (one block, this launch, early starts).
+sf_status_t bwd_sweeps(Path path, const sf_seg_desc_t* d, const SegParams& s, const BwdPtrs& x, const BwdWs& w, const float* Hs, const float* g_init,
+                       cudaStream_t st) {
+    if (path == Path::Tc && !g_timing_on && 2LL * s.B * s.H * s.NB <= sm_count()) {
+        long long n = 0;
+        sf::tc::PairArgs a{Hs, w.GU, static_cast<const __nv_bfloat16*>(x.q), static_cast<const __nv_bfloat16*>(x.k), static_cast<__nv_bfloat16*>(x.dq),
+                           static_cast<__nv_bfloat16*>(x.dk), static_cast<__nv_bfloat16*>(x.dv), w.xq, w.xk, g_init};
+        const sf_status_t r = sf::tc::launch_pair(s, x.q, x.k, x.v, x.dO, x.g, a, true, st, &n);
+        g_launches.fetch_add(n, std::memory_order_relaxed);
+        return r;
+    }
+    SF_TRY(bwd_dq(path, d, s, x, w, Hs, st, true));
+    SegParams t = s;
+    t.s_init = g_init;
+    t.wait_first = 0;
+    return bwd_dkdv(path, d, t, x, w, st, true);
 }
 
 // `saved`: the forward's workspace, or NULL to replay the block states into replay (its state-out goes to sfin).
@@ -430,24 +461,21 @@ sf_status_t segment_bwd(Path path, const sf_seg_desc_t* d, const SegParams& p, c
                         const FwdWs& replay, float* sfin, cudaStream_t st) {
     if (one_block(path, p)) {
         const float* H = saved ? saved->UH : x.S_in;
-        SegParams s = p;
-        s.single = 1; s.s_init = H;
-        SF_TRY(bwd_dq(path, d, s, x, w, nullptr, st));
-        s.s_init = x.dS_out; s.s_final = x.dS_in;
-        SF_TRY(bwd_dkdv(path, d, s, x, w, st, true));
+        SegParams s = first_kernel(p);
+        s.single = 1; s.s_init = H; s.s_final = x.dS_in;
+        SF_TRY(bwd_sweeps(path, d, s, x, w, nullptr, x.dS_out, st));
         return bwd_dg(d, p, x, w, H, st, true);
     }
     const bool replayed = !saved;
     if (replayed) {
         FwdPtrs fx{x.q, x.k, x.v, x.g, x.S_in, nullptr, sfin};               // SR: block-entering states from S_in
-        SF_TRY(fwd_pre(path, d, p, fx, replay, st));
+        SF_TRY(fwd_pre(path, d, first_kernel(p), fx, replay, st, true));
         SF_TRY(fwd_scan(d, p, fx, replay, st, true));
         saved = &replay;
     }
-    SF_TRY(bwd_pre(path, d, p, x, w, nullptr, st, replayed));
+    SF_TRY(bwd_pre(path, d, replayed ? p : first_kernel(p), x, w, nullptr, st, true));
     SF_TRY(bwd_scan(d, p, x, w, saved->beta, st, true));
-    SF_TRY(bwd_dq(path, d, p, x, w, saved->UH, st, true));
-    SF_TRY(bwd_dkdv(path, d, p, x, w, st, true));
+    SF_TRY(bwd_sweeps(path, d, p, x, w, saved->UH, nullptr, st));
     return bwd_dg(d, p, x, w, saved->UH, st, true);
 }
 

@@ -82,8 +82,8 @@ def test_chunked_operator_rows_without_vector_alignment(kind, dtype, tol):
 
 
 # Tensor-core segments of one block start from the boundary state itself (no aggregate, no scan): one token, one chunk and its
-# neighbours, the longest one-block segment of the library's choice, a longer one by request; boundary states present and absent.
-@pytest.mark.parametrize("L,cpb", [(1, 0), (63, 0), (64, 0), (65, 0), (500, 0), (512, 0), (1100, 18)])
+# neighbours, longer ones by request; boundary states present and absent.
+@pytest.mark.parametrize("L,cpb", [(1, 0), (63, 0), (64, 0), (65, 0), (500, 8), (512, 8), (1100, 18)])
 @pytest.mark.parametrize("states", [True, False])
 @pytest.mark.parametrize("saved", [True, False])
 def test_one_block_segments(L, cpb, states, saved):
