@@ -154,14 +154,25 @@ __global__ void __launch_bounds__(DG_NT) dg_epilogue_kernel(SegParams p, int m, 
     const float* Hj = Hs ? Hs + (bh * p.NB + j) * (long long)m : nullptr;       // NULL: states of zeros
     const float* Gin = (j == 0) ? (dS_in + bh * (long long)m) : (Gs + (bh * p.NB + (j - 1)) * (long long)m);
 
-    // anchor: fixed-order tree reduction so that the result is reproducible run to run
+    // anchor: fixed-order tree reduction so that the result is reproducible run to run.  The kernel is a chain of memory round
+    // trips (its bytes take about 1 us), so the loads of AN rows of threads, and below those of XN chunks, go out together.
     float part = 0.f;
-    if (Hj) for (int e = threadIdx.x * 4; e < m; e += DG_NT * 4) {
-        const float4 hv = *reinterpret_cast<const float4*>(Hj + e);
-        const float4 gv = *reinterpret_cast<const float4*>(Gin + e);
-        part = fmaf(hv.x, gv.x, part); part = fmaf(hv.y, gv.y, part);
-        part = fmaf(hv.z, gv.z, part); part = fmaf(hv.w, gv.w, part);
-    }
+    constexpr int AN = 8;
+    if (Hj)
+        for (int e0 = threadIdx.x * 4; e0 < m; e0 += AN * DG_NT * 4) {
+            float4 hv[AN], gv[AN];
+#pragma unroll
+            for (int i = 0; i < AN; ++i) {
+                const int e = e0 + i * DG_NT * 4;
+                if (e < m) { hv[i] = *reinterpret_cast<const float4*>(Hj + e); gv[i] = *reinterpret_cast<const float4*>(Gin + e); }
+            }
+#pragma unroll
+            for (int i = 0; i < AN; ++i)
+                if (e0 + i * DG_NT * 4 < m) {
+                    part = fmaf(hv[i].x, gv[i].x, part); part = fmaf(hv[i].y, gv[i].y, part);
+                    part = fmaf(hv[i].z, gv[i].z, part); part = fmaf(hv[i].w, gv[i].w, part);
+                }
+        }
     for (int off = 16; off > 0; off >>= 1) part += __shfl_xor_sync(0xffffffffu, part, off);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = part;
 
@@ -170,21 +181,33 @@ __global__ void __launch_bounds__(DG_NT) dg_epilogue_kernel(SegParams p, int m, 
     const int ntok = min(nch * C, p.L - c0 * C);          // tokens of this block (the segment's last chunk may be partial)
     const float* xqh = xq + bh * p.L;
     const float* xkh = xk + bh * p.L;
-    for (int c = warp; c < nch; c += DG_NT / 32) {
-        const long long t0 = (long long)(c0 + c) * C;
+    constexpr int XN = 8;
+    for (int cb = warp; cb < nch; cb += XN * (DG_NT / 32)) {
+        float x0[XN], x1[XN];
         const int r0 = 2 * lane, r1 = 2 * lane + 1;
-        // tokens past the end of the segment (ragged last chunk) contribute nothing
-        const int lim = min(C, ntok - c * C), i0 = min(r0, lim - 1), i1 = min(r1, lim - 1);
-        const float x0 = (xqh[t0 + i0] - xkh[t0 + i0]) * (r0 < lim ? 1.f : 0.f);
-        const float x1 = (xqh[t0 + i1] - xkh[t0 + i1]) * (r1 < lim ? 1.f : 0.f);
-        float incl = x0 + x1;                       // inclusive suffix sum over lanes
-        for (int off = 1; off < 32; off <<= 1) {
-            const float up = __shfl_down_sync(0xffffffffu, incl, off);
-            if (lane + off < 32) incl += up;
+#pragma unroll
+        for (int k = 0; k < XN; ++k) {
+            const int c = min(cb + k * (DG_NT / 32), nch - 1);
+            const long long t0 = (long long)(c0 + c) * C;
+            // tokens past the end of the segment (ragged last chunk) contribute nothing
+            const int lim = min(C, ntok - c * C), i0 = min(r0, lim - 1), i1 = min(r1, lim - 1);
+            x0[k] = (xqh[t0 + i0] - xkh[t0 + i0]) * (r0 < lim ? 1.f : 0.f);
+            x1[k] = (xqh[t0 + i1] - xkh[t0 + i1]) * (r1 < lim ? 1.f : 0.f);
         }
-        if (r0 < C) suffix[c * 64 + r0] = incl;
-        if (r1 < C) suffix[c * 64 + r1] = incl - x0;
-        if (lane == 0) sx[c] = incl;
+#pragma unroll
+        for (int k = 0; k < XN; ++k) {
+            const int c = cb + k * (DG_NT / 32);
+            if (c < nch) {
+                float incl = x0[k] + x1[k];             // inclusive suffix sum over lanes
+                for (int off = 1; off < 32; off <<= 1) {
+                    const float up = __shfl_down_sync(0xffffffffu, incl, off);
+                    if (lane + off < 32) incl += up;
+                }
+                if (r0 < C) suffix[c * 64 + r0] = incl;
+                if (r1 < C) suffix[c * 64 + r1] = incl - x0[k];
+                if (lane == 0) sx[c] = incl;
+            }
+        }
     }
     __syncthreads();
     if (threadIdx.x == 0) {
