@@ -1,0 +1,447 @@
+// Warp-level tensor-core kernels (mma.sync) of the chunkwise gated linear recurrence for bf16 storage and small heads
+// (d_k, d_v in {32, 64}); same algebra, launch shape and results as the CUDA-core kernels (sf_simt.cuh), which keep float32
+// storage.  These heads are too narrow for the 128-wide tcgen05 tiles of sf_tc.cuh.
+//
+// Precision is that of float32 arithmetic.  q, k, v, dO are exact bf16 operands.  Everything float32 that enters a product (masked
+// scores, states, weighted rows) is split into three bf16 terms, x = h + m + l with the residuals taken exactly, which carries
+// its full 24-bit significand: the three MMAs of a product have exact products and float32 accumulation.  Scores (bf16 x
+// bf16) take one MMA.
+//
+// One CTA (4 warps) walks a block in tiles of 64 tokens; a warp owns 16 token rows of the outputs, so masked scores go from
+// accumulators to the next product's A operand in registers; the d_k x d_v state lives in the warps' accumulators (16 rows
+// each, or 16 rows x half the columns for 32 rows) and is published once per tile as three bf16 planes in shared memory.
+// Tiles arrive by cp.async one tile ahead.  Rows in shared memory are padded by 16 bytes: ldmatrix without bank conflicts.
+#pragma once
+#include "sf_common.cuh"
+#include "sf_simt.cuh"
+
+namespace sf {
+namespace wmm {
+
+using simt::CT;
+using simt::Decay;
+typedef __nv_bfloat16 bf16;
+constexpr int NT = 128;
+template <int D> constexpr int LD = D + 8;
+template <int D> constexpr int TILE = CT * LD<D>;
+
+__device__ __forceinline__ uint32_t saddr(const bf16* p) { return static_cast<uint32_t>(__cvta_generic_to_shared(p)); }
+__device__ __forceinline__ void ldsm(uint32_t (&r)[4], const bf16* p) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(saddr(p)) : "memory");
+}
+__device__ __forceinline__ void ldsm_t(uint32_t (&r)[4], const bf16* p) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(saddr(p)) : "memory");
+}
+__device__ __forceinline__ void mma(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+// Operand addresses inside a tile whose rows are LDX elements apart (lane l supplies one of the 32 row addresses).
+//   a_rows:  A[m][k] from rows m, columns k        a_cols: A[m][k] from rows k, columns m (transposing load)
+//   b_rows:  B[k][n] from rows n, columns k        b_cols: B[k][n] from rows k, columns n (transposing load)
+// The B loads give two neighbouring n-tiles: registers 0, 1 and 2, 3.
+template <int LDX> __device__ __forceinline__ const bf16* a_rows(const bf16* t, int m, int k) { const int l = threadIdx.x & 31; return t + (m + (l & 15)) * LDX + k + (l >> 4) * 8; }
+template <int LDX> __device__ __forceinline__ const bf16* a_cols(const bf16* t, int m, int k) { const int l = threadIdx.x & 31; return t + (k + (l & 7) + (l >> 4) * 8) * LDX + m + ((l >> 3) & 1) * 8; }
+template <int LDX> __device__ __forceinline__ const bf16* b_rows(const bf16* t, int k, int n) { const int l = threadIdx.x & 31; return t + (n + (l & 7) + (l >> 4) * 8) * LDX + k + ((l >> 3) & 1) * 8; }
+template <int LDX> __device__ __forceinline__ const bf16* b_cols(const bf16* t, int k, int n) { const int l = threadIdx.x & 31; return t + (k + (l & 15)) * LDX + n + (l >> 4) * 8; }
+
+__device__ __forceinline__ uint32_t pack(float a, float b) {
+    const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+    return *reinterpret_cast<const uint32_t*>(&h);
+}
+__device__ __forceinline__ float2 unpack(uint32_t v) { return make_float2(__uint_as_float(v << 16), __uint_as_float(v & 0xffff0000u)); }
+// (a, b) = sum of three bf16 pairs
+__device__ __forceinline__ void split(float a, float b, uint32_t& h, uint32_t& m, uint32_t& l) {
+    h = pack(a, b);
+    float2 f = unpack(h);
+    a -= f.x; b -= f.y;
+    m = pack(a, b);
+    f = unpack(m);
+    l = pack(a - f.x, b - f.y);
+}
+
+// CT x D tile from global rows `stride` elements apart, rows at or beyond `valid` zero; asynchronous.
+template <int D>
+__device__ __forceinline__ void fetch(bf16* dst, const bf16* __restrict__ src, long long stride, int valid) {
+#pragma unroll
+    for (int i = 0; i < CT * D / 8 / NT; ++i) {
+        const int idx = threadIdx.x + i * NT, r = idx / (D / 8), u = (idx % (D / 8)) * 8;
+        const int bytes = r < valid ? 16 : 0;
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(saddr(dst + r * LD<D> + u)), "l"(src + (long long)min(r, valid - 1) * stride + u), "r"(bytes) : "memory");
+    }
+}
+__device__ __forceinline__ void fetch_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void fetch_wait() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
+
+// Decay tables of a tile by one warp (simt::tile_decay, two tokens per lane, sums in double).
+__device__ __forceinline__ void tile_tables(Decay& d, const float* __restrict__ g, long long tg, int valid) {
+    const int l = threadIdx.x & 31, r0 = 2 * l, r1 = r0 + 1;
+    const double g0 = r0 < valid ? (double)g[r0 * tg] : 0.0, g1 = r1 < valid ? (double)g[r1 * tg] : 0.0;
+    double incl = g0 + g1;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const double up = __shfl_up_sync(0xffffffffu, incl, off);
+        if (l >= off) incl += up;
+    }
+    const double tot = __shfl_sync(0xffffffffu, incl, 31);
+    const double b[2] = {incl - g1, incl};
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+        const float hi = (float)b[e];
+        d.bh[r0 + e] = hi;
+        d.bl[r0 + e] = (float)(b[e] - (double)hi);
+        d.wsuf[r0 + e] = __expf((float)(tot - b[e]));
+        d.ebc[r0 + e] = __expf(hi);
+    }
+}
+
+// The DA x DB state, in accumulators: warp w holds rows 16 (w % MB) .., columns NCOL * (w / MB) ...
+template <int DA, int DB>
+struct State {
+    static constexpr int MB = DA / 16, NCOL = DB / (4 / MB), NTI = NCOL / 8;
+    float s[NTI][4];
+    int m0, n0;
+    __device__ __forceinline__ State() {
+        const int w = threadIdx.x >> 5;
+        m0 = 16 * (w % MB);
+        n0 = NCOL * (w / MB);
+    }
+    __device__ __forceinline__ void zero() {
+#pragma unroll
+        for (int j = 0; j < NTI; ++j)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) s[j][e] = 0.f;
+    }
+    // f(row, column) for the accumulator's elements
+    template <typename F> __device__ __forceinline__ void each(F f) {
+        const int l = threadIdx.x & 31;
+#pragma unroll
+        for (int j = 0; j < NTI; ++j)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) f(s[j][e], m0 + (l >> 2) + (e >> 1) * 8, n0 + 8 * j + 2 * (l & 3) + (e & 1));
+    }
+    // three bf16 planes [DA][DB] in shared memory
+    __device__ __forceinline__ void publish(bf16* planes) const {
+        const int l = threadIdx.x & 31;
+#pragma unroll
+        for (int j = 0; j < NTI; ++j)
+#pragma unroll
+            for (int hf = 0; hf < 2; ++hf) {
+                uint32_t p[3];
+                split(s[j][2 * hf], s[j][2 * hf + 1], p[0], p[1], p[2]);
+                const int off = (m0 + (l >> 2) + hf * 8) * LD<DB> + n0 + 8 * j + 2 * (l & 3);
+#pragma unroll
+                for (int t = 0; t < 3; ++t) *reinterpret_cast<uint32_t*>(planes + t * DA * LD<DB> + off) = p[t];
+            }
+    }
+    // s = decay s + sum_t wt[t] x_t^T z_t over the tile's tokens
+    __device__ __forceinline__ void step(const bf16* X, const float* wt, const bf16* Z, float decay) {
+        const int t2 = 2 * (threadIdx.x & 3);
+#pragma unroll
+        for (int j = 0; j < NTI; ++j)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) s[j][e] *= decay;
+#pragma unroll
+        for (int k = 0; k < CT; k += 16) {
+            uint32_t a[4], h[4], m[4], lo[4];
+            ldsm_t(a, a_cols<LD<DA>>(X, m0, k));
+            const float2 w0 = *reinterpret_cast<const float2*>(wt + k + t2), w1 = *reinterpret_cast<const float2*>(wt + k + 8 + t2);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float2 f = unpack(a[i]), w = i < 2 ? w0 : w1;
+                split(f.x * w.x, f.y * w.y, h[i], m[i], lo[i]);
+            }
+#pragma unroll
+            for (int jp = 0; jp < NTI / 2; ++jp) {
+                uint32_t b[4];
+                ldsm_t(b, b_cols<LD<DB>>(Z, k, n0 + 16 * jp));
+                mma(s[2 * jp], lo, b[0], b[1]); mma(s[2 * jp + 1], lo, b[2], b[3]);
+                mma(s[2 * jp], m, b[0], b[1]);  mma(s[2 * jp + 1], m, b[2], b[3]);
+                mma(s[2 * jp], h, b[0], b[1]);  mma(s[2 * jp + 1], h, b[2], b[3]);
+            }
+        }
+    }
+};
+
+// acc[16 rows of X][N] += X P, P [K][N] given as three planes with rows LDP apart: P[k][n] (COLS) or P^T stored, rows n (else)
+template <int K, int N, int LDP, bool COLS>
+__device__ __forceinline__ void times_planes(float (&acc)[N / 8][4], const uint32_t (&x)[K / 16][4], const bf16* planes, int plane_size) {
+#pragma unroll
+    for (int kk = 0; kk < K / 16; ++kk)
+#pragma unroll
+        for (int np = 0; np < N / 16; ++np)
+#pragma unroll
+            for (int t = 2; t >= 0; --t) {
+                uint32_t b[4];
+                if (COLS) ldsm_t(b, b_cols<LDP>(planes + t * plane_size, 16 * kk, 16 * np));
+                else      ldsm(b, b_rows<LDP>(planes + t * plane_size, 16 * kk, 16 * np));
+                mma(acc[2 * np], x[kk], b[0], b[1]);
+                mma(acc[2 * np + 1], x[kk], b[2], b[3]);
+            }
+}
+template <int D>
+__device__ __forceinline__ void row_operand(uint32_t (&x)[D / 16][4], const bf16* tile, int m0) {
+#pragma unroll
+    for (int kk = 0; kk < D / 16; ++kk) ldsm(x[kk], a_rows<LD<D>>(tile, m0, 16 * kk));
+}
+// Masked scores of the warp's 16 rows against 16 columns c0 .. c0 + 15 of the tile (rows of Y), then acc += scores Z.
+//   FWD: (x_r . y_s) exp(b_r - b_s) for s <= r;  else (x_s . y_r) exp(b_r - b_s) for r >= s (rows s, columns r)
+template <int DX, int DZ, bool FWD>
+__device__ __forceinline__ void scores_times(float (&acc)[DZ / 8][4], const uint32_t (&x)[DX / 16][4], const bf16* Y, const bf16* Z, const Decay& d,
+                                             int m0, int c0) {
+    const int l = threadIdx.x & 31, g = l >> 2, t2 = 2 * (l & 3);
+    float sc[2][4] = {};
+#pragma unroll
+    for (int kk = 0; kk < DX / 16; ++kk) {
+        uint32_t b[4];
+        ldsm(b, b_rows<LD<DX>>(Y, 16 * kk, c0));
+        mma(sc[0], x[kk], b[0], b[1]);
+        mma(sc[1], x[kk], b[2], b[3]);
+    }
+    uint32_t a[3][4];
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+#pragma unroll
+        for (int hf = 0; hf < 2; ++hf) {
+            const int row = m0 + g + 8 * hf;
+            const float rh = d.bh[row], rl = d.bl[row];
+            float v[2];
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const int col = c0 + 8 * j + t2 + e;
+                const float diff = FWD ? (rh - d.bh[col]) + (rl - d.bl[col]) : (d.bh[col] - rh) + (d.bl[col] - rl);
+                v[e] = (FWD ? col <= row : col >= row) ? sc[j][2 * hf + e] * __expf(diff) : 0.f;
+            }
+            split(v[0], v[1], a[0][2 * j + hf], a[1][2 * j + hf], a[2][2 * j + hf]);
+        }
+#pragma unroll
+    for (int np = 0; np < DZ / 16; ++np) {
+        uint32_t b[4];
+        ldsm_t(b, b_cols<LD<DZ>>(Z, c0, 16 * np));
+#pragma unroll
+        for (int t = 2; t >= 0; --t) {
+            mma(acc[2 * np], a[t], b[0], b[1]);
+            mma(acc[2 * np + 1], a[t], b[2], b[3]);
+        }
+    }
+}
+template <int N>
+__device__ __forceinline__ void scale(float (&acc)[N / 8][4], const float* w, int m0) {
+    const int g = (threadIdx.x & 31) >> 2;
+    const float w0 = w[m0 + g], w1 = w[m0 + g + 8];
+#pragma unroll
+    for (int j = 0; j < N / 8; ++j) { acc[j][0] *= w0; acc[j][1] *= w0; acc[j][2] *= w1; acc[j][3] *= w1; }
+}
+// rows below `valid` to global memory
+template <int N>
+__device__ __forceinline__ void store(bf16* __restrict__ dst, long long stride, int valid, const float (&acc)[N / 8][4], int m0) {
+    const int l = threadIdx.x & 31, t2 = 2 * (l & 3);
+#pragma unroll
+    for (int hf = 0; hf < 2; ++hf) {
+        const int r = m0 + (l >> 2) + 8 * hf;
+        if (r < valid)
+#pragma unroll
+            for (int j = 0; j < N / 8; ++j) *reinterpret_cast<uint32_t*>(dst + r * stride + 8 * j + t2) = pack(acc[j][2 * hf], acc[j][2 * hf + 1]);
+    }
+}
+// x[row] = <acc row, row of the tile E> in float32
+template <int N>
+__device__ __forceinline__ void dots(float* __restrict__ x, int valid, const float (&acc)[N / 8][4], const bf16* E, int m0) {
+    const int l = threadIdx.x & 31, t2 = 2 * (l & 3);
+#pragma unroll
+    for (int hf = 0; hf < 2; ++hf) {
+        const int r = m0 + (l >> 2) + 8 * hf;
+        float s = 0.f;
+#pragma unroll
+        for (int j = 0; j < N / 8; ++j) {
+            const float2 e = unpack(*reinterpret_cast<const uint32_t*>(E + r * LD<N> + 8 * j + t2));
+            s = fmaf(acc[j][2 * hf], e.x, s);
+            s = fmaf(acc[j][2 * hf + 1], e.y, s);
+        }
+        s += __shfl_xor_sync(0xffffffffu, s, 1);
+        s += __shfl_xor_sync(0xffffffffu, s, 2);
+        if ((l & 3) == 0 && r < valid) x[r] = s;
+    }
+}
+template <int N>
+__device__ __forceinline__ void zero(float (&acc)[N / 8][4]) {
+#pragma unroll
+    for (int j = 0; j < N / 8; ++j)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) acc[j][e] = 0.f;
+}
+
+// ---- block aggregates: the state recurrence from zero, over the block's tiles forward (mode 0: k, v) or reversed (mode 1: q, dO) ----
+template <int DK, int DV>
+struct AggSmem {
+    alignas(16) bf16 X[2][TILE<DK>];
+    alignas(16) bf16 Y[2][TILE<DV>];
+    Decay d[2];
+    double beta;
+};
+template <int DK, int DV>
+__global__ void __launch_bounds__(NT, 3) aggregate_kernel(SegParams p, const bf16* __restrict__ X, const bf16* __restrict__ Y, const float* __restrict__ g,
+                                                          int mode, float* __restrict__ U, float* __restrict__ beta_out) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    AggSmem<DK, DV>& sm = *reinterpret_cast<AggSmem<DK, DV>*>(smem_raw);
+    const int j = blockIdx.x, h = blockIdx.y, b = blockIdx.z, warp = threadIdx.x >> 5;
+    const int t_begin = j * p.R * p.C, t_end = min(p.L, t_begin + p.R * p.C), n = (t_end - t_begin + CT - 1) / CT;
+    const float* gh = g + (long long)b * p.bg + h;
+    const bf16* Xh = X + (long long)b * p.bqk + (long long)h * DK;
+    const bf16* Yh = Y + (long long)b * p.bv + (long long)h * DV;
+    auto tile0 = [&](int i) { return t_begin + (mode == 0 ? i : n - 1 - i) * CT; };
+    auto load = [&](int i) {
+        const int t0 = tile0(i), valid = min(CT, t_end - t0);
+        fetch<DK>(sm.X[i & 1], Xh + t0 * p.tqk, p.tqk, valid);
+        fetch<DV>(sm.Y[i & 1], Yh + t0 * p.tv, p.tv, valid);
+        fetch_commit();
+    };
+    auto tables = [&](int i) { const int t0 = tile0(i); tile_tables(sm.d[i & 1], gh + t0 * p.tg, p.tg, min(CT, t_end - t0)); };
+    State<DK, DV> st;
+    st.zero();
+    load(0);
+    if (warp == 0) tables(0);
+    double beta = 0.0;
+    for (int i = 0; i < n; ++i) {
+        fetch_wait();
+        __syncthreads();
+        if (i + 1 < n) { load(i + 1); if (warp == 0) tables(i + 1); }
+        const Decay& d = sm.d[i & 1];
+        beta += (double)d.bh[CT - 1] + (double)d.bl[CT - 1];
+        st.step(sm.X[i & 1], mode == 0 ? d.wsuf : d.ebc, sm.Y[i & 1], d.ebc[CT - 1]);
+    }
+    const long long blk = ((long long)b * p.H + h) * p.NB + j;
+    if (beta_out && threadIdx.x == 0) beta_out[blk] = (float)beta;
+    float* Uo = U + blk * (long long)(DK * DV);
+    st.each([&](float& x, int r, int c) { Uo[r * DV + c] = x; });
+}
+
+// ---- forward output pass / dq pass: rows x, keys y (DA wide), values z (DB wide), state sum y^T z (DA x DB) ----------------------
+//   forward: (x, y, z) = (q, k, v), state H;   dq: (dO, v, k), state H^T (read transposed), plus xq = <q, dq> from q rows e
+template <int DA, int DB, bool DQ>
+struct SweepSmem {
+    alignas(16) bf16 X[2][TILE<DA>];
+    alignas(16) bf16 Y[2][TILE<DA>];
+    alignas(16) bf16 Z[2][TILE<DB>];
+    alignas(16) bf16 E[DQ ? 2 : 1][DQ ? TILE<DB> : 8];
+    alignas(16) bf16 planes[3 * DA * LD<DB>];
+    Decay d[2];
+};
+template <int DA, int DB, bool DQ>
+__global__ void __launch_bounds__(NT, 2) sweep_kernel(SegParams p, const bf16* __restrict__ x, const bf16* __restrict__ y, const bf16* __restrict__ z,
+                                                      const float* __restrict__ g, const float* __restrict__ Hs, const bf16* __restrict__ e,
+                                                      bf16* __restrict__ out, float* __restrict__ xq) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    SweepSmem<DA, DB, DQ>& sm = *reinterpret_cast<SweepSmem<DA, DB, DQ>*>(smem_raw);
+    const int j = blockIdx.x, h = blockIdx.y, b = blockIdx.z, warp = threadIdx.x >> 5, m0 = 16 * warp;
+    const int t_begin = j * p.R * p.C, t_end = min(p.L, t_begin + p.R * p.C), n = (t_end - t_begin + CT - 1) / CT;
+    const float* gh = g + (long long)b * p.bg + h;
+    const long long ta = DQ ? p.tv : p.tqk, tb = DQ ? p.tqk : p.tv;                       // token strides of the DA / DB wide tensors
+    const long long oa = (long long)b * (DQ ? p.bv : p.bqk) + (long long)h * DA, ob = (long long)b * (DQ ? p.bqk : p.bv) + (long long)h * DB;
+    const long long bh = (long long)b * p.H + h;
+    auto load = [&](int i) {
+        const int t0 = t_begin + i * CT, valid = min(CT, t_end - t0);
+        fetch<DA>(sm.X[i & 1], x + oa + t0 * ta, ta, valid);
+        fetch<DA>(sm.Y[i & 1], y + oa + t0 * ta, ta, valid);
+        fetch<DB>(sm.Z[i & 1], z + ob + t0 * tb, tb, valid);
+        if constexpr (DQ) fetch<DB>(sm.E[i & 1], e + ob + t0 * tb, tb, valid);
+        fetch_commit();
+    };
+    auto tables = [&](int i) { const int t0 = t_begin + i * CT; tile_tables(sm.d[i & 1], gh + t0 * p.tg, p.tg, min(CT, t_end - t0)); };
+    load(0);
+    if (warp == 0) tables(0);
+    State<DA, DB> st;
+    const float* H0 = Hs + (bh * p.NB + j) * (long long)(DA * DB);
+    st.each([&](float& v, int r, int c) { v = DQ ? H0[c * DA + r] : H0[r * DB + c]; });
+    for (int i = 0; i < n; ++i) {
+        const int t0 = t_begin + i * CT, valid = min(CT, t_end - t0), s = i & 1;
+        st.publish(sm.planes);
+        fetch_wait();
+        __syncthreads();
+        if (i + 1 < n) { load(i + 1); if (warp == 0) tables(i + 1); }
+        const Decay& d = sm.d[s];
+        uint32_t xa[DA / 16][4];
+        row_operand<DA>(xa, sm.X[s], m0);
+        float acc[DB / 8][4];
+        zero<DB>(acc);
+        times_planes<DA, DB, LD<DB>, true>(acc, xa, sm.planes, DA * LD<DB>);
+        scale<DB>(acc, d.ebc, m0);
+        for (int c = 0; c <= warp; ++c) scores_times<DA, DB, true>(acc, xa, sm.Y[s], sm.Z[s], d, m0, 16 * c);
+        store<DB>(out + ob + t0 * tb, tb, valid, acc, m0);
+        if constexpr (DQ) dots<DB>(xq + bh * p.L + t0, valid, acc, sm.E[s], m0);
+        if (i + 1 < n) st.step(sm.Y[s], d.wsuf, sm.Z[s], d.ebc[CT - 1]);
+        __syncthreads();                                         // the planes may be rewritten
+    }
+}
+
+// ---- dk/dv pass: reverse sweep carrying G (DK x DV), rows s -----------------------------------------------------------------------
+template <int DK, int DV>
+struct DkdvSmem {
+    alignas(16) bf16 Q[2][TILE<DK>];
+    alignas(16) bf16 K[2][TILE<DK>];
+    alignas(16) bf16 V[2][TILE<DV>];
+    alignas(16) bf16 D[2][TILE<DV>];
+    alignas(16) bf16 planes[3 * DK * LD<DV>];
+    Decay d[2];
+};
+template <int DK, int DV>
+__global__ void __launch_bounds__(NT, 2) dkdv_kernel(SegParams p, const bf16* __restrict__ q, const bf16* __restrict__ k, const bf16* __restrict__ v,
+                                                     const float* __restrict__ g, const bf16* __restrict__ dO, const float* __restrict__ Gs,
+                                                     bf16* __restrict__ dk, bf16* __restrict__ dv, float* __restrict__ xk) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    DkdvSmem<DK, DV>& sm = *reinterpret_cast<DkdvSmem<DK, DV>*>(smem_raw);
+    const int j = blockIdx.x, h = blockIdx.y, b = blockIdx.z, warp = threadIdx.x >> 5, m0 = 16 * warp;
+    const int t_begin = j * p.R * p.C, t_end = min(p.L, t_begin + p.R * p.C), n = (t_end - t_begin + CT - 1) / CT;
+    const float* gh = g + (long long)b * p.bg + h;
+    const long long oqk = (long long)b * p.bqk + (long long)h * DK, ov = (long long)b * p.bv + (long long)h * DV;
+    const long long bh = (long long)b * p.H + h;
+    auto tile0 = [&](int i) { return t_begin + (n - 1 - i) * CT; };
+    auto load = [&](int i) {
+        const int t0 = tile0(i), valid = min(CT, t_end - t0);
+        fetch<DK>(sm.Q[i & 1], q + oqk + t0 * p.tqk, p.tqk, valid);
+        fetch<DK>(sm.K[i & 1], k + oqk + t0 * p.tqk, p.tqk, valid);
+        fetch<DV>(sm.V[i & 1], v + ov + t0 * p.tv, p.tv, valid);
+        fetch<DV>(sm.D[i & 1], dO + ov + t0 * p.tv, p.tv, valid);
+        fetch_commit();
+    };
+    auto tables = [&](int i) { const int t0 = tile0(i); tile_tables(sm.d[i & 1], gh + t0 * p.tg, p.tg, min(CT, t_end - t0)); };
+    load(0);
+    if (warp == 3) tables(0);
+    State<DK, DV> st;
+    const float* G0 = Gs + (bh * p.NB + j) * (long long)(DK * DV);
+    st.each([&](float& x, int r, int c) { x = G0[r * DV + c]; });
+    for (int i = 0; i < n; ++i) {
+        const int t0 = tile0(i), valid = min(CT, t_end - t0), s = i & 1;
+        st.publish(sm.planes);
+        fetch_wait();
+        __syncthreads();
+        if (i + 1 < n) { load(i + 1); if (warp == 3) tables(i + 1); }      // warp 3 has the shortest rows
+        const Decay& d = sm.d[s];
+        {   // dv = A^T dO + w K G
+            uint32_t a[DK / 16][4];
+            row_operand<DK>(a, sm.K[s], m0);
+            float acc[DV / 8][4];
+            zero<DV>(acc);
+            times_planes<DK, DV, LD<DV>, true>(acc, a, sm.planes, DK * LD<DV>);
+            scale<DV>(acc, d.wsuf, m0);
+            for (int c = warp; c < 4; ++c) scores_times<DK, DV, false>(acc, a, sm.Q[s], sm.D[s], d, m0, 16 * c);
+            store<DV>(dv + ov + t0 * p.tv, p.tv, valid, acc, m0);
+        }
+        {   // dk = dA^T Q + w V G^T
+            uint32_t a[DV / 16][4];
+            row_operand<DV>(a, sm.V[s], m0);
+            float acc[DK / 8][4];
+            zero<DK>(acc);
+            times_planes<DV, DK, LD<DV>, false>(acc, a, sm.planes, DK * LD<DV>);
+            scale<DK>(acc, d.wsuf, m0);
+            for (int c = warp; c < 4; ++c) scores_times<DV, DK, false>(acc, a, sm.D[s], sm.Q[s], d, m0, 16 * c);
+            store<DK>(dk + oqk + t0 * p.tqk, p.tqk, valid, acc, m0);
+            dots<DK>(xk + bh * p.L + t0, valid, acc, sm.K[s], m0);
+        }
+        if (i + 1 < n) st.step(sm.Q[s], d.ebc, sm.D[s], d.ebc[CT - 1]);
+        __syncthreads();
+    }
+}
+
+}  // namespace wmm
+}  // namespace sf

@@ -12,6 +12,7 @@
 
 #include "sf_common.cuh"
 #include "sf_scan.cuh"
+#include "sf_mma.cuh"
 #include "sf_simt.cuh"
 #include "sf_tc.cuh"
 
@@ -291,6 +292,47 @@ sf_status_t launch_simt(Role role, const SegParams& p, const RoleArgs& a, cudaSt
     return check_launch();
 }
 
+// bf16 storage, small heads: the warp-level tensor-core kernels
+template <int DK, int DV>
+sf_status_t launch_mma(Role role, const SegParams& p, const RoleArgs& a, cudaStream_t st) {
+    using namespace sf::wmm;
+    dim3 grid(p.NB, p.H, p.B), block(NT);
+    const bf16 *q = static_cast<const bf16*>(a.q), *k = static_cast<const bf16*>(a.k), *v = static_cast<const bf16*>(a.v), *dO = static_cast<const bf16*>(a.dO);
+    switch (role) {
+        case Role::Aggregate: {
+            constexpr size_t sm = sizeof(AggSmem<DK, DV>);
+            SF_TRY(set_smem(aggregate_kernel<DK, DV>, sm));
+            aggregate_kernel<DK, DV><<<grid, block, sm, st>>>(p, a.mode == 0 ? k : q, a.mode == 0 ? v : dO, a.g, a.mode, a.U, a.beta);
+            break;
+        }
+        case Role::FwdOut: {
+            constexpr size_t sm = sizeof(SweepSmem<DK, DV, false>);
+            SF_TRY(set_smem(sweep_kernel<DK, DV, false>, sm));
+            sweep_kernel<DK, DV, false><<<grid, block, sm, st>>>(p, q, k, v, a.g, a.states, nullptr, static_cast<bf16*>(a.o), nullptr);
+            break;
+        }
+        case Role::BwdDq: {
+            constexpr size_t sm = sizeof(SweepSmem<DV, DK, true>);
+            SF_TRY(set_smem(sweep_kernel<DV, DK, true>, sm));
+            sweep_kernel<DV, DK, true><<<grid, block, sm, st>>>(p, dO, v, k, a.g, a.states, q, static_cast<bf16*>(a.dq), a.xq);
+            break;
+        }
+        case Role::BwdDkDv: {
+            constexpr size_t sm = sizeof(DkdvSmem<DK, DV>);
+            SF_TRY(set_smem(dkdv_kernel<DK, DV>, sm));
+            dkdv_kernel<DK, DV><<<grid, block, sm, st>>>(p, q, k, v, a.g, dO, a.states, static_cast<bf16*>(a.dk), static_cast<bf16*>(a.dv), a.xk);
+            break;
+        }
+    }
+    return check_launch();
+}
+sf_status_t launch_mma_d(Role role, const sf_seg_desc_t* d, const SegParams& p, const RoleArgs& a, cudaStream_t st) {
+    if (d->d_k == 32 && d->d_v == 32) return launch_mma<32, 32>(role, p, a, st);
+    if (d->d_k == 64 && d->d_v == 64) return launch_mma<64, 64>(role, p, a, st);
+    if (d->d_k == 32 && d->d_v == 64) return launch_mma<32, 64>(role, p, a, st);
+    return SF_ERR_UNSUPPORTED;
+}
+
 template <typename T>
 sf_status_t launch_simt_d(Role role, const sf_seg_desc_t* d, const SegParams& p, const RoleArgs& a, cudaStream_t st) {
     if (d->d_k == 32 && d->d_v == 32) return launch_simt<T, 32, 32>(role, p, a, st);
@@ -317,7 +359,7 @@ sf_status_t launch_role(Path path, Role role, const sf_seg_desc_t* d, const SegP
         return s;
     }
     if (d->dtype == SF_F32) return launch_simt_d<float>(role, d, p, a, st);
-    return launch_simt_d<__nv_bfloat16>(role, d, p, a, st);
+    return launch_mma_d(role, d, p, a, st);
 }
 
 sf_status_t launch_scan(const sf_seg_desc_t* d, const SegParams& p, int reverse, const float* ld, const float* U,
