@@ -304,7 +304,7 @@ template <> struct ConvVec<1> {
     __device__ __forceinline__ void load(const float* p) { v[0] = *p; }
     __device__ __forceinline__ void store(float* p) const { *p = v[0]; }
 };
-template <> struct ConvVec<2> {
+template <> struct __align__(8) ConvVec<2> {
     float v[2];
     __device__ __forceinline__ void load(const float* p) { const float2 t = *reinterpret_cast<const float2*>(p); v[0] = t.x; v[1] = t.y; }
     __device__ __forceinline__ void store(float* p) const { *reinterpret_cast<float2*>(p) = make_float2(v[0], v[1]); }
@@ -369,11 +369,17 @@ conv_fwd_kernel(int B, int L, int C, const float* __restrict__ x, const float* _
 // of ext in registers and adds into one double-precision sum per tap; the units are dealt out over all row slices of a cluster
 // of CTAs that together cover every row of a group of channels, so the sums meet in the cluster's shared memory, in a fixed
 // order, and no workspace is needed.  block (LN lanes of V channels, 256 / LN slices); grid (channel groups, cluster).
-// Bound by memory latency at 16 warps per SM: 16384 rows x 1024 channels, W = 4, 201 MB in about 55 us; as two kernels, dx 27 us
-// and dw (scalar loads, one CTA per 8 channels) 38 us.  Forward + backward 102 -> 81 us; with four channels per thread 118
-// (registers), with one 92.
+// Bound by memory at the rate of many narrow row streams: 16384 rows x 1024 channels, W = 4, 201 MB in about 47 us (4.3 TB/s),
+// the same with clusters of 6 to 8 and with a ring twice as deep; 512-byte rows per warp were slower (89 us forward + backward).
+// As two kernels, dx took 27 us and dw (scalar loads, one CTA per 8 channels) 38 us.  Forward + backward: 102 us with those, 81
+// with rows loaded into registers four ahead, 73 with the ring.
 constexpr int CONV_UNIT_MIN = 32, CONV_NT = 256;
+constexpr int CONV_DEPTH = 8;
 template <int V> constexpr int kConvLanes = V == 2 ? 16 : 32;
+template <int V>
+__device__ __forceinline__ void conv_copy(ConvVec<V>* dst, const float* src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(static_cast<uint32_t>(__cvta_generic_to_shared(dst))), "l"(src), "n"(4 * V) : "memory");
+}
 template <int V, int W>
 __global__ void __launch_bounds__(CONV_NT, 2)
 conv_bwd_kernel(int B, int L, int C, const float* __restrict__ x, const float* __restrict__ w, const float* __restrict__ tail_in,
@@ -383,6 +389,7 @@ conv_bwd_kernel(int B, int L, int C, const float* __restrict__ x, const float* _
     namespace cg = cooperative_groups;
     cg::cluster_group cl = cg::this_cluster();
     __shared__ double part[CONV_NT / 32][W * V][LN];
+    __shared__ ConvVec<V> ring[CONV_DEPTH][2][CONV_NT];
     const int ln = threadIdx.x % LN, sl = threadIdx.x / LN;
     const int c = (blockIdx.x * LN + ln) * V;
     const bool on = c < C;
@@ -459,34 +466,35 @@ conv_bwd_kernel(int B, int L, int C, const float* __restrict__ x, const float* _
             }
             int e = e0;
             for (; e < min(e1, W - 1); ++e) edge_step(e);
-            // rows inside the segment, AHEAD at a time: the next ones are loaded while these are worked on
-            constexpr int AHEAD = 4;
-            const int inner = min(e1, L);
-            ConvVec<V> ny[AHEAD], nx[AHEAD];
+            // Rows inside the segment come through a ring in shared memory, CONV_DEPTH - 1 rows ahead: every thread copies the
+            // elements that it will use itself, so no barrier is needed.  A slot is refilled one row after it was read.
+            const int rows = min(e1, L) - e;
             const float *yp = db + (long long)e * C, *xp = xb + (long long)e * C;
             float* op = ob + (long long)(e - (W - 1)) * C;
-            const int quads = (inner - e) / AHEAD;
-            auto fetch = [&]() {
-#pragma unroll
-                for (int r = 0; r < AHEAD; ++r) { ny[r].load(yp); nx[r].load(xp); yp += C; xp += C; }
-            };
-            if (quads > 0) fetch();
-            for (int k = 0; k < quads; ++k, e += AHEAD) {
-                ConvVec<V> cy[AHEAD], cx[AHEAD];
-#pragma unroll
-                for (int r = 0; r < AHEAD; ++r) { cy[r] = ny[r]; cx[r] = nx[r]; }
-                if (k + 1 < quads) fetch();
-#pragma unroll
-                for (int r = 0; r < AHEAD; ++r) {
-                    wy[W - 1] = cy[r];
-                    widen(wx[W - 1], cx[r]);
-                    ConvVec<V> o;
-                    zero(o);
-                    step(o);
-                    o.store(op);
-                    op += C;
+            auto issue = [&](int k) {
+                if (k < rows) {
+                    conv_copy<V>(&ring[k % CONV_DEPTH][0][threadIdx.x], yp);
+                    conv_copy<V>(&ring[k % CONV_DEPTH][1][threadIdx.x], xp);
+                    yp += C; xp += C;
                 }
+                asm volatile("cp.async.commit_group;" ::: "memory");
+            };
+#pragma unroll
+            for (int k = 0; k < CONV_DEPTH - 1; ++k) issue(k);
+#pragma unroll 4
+            for (int k = 0; k < rows; ++k) {
+                asm volatile("cp.async.wait_group %0;" ::"n"(CONV_DEPTH - 2) : "memory");
+                wy[W - 1] = ring[k % CONV_DEPTH][0][threadIdx.x];
+                widen(wx[W - 1], ring[k % CONV_DEPTH][1][threadIdx.x]);
+                issue(k + CONV_DEPTH - 1);
+                ConvVec<V> o;
+                zero(o);
+                step(o);
+                o.store(op);
+                op += C;
             }
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+            e += max(rows, 0);
             for (; e < e1; ++e) edge_step(e);
         }
     // lanes with the same channel in a warp, then the warps, then the cluster's CTAs
