@@ -67,9 +67,9 @@ typedef enum { SF_BF16 = 0, SF_F32 = 1 } sf_dtype_t;
 
 /*
  * Shape of one segment.  Supported sets:
- *   SF_F32  : d_k, d_v in {32, 64, 128}, chunk in {16, 32, 64}          (CUDA-core kernels)
+ *   SF_F32  : d_k, d_v in {32, 64, 128}, chunk in {16, 32, 64}          (warp-level kernels)
  *   SF_BF16 : d_k = d_v = 128, chunk = 64                               (tcgen05 / TMEM / TMA kernels)
- *             d_k, d_v in {32, 64}, chunk in {16, 32, 64}               (CUDA-core kernels)
+ *             d_k, d_v in {32, 64}, chunk in {16, 32, 64}               (warp-level kernels)
  * seg_len is any positive number of tokens.  The paper rounds boundaries to multiples of 128 (Section 3.2), so
  * its workloads never leave a partial chunk; when seg_len is not a multiple of chunk the last chunk simply has
  * fewer tokens (its missing rows count as zero keys, values and gradients with log-decay 0, and are never
@@ -264,7 +264,7 @@ void sf_chain_graph_destroy(sf_chain_graph_t* graph);
  *                           one scan, one sweep, ...) instead of once per segment.  Tensor-core path: whenever all segments
  *                           but the last are whole chunks; the blocks then ignore the segment boundaries (block length =
  *                           chunks_per_block, else the library's choice for the whole sequence) and the forward sweep
- *                           itself writes the state entering each segment to S_bounds.  CUDA-core path: when every segment
+ *                           itself writes the state entering each segment to S_bounds.  Warp-level path: when every segment
  *                           but the last is a whole number of blocks of one common length.  Other chains run segment by
  *                           segment as with 0.  Same kernels; where the blocks coincide with the segments' own the
  *                           results are bit-identical, else equal to rounding.  The forward workspace is laid out

@@ -1,25 +1,45 @@
 // Warp-level tensor-core kernels (mma.sync) of the chunkwise gated linear recurrence for bf16 storage and small heads
-// (d_k, d_v in {32, 64}); same algebra, launch shape and results as the CUDA-core kernels (sf_simt.cuh), which keep float32
-// storage.  These heads are too narrow for the 128-wide tcgen05 tiles of sf_tc.cuh.
+// (d_k, d_v in {32, 64}); float32 storage: sf_mma3.cuh.  These heads are too narrow for the 128-wide tcgen05 tiles of sf_tc.cuh.
 //
 // Precision is that of float32 arithmetic.  q, k, v, dO are exact bf16 operands.  Everything float32 that enters a product (masked
 // scores, states, weighted rows) is split into three bf16 terms, x = h + m + l with the residuals taken exactly, which carries
-// its full 24-bit significand: the three MMAs of a product have exact products and float32 accumulation.  Scores (bf16 x
+// its full 24-bit significand: the three MMAs of a product have exact products and add up from zero; the 16-deep steps are added with rounding (add()).  Scores (bf16 x
 // bf16) take one MMA.
 //
 // One CTA (4 warps) walks a block in tiles of 64 tokens; a warp owns 16 token rows of the outputs, so masked scores go from
 // accumulators to the next product's A operand in registers; the d_k x d_v state lives in the warps' accumulators (16 rows
 // each, or 16 rows x half the columns for 32 rows) and is published once per tile as three bf16 planes in shared memory.
 // Tiles arrive by cp.async one tile ahead.  Rows in shared memory are padded by 16 bytes: ldmatrix without bank conflicts.
+// Measured: chain forward + backward, d = 64, 16384 tokens x 16 heads: 447 us (float32 products on CUDA cores 990).
+//
+// Algebra per tile (64 tokens; 32 for float32 storage) (b_r = inclusive cumulative log-decay inside the tile, b_C its total,
+// D[r,s] = exp(b_r - b_s) for s <= r, H_c the state entering the tile; paper Eq. 2 with
+// V_new = {} specialised to F_t = exp(g_t) I):
+//   Pre : A = (Q K^T) * D
+//   Out : O = A V + diag(exp(b)) Q H_c
+//   ST  : H_{c+1} = exp(b_C) H_c + sum_s exp(b_C - b_s) k_s^T v_s
+// and the adjoint stages named in Section 3.4 (SR, OG, STB, PG):
+//   OG  : dA = (dO V^T) * D ;  dq = dA K + diag(exp(b)) dO H_c^T
+//   STB : dH_c = exp(b_C) dH_{c+1} + sum_r exp(b_r) q_r^T dO_r
+//   PG  : dk = dA^T Q + diag(w) V dH_{c+1}^T ;  dv = A^T dO + diag(w) K dH_{c+1},  w_s = exp(b_C - b_s)
+// The tile is the kernels' own: a block of chunks_per_block * chunk tokens is walked in tiles whatever the chunk.
+// Every exponent is a sum of g over a token range (never a difference of long prefix sums), so all weights are <= 1 for
+// g <= 0 and nothing overflows; differences of the tile's prefix sums are taken on float pairs (sums in double).
 #pragma once
 #include "sf_common.cuh"
-#include "sf_simt.cuh"
 
 namespace sf {
 namespace wmm {
 
-using simt::CT;
-using simt::Decay;
+constexpr int CT = 64;         // tokens per tile
+constexpr int MAXR = 64;       // largest chunks_per_block
+constexpr int MAXC = 64;       // largest chunk
+
+struct Decay {
+    float bh[CT], bl[CT];      // inclusive cumulative log-decay as a float pair
+    float wsuf[CT];            // exp(sum_{u>r} g_u)
+    float ebc[CT];             // exp(sum_{u<=r} g_u)
+};
 typedef __nv_bfloat16 bf16;
 constexpr int NT = 128;
 template <int D> constexpr int LD = D + 8;
@@ -35,6 +55,15 @@ __device__ __forceinline__ void ldsm_t(uint32_t (&r)[4], const bf16* p) {
 __device__ __forceinline__ void mma(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
     asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
                  : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+// acc += u for N n-tiles.  The MMAs of one 16-deep step start from zero and their sum is added here, rounded: the tensor core
+// truncates when it adds to an accumulator, which over a long contraction costs up to five times the error (measured).
+template <int N>
+__device__ __forceinline__ void add(float (*acc)[4], const float (&u)[N][4]) {
+#pragma unroll
+    for (int j = 0; j < N; ++j)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) acc[j][e] += u[j][e];
 }
 // Operand addresses inside a tile whose rows are LDX elements apart (lane l supplies one of the 32 row addresses).
 //   a_rows:  A[m][k] from rows m, columns k        a_cols: A[m][k] from rows k, columns m (transposing load)
@@ -73,7 +102,8 @@ __device__ __forceinline__ void fetch(bf16* dst, const bf16* __restrict__ src, l
 __device__ __forceinline__ void fetch_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void fetch_wait() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
 
-// Decay tables of a tile by one warp (simt::tile_decay, two tokens per lane, sums in double).
+// Decay tables of the tile whose `valid` tokens start at g (token stride tg), by one warp, two tokens per lane.  A tile with
+// fewer than CT tokens counts as if padded with zero rows of log-decay 0, which changes no sum; its missing rows are never stored.
 __device__ __forceinline__ void tile_tables(Decay& d, const float* __restrict__ g, long long tg, int valid) {
     const int l = threadIdx.x & 31, r0 = 2 * l, r1 = r0 + 1;
     const double g0 = r0 < valid ? (double)g[r0 * tg] : 0.0, g1 = r1 < valid ? (double)g[r1 * tg] : 0.0;
@@ -155,9 +185,11 @@ struct State {
             for (int jp = 0; jp < NTI / 2; ++jp) {
                 uint32_t b[4];
                 ldsm_t(b, b_cols<LD<DB>>(Z, k, n0 + 16 * jp));
-                mma(s[2 * jp], lo, b[0], b[1]); mma(s[2 * jp + 1], lo, b[2], b[3]);
-                mma(s[2 * jp], m, b[0], b[1]);  mma(s[2 * jp + 1], m, b[2], b[3]);
-                mma(s[2 * jp], h, b[0], b[1]);  mma(s[2 * jp + 1], h, b[2], b[3]);
+                float u[2][4] = {};
+                mma(u[0], lo, b[0], b[1]); mma(u[1], lo, b[2], b[3]);
+                mma(u[0], m, b[0], b[1]);  mma(u[1], m, b[2], b[3]);
+                mma(u[0], h, b[0], b[1]);  mma(u[1], h, b[2], b[3]);
+                add(&s[2 * jp], u);
             }
         }
     }
@@ -167,17 +199,20 @@ struct State {
 template <int K, int N, int LDP, bool COLS>
 __device__ __forceinline__ void times_planes(float (&acc)[N / 8][4], const uint32_t (&x)[K / 16][4], const bf16* planes, int plane_size) {
 #pragma unroll
-    for (int kk = 0; kk < K / 16; ++kk)
+    for (int kk = 0; kk < K / 16; ++kk) {
+        float u[N / 8][4] = {};
 #pragma unroll
-        for (int np = 0; np < N / 16; ++np)
+        for (int t = 2; t >= 0; --t)
 #pragma unroll
-            for (int t = 2; t >= 0; --t) {
+            for (int np = 0; np < N / 16; ++np) {
                 uint32_t b[4];
                 if (COLS) ldsm_t(b, b_cols<LDP>(planes + t * plane_size, 16 * kk, 16 * np));
                 else      ldsm(b, b_rows<LDP>(planes + t * plane_size, 16 * kk, 16 * np));
-                mma(acc[2 * np], x[kk], b[0], b[1]);
-                mma(acc[2 * np + 1], x[kk], b[2], b[3]);
+                mma(u[2 * np], x[kk], b[0], b[1]);
+                mma(u[2 * np + 1], x[kk], b[2], b[3]);
             }
+        add(acc, u);
+    }
 }
 template <int D>
 __device__ __forceinline__ void row_operand(uint32_t (&x)[D / 16][4], const bf16* tile, int m0) {
@@ -218,11 +253,13 @@ __device__ __forceinline__ void scores_times(float (&acc)[DZ / 8][4], const uint
     for (int np = 0; np < DZ / 16; ++np) {
         uint32_t b[4];
         ldsm_t(b, b_cols<LD<DZ>>(Z, c0, 16 * np));
+        float u[2][4] = {};
 #pragma unroll
         for (int t = 2; t >= 0; --t) {
-            mma(acc[2 * np], a[t], b[0], b[1]);
-            mma(acc[2 * np + 1], a[t], b[2], b[3]);
+            mma(u[0], a[t], b[0], b[1]);
+            mma(u[1], a[t], b[2], b[3]);
         }
+        add(&acc[2 * np], u);
     }
 }
 template <int N>

@@ -1,0 +1,528 @@
+// Warp-level tensor-core kernels (mma.sync) of the chunkwise gated linear recurrence for float32 storage; algebra as in
+// sf_mma.cuh.
+//
+// Precision is that of float32 arithmetic: every operand is split into three bf16 terms, x = h + m + l with the residuals taken
+// exactly, which carries its full 24-bit significand.  Of the nine term products the six largest are taken; each of the
+// three left out is below 2^-25 of the full product, less than the rounding of a float32 product.  Products are exact, the MMAs
+// of a 16-deep step add up from zero, and the steps are added with rounding.  Measured against the fp64 oracle (4096 tokens,
+// slow decay, d = 128): o 5.1e-7 max / 4.0e-7 rms, with multiply-adds on CUDA cores 6.1e-7 / 3.5e-7.
+//
+// Why: a token and head cost about 170 k multiply-adds forward + backward at d = 128 against 2.8 KB of traffic, so the arithmetic
+// bounds these kernels.  Six MMAs at the 275 T/s measured for mma.sync are 46 T float32 multiply-adds/s; the FMA pipe gives
+// 35, of which the register-tiled kernels that stood here reached 17.  Chains forward + backward, before and now (us):
+// d = 128, 8144 tokens x 16 heads 1608 -> 1208; 8192 x 32 3137 -> 2321; 512 x 2 113 -> 105; d = 64, 8192 x 16 592 -> 444, 256 x 2
+// 70 -> 66; d = 32, 16384 x 40 1267 -> 946.  The tensor pipe is 57 % busy on the SMs that have a block; the rest is
+// splitting tiles and states and the barriers between the stages of a tile.
+//
+// One CTA walks a block in tiles of 32 tokens, RB = 2 row blocks of 16 x WC column groups of warps.  Tiles, and the state entering
+// the tile, are three bf16 planes in shared memory (rows padded by 16 bytes: ldmatrix without bank conflicts); 32 tokens because
+// four tiles and the state of 128 x 128 heads then fill the 227 KB.  The state lives in the warps' accumulators and its planes are
+// rewritten as it is updated, while the next tile is on its way to registers.  The scores' contraction over features is shared
+// by groups of warps and added up through shared memory.  16 warps per SM: with 8, each with twice the columns, the d = 128
+// kernels take 3 % longer.
+#pragma once
+#include "sf_mma.cuh"
+
+namespace sf {
+namespace w3 {
+
+using wmm::add;
+using wmm::bf16;
+using wmm::LD;
+using wmm::ldsm;
+using wmm::ldsm_t;
+using wmm::mma;
+using wmm::split;
+using wmm::unpack;
+constexpr int CT = 32, RB = 2;
+constexpr int LDP = CT + 4;                                      // row of the score partials
+template <int DK> constexpr int kWarps = DK / 8;                  // 16 warps per SM in one, two or four CTAs
+template <int D> constexpr int PLANE = CT * LD<D>;
+
+struct Decay { float bh[CT], bl[CT], wsuf[CT], ebc[CT]; };       // as wmm::Decay
+__device__ __forceinline__ void tile_tables(Decay& d, const float* __restrict__ g, long long tg, int valid) {
+    const int l = threadIdx.x & 31;
+    const double g0 = l < valid ? (double)g[l * tg] : 0.0;
+    double b = g0;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const double up = __shfl_up_sync(0xffffffffu, b, off);
+        if (l >= off) b += up;
+    }
+    const double tot = __shfl_sync(0xffffffffu, b, 31);
+    const float hi = (float)b;
+    d.bh[l] = hi;
+    d.bl[l] = (float)(b - (double)hi);
+    d.wsuf[l] = __expf((float)(tot - b));
+    d.ebc[l] = __expf(hi);
+}
+
+// CT x D tile: global rows to registers, registers to planes.
+template <int D, int NT>
+struct Raw {
+    static constexpr int N = CT * D / 4 / NT;
+    float4 v[N];
+    __device__ __forceinline__ void fetch(const float* __restrict__ src, long long stride, int valid) {
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            const int idx = threadIdx.x + i * NT, r = idx / (D / 4), c = (idx % (D / 4)) * 4;
+            v[i] = r < valid ? __ldg(reinterpret_cast<const float4*>(src + (long long)r * stride + c)) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+    }
+    __device__ __forceinline__ void put(bf16* planes) const {
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            const int idx = threadIdx.x + i * NT, r = idx / (D / 4), c = (idx % (D / 4)) * 4;
+            uint32_t a[3], b[3];
+            split(v[i].x, v[i].y, a[0], a[1], a[2]);
+            split(v[i].z, v[i].w, b[0], b[1], b[2]);
+#pragma unroll
+            for (int t = 0; t < 3; ++t) *reinterpret_cast<uint2*>(planes + t * PLANE<D> + r * LD<D> + c) = make_uint2(a[t], b[t]);
+        }
+    }
+};
+
+// c[0 .. 2 N - 1] += the six leading term products of the three-term operands a and b (small ones first); b holds N pairs of n-tiles.
+// The accumulators of all n-tiles take a term before the next term: 2 N independent MMAs in a row.
+template <int N>
+__device__ __forceinline__ void mma6(float (*c)[4], const uint32_t (&a)[3][4], const uint32_t (&b)[N][3][4]) {
+    constexpr int TA[6] = {2, 0, 1, 1, 0, 0}, TB[6] = {0, 2, 1, 0, 1, 0};
+#pragma unroll
+    for (int t = 0; t < 6; ++t)
+#pragma unroll
+        for (int n = 0; n < N; ++n) {
+            mma(c[2 * n], a[TA[t]], b[n][TB[t]][0], b[n][TB[t]][1]);
+            mma(c[2 * n + 1], a[TA[t]], b[n][TB[t]][2], b[n][TB[t]][3]);
+        }
+}
+
+// The DA x DB state in accumulators, NW warps: warp w holds rows 16 (w % MB) .., columns NCOL * (w / MB) ..
+template <int DA, int DB, int NW>
+struct State {
+    static constexpr int MB = DA / 16, NCOL = DB / (NW / MB), NTI = NCOL / 8;
+    static_assert(NW % MB == 0 && NTI % 2 == 0, "state split");
+    float s[NTI][4];
+    int m0, n0;
+    __device__ __forceinline__ State() {
+        const int w = threadIdx.x >> 5;
+        m0 = 16 * (w % MB);
+        n0 = NCOL * (w / MB);
+    }
+    template <typename F> __device__ __forceinline__ void each(F f) {
+        const int l = threadIdx.x & 31;
+#pragma unroll
+        for (int j = 0; j < NTI; ++j)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) f(s[j][e], m0 + (l >> 2) + (e >> 1) * 8, n0 + 8 * j + 2 * (l & 3) + (e & 1));
+    }
+    __device__ __forceinline__ void publish(bf16* planes, int j) const {
+        const int l = threadIdx.x & 31;
+#pragma unroll
+        for (int hf = 0; hf < 2; ++hf) {
+            uint32_t p[3];
+            split(s[j][2 * hf], s[j][2 * hf + 1], p[0], p[1], p[2]);
+            const int off = (m0 + (l >> 2) + hf * 8) * LD<DB> + n0 + 8 * j + 2 * (l & 3);
+#pragma unroll
+            for (int t = 0; t < 3; ++t) *reinterpret_cast<uint32_t*>(planes + t * DA * LD<DB> + off) = p[t];
+        }
+    }
+    __device__ __forceinline__ void publish(bf16* planes) const {
+#pragma unroll
+        for (int j = 0; j < NTI; ++j) publish(planes, j);
+    }
+    // s = decay s + sum_t wt[t] x_t^T z_t over the tile's tokens; the sum starts from zero; the new state to planes
+    __device__ __forceinline__ void step(const bf16* X, const float* wt, const bf16* Z, float decay, bf16* planes) {
+        constexpr int JP = 1;
+        const int t2 = 2 * (threadIdx.x & 3);
+        uint32_t a[CT / 16][3][4];
+#pragma unroll
+        for (int k = 0; k < CT / 16; ++k) {
+            uint32_t x[3][4];
+#pragma unroll
+            for (int t = 0; t < 3; ++t) ldsm_t(x[t], wmm::a_cols<LD<DA>>(X + t * PLANE<DA>, m0, 16 * k));
+            const float2 w0 = *reinterpret_cast<const float2*>(wt + 16 * k + t2), w1 = *reinterpret_cast<const float2*>(wt + 16 * k + 8 + t2);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float2 h = unpack(x[0][i]), m = unpack(x[1][i]), l = unpack(x[2][i]), w = i < 2 ? w0 : w1;
+                split(((h.x + m.x) + l.x) * w.x, ((h.y + m.y) + l.y) * w.y, a[k][0][i], a[k][1][i], a[k][2][i]);       // the sums are exact
+            }
+        }
+#pragma unroll
+        for (int jp = 0; jp < NTI / 2; jp += JP) {
+            float u[2 * JP][4] = {};
+#pragma unroll
+            for (int k = 0; k < CT / 16; ++k) {
+                uint32_t b[JP][3][4];
+#pragma unroll
+                for (int i = 0; i < JP; ++i)
+#pragma unroll
+                    for (int t = 0; t < 3; ++t) ldsm_t(b[i][t], wmm::b_cols<LD<DB>>(Z + t * PLANE<DB>, 16 * k, n0 + 16 * (jp + i)));
+                mma6<JP>(u, a[k], b);
+            }
+#pragma unroll
+            for (int i = 0; i < 2 * JP; ++i) {
+#pragma unroll
+                for (int e = 0; e < 4; ++e) s[2 * jp + i][e] = fmaf(s[2 * jp + i][e], decay, u[i][e]);
+                if (planes) publish(planes, 2 * jp + i);
+            }
+        }
+    }
+};
+
+// acc[16 rows m0.. of X][NC columns from n0] += X P over K features; P[k][n] stored by rows k (COLS) or P^T, rows n
+template <int K, int NC, int LDB, bool COLS>
+__device__ __forceinline__ void times_planes(float (&acc)[NC / 8][4], const bf16* X, int m0, const bf16* planes, int plane_size, int n0) {
+#pragma unroll 2
+    for (int kk = 0; kk < K / 16; ++kk) {
+        uint32_t a[3][4], b[NC / 16][3][4];
+#pragma unroll
+        for (int t = 0; t < 3; ++t) ldsm(a[t], wmm::a_rows<LD<K>>(X + t * PLANE<K>, m0, 16 * kk));
+#pragma unroll
+        for (int np = 0; np < NC / 16; ++np)
+#pragma unroll
+            for (int t = 0; t < 3; ++t) {
+                if (COLS) ldsm_t(b[np][t], wmm::b_cols<LDB>(planes + t * plane_size, 16 * kk, n0 + 16 * np));
+                else      ldsm(b[np][t], wmm::b_rows<LDB>(planes + t * plane_size, 16 * kk, n0 + 16 * np));
+            }
+        float u[NC / 8][4] = {};
+        mma6<NC / 16>(u, a, b);
+        add(acc, u);
+    }
+}
+// The scores X Y^T of the tile, as partial sums over KG groups of features: 16 x 16 blocks, SC column blocks beside each other.
+// FWD: the blocks up to the diagonal, else from it on.
+template <int NW> struct Split {
+    static constexpr int SC = NW >= 8 ? 2 : 1, KG = NW / (RB * SC);
+};
+template <int D, int NW, bool FWD>
+__device__ __forceinline__ void score_partials(float* part, const bf16* X, const bf16* Y) {
+    constexpr int SC = Split<NW>::SC, KG = Split<NW>::KG, F = D / KG;
+    const int l = threadIdx.x & 31, w = threadIdx.x >> 5, rb = w % RB, kg = (w / RB) % KG, m0 = 16 * rb, f0 = F * kg;
+    for (int c = SC == 1 ? 0 : w / (RB * KG); c < RB; c += SC) {
+        if (FWD ? c > rb : c < rb) continue;
+        float sc[2][4] = {};
+#pragma unroll
+        for (int f = 0; f < F; f += 16) {
+            uint32_t a[3][4], b[1][3][4];
+#pragma unroll
+            for (int t = 0; t < 3; ++t) {
+                ldsm(a[t], wmm::a_rows<LD<D>>(X + t * PLANE<D>, m0, f0 + f));
+                ldsm(b[0][t], wmm::b_rows<LD<D>>(Y + t * PLANE<D>, f0 + f, 16 * c));
+            }
+            mma6<1>(sc, a, b);
+        }
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+#pragma unroll
+            for (int hf = 0; hf < 2; ++hf)
+                *reinterpret_cast<float2*>(part + (kg * CT + m0 + (l >> 2) + 8 * hf) * LDP + 16 * c + 8 * j + 2 * (l & 3)) = make_float2(sc[j][2 * hf], sc[j][2 * hf + 1]);
+    }
+}
+// Sums of the partials times the decay mask, split into three bf16 pairs that replace partials 0 and 1 of the same place.
+template <int NW, bool FWD>
+__device__ __forceinline__ void mask_scores(float* part, const Decay& d) {
+#pragma unroll
+    for (int i = threadIdx.x; i < CT * CT / 2; i += 32 * NW) {
+        const int row = i / (CT / 2), col = (i % (CT / 2)) * 2;
+        if (FWD ? (col & 16) > (row & 16) : (col & 16) < (row & 16)) continue;
+        float* p0 = part + row * LDP + col;
+        float2 s = *reinterpret_cast<const float2*>(p0);
+#pragma unroll
+        for (int w = 1; w < Split<NW>::KG; ++w) {
+            const float2 o = *reinterpret_cast<const float2*>(p0 + w * CT * LDP);
+            s.x += o.x; s.y += o.y;
+        }
+        const float rh = d.bh[row], rl = d.bl[row];
+        const float2 ch = *reinterpret_cast<const float2*>(d.bh + col), cl = *reinterpret_cast<const float2*>(d.bl + col);
+        const float e0 = FWD ? (rh - ch.x) + (rl - cl.x) : (ch.x - rh) + (cl.x - rl);
+        const float e1 = FWD ? (rh - ch.y) + (rl - cl.y) : (ch.y - rh) + (cl.y - rl);
+        uint32_t h, m, lo;
+        split((FWD ? col <= row : col >= row) ? s.x * __expf(e0) : 0.f, (FWD ? col + 1 <= row : col + 1 >= row) ? s.y * __expf(e1) : 0.f, h, m, lo);
+        *reinterpret_cast<uint2*>(p0) = make_uint2(h, m);
+        *reinterpret_cast<uint32_t*>(p0 + CT * LDP) = lo;
+    }
+}
+// acc += (masked scores) Z for NC columns from n0
+template <int DZ, int NC, bool FWD>
+__device__ __forceinline__ void scores_times(float (&acc)[NC / 8][4], const float* part, const bf16* Z, int rb, int n0) {
+    const int l = threadIdx.x & 31;
+    for (int c = FWD ? 0 : rb; c < (FWD ? rb + 1 : RB); ++c) {
+        uint32_t a[3][4], b[NC / 16][3][4];
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+#pragma unroll
+            for (int hf = 0; hf < 2; ++hf) {
+                const float* p0 = part + (16 * rb + (l >> 2) + 8 * hf) * LDP + 16 * c + 8 * j + 2 * (l & 3);
+                const uint2 hm = *reinterpret_cast<const uint2*>(p0);
+                a[0][2 * j + hf] = hm.x;
+                a[1][2 * j + hf] = hm.y;
+                a[2][2 * j + hf] = *reinterpret_cast<const uint32_t*>(p0 + CT * LDP);
+            }
+#pragma unroll
+        for (int np = 0; np < NC / 16; ++np)
+#pragma unroll
+            for (int t = 0; t < 3; ++t) ldsm_t(b[np][t], wmm::b_cols<LD<DZ>>(Z + t * PLANE<DZ>, 16 * c, n0 + 16 * np));
+        float u[NC / 8][4] = {};
+        mma6<NC / 16>(u, a, b);
+        add(acc, u);
+    }
+}
+// f(accumulator pair, row in the tile, column) for the warp's 16 x NC outputs
+template <int NC, typename F>
+__device__ __forceinline__ void each_pair(const float (&acc)[NC / 8][4], int rb, int n0, F f) {
+    const int l = threadIdx.x & 31;
+#pragma unroll
+    for (int hf = 0; hf < 2; ++hf)
+#pragma unroll
+        for (int j = 0; j < NC / 8; ++j) f(acc[j][2 * hf], acc[j][2 * hf + 1], 16 * rb + (l >> 2) + 8 * hf, n0 + 8 * j + 2 * (l & 3), hf, j);
+}
+template <int NC>
+__device__ __forceinline__ void store(float* __restrict__ dst, long long stride, int valid, const float (&acc)[NC / 8][4], int rb, int n0) {
+    each_pair<NC>(acc, rb, n0, [&](float a, float b, int r, int c, int, int) {
+        if (r < valid) *reinterpret_cast<float2*>(dst + r * stride + c) = make_float2(a, b);
+    });
+}
+// row sums of acc * e into red[row]; e[hf][j] is the pair beside acc[j][2 hf]
+template <int NC>
+__device__ __forceinline__ void row_dots(float* red, const float (&acc)[NC / 8][4], const float2 (&e)[2][NC / 8], int rb) {
+    const int l = threadIdx.x & 31;
+#pragma unroll
+    for (int hf = 0; hf < 2; ++hf) {
+        float s = 0.f;
+#pragma unroll
+        for (int j = 0; j < NC / 8; ++j) { s = fmaf(acc[j][2 * hf], e[hf][j].x, s); s = fmaf(acc[j][2 * hf + 1], e[hf][j].y, s); }
+        s += __shfl_xor_sync(0xffffffffu, s, 1);
+        s += __shfl_xor_sync(0xffffffffu, s, 2);
+        if ((l & 3) == 0) red[16 * rb + (l >> 2) + 8 * hf] = s;
+    }
+}
+template <int WC>
+__device__ __forceinline__ void store_dots(float* __restrict__ x, const float* red, int valid) {
+    if ((int)threadIdx.x < valid) {
+        float s = red[threadIdx.x];
+#pragma unroll
+        for (int w = 1; w < WC; ++w) s += red[w * CT + threadIdx.x];
+        x[threadIdx.x] = s;
+    }
+}
+
+// ---- block aggregates: the state recurrence from zero, tiles forward (mode 0: k, v) or reversed (mode 1: q, dO) -------------------
+template <int DK, int DV>
+struct AggSmem {
+    alignas(16) bf16 X[3 * PLANE<DK>];
+    alignas(16) bf16 Y[3 * PLANE<DV>];
+    Decay d[2];
+};
+template <int DK, int DV>
+__global__ void __launch_bounds__(32 * kWarps<DK>, 16 / kWarps<DK>)
+aggregate_kernel(SegParams p, const float* __restrict__ X, const float* __restrict__ Y, const float* __restrict__ g, int mode, float* __restrict__ U,
+                 float* __restrict__ beta_out) {
+    constexpr int NW = kWarps<DK>, NT = 32 * NW;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    AggSmem<DK, DV>& sm = *reinterpret_cast<AggSmem<DK, DV>*>(smem_raw);
+    const int j = blockIdx.x, h = blockIdx.y, b = blockIdx.z, warp = threadIdx.x >> 5;
+    const int t_begin = j * p.R * p.C, t_end = min(p.L, t_begin + p.R * p.C), n = (t_end - t_begin + CT - 1) / CT;
+    const float* gh = g + (long long)b * p.bg + h;
+    const float* Xh = X + (long long)b * p.bqk + (long long)h * DK;
+    const float* Yh = Y + (long long)b * p.bv + (long long)h * DV;
+    auto tile0 = [&](int i) { return t_begin + (mode == 0 ? i : n - 1 - i) * CT; };
+    Raw<DK, NT> rx;
+    Raw<DV, NT> ry;
+    auto load = [&](int i) {
+        const int t0 = tile0(i), valid = min(CT, t_end - t0);
+        rx.fetch(Xh + t0 * p.tqk, p.tqk, valid);
+        ry.fetch(Yh + t0 * p.tv, p.tv, valid);
+    };
+    auto tables = [&](int i) { const int t0 = tile0(i); tile_tables(sm.d[i & 1], gh + t0 * p.tg, p.tg, min(CT, t_end - t0)); };
+    State<DK, DV, NW> st;
+    st.each([](float& x, int, int) { x = 0.f; });
+    load(0);
+    if (warp == 0) tables(0);
+    double beta = 0.0;
+    for (int i = 0; i < n; ++i) {
+        rx.put(sm.X);
+        ry.put(sm.Y);
+        __syncthreads();
+        if (i + 1 < n) { load(i + 1); if (warp == 0) tables(i + 1); }
+        const Decay& d = sm.d[i & 1];
+        beta += (double)d.bh[CT - 1] + (double)d.bl[CT - 1];
+        st.step(sm.X, mode == 0 ? d.wsuf : d.ebc, sm.Y, d.ebc[CT - 1], nullptr);
+        __syncthreads();
+    }
+    const long long blk = ((long long)b * p.H + h) * p.NB + j;
+    if (beta_out && threadIdx.x == 0) beta_out[blk] = (float)beta;
+    float* Uo = U + blk * (long long)(DK * DV);
+    st.each([&](float& x, int r, int c) { Uo[r * DV + c] = x; });
+}
+
+// ---- forward output pass / dq pass (tile roles as wmm::sweep_kernel) --------------------------------------------------------------
+template <int DA, int DB, int NW>
+struct SweepSmem {
+    alignas(16) bf16 X[3 * PLANE<DA>];
+    alignas(16) bf16 Y[3 * PLANE<DA>];
+    alignas(16) bf16 Z[3 * PLANE<DB>];
+    alignas(16) bf16 planes[3 * DA * LD<DB>];
+    float part[Split<NW>::KG * CT * LDP];
+    float red[NW / RB * CT];
+    Decay d[2];
+};
+template <int DA, int DB, int NW, bool DQ>
+__global__ void __launch_bounds__(32 * NW, 16 / NW)
+sweep_kernel(SegParams p, const float* __restrict__ x, const float* __restrict__ y, const float* __restrict__ z, const float* __restrict__ g,
+             const float* __restrict__ Hs, const float* __restrict__ e, float* __restrict__ out, float* __restrict__ xq) {
+    constexpr int NT = 32 * NW, WC = NW / RB, NC = DB / WC;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    SweepSmem<DA, DB, NW>& sm = *reinterpret_cast<SweepSmem<DA, DB, NW>*>(smem_raw);
+    const int j = blockIdx.x, h = blockIdx.y, b = blockIdx.z, warp = threadIdx.x >> 5, rb = warp % RB, wc = warp / RB, n0 = NC * wc;
+    const int t_begin = j * p.R * p.C, t_end = min(p.L, t_begin + p.R * p.C), n = (t_end - t_begin + CT - 1) / CT;
+    const float* gh = g + (long long)b * p.bg + h;
+    const long long ta = DQ ? p.tv : p.tqk, tb = DQ ? p.tqk : p.tv;
+    const long long oa = (long long)b * (DQ ? p.bv : p.bqk) + (long long)h * DA, ob = (long long)b * (DQ ? p.bqk : p.bv) + (long long)h * DB;
+    const long long bh = (long long)b * p.H + h;
+    Raw<DA, NT> rx, ry;
+    Raw<DB, NT> rz;
+    auto load = [&](int i) {
+        const int t0 = t_begin + i * CT, valid = min(CT, t_end - t0);
+        rx.fetch(x + oa + t0 * ta, ta, valid);
+        ry.fetch(y + oa + t0 * ta, ta, valid);
+        rz.fetch(z + ob + t0 * tb, tb, valid);
+    };
+    auto tables = [&](int i) { const int t0 = t_begin + i * CT; tile_tables(sm.d[i & 1], gh + t0 * p.tg, p.tg, min(CT, t_end - t0)); };
+    load(0);
+    if (warp == 0) tables(0);
+    State<DA, DB, NW> st;
+    const float* H0 = Hs + (bh * p.NB + j) * (long long)(DA * DB);
+    st.each([&](float& v, int r, int c) { v = DQ ? H0[c * DA + r] : H0[r * DB + c]; });
+    st.publish(sm.planes);
+    for (int i = 0; i < n; ++i) {
+        const int t0 = t_begin + i * CT, valid = min(CT, t_end - t0);
+        rx.put(sm.X);
+        ry.put(sm.Y);
+        rz.put(sm.Z);
+        __syncthreads();
+        if (warp == 0 && i + 1 < n) tables(i + 1);
+        const Decay& d = sm.d[i & 1];
+        float2 er[2][NC / 8];
+        float acc[NC / 8][4] = {};
+        if constexpr (DQ)                                        // the q rows of the dot products are on their way meanwhile
+            each_pair<NC>(acc, rb, n0, [&](float, float, int r, int c, int hf, int jj) {
+                er[hf][jj] = r < valid ? __ldg(reinterpret_cast<const float2*>(e + ob + (t0 + r) * tb + c)) : make_float2(0.f, 0.f);
+            });
+        score_partials<DA, NW, true>(sm.part, sm.X, sm.Y);
+        times_planes<DA, NC, LD<DB>, true>(acc, sm.X, 16 * rb, sm.planes, DA * LD<DB>, n0);
+        {
+            const int l = threadIdx.x & 31;
+            const float w0 = d.ebc[16 * rb + (l >> 2)], w1 = d.ebc[16 * rb + (l >> 2) + 8];
+#pragma unroll
+            for (int jj = 0; jj < NC / 8; ++jj) { acc[jj][0] *= w0; acc[jj][1] *= w0; acc[jj][2] *= w1; acc[jj][3] *= w1; }
+        }
+        __syncthreads();
+        mask_scores<NW, true>(sm.part, d);
+        __syncthreads();
+        scores_times<DB, NC, true>(acc, sm.part, sm.Z, rb, n0);
+        store<NC>(out + ob + t0 * tb, tb, valid, acc, rb, n0);
+        if constexpr (DQ) row_dots<NC>(sm.red + wc * CT, acc, er, rb);
+        if (i + 1 < n) {
+            load(i + 1);
+            st.step(sm.Y, d.wsuf, sm.Z, d.ebc[CT - 1], sm.planes);
+        }
+        __syncthreads();
+        if constexpr (DQ) store_dots<WC>(xq + bh * p.L + t0, sm.red, valid);
+    }
+}
+
+// ---- dk/dv pass: reverse sweep carrying G, rows s ---------------------------------------------------------------------------------
+template <int DK, int DV, int NW>
+struct DkdvSmem {
+    alignas(16) bf16 Q[3 * PLANE<DK>];
+    alignas(16) bf16 K[3 * PLANE<DK>];
+    alignas(16) bf16 V[3 * PLANE<DV>];
+    alignas(16) bf16 D[3 * PLANE<DV>];
+    alignas(16) bf16 planes[3 * DK * LD<DV>];
+    float part[Split<NW>::KG * CT * LDP];
+    float red[NW / RB * CT];
+    Decay d[2];
+};
+template <int DK, int DV, int NW>
+__global__ void __launch_bounds__(32 * NW, 16 / NW)
+dkdv_kernel(SegParams p, const float* __restrict__ q, const float* __restrict__ k, const float* __restrict__ v, const float* __restrict__ g,
+            const float* __restrict__ dO, const float* __restrict__ Gs, float* __restrict__ dk, float* __restrict__ dv, float* __restrict__ xk) {
+    constexpr int NT = 32 * NW, WC = NW / RB, NV = DV / WC, NK = DK / WC;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    DkdvSmem<DK, DV, NW>& sm = *reinterpret_cast<DkdvSmem<DK, DV, NW>*>(smem_raw);
+    const int j = blockIdx.x, h = blockIdx.y, b = blockIdx.z, warp = threadIdx.x >> 5, rb = warp % RB, wc = warp / RB, l = threadIdx.x & 31;
+    const int t_begin = j * p.R * p.C, t_end = min(p.L, t_begin + p.R * p.C), n = (t_end - t_begin + CT - 1) / CT;
+    const float* gh = g + (long long)b * p.bg + h;
+    const long long oqk = (long long)b * p.bqk + (long long)h * DK, ov = (long long)b * p.bv + (long long)h * DV;
+    const long long bh = (long long)b * p.H + h;
+    auto tile0 = [&](int i) { return t_begin + (n - 1 - i) * CT; };
+    Raw<DK, NT> rq, rk;
+    Raw<DV, NT> rv, rd;
+    auto load = [&](int i) {
+        const int t0 = tile0(i), valid = min(CT, t_end - t0);
+        rq.fetch(q + oqk + t0 * p.tqk, p.tqk, valid);
+        rk.fetch(k + oqk + t0 * p.tqk, p.tqk, valid);
+        rv.fetch(v + ov + t0 * p.tv, p.tv, valid);
+        rd.fetch(dO + ov + t0 * p.tv, p.tv, valid);
+    };
+    auto tables = [&](int i) { const int t0 = tile0(i); tile_tables(sm.d[i & 1], gh + t0 * p.tg, p.tg, min(CT, t_end - t0)); };
+    load(0);
+    if (warp == 1) tables(0);
+    State<DK, DV, NW> st;
+    const float* G0 = Gs + (bh * p.NB + j) * (long long)(DK * DV);
+    st.each([&](float& x, int r, int c) { x = G0[r * DV + c]; });
+    st.publish(sm.planes);
+    for (int i = 0; i < n; ++i) {
+        const int t0 = tile0(i), valid = min(CT, t_end - t0);
+        rq.put(sm.Q);
+        rk.put(sm.K);
+        rv.put(sm.V);
+        rd.put(sm.D);
+        __syncthreads();
+        if (warp == 1 && i + 1 < n) tables(i + 1);
+        const Decay& d = sm.d[i & 1];
+        const float w0 = d.wsuf[16 * rb + (l >> 2)], w1 = d.wsuf[16 * rb + (l >> 2) + 8];
+        {   // dv = A^T dO + w K G
+            float acc[NV / 8][4] = {};
+            score_partials<DK, NW, false>(sm.part, sm.K, sm.Q);
+            times_planes<DK, NV, LD<DV>, true>(acc, sm.K, 16 * rb, sm.planes, DK * LD<DV>, NV * wc);
+#pragma unroll
+            for (int jj = 0; jj < NV / 8; ++jj) { acc[jj][0] *= w0; acc[jj][1] *= w0; acc[jj][2] *= w1; acc[jj][3] *= w1; }
+            __syncthreads();
+            mask_scores<NW, false>(sm.part, d);
+            __syncthreads();
+            scores_times<DV, NV, false>(acc, sm.part, sm.D, rb, NV * wc);
+            store<NV>(dv + ov + t0 * p.tv, p.tv, valid, acc, rb, NV * wc);
+        }
+        {   // dk = dA^T Q + w V G^T
+            float acc[NK / 8][4] = {};
+            times_planes<DV, NK, LD<DV>, false>(acc, sm.V, 16 * rb, sm.planes, DK * LD<DV>, NK * wc);
+#pragma unroll
+            for (int jj = 0; jj < NK / 8; ++jj) { acc[jj][0] *= w0; acc[jj][1] *= w0; acc[jj][2] *= w1; acc[jj][3] *= w1; }
+            __syncthreads();                                     // the partials of A have been read
+            score_partials<DV, NW, false>(sm.part, sm.V, sm.D);
+            __syncthreads();
+            mask_scores<NW, false>(sm.part, d);
+            __syncthreads();
+            scores_times<DK, NK, false>(acc, sm.part, sm.Q, rb, NK * wc);
+            store<NK>(dk + oqk + t0 * p.tqk, p.tqk, valid, acc, rb, NK * wc);
+            float2 er[2][NK / 8];
+            each_pair<NK>(acc, rb, NK * wc, [&](float, float, int r, int c, int hf, int jj) {
+                const bf16* kp = sm.K + r * LD<DK> + c;
+                const float2 x0 = unpack(*reinterpret_cast<const uint32_t*>(kp)), x1 = unpack(*reinterpret_cast<const uint32_t*>(kp + PLANE<DK>)),
+                             x2 = unpack(*reinterpret_cast<const uint32_t*>(kp + 2 * PLANE<DK>));
+                er[hf][jj] = make_float2((x0.x + x1.x) + x2.x, (x0.y + x1.y) + x2.y);
+            });
+            row_dots<NK>(sm.red + wc * CT, acc, er, rb);
+        }
+        if (i + 1 < n) {
+            load(i + 1);
+            st.step(sm.Q, d.ebc, sm.D, d.ebc[CT - 1], sm.planes);
+        }
+        __syncthreads();
+        store_dots<WC>(xk + bh * p.L + t0, sm.red, valid);
+    }
+}
+
+}  // namespace w3
+}  // namespace sf

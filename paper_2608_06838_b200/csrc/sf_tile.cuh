@@ -1,5 +1,4 @@
-// Register-tiled float32 products on CUDA cores, shared by the float32 / small-head kernels and the chunkwise forms of the
-// extension operators.
+// Register-tiled float32 products on CUDA cores, for the chunkwise forms of the extension operators.
 //
 // Operands live in shared memory as row-major float32 tiles whose 16-byte units are XOR-swizzled with the row's index over
 // four: unit u of row r sits at position u ^ ((r >> 2) & 7).  A product C[m][n] += sum_k A(m,k) B(k,n) reads an operand

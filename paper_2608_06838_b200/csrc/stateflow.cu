@@ -13,7 +13,7 @@
 #include "sf_common.cuh"
 #include "sf_scan.cuh"
 #include "sf_mma.cuh"
-#include "sf_simt.cuh"
+#include "sf_mma3.cuh"
 #include "sf_tc.cuh"
 
 namespace {
@@ -69,7 +69,7 @@ enum class Path { Invalid, Unsupported, Simt, Tc };
 Path classify(const sf_seg_desc_t* d) {
     if (!d) return Path::Invalid;
     if (d->B <= 0 || d->H <= 0 || d->d_k <= 0 || d->d_v <= 0 || d->chunk <= 0 || d->seg_len <= 0) return Path::Invalid;
-    if (d->chunks_per_block < 0 || d->chunks_per_block > sf::simt::MAXR) return Path::Invalid;
+    if (d->chunks_per_block < 0 || d->chunks_per_block > sf::wmm::MAXR) return Path::Invalid;
     if (d->dtype != SF_BF16 && d->dtype != SF_F32) return Path::Invalid;
     if (d->tok_stride_qk < (long long)d->H * d->d_k || d->tok_stride_v < (long long)d->H * d->d_v || d->tok_stride_g < d->H)
         return Path::Invalid;
@@ -141,12 +141,12 @@ int chain_chunks_per_block(int NC, long long bh) {
     return (int)((NC + nb - 1) / nb);
 }
 
-// Block length of the CUDA-core kernels, which walk a block in tiles of 64 tokens: waves * (tiles per block + what a CTA costs
-// besides its tiles), one wave being all CTAs that fit on the device at once.  A tile is 10-25 us of arithmetic, so unlike
+// Block length of the warp-level kernels (sf_mma.cuh, sf_mma3.cuh), in tiles of 64 tokens: waves * (tiles per block + what a CTA costs
+// besides its tiles), one wave being all CTAs that fit on the device at once.  A tile is 5-15 us of arithmetic, so unlike
 // on the tensor-core path short blocks cost little; at most 16 tiles, beyond which the block states no longer count.
 // Ties go to the longer block.
-int simt_chunks_per_block(const sf_seg_desc_t* d) {
-    const int tile = sf::simt::CT, cpt = tile / d->chunk;                 // chunks per tile
+int tile_chunks_per_block(const sf_seg_desc_t* d) {
+    const int tile = sf::wmm::CT, cpt = tile / d->chunk;                 // chunks per tile
     const long long ntile = ((long long)d->seg_len + tile - 1) / tile, bh = (long long)d->B * d->H;
     const long long slots = (long long)sm_count() * (d->d_k == 128 ? 1 : (d->d_k == 64 ? 2 : 3));
     long long best_cost = -1;
@@ -174,7 +174,7 @@ SegParams make_params(const sf_seg_desc_t* d, int cpb_override = 0) {
     p.B = d->B; p.H = d->H; p.L = d->seg_len; p.C = d->chunk;
     p.NC = (d->seg_len + d->chunk - 1) / d->chunk;      // the last chunk may be partial
     int r = cpb_override > 0 ? cpb_override : d->chunks_per_block;
-    p.R = r > 0 ? r : (on_tensor_cores(d) ? auto_chunks_per_block(p.NC, (long long)d->B * d->H) : simt_chunks_per_block(d));
+    p.R = r > 0 ? r : (on_tensor_cores(d) ? auto_chunks_per_block(p.NC, (long long)d->B * d->H) : tile_chunks_per_block(d));
     p.NB = (p.NC + p.R - 1) / p.R;
     p.tqk = d->tok_stride_qk; p.tv = d->tok_stride_v; p.tg = d->tok_stride_g;
     p.bqk = d->batch_stride_qk; p.bv = d->batch_stride_v; p.bg = d->batch_stride_g;
@@ -248,50 +248,6 @@ struct RoleArgs {
     float *xq, *xk;
 };
 
-template <typename T, int DK, int DV>
-sf_status_t launch_simt(Role role, const SegParams& p, const RoleArgs& a, cudaStream_t st) {
-    using namespace sf::simt;
-    dim3 grid(p.NB, p.H, p.B), block(kThreads<DK>);
-    switch (role) {
-        case Role::Aggregate: {
-            auto kern = block_aggregate_kernel<T, DK, DV>;
-            constexpr size_t sm = sizeof(AggSmem<DK, DV>);
-            SF_TRY(set_smem(kern, sm));
-            const T* X = static_cast<const T*>(a.mode == 0 ? a.k : a.q);
-            const T* Y = static_cast<const T*>(a.mode == 0 ? a.v : a.dO);
-            kern<<<grid, block, sm, st>>>(p, X, Y, a.g, a.mode, a.U, a.beta);
-            break;
-        }
-        case Role::FwdOut: {
-            auto kern = fwd_out_kernel<T, DK, DV>;
-            constexpr size_t sm = sizeof(FwdSmem<DK, DV>);
-            SF_TRY(set_smem(kern, sm));
-            kern<<<grid, block, sm, st>>>(p, static_cast<const T*>(a.q), static_cast<const T*>(a.k),
-                                          static_cast<const T*>(a.v), a.g, a.states, static_cast<T*>(a.o));
-            break;
-        }
-        case Role::BwdDq: {
-            auto kern = bwd_dq_kernel<T, DK, DV>;
-            constexpr size_t sm = sizeof(DqSmem<DK, DV>);
-            SF_TRY(set_smem(kern, sm));
-            kern<<<grid, block, sm, st>>>(p, static_cast<const T*>(a.q), static_cast<const T*>(a.k),
-                                          static_cast<const T*>(a.v), a.g, static_cast<const T*>(a.dO), a.states,
-                                          static_cast<T*>(a.dq), a.xq);
-            break;
-        }
-        case Role::BwdDkDv: {
-            auto kern = bwd_dkdv_kernel<T, DK, DV>;
-            constexpr size_t sm = sizeof(DkdvSmem<DK, DV>);
-            SF_TRY(set_smem(kern, sm));
-            kern<<<grid, block, sm, st>>>(p, static_cast<const T*>(a.q), static_cast<const T*>(a.k),
-                                          static_cast<const T*>(a.v), a.g, static_cast<const T*>(a.dO), a.states,
-                                          static_cast<T*>(a.dk), static_cast<T*>(a.dv), a.xk);
-            break;
-        }
-    }
-    return check_launch();
-}
-
 // bf16 storage, small heads: the warp-level tensor-core kernels
 template <int DK, int DV>
 sf_status_t launch_mma(Role role, const SegParams& p, const RoleArgs& a, cudaStream_t st) {
@@ -333,19 +289,51 @@ sf_status_t launch_mma_d(Role role, const sf_seg_desc_t* d, const SegParams& p, 
     return SF_ERR_UNSUPPORTED;
 }
 
-template <typename T>
-sf_status_t launch_simt_d(Role role, const sf_seg_desc_t* d, const SegParams& p, const RoleArgs& a, cudaStream_t st) {
-    if (d->d_k == 32 && d->d_v == 32) return launch_simt<T, 32, 32>(role, p, a, st);
-    if (d->d_k == 64 && d->d_v == 64) return launch_simt<T, 64, 64>(role, p, a, st);
-    if (d->d_k == 32 && d->d_v == 64) return launch_simt<T, 32, 64>(role, p, a, st);
-    if constexpr (sizeof(T) == 4) {
-        if (d->d_k == 128 && d->d_v == 128) return launch_simt<T, 128, 128>(role, p, a, st);
+// float32 storage
+template <int DK, int DV>
+sf_status_t launch_mma3(Role role, const SegParams& p, const RoleArgs& a, cudaStream_t st) {
+    using namespace sf::w3;
+    constexpr int NW = kWarps<DK>;
+    dim3 grid(p.NB, p.H, p.B), block(32 * NW);
+    const float *q = static_cast<const float*>(a.q), *k = static_cast<const float*>(a.k), *v = static_cast<const float*>(a.v), *dO = static_cast<const float*>(a.dO);
+    switch (role) {
+        case Role::Aggregate: {
+            constexpr size_t sm = sizeof(AggSmem<DK, DV>);
+            SF_TRY(set_smem(aggregate_kernel<DK, DV>, sm));
+            aggregate_kernel<DK, DV><<<grid, block, sm, st>>>(p, a.mode == 0 ? k : q, a.mode == 0 ? v : dO, a.g, a.mode, a.U, a.beta);
+            break;
+        }
+        case Role::FwdOut: {
+            constexpr size_t sm = sizeof(SweepSmem<DK, DV, NW>);
+            SF_TRY(set_smem(sweep_kernel<DK, DV, NW, false>, sm));
+            sweep_kernel<DK, DV, NW, false><<<grid, block, sm, st>>>(p, q, k, v, a.g, a.states, nullptr, static_cast<float*>(a.o), nullptr);
+            break;
+        }
+        case Role::BwdDq: {
+            constexpr size_t sm = sizeof(SweepSmem<DV, DK, NW>);
+            SF_TRY(set_smem(sweep_kernel<DV, DK, NW, true>, sm));
+            sweep_kernel<DV, DK, NW, true><<<grid, block, sm, st>>>(p, dO, v, k, a.g, a.states, q, static_cast<float*>(a.dq), a.xq);
+            break;
+        }
+        case Role::BwdDkDv: {
+            constexpr size_t sm = sizeof(DkdvSmem<DK, DV, NW>);
+            SF_TRY(set_smem(dkdv_kernel<DK, DV, NW>, sm));
+            dkdv_kernel<DK, DV, NW><<<grid, block, sm, st>>>(p, q, k, v, a.g, dO, a.states, static_cast<float*>(a.dk), static_cast<float*>(a.dv), a.xk);
+            break;
+        }
     }
+    return check_launch();
+}
+sf_status_t launch_mma3_d(Role role, const sf_seg_desc_t* d, const SegParams& p, const RoleArgs& a, cudaStream_t st) {
+    if (d->d_k == 32 && d->d_v == 32) return launch_mma3<32, 32>(role, p, a, st);
+    if (d->d_k == 64 && d->d_v == 64) return launch_mma3<64, 64>(role, p, a, st);
+    if (d->d_k == 32 && d->d_v == 64) return launch_mma3<32, 64>(role, p, a, st);
+    if (d->d_k == 128 && d->d_v == 128) return launch_mma3<128, 128>(role, p, a, st);
     return SF_ERR_UNSUPPORTED;
 }
 
 // `early`: the kernel may start while the one before it in the stream finishes (launch_after()); it must then follow a kernel of
-// the same call.  The CUDA-core kernels do not take part.
+// the same call.  The warp-level kernels do not take part.
 sf_status_t launch_role(Path path, Role role, const sf_seg_desc_t* d, const SegParams& p, const RoleArgs& a, cudaStream_t st, bool early) {
     const int stage = role == Role::Aggregate ? (a.mode == 0 ? ST_AGG_KV : ST_AGG_QDO)
                     : role == Role::FwdOut ? ST_FWD_OUT : role == Role::BwdDq ? ST_DQ : ST_DKDV;
@@ -358,7 +346,7 @@ sf_status_t launch_role(Path path, Role role, const sf_seg_desc_t* d, const SegP
         g_launches.fetch_add(n, std::memory_order_relaxed);
         return s;
     }
-    if (d->dtype == SF_F32) return launch_simt_d<float>(role, d, p, a, st);
+    if (d->dtype == SF_F32) return launch_mma3_d(role, d, p, a, st);
     return launch_mma_d(role, d, p, a, st);
 }
 
@@ -631,7 +619,7 @@ sf_status_t validate_chain(const sf_seg_desc_t* d, const int32_t* seg_lens, int3
 }
 
 // ---- merged launches (sf_tuning_t.merge_launches) ------------------------------------------------------------------
-// When the segments are whole chunks (tensor-core path) or, on the CUDA-core path, every segment but the last is a whole
+// When the segments are whole chunks (tensor-core path) or, on the warp-level path, every segment but the last is a whole
 // number of blocks of one common length R, the chain is ONE segment that spans the sequence: each stage then runs once over the whole chain (one aggregate launch,
 // one scan, one sweep, ...) instead of once per segment, with the same blocks, the same kernels and the same arithmetic
 // (results are bit-identical).  The boundary states S_bounds[i] are the states entering the first block of each segment.
@@ -661,12 +649,12 @@ bool merged_desc(const sf_seg_desc_t* desc, const int32_t* seg_lens, int32_t n_s
     int R = desc->chunks_per_block;
     if (R == 0) {
         // the longest block length up to the library's choice that divides the chunk count of every segment but the last
-        for (R = simt_chunks_per_block(&t); R >= 1; --R) {
+        for (R = tile_chunks_per_block(&t); R >= 1; --R) {
             bool ok = true;
             for (int i = 0; i + 1 < n_seg && ok; ++i) ok = (seg_lens[i] / C) % R == 0;
             if (ok) break;
         }
-        if (R * C < sf::simt::CT) return false;
+        if (R * C < sf::wmm::CT) return false;
     } else {
         for (int i = 0; i + 1 < n_seg; ++i)
             if ((seg_lens[i] / C) % R) return false;
@@ -843,7 +831,7 @@ sf_status_t sf_segment_fwd_static(const sf_seg_desc_t* desc, const void* q, cons
     // The scratch array bounds the number of blocks: where the library's choice has more than fit, the longest that fit.
     sf_seg_desc_t d = *desc;
     if (d.chunks_per_block == 0)
-        for (int r = make_params(&d).R; sf_workspace_bytes(&d, 0) > SF_STATIC_SCRATCH_BYTES && r < sf::simt::MAXR;) d.chunks_per_block = ++r;
+        for (int r = make_params(&d).R; sf_workspace_bytes(&d, 0) > SF_STATIC_SCRATCH_BYTES && r < sf::wmm::MAXR;) d.chunks_per_block = ++r;
     if (sf_workspace_bytes(&d, 0) > SF_STATIC_SCRATCH_BYTES) return SF_ERR_WORKSPACE;
     // device address of the scratch array, looked up once per device with that device current
     constexpr int kMaxDevices = 64;
@@ -870,7 +858,7 @@ sf_status_t sf_state_scan(const sf_seg_desc_t* desc, int32_t chunks_per_block, i
     Path path = classify(desc);
     if (path == Path::Invalid) return SF_ERR_INVALID_ARG;
     if (path == Path::Unsupported) return SF_ERR_UNSUPPORTED;
-    if (chunks_per_block < 0 || chunks_per_block > sf::simt::MAXR) return SF_ERR_INVALID_ARG;
+    if (chunks_per_block < 0 || chunks_per_block > sf::wmm::MAXR) return SF_ERR_INVALID_ARG;
     if (!log_decay || !U || !states || !S_boundary_out || S_boundary_in == S_boundary_out) return SF_ERR_INVALID_ARG;
     if (!aligned16(U) || !aligned16(states) || !aligned16(S_boundary_out) || (S_boundary_in && !aligned16(S_boundary_in)))
         return SF_ERR_INVALID_ARG;

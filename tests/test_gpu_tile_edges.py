@@ -12,7 +12,7 @@ pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
 
 
-# The CUDA-core kernels walk a block in tiles of 64 tokens whatever the chunk: blocks shorter than a tile (3 chunks of 16),
+# The warp-level kernels walk a block in tiles of 64 tokens (float32: 32) whatever the chunk: blocks shorter than a tile (3 chunks of 16),
 # of one tile and a remainder (5 of 16, 3 of 32), of whole tiles; segments that end one token before, at and after a tile.
 @pytest.mark.parametrize("chunk,cpb", [(16, 3), (16, 5), (32, 3), (64, 2), (64, 0)])
 @pytest.mark.parametrize("dk,dv,dtype", [(32, 32, "f32"), (32, 64, "bf16"), (64, 64, "f32"), (64, 64, "bf16"), (128, 128, "f32")])
