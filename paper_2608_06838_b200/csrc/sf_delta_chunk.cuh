@@ -575,23 +575,25 @@ __global__ void __launch_bounds__(kThreads<DK, DV>) out_kernel(Params p, const T
 }
 
 // ---- backward, tile-parallel: every input gradient of the tile from the stored Hc, dHc, T, A, KM.  grid (tiles, H, B) ------
-// The shared memory of a 128-wide head holds one of the two states at a time; H is then fetched twice.
+// From 64 x 64 on the shared memory holds one of the two states at a time and H is fetched twice: three CTAs of a 64 x 64 head then
+// share an SM instead of two (KM is read from global memory for the same reason), 684 -> 597 us at 16 heads x 512 tiles.
 template <int DK, int DV>
 struct BwdSmem {
-    static constexpr bool BOTH = DK * DV <= 64 * 64;
+    static constexpr bool BOTH = DK * DV < 64 * 64;
+    static constexpr int RW = kThreads<DK, DV> == 256 ? 4 : 2;
     float Q[CT * DK], K[CT * DK], V[CT * DV], D[CT * DV];
     float R[CT * DV];                   // beta*V - beta*gam*(K H), then dW, then the two C x C products
     float W[CT * DV];
     float H[DK * DV], G[BOTH ? DK * DV : 4];
-    float T[CC], A[CC], KM[CC];
+    float T[CC], A[CC];
     Decay d;
-    float qd[CT * 4], kw[CT * 4], kz[CT * 4], zv[CT * 4];              // row sums, per warp that shares a row
+    float qd[CT * RW], kw[CT * RW], kz[CT * RW], zv[CT * RW];          // row sums, per warp that shares a row
     float rs[CT], rl[CT], part[8];
 };
-// Row sums of acc(m, n) e(m, n) into red[m * 4 + warp column]: a butterfly over the eight lanes that share the row.
-template <class Mp, typename F>
+// Row sums of acc(m, n) e(m, n) into red[m * RW + warp column]: a butterfly over the eight lanes that share the row.
+template <int RW, class Mp, typename F>
 __device__ __forceinline__ void row_dots(const float (&acc)[Mp::TM][Mp::TN], const Mp& mp, float* red, F e) {
-    static_assert(Mp::TXN / 8 <= 4, "red holds four partial sums per row");
+    static_assert(Mp::TXN / 8 <= RW, "red holds RW partial sums per row");
 #pragma unroll
     for (int i = 0; i < Mp::TM; ++i) {
         float s = 0.f;
@@ -602,14 +604,14 @@ __device__ __forceinline__ void row_dots(const float (&acc)[Mp::TM][Mp::TN], con
             s = fmaf(acc[i][4 * gq + 2], v.z, s); s = fmaf(acc[i][4 * gq + 3], v.w, s);
         }
         s = tile::sum_x(s);
-        if ((mp.tx & 7) == 0) red[mp.m(i) * 4 + (mp.tx >> 3)] = s;
+        if ((mp.tx & 7) == 0) red[mp.m(i) * RW + (mp.tx >> 3)] = s;
     }
 }
-template <class Mp>
+template <int RW, class Mp>
 __device__ __forceinline__ float row_sum(const float* red, int t) {
-    float s = red[t * 4];
+    float s = red[t * RW];
 #pragma unroll
-    for (int w = 1; w < Mp::TXN / 8; ++w) s += red[t * 4 + w];
+    for (int w = 1; w < Mp::TXN / 8; ++w) s += red[t * RW + w];
     return s;
 }
 template <typename T, int DK, int DV>
@@ -640,7 +642,6 @@ __global__ void __launch_bounds__(kThreads<DK, DV>) bwd_out_kernel(Params p, con
     tile::load<CT, DK, NT>(sm.Q, q + oqk, p.tqk, n, p.vec);
     load_square<NT>(sm.T, w.T + (long long)c * CC);
     load_square<NT>(sm.A, w.A + (long long)c * CC);
-    load_square<NT>(sm.KM, w.KM + (long long)c * CC);
     if (Smem::BOTH) tile::load<DK, DV, NT>(G, Gg, DV, DK);
     // <dH', H>, the gradient of the tile's total decay through gam_n
     {
@@ -672,7 +673,7 @@ __global__ void __launch_bounds__(kThreads<DK, DV>) bwd_out_kernel(Params p, con
     }
     if (mk.on) {
         tile::product<MK, true, true, DV, DV>(adq, sm.D, sm.H, 0, DV, mk);                    // dO H^T
-        row_dots(adq, mk, sm.qd, [&](int m, int nn) { return tile::ld4(sm.Q + tile::at<DK>(m, nn)); });
+        row_dots<Smem::RW>(adq, mk, sm.qd, [&](int m, int nn) { return tile::ld4(sm.Q + tile::at<DK>(m, nn)); });
         scale_acc(adq, mk, [&](int m) { return sm.d.gam[m]; });
     }
     __syncthreads();
@@ -698,7 +699,7 @@ __global__ void __launch_bounds__(kThreads<DK, DV>) bwd_out_kernel(Params p, con
     }
     if (mk.on) {
         tile::product<MK, true, true, DV, DV>(adk, sm.W, G, 0, DV, mk);                       // W dH'^T
-        row_dots(adk, mk, sm.kw, [&](int m, int nn) { return tile::ld4(sm.K + tile::at<DK>(m, nn)); });
+        row_dots<Smem::RW>(adk, mk, sm.kw, [&](int m, int nn) { return tile::ld4(sm.K + tile::at<DK>(m, nn)); });
         scale_acc(adk, mk, [&](int m) { return sm.d.om[m]; });
     }
     __syncthreads();
@@ -708,7 +709,7 @@ __global__ void __launch_bounds__(kThreads<DK, DV>) bwd_out_kernel(Params p, con
         tile::zero<MV>(a);
         if (mv.on) {
             tile::product<MV, false, false, CT, DV>(a, sm.T, sm.R, mv.warp_m0(), CT, mv);     // Z = T^T dW
-            row_dots(a, mv, sm.zv, [&](int m, int nn) { return tile::ld4(sm.V + tile::at<DV>(m, nn)); });
+            row_dots<Smem::RW>(a, mv, sm.zv, [&](int m, int nn) { return tile::ld4(sm.V + tile::at<DV>(m, nn)); });
             tile::put<MV, DV>(sm.V, a, mv, same);                                             // V has served: Z takes its place
             store_rows(dv_out + ov, p.tv, n, a, mv, p.vec, [&](int m) { return sm.d.beta[m]; });
         }
@@ -723,7 +724,7 @@ __global__ void __launch_bounds__(kThreads<DK, DV>) bwd_out_kernel(Params p, con
         float a[MK::TM][MK::TN];
         tile::zero<MK>(a);
         tile::product<MK, true, true, DV, DV>(a, sm.V, sm.H, 0, DV, mk);                      // Z H^T
-        row_dots(a, mk, sm.kz, [&](int m, int nn) { return tile::ld4(sm.K + tile::at<DK>(m, nn)); });
+        row_dots<Smem::RW>(a, mk, sm.kz, [&](int m, int nn) { return tile::ld4(sm.K + tile::at<DK>(m, nn)); });
 #pragma unroll
         for (int i = 0; i < MK::TM; ++i) {
             const float f = -sm.d.beta[mk.m(i)] * sm.d.gam[mk.m(i)];
@@ -737,11 +738,14 @@ __global__ void __launch_bounds__(kThreads<DK, DV>) bwd_out_kernel(Params p, con
         const int t = tid >> 2, s0 = (tid & 3) * 8;
         const float bt = sm.d.beta[t];
         float re = 0.f, rl = 0.f;
+        const float* kmg = w.KM + (long long)c * CC + t * CT + s0;
+        const float4 k0 = tile::load4(kmg), k1 = tile::load4(kmg + 4);
+        const float km[8] = {k0.x, k0.y, k0.z, k0.w, k1.x, k1.y, k1.z, k1.w};
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
             const int s = s0 + e, x = tile::at<CT>(t, s);
             const float m = s <= t ? mexp(sm.d, t, s) : 0.f;
-            const float da = DA[x], dl = s < t ? -ZW[x] : 0.f, lk = dl * sm.KM[x];
+            const float da = DA[x], dl = s < t ? -ZW[x] : 0.f, lk = dl * km[e];
             const float ee = fmaf(da, sm.A[x], bt * lk);               // A and KM hold M * QK^T (s <= t) and M * KK^T (s < t), else 0
             DA[x] = da * m;
             ZW[x] = bt * dl * m;
@@ -754,10 +758,10 @@ __global__ void __launch_bounds__(kThreads<DK, DV>) bwd_out_kernel(Params p, con
         if ((tid & 3) == 0) { sm.rs[t] = re; sm.rl[t] = rl; }
     }
     __syncthreads();
-    // P + P^T into KM's place; warp 0 meanwhile turns the row and column sums into dg and dbeta
+    // P + P^T into the place of dO, which has served; warp 0 meanwhile turns the row and column sums into dg and dbeta
     for (int i = tid; i < CC; i += NT) {
         const int t = i / CT, s = i % CT;
-        sm.KM[tile::at<CT>(t, s)] = ZW[tile::at<CT>(t, s)] + ZW[tile::at<CT>(s, t)];
+        sm.D[tile::at<CT>(t, s)] = ZW[tile::at<CT>(t, s)] + ZW[tile::at<CT>(s, t)];
     }
     if (tid < CT) {
         const int t = tid;
@@ -765,7 +769,7 @@ __global__ void __launch_bounds__(kThreads<DK, DV>) bwd_out_kernel(Params p, con
 #pragma unroll 8
         for (int s = 0; s < CT; ++s) cs += sm.A[tile::at<CT>(s, t)];
         const float gam = sm.d.gam[t], om = sm.d.om[t], bt = sm.d.beta[t];
-        const float kz = row_sum<MK>(sm.kz, t), kw = row_sum<MK>(sm.kw, t), qd = row_sum<MK>(sm.qd, t), zv = row_sum<MV>(sm.zv, t);
+        const float kz = row_sum<Smem::RW, MK>(sm.kz, t), kw = row_sum<Smem::RW, MK>(sm.kw, t), qd = row_sum<Smem::RW, MK>(sm.qd, t), zv = row_sum<Smem::RW, MV>(sm.zv, t);
         float tot = kw * om;                                        // chunk-total terms: they belong to the last token, so to every suffix
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, off);
@@ -788,7 +792,7 @@ __global__ void __launch_bounds__(kThreads<DK, DV>) bwd_out_kernel(Params p, con
     if (mk.on) {
         tile::product<MK, true, false, CT, DK>(adq, DA, sm.K, 0, mk.warp_m0() + 16, mk);
         tile::product<MK, false, false, CT, DK>(adk, DA, sm.Q, mk.warp_m0(), CT, mk);
-        tile::product<MK, true, false, CT, DK>(adk, sm.KM, sm.K, 0, CT, mk);
+        tile::product<MK, true, false, CT, DK>(adk, sm.D, sm.K, 0, CT, mk);
         store_rows(dq + oqk, p.tqk, n, adq, mk, p.vec, [](int) { return 1.f; });
         store_rows(dk_out + oqk, p.tqk, n, adk, mk, p.vec, [](int) { return 1.f; });
     }
