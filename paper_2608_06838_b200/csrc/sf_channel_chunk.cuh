@@ -388,13 +388,17 @@ __device__ __forceinline__ void store_rows(T* __restrict__ dst, long long stride
 }
 
 // ---- Out: O = A V + (q*gam) Hc.  grid (tiles, H, B) ---------------------------------------------------------------------
+// The product with Hc comes first and the level arrays take its operands' place: four CTAs of a 64-wide head per SM instead of
+// three (195 -> 179 us on 16384 tokens x 16 heads).
 template <int DK, int DV>
 struct OutSmem {
-    float S[3 * CT * DK], Qg[CT * DK], V[CT * DV], H[DK * DV], A[CC], tot[8 * DK];
+    static constexpr int LV = 3 * CT * DK, QH = CT * DK + DK * DV;
+    float S[LV > QH ? LV : QH];                          // q*gam and Hc, then the level arrays
+    float V[CT * DV], A[CC], tot[8 * DK];
     float red[8 * (DK / 32) * 16];
 };
 template <typename T, int DK, int DV>
-__global__ void __launch_bounds__(kThreads<DK, DV>) out_kernel(Params p, const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v,
+__global__ void __launch_bounds__(kThreads<DK, DV>, kThreads<DK, DV> == 128 ? 4 : 1) out_kernel(Params p, const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v,
                                                                const float* __restrict__ g, T* __restrict__ o, const float* ws) {
     constexpr int NT = kThreads<DK, DV>;
     using MK = tile::Map<CT, DK, NT>;
@@ -416,21 +420,26 @@ __global__ void __launch_bounds__(kThreads<DK, DV>) out_kernel(Params p, const T
         put_total<DK>(sm.tot, gq, mk);
     }
     tile::load<CT, DV, NT>(sm.V, v + ov, p.tv, n, p.vec);
-    tile::load<DK, DV, NT>(sm.H, w.Hc + (long long)c * DK * DV, DV, DK);
+    float *Qg = sm.S, *H = sm.S + CT * DK;
+    tile::load<DK, DV, NT>(H, w.Hc + (long long)c * DK * DV, DV, DK);
+    __syncthreads();
+    if (mk.on) {
+        float f[4];
+        exp_blocks<DK>(f, sm.tot, 0, mk.ty, mk);
+        put_quad<DK>(Qg, times(qq, exp_prefix(gq), f), mk);
+    }
+    __syncthreads();
+    float acc[MV::TM][MV::TN];
+    tile::zero<MV>(acc);
+    if (mv.on) tile::product<MV, true, false, DK, DV>(acc, Qg, H, 0, DK, mv);
     __syncthreads();
     if (mk.on) {
         const Quad ep = exp_prefix(gq), es = exp_suffix(gq);
         diag_partials(sm.red, qq, kq, near_weights(gq), es, mk);
         put_levels<DK>(sm.S, qq, kq, ep, es, sm.tot, mk);
-        float f[4];
-        exp_blocks<DK>(f, sm.tot, 0, mk.ty, mk);
-        put_quad<DK>(sm.Qg, times(qq, ep, f), mk);
     }
     __syncthreads();
     assemble_scores<DK, NT, MK::TXN / 8>(sm.A, sm.S, sm.red);
-    float acc[MV::TM][MV::TN];
-    tile::zero<MV>(acc);
-    if (mv.on) tile::product<MV, true, false, DK, DV>(acc, sm.Qg, sm.H, 0, DK, mv);
     __syncthreads();
     if (mv.on) {
         tile::product<MV, true, false, CT, DV>(acc, sm.A, sm.V, 0, mv.warp_m0() + 16, mv);

@@ -228,10 +228,12 @@ __device__ __forceinline__ void scale_acc(float (&acc)[Mp::TM][Mp::TN], const Mp
 }
 
 // ---- Pre: T, Phi, Psi; with BWD also A, KM and Theta.  grid (tiles, H, B) --------------------------------------------
+// With BWD q shares a buffer with the right-hand side Wk is formed from and is loaded twice: five CTAs of a 64 x 64 head per SM
+// instead of four (425 -> 411 us at 16 heads x 512 tiles).
 template <int DK, int DV, bool BWD>
 struct PreSmem {
     float K[CT * DK], X[CT * DV], Y[CT * DK], T[CC], tmp[256];
-    float Q[BWD ? CT * DK : 4], D[BWD ? CT * DV : 4], A[BWD ? CC : 4];
+    float D[BWD ? CT * DV : 4], A[BWD ? CC : 4];
     Decay d;
 };
 template <typename T, int DK, int DV, bool BWD>
@@ -255,7 +257,7 @@ __global__ void __launch_bounds__(kThreads<DK, DV>) pre_kernel(Params p, const T
     tile::load<CT, DK, NT>(sm.K, k + oqk, p.tqk, n, p.vec);
     tile::load<CT, DV, NT>(sm.X, v + ov, p.tv, n, p.vec);
     if constexpr (BWD) {
-        tile::load<CT, DK, NT>(sm.Q, q + oqk, p.tqk, n, p.vec);
+        tile::load<CT, DK, NT>(sm.Y, q + oqk, p.tqk, n, p.vec);      // Y's other uses come later; q is loaded again for Theta
         tile::load<CT, DV, NT>(sm.D, dO + ov, p.tv, n, p.vec);
     }
     __syncthreads();
@@ -276,7 +278,8 @@ __global__ void __launch_bounds__(kThreads<DK, DV>) pre_kernel(Params p, const T
             tile::store4(w.A + (long long)c * CC + m * CT + n0, f);
             tile::st4(sm.A + tile::at<CT>(m, n0), f);
         };
-        two_square_products<NT, DK, DK>(sm.K, sm.K, put_l, sm.Q, sm.K, put_a);
+        two_square_products<NT, DK, DK>(sm.K, sm.K, put_l, sm.Y, sm.K, put_a);
+        __syncthreads();
     } else {
         if (threadIdx.x < 128) square_product<DK>(sm.K, sm.K, threadIdx.x, put_l);
     }
@@ -330,8 +333,9 @@ __global__ void __launch_bounds__(kThreads<DK, DV>) pre_kernel(Params p, const T
         float az[MV::TM][MV::TN];
         tile::zero<MV>(az);
         if (mv.on) tile::product<MV, false, false, CT, DV>(az, sm.A, sm.D, mv.warp_m0(), CT, mv);         // A^T dO
-        __syncthreads();                                            // X and A, dO have been read
+        __syncthreads();                                            // X, Y and A, dO have been read
         if (mv.on) tile::put<MV, DV>(sm.X, az, mv, same);
+        tile::load<CT, DK, NT>(sm.Y, q + oqk, p.tqk, n, p.vec);
         tile::scale_rows<CT, DV, NT>(sm.D, sm.d.gam);
         __syncthreads();
         tile::zero<MV>(az);
@@ -343,7 +347,7 @@ __global__ void __launch_bounds__(kThreads<DK, DV>) pre_kernel(Params p, const T
         float acc[MPsi::TM][MPsi::TN];
         tile::zero<MPsi>(acc);
         if (m.on) {
-            tile::product<MPsi, false, false, DK, DV>(acc, sm.Q, sm.D, 0, CT, m);
+            tile::product<MPsi, false, false, DK, DV>(acc, sm.Y, sm.D, 0, CT, m);
             tile::product<MPsi, false, false, DK, DV>(acc, sm.K, sm.X, 0, CT, m);
             store_dense<MPsi, DV>(w.Theta + (long long)c * DK * DV, acc, m, same);
         }
