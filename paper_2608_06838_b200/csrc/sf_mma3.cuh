@@ -10,8 +10,8 @@
 // Why: a token and head cost about 170 k multiply-adds forward + backward at d = 128 against 2.8 KB of traffic, so the arithmetic
 // bounds these kernels.  Six MMAs at the 275 T/s measured for mma.sync are 46 T float32 multiply-adds/s; the FMA pipe gives
 // 35, of which the register-tiled kernels that stood here reached 17.  Chains forward + backward, before and now (us):
-// d = 128, 8144 tokens x 16 heads 1608 -> 1208; 8192 x 32 3137 -> 2321; 512 x 2 113 -> 105; d = 64, 8192 x 16 592 -> 444, 256 x 2
-// 70 -> 66; d = 32, 16384 x 40 1267 -> 946.  The tensor pipe is 57 % busy on the SMs that have a block; the rest is
+// d = 128, 8144 tokens x 16 heads 1608 -> 1201; 8192 x 32 3137 -> 2307; 512 x 2 113 -> 104; d = 64, 8192 x 16 592 -> 441, 256 x 2
+// 70 -> 65; d = 32, 16384 x 40 1267 -> 923.  The tensor pipe is 57 % busy on the SMs that have a block; the rest is
 // splitting tiles and states and the barriers between the stages of a tile.
 //
 // One CTA walks a block in tiles of 32 tokens, RB = 2 row blocks of 16 x WC column groups of warps.  Tiles, and the state entering
@@ -307,10 +307,12 @@ __device__ __forceinline__ void store_dots(float* __restrict__ x, const float* r
 }
 
 // ---- block aggregates: the state recurrence from zero, tiles forward (mode 0: k, v) or reversed (mode 1: q, dO) -------------------
+// Two tiles in shared memory, one barrier per tile: a warp splits the next tile while others are in this one's MMAs (chains 0.6 %
+// faster than with one tile and two barriers).
 template <int DK, int DV>
 struct AggSmem {
-    alignas(16) bf16 X[3 * PLANE<DK>];
-    alignas(16) bf16 Y[3 * PLANE<DV>];
+    alignas(16) bf16 X[2][3 * PLANE<DK>];
+    alignas(16) bf16 Y[2][3 * PLANE<DV>];
     Decay d[2];
 };
 template <int DK, int DV>
@@ -339,15 +341,18 @@ aggregate_kernel(SegParams p, const float* __restrict__ X, const float* __restri
     load(0);
     if (warp == 0) tables(0);
     double beta = 0.0;
+    rx.put(sm.X[0]);
+    ry.put(sm.Y[0]);
     for (int i = 0; i < n; ++i) {
-        rx.put(sm.X);
-        ry.put(sm.Y);
-        __syncthreads();
+        __syncthreads();                                         // tile i is complete; tile i - 1 has been read
         if (i + 1 < n) { load(i + 1); if (warp == 0) tables(i + 1); }
         const Decay& d = sm.d[i & 1];
         beta += (double)d.bh[CT - 1] + (double)d.bl[CT - 1];
-        st.step(sm.X, mode == 0 ? d.wsuf : d.ebc, sm.Y, d.ebc[CT - 1], nullptr);
-        __syncthreads();
+        st.step(sm.X[i & 1], mode == 0 ? d.wsuf : d.ebc, sm.Y[i & 1], d.ebc[CT - 1], nullptr);
+        if (i + 1 < n) {
+            rx.put(sm.X[(i + 1) & 1]);
+            ry.put(sm.Y[(i + 1) & 1]);
+        }
     }
     const long long blk = ((long long)b * p.H + h) * p.NB + j;
     if (beta_out && threadIdx.x == 0) beta_out[blk] = (float)beta;
