@@ -232,27 +232,6 @@ __device__ __forceinline__ void load(float* dst, const T* __restrict__ src, long
         }
     }
 }
-// The same with a factor per row.
-template <int ROWS, int D, int NT, typename T>
-__device__ __forceinline__ void load_scaled(float* dst, const T* __restrict__ src, long long stride, int valid, const float* w) {
-    constexpr int U = D / 4, IT = ROWS * U / NT;
-    static_assert(ROWS * U % NT == 0, "tile does not divide among the threads");
-#pragma unroll
-    for (int i0 = 0; i0 < IT; i0 += 8) {
-        float4 v[8];
-#pragma unroll
-        for (int i = 0; i < 8 && i0 + i < IT; ++i) {
-            const int idx = threadIdx.x + (i0 + i) * NT, r = idx / U, c = (idx % U) * 4;
-            v[i] = r < valid ? load4(src + r * stride + c) : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-#pragma unroll
-        for (int i = 0; i < 8 && i0 + i < IT; ++i) {
-            const int idx = threadIdx.x + (i0 + i) * NT, r = idx / U, c = (idx % U) * 4;
-            const float f = w[r];
-            st4(dst + at<D>(r, c), make_float4(v[i].x * f, v[i].y * f, v[i].z * f, v[i].w * f));
-        }
-    }
-}
 // Rows of a tile times a factor per row, in place.
 template <int ROWS, int D, int NT>
 __device__ __forceinline__ void scale_rows(float* x, const float* w) {
