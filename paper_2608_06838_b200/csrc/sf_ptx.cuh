@@ -7,6 +7,8 @@
 namespace sf {
 namespace ptx {
 
+__device__ int g_dev_status = 0;            // what a bounded wait that ran out leaves behind (one word per device)
+
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return static_cast<uint32_t>(__cvta_generic_to_shared(p)); }
 
 // ---- mbarrier ------------------------------------------------------------------------------------
@@ -27,36 +29,69 @@ __device__ __forceinline__ void mbar_arrive_warp(uint64_t* bar) {
     __syncwarp();
     if ((threadIdx.x & 31) == 0) mbar_arrive(bar);
 }
-__device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
+__device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
     uint32_t ok;
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
         "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
         "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity) : "memory");
+        : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
     return ok != 0;
 }
+__device__ __forceinline__ bool mbar_test_wait(uint32_t bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+    return ok != 0;
+}
+__device__ __forceinline__ int ld_shared_volatile(uint32_t a) {
+    int v;
+    asm volatile("ld.volatile.shared.s32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
+    return v;
+}
 
-// Bounded wait: gives up after `limit` clock cycles (about a second by default), records `code` in *status (global)
+// Bounded wait: gives up after `limit` clock cycles (about a second by default), records `code` in the device's status word
 // and sets the CTA-wide sticky flag *abort_flag (shared) so that every later wait in this CTA returns at once.
 // The kernel then runs to its end on undefined data and releases its TMEM normally.
+// SPIN: without suspending the thread between tries, for the one warp whose next instructions everything else waits for.
+// Not inlined: a kernel has dozens of waits, and its code has to fit the instruction cache.
 constexpr long long WAIT_LIMIT_CYCLES = 2000000000LL;
-__device__ __forceinline__ void mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int* status, int code,
-                                          long long limit = WAIT_LIMIT_CYCLES) {
-    if (mbar_try_wait(bar, parity)) return;
-    if (*abort_flag) return;
+template <bool SPIN>
+__device__ __forceinline__ void mbar_wait_limit(uint32_t bar, uint32_t parity, uint32_t abort_flag, int code, long long limit) {
+    if (ld_shared_volatile(abort_flag)) return;
     const long long t0 = clock64();
-    for (uint32_t it = 0;; ++it) {
-        if (mbar_try_wait(bar, parity)) return;
-        if ((it & 255u) == 255u) {
-            if (*abort_flag) return;
+    for (uint32_t it = 1;; ++it) {
+        if (SPIN ? mbar_test_wait(bar, parity) : mbar_try_wait(bar, parity)) return;
+        if ((it & 255u) == 0u) {
+            if (ld_shared_volatile(abort_flag)) return;
             if (clock64() - t0 > limit) {
-                *abort_flag = 1;
-                atomicExch(status, code);
+                asm volatile("st.volatile.shared.s32 [%0], %1;" ::"r"(abort_flag), "r"(1) : "memory");
+                atomicExch(&g_dev_status, code);
                 return;
             }
         }
     }
+}
+// `pc`: parity + 2 code
+template <bool SPIN>
+__device__ __noinline__ void mbar_wait_call(uint32_t bar, uint32_t pc, uint32_t abort_flag) {
+    if (mbar_try_wait(bar, pc & 1)) return;
+    mbar_wait_limit<SPIN>(bar, pc & 1, abort_flag, (int)(pc >> 1), WAIT_LIMIT_CYCLES);
+}
+template <bool SPIN = false>
+__device__ __forceinline__ void mbar_wait(uint64_t* bar, uint32_t parity, int* abort_flag, int code) {
+    mbar_wait_call<SPIN>(smem_u32(bar), parity + 2 * code, smem_u32(abort_flag));
+}
+
+// One lane of a converged warp, always the same.  Code that only it runs keeps the warp's uniform values in uniform registers, which the
+// operands of MMAs and tile copies have to be in; after `lane == 0` each of them is moved there anew (12 KB for 32 MMAs instead of 6).
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\tselp.u32 %0, 1, 0, q;\n\t}" : "=r"(p));
+    return p != 0;
 }
 
 // ---- fences ----------------------------------------------------------------------------------------
@@ -85,6 +120,21 @@ __device__ __forceinline__ void tma_load_4d(void* smem_dst, const void* tmap, ui
         : "memory");
 }
 
+// the same tile into L2 only
+__device__ __forceinline__ void tma_prefetch_4d(const void* tmap, int c0, int c1, int c2, int c3) {
+    asm volatile("cp.async.bulk.prefetch.tensor.4d.L2.global.tile [%0, {%1, %2, %3, %4}];"
+                 ::"l"(reinterpret_cast<uint64_t>(tmap)), "r"(c0), "r"(c1), "r"(c2), "r"(c3) : "memory");
+}
+// 4-D tiled store of shared memory (written before a fence_proxy_async()); parts outside the tensor are not written.
+__device__ __forceinline__ void tma_store_4d(const void* tmap, const void* smem_src, int c0, int c1, int c2, int c3) {
+    asm volatile("cp.async.bulk.tensor.4d.global.shared::cta.tile.bulk_group [%0, {%2, %3, %4, %5}], [%1];"
+                 ::"l"(reinterpret_cast<uint64_t>(tmap)), "r"(smem_u32(smem_src)), "r"(c0), "r"(c1), "r"(c2), "r"(c3) : "memory");
+}
+__device__ __forceinline__ void tma_store_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
+// shared memory of this thread's stores has been read / the stores have been performed
+__device__ __forceinline__ void tma_store_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
+__device__ __forceinline__ void tma_store_wait() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
+
 // ---- TMEM ------------------------------------------------------------------------------------------
 // One full warp allocates `ncols` (power of two >= 32) columns; the base address lands in *dst_smem.
 __device__ __forceinline__ void tmem_alloc(uint32_t* dst_smem, uint32_t ncols) {
@@ -108,16 +158,6 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
           "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
         : "r"(taddr) : "memory");
 }
-// 16 lanes x 32 columns, same thread mapping as tmem_ld_16x64 with 4 column groups
-__device__ __forceinline__ void tmem_ld_16x32(uint32_t taddr, float* v) {
-    uint32_t* r = reinterpret_cast<uint32_t*>(v);
-    asm volatile(
-        "tcgen05.ld.sync.aligned.16x256b.x4.b32 "
-        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr) : "memory");
-}
 // 32 lanes x 16 columns
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
     uint32_t* r = reinterpret_cast<uint32_t*>(v);
@@ -137,26 +177,19 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const float* v) {
           "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]),
           "r"(taddr) : "memory");
 }
+// two float32 multiplications in one instruction
+__device__ __forceinline__ void mul2(float& a, float& b, float f, float g) {
+    asm("{\n\t.reg .b64 x, y;\n\t"
+        "mov.b64 x, {%0, %1};\n\t"
+        "mov.b64 y, {%2, %3};\n\t"
+        "mul.rn.f32x2 x, x, y;\n\t"
+        "mov.b64 {%0, %1}, x;\n\t}" : "+f"(a), "+f"(b) : "f"(f), "f"(g));
+}
 // 2^x with the single-instruction approximation (inputs here are <= 0 or moderate; flush-to-zero underflow is the wanted limit)
 __device__ __forceinline__ float ex2(float x) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
-}
-// 16 lanes x 64 columns: thread t gets, for each group j of 8 columns, v[4j], v[4j+1] = (lane t/4, columns
-// 8j + 2(t%4), +1) and v[4j+2], v[4j+3] = (lane t/4 + 8, same columns) - the layout of an M = 64 accumulator
-// row block, spread over all 32 threads of the warp.
-__device__ __forceinline__ void tmem_ld_16x64(uint32_t taddr, float* v) {
-    uint32_t* r = reinterpret_cast<uint32_t*>(v);
-    asm volatile(
-        "tcgen05.ld.sync.aligned.16x256b.x8.b32 "
-        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-        "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-          "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-          "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-        : "r"(taddr) : "memory");
 }
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tmem_st32(uint32_t taddr, const float* v) {
@@ -192,21 +225,29 @@ __host__ __device__ constexpr uint32_t idesc_bf16(int M, int N, int a_mn_major, 
 }
 
 // D[tmem] (+)= A[smem] * B[smem]; issued by ONE thread, descriptors passed as 32-bit pieces.
-// The issuing thread has no queue to hide behind: whatever it executes between two tcgen05.mma instructions
-// is idle time of the tensor pipe, so the descriptors of a K loop are formed with one integer add each: the high word of every descriptor here is the same constant and a K step only moves
+// The descriptors of a K loop are formed with one integer add each: the high word of every descriptor here is the same constant and a K step only moves
 // the 14-bit start-address field of the low word (shared memory is smaller than 2^18 bytes: no carry out of it).
 constexpr uint32_t DESC_HI = (1024u >> 4) | (1u << 14) | (2u << 29);
 __device__ __forceinline__ uint32_t desc_lo(uint32_t saddr, uint32_t lbo_bytes) {
     return ((saddr & 0x3FFFFu) >> 4) | ((lbo_bytes >> 4) << 16);
 }
-template <int ACC>
-__device__ __forceinline__ void mma_lo(uint32_t d_tmem, uint32_t alo, uint32_t blo, uint32_t idesc) {
+__device__ __forceinline__ void mma_lo(uint32_t d_tmem, uint32_t alo, uint32_t blo, uint32_t idesc, bool acc) {
     asm volatile(
-        "{\n\t.reg .b64 da, db;\n\t"
+        "{\n\t.reg .b64 da, db;\n\t.reg .pred p;\n\t"
         "mov.b64 da, {%1, %4};\n\t"
         "mov.b64 db, {%2, %4};\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %3, %5;\n\t}"
-        ::"r"(d_tmem), "r"(alo), "r"(blo), "r"(idesc), "r"(DESC_HI), "n"(ACC) : "memory");
+        "setp.ne.u32 p, %5, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %3, p;\n\t}"
+        ::"r"(d_tmem), "r"(alo), "r"(blo), "r"(idesc), "r"(DESC_HI), "r"((uint32_t)acc) : "memory");
+}
+// D[tmem] (+)= A[tmem] * B[smem]: row r of A in lane r, two bf16 per column.  Lanes of D with their bit set in `off` are left as they are.
+__device__ __forceinline__ void mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint32_t blo, uint32_t idesc, bool acc, const uint32_t (&off)[4]) {
+    asm volatile(
+        "{\n\t.reg .b64 db;\n\t.reg .pred p;\n\t"
+        "mov.b64 db, {%2, %4};\n\t"
+        "setp.ne.u32 p, %5, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], db, %3, {%6, %7, %8, %9}, p;\n\t}"
+        ::"r"(d_tmem), "r"(a_tmem), "r"(blo), "r"(idesc), "r"(DESC_HI), "r"((uint32_t)acc), "r"(off[0]), "r"(off[1]), "r"(off[2]), "r"(off[3]) : "memory");
 }
 // Arrive on an mbarrier once all MMAs issued so far by this thread have completed.
 __device__ __forceinline__ void mma_commit(uint64_t* bar) {

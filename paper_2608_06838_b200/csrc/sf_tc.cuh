@@ -1,11 +1,11 @@
 // tcgen05 / TMEM / TMA kernels for the bf16, d_k = d_v = 128, chunk = 64 shape.
 //
-// Thread roles in every kernel here: warps 0-3 are the compute warpgroup (TMEM loads/stores, decay
-// masks, epilogues; warp w owns TMEM lanes 32(w mod 4)..+31), then one TMA producer warp and one warp that
+// Thread roles in every kernel here: the first warps compute (TMEM loads/stores, decay masks, epilogues;
+// warp w owns TMEM lanes 32(w mod 4)..+31), then one TMA producer warp and one warp that
 // issues the MMAs (lane 0 each).  All waits are bounded (see ptx::mbar_wait).
 //
-// Shared-memory operand storage: every [64 tokens x 128 features] bf16 tile is two TMA boxes of
-// [64 rows x 64 columns] (128-byte rows, SWIZZLE_128B, 8 KB each, features 0-63 then 64-127).  The
+// Shared-memory operand storage: every bf16 tile of 64 (aggregates) or 128 (sweeps) tokens x 128 features is two TMA boxes of
+// [tokens x 64 columns] (128-byte rows, SWIZZLE_128B, features 0-63 then 64-127).  The
 // same storage is read K-major when the contraction runs over features and MN-major when it runs
 // over tokens (ptx::desc_lo).
 #pragma once
@@ -19,7 +19,7 @@
 namespace sf {
 namespace tc {
 
-__device__ int g_dev_status = 0;
+using ptx::g_dev_status;
 
 inline int read_device_status() {
     int v = 0;
@@ -61,29 +61,29 @@ inline EncodeTiledFn encode_fn() {
     return fn;
 }
 
-// Map of a [B, L, H, 128] bf16 view: dims (feature, head, token, batch), box = 64 features x 1 x 64 tokens x 1.
+// Map of a [B, L, H, 128] bf16 view: dims (feature, head, token, batch), box = 64 features x 1 x `rows` tokens x 1.
 // A map is a pure function of (base, B, L, H, strides) and encoding one never reads device memory, so each host
 // thread keeps the last TMAP_CACHE maps it encoded: a chain that is launched again from the host (no graph) with the
 // same buffers re-encodes nothing.
 constexpr int TMAP_CACHE = 64;
 struct TmapKey {
-    const void* base; int B, L, H; long long tok_stride, batch_stride;
+    const void* base; int rows, B, L, H; long long tok_stride, batch_stride;
     bool operator==(const TmapKey& o) const {
-        return base == o.base && B == o.B && L == o.L && H == o.H && tok_stride == o.tok_stride && batch_stride == o.batch_stride;
+        return base == o.base && rows == o.rows && B == o.B && L == o.L && H == o.H && tok_stride == o.tok_stride && batch_stride == o.batch_stride;
     }
 };
 struct TmapCache { TmapKey key[TMAP_CACHE]; CUtensorMap map[TMAP_CACHE]; int used = 0, next = 0; };
 
-inline bool make_tmap(CUtensorMap* m, const void* base, int B, int L, int H, long long tok_stride, long long batch_stride) {
+inline bool make_tmap(CUtensorMap* m, int rows, const void* base, int B, int L, int H, long long tok_stride, long long batch_stride) {
     thread_local TmapCache cache;
-    const TmapKey key{base, B, L, H, tok_stride, batch_stride};
+    const TmapKey key{base, rows, B, L, H, tok_stride, batch_stride};
     for (int i = 0; i < cache.used; ++i)
         if (cache.key[i] == key) { *m = cache.map[i]; return true; }
     EncodeTiledFn fn = encode_fn();
     if (!fn) return false;
     cuuint64_t dims[4] = {(cuuint64_t)D, (cuuint64_t)H, (cuuint64_t)L, (cuuint64_t)B};
     cuuint64_t strides[3] = {(cuuint64_t)D * 2, (cuuint64_t)tok_stride * 2, (cuuint64_t)(B > 1 ? batch_stride : (long long)L * tok_stride) * 2};
-    cuuint32_t box[4] = {64, 1, 64, 1};
+    cuuint32_t box[4] = {64, 1, (cuuint32_t)rows, 1};
     cuuint32_t estr[4] = {1, 1, 1, 1};
     if (fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
            CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
@@ -190,111 +190,47 @@ __device__ __forceinline__ void scale_tile(unsigned char* dst, const unsigned ch
     }
 }
 
-// TMEM accumulators of token-row results (M = 64) occupy lanes 0-15 of each 32-lane quarter, so two of
-// them are interleaved in the same columns: X at lane offset 0, Y at lane offset 16.  They are read
-// with the 16-lane load shape (ptx::tmem_ld_16x64): in the warp with index q (mod 4), thread t holds
-// rows 16q + t/4 and 16q + t/4 + 8, two adjacent columns out of every eight.
-
-// Decay mask on the [64 x 64] score accumulators at TMEM columns `sc`:
-//   dst[r][s] = bf16( acc[r][s] * exp(b_r - b_s) )  for s <= r, else 0        (row-major, one box)
-// X -> dst0 and, if dst1 != nullptr, Y -> dst1 (same mask).
-__device__ __forceinline__ void mask_pass(uint32_t sc, const float* bch, unsigned char* dst0, unsigned char* dst1) {
-    const int q = (threadIdx.x >> 5) & 3, lane = threadIdx.x & 31;
-    const int rA = 16 * q + (lane >> 2), rB = rA + 8, cq = 2 * (lane & 3);
-    const uint32_t taddr = sc + ((uint32_t)(q * 32) << 16);
-    const float bA = bch[rA] * LOG2E, bB = bch[rB] * LOG2E;
-#pragma unroll
-    for (int hf = 0; hf < 2; ++hf) {
-        float x[16], y[16];
-        ptx::tmem_ld_16x32(taddr + hf * 32, x);
-        if (dst1) ptx::tmem_ld_16x32(taddr + (16u << 16) + hf * 32, y);
-        ptx::tmem_ld_wait();
-#pragma unroll
-        for (int jj = 0; jj < 4; ++jj) {
-            const int j = hf * 4 + jj, s0 = 8 * j + cq;
-            const float2 bs = *reinterpret_cast<const float2*>(bch + s0);
-            const float e0 = -LOG2E * bs.x, e1 = -LOG2E * bs.y;
-            const float dA0 = s0 <= rA ? ptx::ex2(bA + e0) : 0.f, dA1 = s0 + 1 <= rA ? ptx::ex2(bA + e1) : 0.f;
-            const float dB0 = s0 <= rB ? ptx::ex2(bB + e0) : 0.f, dB1 = s0 + 1 <= rB ? ptx::ex2(bB + e1) : 0.f;
-            const int offA = rA * 128 + ((j ^ (rA & 7)) << 4) + 2 * cq, offB = rB * 128 + ((j ^ (rB & 7)) << 4) + 2 * cq;
-            *reinterpret_cast<uint32_t*>(dst0 + offA) = pack2(x[4 * jj] * dA0, x[4 * jj + 1] * dA1);
-            *reinterpret_cast<uint32_t*>(dst0 + offB) = pack2(x[4 * jj + 2] * dB0, x[4 * jj + 3] * dB1);
-            if (dst1) {
-                *reinterpret_cast<uint32_t*>(dst1 + offA) = pack2(y[4 * jj] * dA0, y[4 * jj + 1] * dA1);
-                *reinterpret_cast<uint32_t*>(dst1 + offB) = pack2(y[4 * jj + 2] * dB0, y[4 * jj + 3] * dB1);
-            }
-        }
-    }
-}
-
-// State pass over NU consecutive 16-column units starting at unit u0 of a [128 x 128] float32
-// accumulator at TMEM columns `acc`; the thread owns lane a = threadIdx.x & 127.  Writes the bf16 copy
-// of the state to `sb` (two boxes of [128 rows x 64 columns], 16 KB apart) and scales the accumulator
-// by `decay`.  If init != nullptr the state is taken from global memory (init[a*128 + i], or
-// init[i*128 + a] when `transposed`) instead of TMEM; `first` without it means a state of zeros.
+// Passes over the [128 x 128] float32 state at TMEM columns `acc`; a thread owns lane threadIdx.x & 127 and NU units of 16 columns from u0
+// on.  They are loops, not straight code: what a CTA runs has to stay in the instruction cache (see the sweeps).
+//
+// The state from global memory (init[a*128 + i], or init[i*128 + a] when `transposed`; NULL: zero) to tensor memory.
 template <int NU>
-__device__ __forceinline__ void state_pass(uint32_t acc, unsigned char* sb, float decay, bool first, const float* init, bool transposed,
-                                           int u0, float* __restrict__ dump = nullptr) {
-    const int a = threadIdx.x & 127, warp = a >> 5;
-    const uint32_t taddr = acc + ((uint32_t)(warp * 32) << 16);
-    // two units (32 registers) at a time keeps the register footprint small enough for the 96-register budget
+__device__ __forceinline__ void state_init(uint32_t acc, const float* init, bool transposed, int u0) {
+    const int a = threadIdx.x & 127;
+    const uint32_t taddr = acc + ((uint32_t)((a >> 5) * 32) << 16);
+#pragma unroll 1
+    for (int u = u0; u < u0 + NU; ++u) {
+        float v[16] = {};
+        if (init && transposed) {
 #pragma unroll
-    for (int k0 = 0; k0 < NU; k0 += 2) {
-        const int nk = (NU - k0) < 2 ? (NU - k0) : 2;
-        float v[2][16];
-        if (first && !init) {
+            for (int i = 0; i < 16; ++i) v[i] = init[(u * 16 + i) * D + a];
+        } else if (init) {
 #pragma unroll
-            for (int k = 0; k < 2; ++k)
-#pragma unroll
-                for (int i = 0; i < 16; ++i) v[k][i] = 0.f;
-        } else if (first) {
-#pragma unroll
-            for (int k = 0; k < 2; ++k) {
-                if (k < nk) {
-                    const int col = (u0 + k0 + k) * 16;
-                    if (transposed) {
-#pragma unroll
-                        for (int i = 0; i < 16; ++i) v[k][i] = init[(col + i) * D + a];
-                    } else {
-#pragma unroll
-                        for (int i = 0; i < 16; i += 4) {
-                            const float4 f = *reinterpret_cast<const float4*>(init + a * D + col + i);
-                            v[k][i] = f.x; v[k][i + 1] = f.y; v[k][i + 2] = f.z; v[k][i + 3] = f.w;
-                        }
-                    }
-                }
-            }
-        } else {
-#pragma unroll
-            for (int k = 0; k < 2; ++k)
-                if (k < nk) ptx::tmem_ld16(taddr + (u0 + k0 + k) * 16, v[k]);
-            ptx::tmem_ld_wait();
+            for (int i = 0; i < 16; i += 4) *reinterpret_cast<float4*>(v + i) = *reinterpret_cast<const float4*>(init + a * D + u * 16 + i);
         }
-        if (dump) {
-            // the state entering this chunk is a boundary state of the chain: row a, this thread's 16-column units
+        ptx::tmem_st16(taddr + u * 16, v);
+    }
+    ptx::tmem_st_wait();
+}
+// The bf16 copy of the state to `sb` (two boxes of [128 rows x 64 columns], 16 KB apart); the accumulator times `decay`.
+template <int NU>
+__device__ __forceinline__ void state_pass(uint32_t acc, unsigned char* sb, float decay, int u0) {
+    static_assert(NU % 2 == 0, "two units at a time");
+    const int a = threadIdx.x & 127;
+    const uint32_t taddr = acc + ((uint32_t)((a >> 5) * 32) << 16);
+#pragma unroll 1
+    for (int u = u0; u < u0 + NU; u += 2) {
+        float v[32];
+        ptx::tmem_ld32(taddr + u * 16, v);
+        ptx::tmem_ld_wait();
+        unsigned char* box = sb + (u >> 2) * 16384;
 #pragma unroll
-            for (int k = 0; k < 2; ++k)
-                if (k < nk) {
-                    float4* o4 = reinterpret_cast<float4*>(dump + a * D + (u0 + k0 + k) * 16);
+        for (int e = 0; e < 4; ++e)
+            st_unit(box, a, (u & 3) * 2 + e, make_uint4(pack2(v[e * 8], v[e * 8 + 1]), pack2(v[e * 8 + 2], v[e * 8 + 3]),
+                                                        pack2(v[e * 8 + 4], v[e * 8 + 5]), pack2(v[e * 8 + 6], v[e * 8 + 7])));
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) o4[i] = make_float4(v[k][4 * i], v[k][4 * i + 1], v[k][4 * i + 2], v[k][4 * i + 3]);
-                }
-        }
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            if (k < nk) {
-                const int u = u0 + k0 + k;
-                unsigned char* box = sb + (u >> 2) * 16384;
-#pragma unroll
-                for (int e = 0; e < 2; ++e)
-                    st_unit(box, a, (u & 3) * 2 + e,
-                            make_uint4(pack2(v[k][e * 8], v[k][e * 8 + 1]), pack2(v[k][e * 8 + 2], v[k][e * 8 + 3]),
-                                       pack2(v[k][e * 8 + 4], v[k][e * 8 + 5]), pack2(v[k][e * 8 + 6], v[k][e * 8 + 7])));
-#pragma unroll
-                for (int i = 0; i < 16; ++i) v[k][i] *= decay;
-                ptx::tmem_st16(taddr + u * 16, v[k]);
-            }
-        }
+        for (int i = 0; i < 32; i += 2) ptx::mul2(v[i], v[i + 1], decay, decay);
+        ptx::tmem_st32(taddr + u * 16, v);
     }
     ptx::tmem_st_wait();
 }
@@ -305,7 +241,7 @@ template <int NU>
 __device__ __forceinline__ void state_out(uint32_t acc, float* __restrict__ dst, int u0) {
     const int a = threadIdx.x & 127;
     const uint32_t taddr = acc + ((uint32_t)((a >> 5) * 32) << 16);
-#pragma unroll
+#pragma unroll 1
     for (int k = 0; k < NU; ++k) {
         float v[16];
         ptx::tmem_ld16(taddr + (u0 + k) * 16, v);
@@ -316,140 +252,28 @@ __device__ __forceinline__ void state_out(uint32_t acc, float* __restrict__ dst,
     }
 }
 
-// Weighted copy of one [64 x 64] box: dst = diag(w) src, by the 128 threads of a warpgroup (t = 0..127);
-// a thread meets rows (t>>3) + {0, 16, 32, 48}.
-template <typename F>
-__device__ __forceinline__ void scale_box(unsigned char* dst, const unsigned char* src, int t, F w_row) {
-    const uint4* in = reinterpret_cast<const uint4*>(src);
-    uint4* out = reinterpret_cast<uint4*>(dst);
-    uint4 v[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) v[i] = in[t + 128 * i];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const float w = w_row((t >> 3) + 16 * i);
-        __nv_bfloat162* h2 = reinterpret_cast<__nv_bfloat162*>(&v[i]);
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const float2 f = __bfloat1622float2(h2[e]);
-            h2[e] = __floats2bfloat162_rn(f.x * w, f.y * w);
-        }
-        out[t + 128 * i] = v[i];
-    }
-}
-
-// 4 x 4 transpose across the four lanes of a row group by two butterfly exchanges (lane ^ 1, then lane ^ 2):
-// lane q gives up w[i] and ends with the w[q] of lanes 0..3, in lane order.  4 shuffles + 12 selects.
-// The mapping is its own inverse.
-__device__ __forceinline__ uint4 lanes4_transpose(uint32_t w0, uint32_t w1, uint32_t w2, uint32_t w3) {
-    const bool p0 = (threadIdx.x & 1) != 0, p1 = (threadIdx.x & 2) != 0;
-    uint32_t s0 = p0 ? w0 : w1, s1 = p0 ? w2 : w3;
-    uint32_t r0 = __shfl_xor_sync(0xffffffffu, s0, 1), r1 = __shfl_xor_sync(0xffffffffu, s1, 1);
-    const uint32_t a0 = p0 ? r0 : w0, a1 = p0 ? w1 : r0, a2 = p0 ? r1 : w2, a3 = p0 ? w3 : r1;
-    s0 = p1 ? a0 : a2; s1 = p1 ? a1 : a3;
-    r0 = __shfl_xor_sync(0xffffffffu, s0, 2); r1 = __shfl_xor_sync(0xffffffffu, s1, 2);
-    return make_uint4(p1 ? r0 : a0, p1 ? r1 : a1, p1 ? a2 : r0, p1 ? a3 : r1);
-}
-
-struct NoWait { __device__ __forceinline__ void operator()() const {} };
-
-// Epilogue of an interleaved accumulator pair at TMEM columns `pair`: out[r][:] = X[r][:] + scale_r * Y[r][:]
-// as bf16 to global rows and, with DOT, the row dot products dot_r = sum_c out[r][c] * e[r][c] (out in float32)
-// against global rows e.  The thread serves rows rA = 16q + t/4 and rB = rA + 8; out_A/out_B (and e_A/e_B)
-// point at their first element.  On return dotA/dotB hold the full row sums in every lane of the row's group.
-//
-// The accumulator layout gives lane q' = t%4 of a row the bf16 column pairs 8j + 2q' (j = 0..15): 4-byte
-// pieces 16 bytes apart.  Global memory is touched in 16-byte pieces instead (the four lanes of a row
-// cover 64 contiguous bytes per instruction: an eighth of the load/store instructions), and the butterfly
-// above converts between the two layouts in registers.  `ready` is called before the first TMEM read: the e
-// rows are fetched and rearranged before it, so the wait for the accumulator hides their latency.
-template <bool DOT, typename W = NoWait>
-__device__ __forceinline__ void pair_epilogue(uint32_t pair, float scaleA, float scaleB, __nv_bfloat16* __restrict__ out_A,
-                                              __nv_bfloat16* __restrict__ out_B, const __nv_bfloat16* __restrict__ e_A,
-                                              const __nv_bfloat16* __restrict__ e_B, float& dotA, float& dotB, bool validA,
-                                              bool validB, W ready = W()) {
-    const int q = (threadIdx.x >> 5) & 3, lane = threadIdx.x & 31;
-    const uint32_t taddr = pair + ((uint32_t)(q * 32) << 16);
-    const int c16 = 8 * (lane & 3);                      // first column of this lane's 16-byte pieces
-    dotA = 0.f;
-    dotB = 0.f;
-    uint32_t pa[DOT ? 16 : 1], pb[DOT ? 16 : 1];
-    if (DOT) {
-        uint4 va[4], vb[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            va[i] = __ldg(reinterpret_cast<const uint4*>(e_A + 32 * i + c16));      // callers pass rows inside the segment
-            vb[i] = __ldg(reinterpret_cast<const uint4*>(e_B + 32 * i + c16));
-        }
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const uint4 ta = lanes4_transpose(va[i].x, va[i].y, va[i].z, va[i].w);
-            const uint4 tb = lanes4_transpose(vb[i].x, vb[i].y, vb[i].z, vb[i].w);
-            pa[4 * i] = ta.x; pa[4 * i + 1] = ta.y; pa[4 * i + 2] = ta.z; pa[4 * i + 3] = ta.w;
-            pb[4 * i] = tb.x; pb[4 * i + 1] = tb.y; pb[4 * i + 2] = tb.z; pb[4 * i + 3] = tb.w;
-        }
-    }
-    ready();
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {                        // 32 columns at a time: j = 4i .. 4i+3
-        float x[16], y[16];
-        ptx::tmem_ld_16x32(taddr + i * 32, x);
-        ptx::tmem_ld_16x32(taddr + (16u << 16) + i * 32, y);
-        ptx::tmem_ld_wait();
-        uint32_t wa[4], wb[4];
-#pragma unroll
-        for (int jj = 0; jj < 4; ++jj) {
-            const float a0 = fmaf(scaleA, y[4 * jj], x[4 * jj]), a1 = fmaf(scaleA, y[4 * jj + 1], x[4 * jj + 1]);
-            const float b0 = fmaf(scaleB, y[4 * jj + 2], x[4 * jj + 2]), b1 = fmaf(scaleB, y[4 * jj + 3], x[4 * jj + 3]);
-            if (DOT) {
-                const float2 fa = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&pa[4 * i + jj]));
-                const float2 fb = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&pb[4 * i + jj]));
-                dotA = fmaf(a0, fa.x, dotA); dotA = fmaf(a1, fa.y, dotA);
-                dotB = fmaf(b0, fb.x, dotB); dotB = fmaf(b1, fb.y, dotB);
-            }
-            wa[jj] = pack2(a0, a1);
-            wb[jj] = pack2(b0, b1);
-        }
-        const uint4 ua = lanes4_transpose(wa[0], wa[1], wa[2], wa[3]), ub = lanes4_transpose(wb[0], wb[1], wb[2], wb[3]);
-        if (validA) *reinterpret_cast<uint4*>(out_A + 32 * i + c16) = ua;      // rows past the end of the segment are not stored
-        if (validB) *reinterpret_cast<uint4*>(out_B + 32 * i + c16) = ub;
-    }
-    if (DOT) {
-        dotA += __shfl_xor_sync(0xffffffffu, dotA, 1); dotA += __shfl_xor_sync(0xffffffffu, dotA, 2);
-        dotB += __shfl_xor_sync(0xffffffffu, dotB, 1); dotB += __shfl_xor_sync(0xffffffffu, dotB, 2);
-    }
-}
-
 // One K loop of MMAs from precomputed low descriptor words.  Offset rules of a K step (16-byte units):
-//   DK8 / DK16: K-major operand (a [rows x 128] tile, K step = features 16*ks .. 16*ks+15: +32 B inside a box, the
-//               second 64 features in the next box 8 KB / 16 KB away);
-//   DMN:        MN-major operand (rows are the contraction index: K step = rows 16*ks .. 16*ks+15 = +2048 B; the
-//               other 64 elements of M/N lie one box away, which is the descriptor's leading offset).
-enum { DK8 = 0, DK16 = 1, DMN = 2 };
+//   DK16: K-major operand (a [128 rows x 128] tile, K step = features 16*ks .. 16*ks+15: +32 B inside a box, the second 64
+//         features in the next box 16 KB away);
+//   DMN:  MN-major operand (rows are the contraction index: K step = rows 16*ks .. 16*ks+15 = +2048 B; the other 64
+//         elements of M/N lie one box away, which is the descriptor's leading offset).
+// Straight code, unlike the elementwise passes: a loop's few dependent instructions per step take longer than the MMA (out_done of a
+// sweep came 1500 cycles after the first issue instead of 800).
+enum { DK16 = 1, DMN = 2 };
 template <int RULE>
-__host__ __device__ constexpr uint32_t dofs(int ks) {
-    return RULE == DMN ? 128u * ks : (RULE == DK8 ? 512u : 1024u) * (ks >> 2) + 2u * (ks & 3);
-}
-template <int NK, int RA, int RB, int ACC0, int KS = 0>
-__device__ __forceinline__ void mma_group(uint32_t d, uint32_t alo, uint32_t blo, uint32_t idesc) {
-    if constexpr (KS < NK) {
-        ptx::mma_lo<(ACC0 || KS > 0) ? 1 : 0>(d, alo + dofs<RA>(KS), blo + dofs<RB>(KS), idesc);
-        mma_group<NK, RA, RB, ACC0, KS + 1>(d, alo, blo, idesc);
+__host__ __device__ constexpr uint32_t dofs(int ks) { return RULE == DMN ? 128u * ks : 1024u * (ks >> 2) + 2u * (ks & 3); }
+template <int FROM, int TO, int RA, int RB>
+__device__ __forceinline__ void mma_group(uint32_t d, uint32_t alo, uint32_t blo, uint32_t idesc, bool acc) {
+    if constexpr (FROM < TO) {
+        ptx::mma_lo(d, alo + dofs<RA>(FROM), blo + dofs<RB>(FROM), idesc, acc);
+        mma_group<FROM + 1, TO, RA, RB>(d, alo, blo, idesc, true);
     }
 }
 __device__ __forceinline__ uint32_t klo(uint32_t tile) { return ptx::desc_lo(tile, 0); }
 __device__ __forceinline__ uint32_t mlo(uint32_t tile, uint32_t box_bytes) { return ptx::desc_lo(tile, box_bytes); }
 
-// Warp roles of the chunk-sweep kernels (20 warps): four compute warpgroups, warp 16 issues the MMAs,
-// warp 17 the TMA loads (lane 0 each), warps 18-19 only fill the fifth warpgroup.  The carried state
-// sits on the critical path (MMA -> rescale -> MMA), so several warpgroups share its rescaling (16-column
-// units) as soon as the previous chunk's state MMAs retire and only then turn to their other jobs:
-//   WG0, WG1: state units, then the weighted tile halves      WG2: state units (forward-state sweeps), decay mask of
-//   the NEXT chunk, dv epilogue (dk/dv pass)                  WG3: epilogues
-// mbarriers carry the dependencies  scores -> mask -> MMAs <- state pass <- previous state MMAs;  MMAs -> epilogue.
-constexpr int SW_THREADS = 640;
-constexpr int W_MMA = 16, W_TMA = 17;
-#define SF_WAIT(bar, parity, code) ptx::mbar_wait(bar, parity, abort_flag, status, code)
+#define SF_SPIN(bar, parity, code) ptx::mbar_wait<true>(bar, parity, abort_flag, code)
+#define SF_WAIT(bar, parity, code) ptx::mbar_wait(bar, parity, abort_flag, code)
 
 // ==================================================================================================
 // Block aggregates on tensor cores: U = sum_s w_s x_s^T y_s over the block (M = N = 128, K = tokens).
@@ -472,14 +296,14 @@ struct AggSmem {
 
 __global__ void __launch_bounds__(AGG_THREADS, 1)
 tc_aggregate_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmY, SegParams p,
-                    const float* __restrict__ g, int mode, float* __restrict__ U, float* __restrict__ beta_out, int* status) {
+                    const float* __restrict__ g, int mode, float* __restrict__ U, float* __restrict__ beta_out) {
     extern __shared__ unsigned char smem_raw[];
     AggSmem& sm = *reinterpret_cast<AggSmem*>(align1024(smem_raw));
     const int h = blockIdx.x, j = blockIdx.y, b = blockIdx.z;   // heads fastest: co-resident CTAs read neighbouring 256-byte pieces of the same tokens
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const int c0 = j * p.R, nch = min(p.R, p.NC - c0);
     const long long t0 = (long long)c0 * C;
-    volatile int* abort_flag = &sm.abort_flag;
+    int* abort_flag = &sm.abort_flag;
     constexpr int WT = AGG_COMP / 32, WM = WT + 1;
 
     if (tid == 0) {
@@ -518,8 +342,7 @@ tc_aggregate_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_consta
                 SF_WAIT(&sm.ready[s], it & 1, DEV_TIMEOUT_TMA);
                 ptx::tc_fence_after_sync();
                 const uint32_t xa = ptx::smem_u32(sm.tiles[s][0]), ya = ptx::smem_u32(sm.tiles[s][1]);
-                if (c == 0) mma_group<4, DMN, DMN, 0>(tmem, mlo(xa, BOX), mlo(ya, BOX), idesc);
-                else        mma_group<4, DMN, DMN, 1>(tmem, mlo(xa, BOX), mlo(ya, BOX), idesc);
+                mma_group<0, 4, DMN, DMN>(tmem, mlo(xa, BOX), mlo(ya, BOX), idesc, c > 0);
                 ptx::mma_commit(&sm.empty[s]);
             }
             ptx::mma_commit(&sm.done);
@@ -568,418 +391,476 @@ tc_aggregate_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_consta
 }
 
 // ==================================================================================================
-// Chunk sweep with a forward-running state (Out + ST of paper Eq. 2; SR + OG of Section 3.4).
-// With tile roles (xq, xk, xv) and the state St[a][b] = sum xk[.][a] * xv[.][b]:
-//     out_r = sum_{s<=r} (xq_r . xk_s) D[r,s] xv_s  +  exp(b_r) * xq_r St_c ;   St_{c+1} = exp(b_C) St_c + xk^T diag(w) xv
-//   forward output pass : (xq, xk, xv) = (q, k, v),  St = H (from Hs[j]),         out = o
-//   dq pass             : (xq, xk, xv) = (dO, v, k), St = H^T (Hs[j] transposed), out = dq, and
-//                         xout[t] = q_t . dq_t (float32), q read from global memory in the epilogue
-// TMEM columns: St 0-127; O pair (intra at lanes +0, inter at lanes +16) double-buffered at 128 / 256;
-// scores double-buffered at 384 / 448.
-constexpr int SW_STAGES = 3;
+// Chunk sweeps of a block: o (Out + ST of paper Eq. 2), dq (SR + OG of Section 3.4), dk and dv (STB + PG).  All four have the
+// same form over tiles of 128 tokens, with x, y, z three of the tensors and a carried state St [128 x 128]:
+//     out_r = sum_s (x_r . y_s) D[r,s] z_s  +  a_r x_r St ;     St <- exp(b_T) St + y^T diag(w) z
+//             x   y   z    St               runs      pairs   D                a_r             w_s
+//       o     q   k   v    H                forward   s <= r  exp(b_r - b_s)   exp(b_r)        exp(b_T - b_s)
+//       dq    dO  v   k    H^T              forward   s <= r  exp(b_r - b_s)   exp(b_r)        exp(b_T - b_s)
+//       dk    v   dO  q    G^T              reverse   s >= r  exp(b_s - b_r)   exp(b_T - b_r)  exp(b_s)
+//       dv    k   q   dO   G                reverse   s >= r  exp(b_s - b_r)   exp(b_T - b_r)  exp(b_s)
+// b: inclusive cumulative log-decay inside the tile, b_T its total, H the state, G the gradient of the state leaving the tile.
+// With b_T - b in the place of b the reverse sweeps' weights are those of the forward ones; the decay tables hold it.
+// dq and dk also store the row dot products x_out[t] = q_t . dq_t and k_t . dk_t (float32), which the log-decay gradient needs.
+//
+// Per tile four groups of eight MMAs of 128 x 128 x 16 (64 cycles each): scores x y^T, x St, the state update, and P z with
+// P = bf16(scores * D) read from tensor memory, where the mask pass leaves it in the columns of the scores.  y is scaled by w in
+// place once the scores have been taken; the output tile replaces z and leaves by TMA, the tile for the dot products arrives
+// in the place of x: so two whole tile sets and the state fit the shared memory, and no operand is copied.
+// K steps of P z write only the lanes whose rows have a pair in them (disable-output-lane), so a row meets no z row beyond
+// its own 16 tokens: there 0 * Inf would be NaN.
+//
+// Why tiles of 128 tokens: a chunk of 64 needs M = 64 MMAs for the token-row products, which run at half rate, and pays every
+// hand-off between MMAs and elementwise passes (commit, wait, fence, 100-250 cycles each) twice as often.
+//
+// Why loops where the code could be unrolled, and one body for the backward's sweeps with the role as a value: the 20 warps run eight
+// different programs, and what they run per tile has to stay in the instruction cache.  Straight code, 62 KB for the forward sweep and 197 KB
+// for the backward's three, took 7700 cycles per tile forward and 16000-20000 in dk and dv, whose CTAs pushed each other's code out; now 31 and
+// 37 KB and 4150 / 5700 (dq, dk) / 5000 (dv).  A short call runs mostly cold code: 200 tokens x 16 heads 21.8 -> 13.6 us with the last 10 KB.
+//
+// What bounds them: per tile scores -> mask -> P z -> epilogue in series (850 + 1650 + 800 + 600 cycles), MMAs 2048 of 4150.  A second set of
+// score columns (x St and P z in one accumulator, rescaled between) to overlap two tiles was slower: 4700 cycles, the elementwise warps
+// then are in series.  Against 64-token tiles with dk and dv in one sweep (16384 tokens x 32 heads): o 116 -> 86 us, dq 150 -> 113,
+// dk and dv 389 -> 311; chains forward + backward 1.13x, 256K tokens x 32 heads 9.43 -> 8.25 ms.
+//
+// A tile is two 64-token chunks, or one before a chunk where a segment of a merged launch begins (SegParams::bslot) and at the end
+// of a block; the rows of a missing half take no part in the state update and in P z and are not stored.
+//
+// Roles (20 warps): WG0, WG1 state pass (TMEM state -> bf16 copy in shared memory, rescaled state), then y *= w;  WG2, WG3
+// decay mask, then epilogue;  warp 16 MMAs, 17 tile loads, 18 output tiles, 19 decay tables.
+// Tensor memory: St 0-127, x St 128-255, P z 256-383, scores / P 384-511.
+constexpr int SW_THREADS = 640;
+constexpr int W_MMA = 16, W_TMA = 17, W_OUT = 18, W_TAB = 19;
+constexpr int TT = 128;                    // tokens per tile
+constexpr int FBOX = TT * 128;             // bytes of [128 tokens x 64 features]
+constexpr int XTILE = 2 * FBOX;            // bytes of [128 tokens x 128 features]
+enum { SWEEP_O = 0, SWEEP_DQ = 1, SWEEP_DK = 2, SWEEP_DV = 3 };
+
 struct SweepSmem {
-    alignas(1024) unsigned char tiles[SW_STAGES][3][TILE];
-    alignas(1024) unsigned char xvw[TILE];
-    alignas(1024) unsigned char am[2][BOX];
-    alignas(1024) unsigned char sb[2 * 16384];
-    float bloc[MAXR * C];
-    float ctot[MAXR];
-    uint64_t full[SW_STAGES], sc_done[2], am_ready[2], st_ready, w_ready, st_done, out_done[2], o_free[2], g_issued;
+    alignas(1024) unsigned char tiles[2][3][XTILE];      // x, y, z
+    alignas(1024) unsigned char sb[2 * FBOX];            // bf16 copy of the state
+    float b[2][TT];                                      // cumulative log-decay of a tile, in units of log 2
+    float u[2][TT];                                      // 2^(b_ref - b_s), ref the token of s's 32 that is nearest to the rows they meet
+                                                         // (both: the halves of the row dot products, once the tile's tables have served)
+    float total[2];
+    uint64_t full_xy[2], full_z[2], sc_done[2], p_ready[2], y_ready[2], st_ready[2], st_done[2], x_done[2], out_done[2], o_free[2], staged[2],
+        e_full[2], z_free[2], tab_full[2], g_issued;
+    unsigned long long cuts;
     uint32_t tmem_base;
     int abort_flag;
 };
+static_assert(sizeof(SweepSmem) <= 227 * 1024, "one CTA per SM");
 
-template <bool DQ>
-__device__ __forceinline__ void sweep_body(const CUtensorMap* tmQ, const CUtensorMap* tmK, const CUtensorMap* tmV, const SegParams& p,
-                                           const float* __restrict__ g, const float* Hs, __nv_bfloat16* __restrict__ out,
-                                           long long out_tok, long long out_bat, const __nv_bfloat16* __restrict__ e_glob,
-                                           float* __restrict__ xout, int* status, int h, int j) {
-    extern __shared__ unsigned char smem_raw[];
-    SweepSmem& sm = *reinterpret_cast<SweepSmem*>(align1024(smem_raw));
-    const int b = blockIdx.z;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int c0 = j * p.R, nch = min(p.R, p.NC - c0);
-    const long long t0 = (long long)c0 * C;
-    volatile int* abort_flag = &sm.abort_flag;
-    constexpr uint32_t T_ST = 0, T_O = 128, T_SC = 384;
-
-    if (tid == 0) {
-        sm.abort_flag = 0;
-        for (int s = 0; s < SW_STAGES; ++s) ptx::mbar_init(&sm.full[s], 1);
-        for (int i = 0; i < 2; ++i) {
-            ptx::mbar_init(&sm.sc_done[i], 1); ptx::mbar_init(&sm.am_ready[i], 4);
-            ptx::mbar_init(&sm.out_done[i], 1); ptx::mbar_init(&sm.o_free[i], 4);
-        }
-        ptx::mbar_init(&sm.st_ready, 12);
-        ptx::mbar_init(&sm.w_ready, 8);
-        ptx::mbar_init(&sm.st_done, 1);
-        ptx::mbar_init(&sm.g_issued, 16);
-        ptx::fence_mbar_init();
+// The tiles of a block of nch chunks, in order: first chunk c and length len (1 or 2 chunks) of the i-th.
+struct Tiles {
+    bool rev;
+    int nch, i, c, len;
+    unsigned long long cuts;                             // forward: bit c set where a tile must begin at chunk c
+    __device__ __forceinline__ Tiles(bool rev_, int nch_, unsigned long long cuts_) : rev(rev_), nch(nch_), i(0), cuts(cuts_) {
+        c = rev ? (nch - 1) & ~1 : 0;
+        measure();
     }
-    if (warp == W_MMA) ptx::tmem_alloc(&sm.tmem_base, 512);
-    ptx::tc_fence_before_sync();
-    __syncthreads();
-    ptx::tc_fence_after_sync();
-    const uint32_t tmem = sm.tmem_base;
-    if (p.wait_first) grid_wait();
-    // the decay tables are built by the compute warps while the first tiles are already on their way
+    __device__ __forceinline__ void measure() { len = c + 1 < nch && !((cuts >> ((c + 1) & 63)) & 1) ? 2 : 1; }
+    __device__ __forceinline__ bool more() const { return rev ? c >= 0 : c < nch; }
+    __device__ __forceinline__ void next() {
+        c = rev ? c - 2 : c + len;
+        ++i;
+        measure();
+    }
+    __device__ __forceinline__ int stage() const { return i & 1; }
+    __device__ __forceinline__ uint32_t phase() const { return (i >> 1) & 1; }
+};
 
-    if (warp == W_TMA) {
-        if (lane == 0) {
-            grid_launch_next();
-            ptx::prefetch_tmap(tmQ); ptx::prefetch_tmap(tmK); ptx::prefetch_tmap(tmV);
-            SF_WAIT(&sm.g_issued, 0, DEV_TIMEOUT_TMA);
-            for (int c = 0; c < nch; ++c) {
-                const int s = c % SW_STAGES;
-                // the stage was last used by chunk c-3, complete once all its MMAs retired
-                if (c >= SW_STAGES) SF_WAIT(&sm.out_done[(c - SW_STAGES) & 1], ((c - SW_STAGES) >> 1) & 1, DEV_TIMEOUT_MMA);
-                ptx::mbar_expect_tx(&sm.full[s], 3 * TILE);
-                const int tok = (int)t0 + c * C;
-                tma_tile(sm.tiles[s][0], tmQ, &sm.full[s], h, tok, b);
-                tma_tile(sm.tiles[s][1], tmK, &sm.full[s], h, tok, b);
-                tma_tile(sm.tiles[s][2], tmV, &sm.full[s], h, tok, b);
+// Loads the tile of head h from token t0 on; tokens at or beyond the end of the tensor are zeros.
+__device__ __forceinline__ void load_tile(unsigned char* dst, const CUtensorMap* m, uint64_t* bar, int h, int t0, int b) {
+    ptx::tma_load_4d(dst, m, bar, 0, h, t0, b);
+    ptx::tma_load_4d(dst + FBOX, m, bar, 64, h, t0, b);
+}
+__device__ __forceinline__ void prefetch_tile(const CUtensorMap* m, int h, int t0, int b) {
+    ptx::tma_prefetch_4d(m, 0, h, t0, b);
+    ptx::tma_prefetch_4d(m, 64, h, t0, b);
+}
+
+// P = bf16(scores * D), D = 2^(b_r - b_s), for the 32 rows of a warp (row 32 q + lane) and every second block of 32 columns that has a
+// pair, from block `half` on; P of a block takes the first half of its own columns.  Off the diagonal D is the product of a factor
+// of the row and one of the column, both at most 1, split at the token of the block that is nearest to the rows: an
+// exponential per element there would keep the SM quarter of the last rows (four of ten blocks) busy for 1000 cycles.
+__device__ __forceinline__ void mask_tile(uint32_t sc, const float* b, const float* u, bool rev, int half) {
+    const int q = (threadIdx.x >> 5) & 3, lane = threadIdx.x & 31;
+    const uint32_t taddr = sc + ((uint32_t)(q * 32) << 16), pairs = rev ? 0xffffffffu << lane : 0xffffffffu >> (31 - lane);
+    const float br = b[32 * q + lane];
+#pragma unroll 1
+    for (int cb = rev ? q + ((q ^ half) & 1) : half; cb < (rev ? 4 : q + 1); cb += 2) {
+        float x[32], y[16];
+        ptx::tmem_ld32(taddr + 32 * cb, x);
+        if (cb == q) {
+            const float* bc = b + 32 * cb;
+            ptx::tmem_ld_wait();
+#pragma unroll
+            for (int j = 0; j < 32; j += 4) {
+                const float4 f = *reinterpret_cast<const float4*>(bc + j);
+                const float bs[4] = {f.x, f.y, f.z, f.w};
+#pragma unroll
+                for (int e = 0; e < 4; ++e) x[j + e] = (pairs >> (j + e)) & 1 ? x[j + e] * ptx::ex2(br - bs[e]) : 0.f;
             }
-        }
-    } else if (warp == W_MMA) {
-        if (lane == 0) {
-            constexpr uint32_t id_sc = ptx::idesc_bf16(64, 64, 0, 0);
-            constexpr uint32_t id_o1 = ptx::idesc_bf16(64, 128, 0, 1);
-            constexpr uint32_t id_st = ptx::idesc_bf16(128, 128, 1, 1);
-            const uint32_t sb = ptx::smem_u32(sm.sb), xvw = ptx::smem_u32(sm.xvw);
-            auto scores = [&](int c) {
-                const int s = c % SW_STAGES;
-                SF_WAIT(&sm.full[s], (c / SW_STAGES) & 1, DEV_TIMEOUT_TMA);
-                ptx::tc_fence_after_sync();
-                const uint32_t xq = ptx::smem_u32(sm.tiles[s][0]), xk = ptx::smem_u32(sm.tiles[s][1]);
-                mma_group<8, DK8, DK8, 0>(tmem + T_SC + (c & 1) * 64, klo(xq), klo(xk), id_sc);
-                ptx::mma_commit(&sm.sc_done[c & 1]);
-            };
-            scores(0);
-            if (nch > 1) scores(1);
-            for (int c = 0; c < nch; ++c) {
-                const int s = c % SW_STAGES, bf = c & 1;
-                const uint32_t xq = ptx::smem_u32(sm.tiles[s][0]), xk = ptx::smem_u32(sm.tiles[s][1]), xv = ptx::smem_u32(sm.tiles[s][2]);
-                const uint32_t am = ptx::smem_u32(sm.am[bf]);
-                const uint32_t to = tmem + T_O + bf * 128;
-                if (c >= 2) SF_WAIT(&sm.o_free[bf], ((c - 2) >> 1) & 1, DEV_TIMEOUT_MMA);
-                SF_WAIT(&sm.st_ready, c & 1, DEV_TIMEOUT_MMA);
-                ptx::tc_fence_after_sync();
-                // the state-dependent MMAs first: inter-chunk output (lanes +16), then the state update
-                mma_group<8, DK8, DMN, 0>(to + (16u << 16), klo(xq), mlo(sb, 16384), id_o1);
-                SF_WAIT(&sm.w_ready, c & 1, DEV_TIMEOUT_MMA);        // the weighted tile is written while the MMAs above run
-                ptx::tc_fence_after_sync();
-                mma_group<4, DMN, DMN, 1>(tmem + T_ST, mlo(xk, BOX), mlo(xvw, BOX), id_st);
-                ptx::mma_commit(&sm.st_done);
-                SF_WAIT(&sm.am_ready[bf], (c >> 1) & 1, DEV_TIMEOUT_MMA);
-                ptx::tc_fence_after_sync();
-                mma_group<4, DK8, DMN, 0>(to, klo(am), mlo(xv, BOX), id_o1);                // intra
-                ptx::mma_commit(&sm.out_done[bf]);
-                if (c + 2 < nch) scores(c + 2);          // into the score buffer the mask of chunk c has released
-            }
-        }
-    } else if (warp < 16) {
-        const long long bh = ((long long)b * p.H + h) * (long long)(D * D);
-        const float* H0 = p.single ? (p.s_init ? p.s_init + bh : nullptr) : Hs + bh * p.NB + (long long)j * (D * D);
-        if (H0) ptx::prefetch_l2(H0 + tid * 32);                 // the block's initial state (512 lines) is on its way while the tables are built
-        prep_decay(g + (long long)b * p.bg + h, p.tg, t0, nch, p.L, sm.bloc, sm.ctot, 16, &sm.g_issued);
-        ptx::named_bar_sync(1, 512);
-        const int wg = warp >> 2, t = tid & 127;
-        const int rA = 16 * (warp & 3) + (lane >> 2), rB = rA + 8;
-        __nv_bfloat16* out_h = out + (long long)b * out_bat + (long long)h * D;
-        const __nv_bfloat16* e_h = DQ ? e_glob + (long long)b * out_bat + (long long)h * D : nullptr;
-        float* xo = DQ ? xout + ((long long)b * p.H + h) * p.L : nullptr;
-        auto mask = [&](int c) {
-            const int bf = c & 1;
-            SF_WAIT(&sm.sc_done[bf], (c >> 1) & 1, DEV_TIMEOUT_MMA);
-            if (c >= 2) SF_WAIT(&sm.out_done[bf], ((c - 2) >> 1) & 1, DEV_TIMEOUT_MMA);      // Am[bf] no longer read
-            ptx::tc_fence_after_sync();
-            mask_pass(tmem + T_SC + bf * 64, sm.bloc + c * C, sm.am[bf], nullptr);
-            ptx::fence_proxy_async();
-            ptx::tc_fence_before_sync();
-            ptx::mbar_arrive_warp(&sm.am_ready[bf]);
-        };
-        auto epilogue = [&](int c) {
-            const int bf = c & 1;
-            const long long tokA = t0 + c * C + rA, tokB = tokA + 8;
-            const float eA = fast_exp(sm.bloc[c * C + rA]), eB = fast_exp(sm.bloc[c * C + rB]);
-            auto ready = [&]() {
-                SF_WAIT(&sm.out_done[bf], (c >> 1) & 1, DEV_TIMEOUT_MMA);
-                ptx::tc_fence_after_sync();
-            };
-            float dotA, dotB;
-            const bool vA = tokA < p.L, vB = tokB < p.L;          // rows past the end of a ragged segment: computed, not stored
-            const long long lastTok = p.L - 1;
-            pair_epilogue<DQ>(tmem + T_O + bf * 128, eA, eB, out_h + tokA * out_tok, out_h + tokB * out_tok,
-                              DQ ? e_h + min(tokA, lastTok) * out_tok : nullptr, DQ ? e_h + min(tokB, lastTok) * out_tok : nullptr,
-                              dotA, dotB, vA, vB, ready);
-            if (DQ && (lane & 3) == 0) {
-                if (vA) xo[tokA] = dotA;
-                if (vB) xo[tokB] = dotB;
-            }
-            ptx::tc_fence_before_sync();
-            ptx::mbar_arrive_warp(&sm.o_free[bf]);
-        };
-        // tables, first tiles, scores and mask need only the caller's inputs: they run while the scan finishes
-        if (wg == 3) {
-            grid_wait();
-            for (int c = 0; c < nch; ++c) epilogue(c);
         } else {
-            if (wg == 2) mask(0);
-            grid_wait();
-            for (int c = 0; c < nch; ++c) {
-                const int s = c % SW_STAGES;
-                const float* bch = sm.bloc + c * C;
-                const float bC = sm.ctot[c];
-                float* dump = nullptr;                   // merged launches: the state entering a segment's first chunk goes out
-                if (!DQ && c == 0 && p.single && p.s_copy) dump = p.s_copy + bh;
-                else if (!DQ && p.bslot) {
-                    const int slot = __ldg(p.bslot + c0 + c);
-                    if (slot >= 0) dump = p.bbase + slot * p.bstride + ((long long)b * p.H + h) * (long long)(D * D);
-                }
-                if (wg < 2) SF_WAIT(&sm.full[s], (c / SW_STAGES) & 1, DEV_TIMEOUT_TMA);
-                if (c > 0) SF_WAIT(&sm.st_done, (c - 1) & 1, DEV_TIMEOUT_MMA);
-                ptx::tc_fence_after_sync();
-                // 16-column units: WG0 0-2, WG1 3-5, WG2 6-7
-                if (wg < 2) state_pass<3>(tmem + T_ST, sm.sb, fast_exp(bC), c == 0, H0, DQ, 3 * wg, dump);
-                else        state_pass<2>(tmem + T_ST, sm.sb, fast_exp(bC), c == 0, H0, DQ, 6, dump);
-                ptx::fence_proxy_async();
-                ptx::tc_fence_before_sync();
-                ptx::mbar_arrive_warp(&sm.st_ready);
-                if (wg < 2) {
-                    scale_box(sm.xvw + wg * BOX, sm.tiles[s][2] + wg * BOX, t, [&](int row) { return fast_exp(bC - bch[row]); });
-                    ptx::fence_proxy_async();
-                    ptx::mbar_arrive_warp(&sm.w_ready);
-                }
-                if (wg == 2 && c + 1 < nch) mask(c + 1);
-            }
-            if (!DQ && p.single) {                       // the state leaving the segment
-                SF_WAIT(&sm.st_done, (nch - 1) & 1, DEV_TIMEOUT_MMA);
-                ptx::tc_fence_after_sync();
-                if (wg < 2) state_out<3>(tmem + T_ST, p.s_final + bh, 3 * wg);
-                else        state_out<2>(tmem + T_ST, p.s_final + bh, 6);
+            const float fr = ptx::ex2(br - b[32 * cb + (rev ? 0 : 31)]);
+            const float* uc = u + 32 * cb;
+            ptx::tmem_ld_wait();
+#pragma unroll
+            for (int j = 0; j < 32; j += 4) {
+                const float4 f = *reinterpret_cast<const float4*>(uc + j);
+                ptx::mul2(x[j], x[j + 1], fr, fr); ptx::mul2(x[j + 2], x[j + 3], fr, fr);
+                ptx::mul2(x[j], x[j + 1], f.x, f.y); ptx::mul2(x[j + 2], x[j + 3], f.z, f.w);
             }
         }
+#pragma unroll
+        for (int j = 0; j < 16; ++j) y[j] = __uint_as_float(pack2(x[2 * j], x[2 * j + 1]));
+        ptx::tmem_st16(taddr + 32 * cb, y);
     }
-    ptx::tc_fence_before_sync();
-    __syncthreads();
-    if (warp == W_MMA) ptx::tmem_dealloc(tmem, 512);
+    ptx::tmem_st_wait();
 }
 
-template <bool DQ>
-__global__ void __launch_bounds__(SW_THREADS, 1)
-tc_sweep_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
-                SegParams p, const float* __restrict__ g, const float* Hs, __nv_bfloat16* __restrict__ out, long long out_tok,
-                long long out_bat, const __nv_bfloat16* __restrict__ e_glob, float* __restrict__ xout, int* status) {
-    // heads fastest: co-resident CTAs read neighbouring 256-byte pieces of the same tokens
-    sweep_body<DQ>(&tmQ, &tmK, &tmV, p, g, Hs, out, out_tok, out_bat, e_glob, xout, status, blockIdx.x, blockIdx.y);
+// y *= w in place, 256 threads; a thread meets the rows t/8 + 32 i
+template <typename F>
+__device__ __forceinline__ void scale_rows(unsigned char* tile, int t, F w_row) {
+    uint4* u = reinterpret_cast<uint4*>(tile);
+    float w[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) w[i] = w_row((t >> 3) + 32 * i);
+#pragma unroll 1
+    for (int hf = 0; hf < 2; ++hf) {
+        uint4 v[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) v[i] = u[hf * (FBOX / 16) + t + 256 * i];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            __nv_bfloat162* h2 = reinterpret_cast<__nv_bfloat162*>(&v[i]);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                float2 f = __bfloat1622float2(h2[e]);
+                ptx::mul2(f.x, f.y, w[i], w[i]);
+                h2[e] = __floats2bfloat162_rn(f.x, f.y);
+            }
+            u[hf * (FBOX / 16) + t + 256 * i] = v[i];
+        }
+    }
 }
 
-// ==================================================================================================
-// dk/dv pass (STB inside the block + PG, Section 3.4): reverse chunk sweep carrying G = dH (the
-// gradient w.r.t. the state leaving the chunk, from Gs[j]):
-//     A = (Q K^T) D,  dA = (dO V^T) D
-//     dv_s = sum_{r>=s} A[r,s] dO_r + w_s k_s G ;   dk_s = sum_{r>=s} dA[r,s] q_r + w_s v_s G^T ;   w_s = exp(b_C - b_s)
-//     G <- exp(b_C) G + (diag(exp(b)) Q)^T dO
-// and xk[t] = k_t . dk_t (float32).
-// TMEM columns: G 0-127; dk pair 128-255; dv pair 256-383; score pair (A at lanes +0, dA at +16)
-// double-buffered at 384 / 448.
-struct DkdvSmem {
-    alignas(1024) unsigned char tiles[2][4][TILE];     // q, k, v, dO
-    alignas(1024) unsigned char qw[TILE];
-    alignas(1024) unsigned char am[2][BOX];
-    alignas(1024) unsigned char dam[2][BOX];
-    alignas(1024) unsigned char gb[2 * 16384];
-    float bloc[MAXR * C];
-    float ctot[MAXR];
-    uint64_t full[2], sc_done[2], am_ready[2], st_ready, w_ready, st_done[2], it_done[2], dv_done, dk_done, dv_free, dk_free, g_issued;
-    uint32_t tmem_base;
-    int abort_flag;
-};
+// Row 32 q + lane of the output, features 64 half ..: a * inter + intra as bf16 into the tile `slot` and, with `with_dot`, its dot product
+// with the tile `e_tile`.  `loaded` is called once the accumulators have been read.
+template <typename F>
+__device__ __forceinline__ float epilogue_tile(uint32_t inter, uint32_t intra, unsigned char* slot, const unsigned char* e_tile, float a, int half,
+                                               bool with_dot, F loaded) {
+    const int q = (threadIdx.x >> 5) & 3, row = 32 * q + (threadIdx.x & 31);
+    const uint32_t from = ((uint32_t)(q * 32) << 16) + 64 * half;
+    unsigned char* box = slot + half * FBOX;
+    float dot = 0.f;
+#pragma unroll 1
+    for (int cb = 0; cb < 2; ++cb) {
+        float x[32], y[32];
+        ptx::tmem_ld32(inter + from + 32 * cb, x);
+        ptx::tmem_ld32(intra + from + 32 * cb, y);
+        ptx::tmem_ld_wait();
+        if (cb == 1) loaded();
+#pragma unroll
+        for (int i = 0; i < 32; ++i) y[i] = fmaf(a, x[i], y[i]);
+        if (with_dot) {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const uint4 v = ld_unit(e_tile + half * FBOX, row, cb * 4 + e);
+                const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&w[i]));
+                    dot = fmaf(y[8 * e + 2 * i], f.x, dot);
+                    dot = fmaf(y[8 * e + 2 * i + 1], f.y, dot);
+                }
+            }
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+            st_unit(box, row, cb * 4 + e, make_uint4(pack2(y[8 * e], y[8 * e + 1]), pack2(y[8 * e + 2], y[8 * e + 3]),
+                                                     pack2(y[8 * e + 4], y[8 * e + 5]), pack2(y[8 * e + 6], y[8 * e + 7])));
+    }
+    return dot;
+}
 
-// The dk and dv accumulator pairs are single-buffered (TMEM is full), so each has its own completion and
-// release barrier.  Per iteration the MMAs that read or update the carried gradient G are issued first and
-// st_done is committed right behind them: the rescaling of G for the next chunk (the serial part of the sweep)
-// then overlaps the intra-chunk MMAs, the epilogues and the next chunk's scores.  it_done closes the iteration.
-__device__ __forceinline__ void dkdv_body(const CUtensorMap* tmQ, const CUtensorMap* tmK, const CUtensorMap* tmV, const CUtensorMap* tmD,
-                                          const SegParams& p, const float* __restrict__ g, const float* Gs,
-                                          const __nv_bfloat16* __restrict__ k_glob, __nv_bfloat16* __restrict__ dk,
-                                          __nv_bfloat16* __restrict__ dv, float* __restrict__ xk, int* status, int h, int j) {
-    extern __shared__ unsigned char smem_raw[];
-    DkdvSmem& sm = *reinterpret_cast<DkdvSmem*>(align1024(smem_raw));
+// P z over K steps of 16 tokens: FROM .. TO - 1 of the eight, counted from the last one in the reverse sweeps, each for the lanes that have a
+// pair in it: rows from 16 ks on (forward) or up to 16 ks + 15 (reverse).  The first step is the one that all rows take part in.
+template <int FROM, int TO>
+__device__ __forceinline__ void mma_intra(uint32_t d, uint32_t p, uint32_t zlo, uint32_t idesc, bool rev, bool acc) {
+    if constexpr (FROM < TO) {
+        constexpr int pc = 32 * (FROM >> 1) + 8 * (FROM & 1), lanes = 16 * FROM;
+        uint32_t off[4];
+#pragma unroll
+        for (int w = 0; w < 4; ++w) {
+            const int n = lanes - 32 * w, m = lanes - 96 + 32 * w;       // lanes of word w that are off: the first n, or the last m
+            const uint32_t fwd = n <= 0 ? 0u : n >= 32 ? ~0u : (1u << n) - 1, bwd = m <= 0 ? 0u : m >= 32 ? ~0u : ~0u << (32 - m);
+            off[w] = rev ? bwd : fwd;
+        }
+        ptx::mma_ts(d, rev ? p + 104 - pc : p + pc, rev ? zlo + dofs<DMN>(7 - FROM) : zlo + dofs<DMN>(FROM), idesc, acc, off);
+        mma_intra<FROM + 1, TO>(d, p, zlo, idesc, rev, true);
+    }
+}
+
+struct SweepMaps { const CUtensorMap *x, *y, *z, *e, *out; };      // out: boxes of 64 tokens, the others of 128
+
+template <bool BWD>
+__device__ __forceinline__ void sweep_body(int role, const SweepMaps& m, const SegParams& p, const float* __restrict__ g, const float* states,
+                                           const float* s_init, float* __restrict__ xout, int h, int j) {
+    const bool rev = BWD && role >= SWEEP_DK, dot = BWD && role != SWEEP_DV;       // dq and dk carry the transposed state
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    SweepSmem& sm = *reinterpret_cast<SweepSmem*>(smem_raw);
     const int b = blockIdx.z;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int c0 = j * p.R, nch = min(p.R, p.NC - c0);
-    const long long t0 = (long long)c0 * C;
-    volatile int* abort_flag = &sm.abort_flag;
-    constexpr uint32_t T_G = 0, T_DK = 128, T_DV = 256, T_SC = 384;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
+    const int c0 = j * p.R, nch = min(p.R, p.NC - c0), t0 = c0 * C;
+    int* abort_flag = &sm.abort_flag;
+    constexpr uint32_t T_ST = 0, T_INTER = 128, T_INTRA = 256, T_SC = 384;
 
     if (tid == 0) {
         sm.abort_flag = 0;
-        for (int i = 0; i < 2; ++i) {
-            ptx::mbar_init(&sm.full[i], 1);
-            ptx::mbar_init(&sm.sc_done[i], 1); ptx::mbar_init(&sm.am_ready[i], 4);
-            ptx::mbar_init(&sm.st_done[i], 1);
-            ptx::mbar_init(&sm.it_done[i], 1);
+        for (int s = 0; s < 2; ++s) {
+            ptx::mbar_init(&sm.full_xy[s], 1); ptx::mbar_init(&sm.full_z[s], 1); ptx::mbar_init(&sm.sc_done[s], 1);
+            ptx::mbar_init(&sm.p_ready[s], 8); ptx::mbar_init(&sm.y_ready[s], 8); ptx::mbar_init(&sm.st_ready[s], 8);
+            ptx::mbar_init(&sm.st_done[s], 1); ptx::mbar_init(&sm.x_done[s], 1); ptx::mbar_init(&sm.out_done[s], 1);
+            ptx::mbar_init(&sm.o_free[s], 8); ptx::mbar_init(&sm.staged[s], 8); ptx::mbar_init(&sm.e_full[s], 1); ptx::mbar_init(&sm.z_free[s], 1);
+            ptx::mbar_init(&sm.tab_full[s], 1);
         }
-        ptx::mbar_init(&sm.st_ready, 8);
-        ptx::mbar_init(&sm.w_ready, 8);
-        ptx::mbar_init(&sm.dv_done, 1);
-        ptx::mbar_init(&sm.dk_done, 1);
-        ptx::mbar_init(&sm.dv_free, 4);
-        ptx::mbar_init(&sm.dk_free, 4);
-        ptx::mbar_init(&sm.g_issued, 16);
+        ptx::mbar_init(&sm.g_issued, 1);
         ptx::fence_mbar_init();
     }
     if (warp == W_MMA) ptx::tmem_alloc(&sm.tmem_base, 512);
+    if (!BWD && warp == 1) {                             // where segments of a merged launch begin (a block has at most 64 chunks)
+        unsigned long long cuts = 0;
+        if (p.bslot) {
+            const bool lo = lane < nch && __ldg(p.bslot + c0 + lane) >= 0, hi = lane + 32 < nch && __ldg(p.bslot + c0 + lane + 32) >= 0;
+            cuts = __ballot_sync(0xffffffffu, lo) | ((unsigned long long)__ballot_sync(0xffffffffu, hi) << 32);
+        }
+        if (lane == 0) sm.cuts = cuts;
+    }
     ptx::tc_fence_before_sync();
     __syncthreads();
     ptx::tc_fence_after_sync();
     const uint32_t tmem = sm.tmem_base;
+    Tiles it(rev, nch, BWD ? 0 : sm.cuts);
     if (p.wait_first) grid_wait();
-    // the decay tables are built by the compute warps while the first tiles are already on their way
 
-    // iteration i handles chunk c = nch-1-i
     if (warp == W_TMA) {
-        if (lane == 0) {
+        const bool leader = ptx::elect_one();
+        if (leader) {
             grid_launch_next();
-            ptx::prefetch_tmap(tmQ); ptx::prefetch_tmap(tmK); ptx::prefetch_tmap(tmV); ptx::prefetch_tmap(tmD);
-            SF_WAIT(&sm.g_issued, 0, DEV_TIMEOUT_TMA);
-            for (int i = 0; i < nch; ++i) {
-                const int s = i & 1;
-                // the stage was last used by iteration i-2; it_done is committed after all of its MMAs
-                if (i >= 2) SF_WAIT(&sm.it_done[s], ((i - 2) >> 1) & 1, DEV_TIMEOUT_MMA);
-                ptx::mbar_expect_tx(&sm.full[s], 4 * TILE);
-                const int tok = (int)t0 + (nch - 1 - i) * C;
-                tma_tile(sm.tiles[s][0], tmQ, &sm.full[s], h, tok, b);
-                tma_tile(sm.tiles[s][1], tmK, &sm.full[s], h, tok, b);
-                tma_tile(sm.tiles[s][2], tmV, &sm.full[s], h, tok, b);
-                tma_tile(sm.tiles[s][3], tmD, &sm.full[s], h, tok, b);
+            ptx::prefetch_tmap(m.x); ptx::prefetch_tmap(m.y); ptx::prefetch_tmap(m.z); ptx::prefetch_tmap(m.out);
+        }
+        SF_WAIT(&sm.g_issued, 0, DEV_TIMEOUT_TMA);
+        for (; it.more(); it.next()) {
+            const int s = it.stage(), tok = t0 + it.c * C;
+            const uint32_t before = it.phase() ^ 1;
+            const bool wait = it.i >= 2;
+            // y of tile i - 2 has served with its state update, x with its product with the state (or as the tile for the dot products), z once
+            // the output tile that took its place has left; what has to wait is on its way to L2 meanwhile.  full_xy is armed only where
+            // tile i - 2 is known to have passed it.
+            if (leader && dot) prefetch_tile(m.x, h, tok, b);
+            if (leader) prefetch_tile(m.z, h, tok, b);
+            if (wait) SF_WAIT(dot ? &sm.st_done[s] : &sm.x_done[s], before, DEV_TIMEOUT_MMA);
+            if (leader) {
+                ptx::mbar_expect_tx(&sm.full_xy[s], 2 * XTILE);
+                load_tile(sm.tiles[s][dot], dot ? m.y : m.x, &sm.full_xy[s], h, tok, b);
+            }
+            if (wait) SF_WAIT(dot ? &sm.staged[s] : &sm.st_done[s], before, DEV_TIMEOUT_MMA);
+            if (leader) load_tile(sm.tiles[s][!dot], dot ? m.x : m.y, &sm.full_xy[s], h, tok, b);
+            if (wait) SF_WAIT(&sm.z_free[s], before, DEV_TIMEOUT_MMA);
+            if (leader) {
+                ptx::mbar_expect_tx(&sm.full_z[s], XTILE);
+                load_tile(sm.tiles[s][2], m.z, &sm.full_z[s], h, tok, b);
+                if (dot) prefetch_tile(m.e, h, tok, b);
             }
         }
     } else if (warp == W_MMA) {
-        if (lane == 0) {
-            constexpr uint32_t id_sc = ptx::idesc_bf16(64, 64, 0, 0);
-            constexpr uint32_t id_tt = ptx::idesc_bf16(64, 128, 1, 1);     // A^T dO, dA^T Q: both operands token-major
-            constexpr uint32_t id_kn = ptx::idesc_bf16(64, 128, 0, 1);     // K G
-            constexpr uint32_t id_kk = ptx::idesc_bf16(64, 128, 0, 0);     // V G^T
-            constexpr uint32_t id_st = ptx::idesc_bf16(128, 128, 1, 1);
-            const uint32_t gb = ptx::smem_u32(sm.gb), qw = ptx::smem_u32(sm.qw);
-            auto scores = [&](int i) {
-                const int s = i & 1;
-                SF_WAIT(&sm.full[s], (i >> 1) & 1, DEV_TIMEOUT_TMA);
-                ptx::tc_fence_after_sync();
-                const uint32_t xq = ptx::smem_u32(sm.tiles[s][0]), xk = ptx::smem_u32(sm.tiles[s][1]);
-                const uint32_t xv = ptx::smem_u32(sm.tiles[s][2]), xd = ptx::smem_u32(sm.tiles[s][3]);
-                const uint32_t sc = tmem + T_SC + (i & 1) * 64;
-                mma_group<8, DK8, DK8, 0>(sc, klo(xq), klo(xk), id_sc);
-                mma_group<8, DK8, DK8, 0>(sc + (16u << 16), klo(xd), klo(xv), id_sc);
-                ptx::mma_commit(&sm.sc_done[i & 1]);
-            };
-            scores(0);
-            for (int i = 0; i < nch; ++i) {
-                const int s = i & 1;
-                const uint32_t xq = ptx::smem_u32(sm.tiles[s][0]), xk = ptx::smem_u32(sm.tiles[s][1]);
-                const uint32_t xv = ptx::smem_u32(sm.tiles[s][2]), xd = ptx::smem_u32(sm.tiles[s][3]);
-                const uint32_t am = ptx::smem_u32(sm.am[s]), dam = ptx::smem_u32(sm.dam[s]);
-                SF_WAIT(&sm.st_ready, i & 1, DEV_TIMEOUT_MMA);
-                if (i >= 1) SF_WAIT(&sm.dv_free, (i - 1) & 1, DEV_TIMEOUT_MMA);
-                ptx::tc_fence_after_sync();
-                // Everything that touches the carried gradient goes first, so that its rescaling for the next chunk
-                // runs while the intra-chunk MMAs and the next scores execute:
-                //   dv (lanes +16) = K G,  dk (lanes +16) = V G^T,  G += (diag(exp(b)) Q)^T dO
-                mma_group<8, DK8, DMN, 0>(tmem + T_DV + (16u << 16), klo(xk), mlo(gb, 16384), id_kn);
-                if (i >= 1) SF_WAIT(&sm.dk_free, (i - 1) & 1, DEV_TIMEOUT_MMA);
-                ptx::tc_fence_after_sync();
-                mma_group<8, DK8, DK16, 0>(tmem + T_DK + (16u << 16), klo(xv), klo(gb), id_kk);
-                SF_WAIT(&sm.w_ready, i & 1, DEV_TIMEOUT_MMA);
-                ptx::tc_fence_after_sync();
-                mma_group<4, DMN, DMN, 1>(tmem + T_G, mlo(qw, BOX), mlo(xd, BOX), id_st);
-                ptx::mma_commit(&sm.st_done[s]);                 // G, its bf16 copy and qw are free again
-                // intra-chunk parts: dv (lanes +0) = A^T dO, dk (lanes +0) = dA^T Q
-                SF_WAIT(&sm.am_ready[s], (i >> 1) & 1, DEV_TIMEOUT_MMA);
-                ptx::tc_fence_after_sync();
-                mma_group<4, DMN, DMN, 0>(tmem + T_DV, mlo(am, BOX), mlo(xd, BOX), id_tt);
-                ptx::mma_commit(&sm.dv_done);
-                mma_group<4, DMN, DMN, 0>(tmem + T_DK, mlo(dam, BOX), mlo(xq, BOX), id_tt);
-                ptx::mma_commit(&sm.dk_done);
-                ptx::mma_commit(&sm.it_done[s]);                 // tiles and masks of this iteration are free again
-                if (i + 1 < nch) scores(i + 1);      // two stages: the next chunk's tiles are already resident
+        const bool leader = ptx::elect_one();
+        constexpr uint32_t id_sc = ptx::idesc_bf16(128, 128, 0, 0), id_o = ptx::idesc_bf16(128, 128, 0, 1), id_st = ptx::idesc_bf16(128, 128, 1, 1);
+        const uint32_t sb = ptx::smem_u32(sm.sb);
+        for (; it.more(); it.next()) {
+            const int s = it.stage();
+            const uint32_t ph = it.phase();
+            const uint32_t x = ptx::smem_u32(sm.tiles[s][0]), y = ptx::smem_u32(sm.tiles[s][1]), z = ptx::smem_u32(sm.tiles[s][2]);
+            SF_SPIN(&sm.full_xy[s], ph, DEV_TIMEOUT_TMA);
+            ptx::tc_fence_after_sync();
+            if (leader) {                                // behind the MMAs that read the last P from these columns
+                mma_group<0, 8, DK16, DK16>(tmem + T_SC, klo(x), klo(y), id_sc, false);
+                ptx::mma_commit(&sm.sc_done[s]);
+            }
+            SF_SPIN(&sm.st_ready[s], ph, DEV_TIMEOUT_MMA);
+            if (it.i > 0) SF_SPIN(&sm.o_free[s ^ 1], (uint32_t)((it.i - 1) >> 1) & 1, DEV_TIMEOUT_MMA);
+            ptx::tc_fence_after_sync();
+            if (leader) {
+                mma_group<0, 8, DK16, DMN>(tmem + T_INTER, klo(x), mlo(sb, FBOX), id_o, false);
+                ptx::mma_commit(&sm.x_done[s]);
+            }
+            SF_SPIN(&sm.full_z[s], ph, DEV_TIMEOUT_TMA);
+            SF_SPIN(&sm.y_ready[s], ph, DEV_TIMEOUT_MMA);
+            ptx::tc_fence_after_sync();
+            if (leader) {
+                mma_group<0, 4, DMN, DMN>(tmem + T_ST, mlo(y, FBOX), mlo(z, FBOX), id_st, true);
+                if (it.len > 1) mma_group<4, 8, DMN, DMN>(tmem + T_ST, mlo(y, FBOX), mlo(z, FBOX), id_st, true);
+                ptx::mma_commit(&sm.st_done[s]);
+            }
+            SF_SPIN(&sm.p_ready[s], ph, DEV_TIMEOUT_MMA);
+            ptx::tc_fence_after_sync();
+            if (leader) {                                // of a tile of one chunk the steps with its tokens: the first four, or the last in the reverse sweeps
+                if (it.len > 1 || !rev) mma_intra<0, 4>(tmem + T_INTRA, tmem + T_SC, mlo(z, FBOX), id_o, rev, false);
+                if (it.len > 1 || rev) mma_intra<4, 8>(tmem + T_INTRA, tmem + T_SC, mlo(z, FBOX), id_o, rev, it.len > 1);
+                ptx::mma_commit(&sm.out_done[s]);
             }
         }
-    } else if (warp < 16) {
-        const long long bh = ((long long)b * p.H + h) * (long long)(D * D);
-        const float* G0 = p.single ? (p.s_init ? p.s_init + bh : nullptr) : Gs + bh * p.NB + (long long)j * (D * D);
-        if (G0) ptx::prefetch_l2(G0 + tid * 32);                 // the block's incoming state gradient, on its way while the tables are built
-        prep_decay(g + (long long)b * p.bg + h, p.tg, t0, nch, p.L, sm.bloc, sm.ctot, 16, &sm.g_issued);
-        ptx::named_bar_sync(1, 512);
-        const int wg = warp >> 2, t = tid & 127;
-        const int rA = 16 * (warp & 3) + (lane >> 2), rB = rA + 8;
-        __nv_bfloat16* dk_h = dk + (long long)b * p.bqk + (long long)h * D;
-        __nv_bfloat16* dv_h = dv + (long long)b * p.bv + (long long)h * D;
-        const __nv_bfloat16* k_h = k_glob + (long long)b * p.bqk + (long long)h * D;
-        float* xo = xk + ((long long)b * p.H + h) * p.L;
-        auto mask = [&](int i) {
-            const int c = nch - 1 - i, bf = i & 1;
-            SF_WAIT(&sm.sc_done[bf], (i >> 1) & 1, DEV_TIMEOUT_MMA);
-            if (i >= 2) SF_WAIT(&sm.it_done[bf], ((i - 2) >> 1) & 1, DEV_TIMEOUT_MMA);     // am/dam[bf] no longer read
-            ptx::tc_fence_after_sync();
-            mask_pass(tmem + T_SC + bf * 64, sm.bloc + c * C, sm.am[bf], sm.dam[bf]);
-            ptx::fence_proxy_async();
-            ptx::tc_fence_before_sync();
-            ptx::mbar_arrive_warp(&sm.am_ready[bf]);
-        };
-        if (wg >= 2) {
-            if (wg == 2) mask(0);
-            grid_wait();
-            for (int i = 0; i < nch; ++i) {
-                const int c = nch - 1 - i;
-                const long long tokA = t0 + c * C + rA, tokB = tokA + 8;
-                const float wA = fast_exp(sm.ctot[c] - sm.bloc[c * C + rA]), wB = fast_exp(sm.ctot[c] - sm.bloc[c * C + rB]);
-                const bool vA = tokA < p.L, vB = tokB < p.L;
-                float dotA, dotB;
-                auto dk_ready = [&]() {
-                    SF_WAIT(&sm.dk_done, i & 1, DEV_TIMEOUT_MMA);
-                    ptx::tc_fence_after_sync();
-                };
-                if (wg == 2) {
-                    SF_WAIT(&sm.dv_done, i & 1, DEV_TIMEOUT_MMA);
-                    ptx::tc_fence_after_sync();
-                    pair_epilogue<false>(tmem + T_DV, wA, wB, dv_h + tokA * p.tv, dv_h + tokB * p.tv, nullptr, nullptr, dotA, dotB, vA, vB);
-                    ptx::tc_fence_before_sync();
-                    ptx::mbar_arrive_warp(&sm.dv_free);
-                    if (i + 1 < nch) mask(i + 1);
-                } else {
-                    pair_epilogue<true>(tmem + T_DK, wA, wB, dk_h + tokA * p.tqk, dk_h + tokB * p.tqk, k_h + min(tokA, (long long)p.L - 1) * p.tqk, k_h + min(tokB, (long long)p.L - 1) * p.tqk, dotA, dotB, vA, vB, dk_ready);
-                    if ((lane & 3) == 0) {
-                        if (vA) xo[tokA] = dotA;
-                        if (vB) xo[tokB] = dotB;
+    } else if (warp == W_OUT) {
+        const bool leader = ptx::elect_one();
+        grid_wait();
+        for (; it.more(); it.next()) {
+            const int s = it.stage(), tok = t0 + it.c * C;
+            if (dot) {
+                SF_WAIT(&sm.x_done[s], it.phase(), DEV_TIMEOUT_MMA);
+                if (leader) {
+                    ptx::mbar_expect_tx(&sm.e_full[s], XTILE);
+                    load_tile(sm.tiles[s][0], m.e, &sm.e_full[s], h, tok, b);
+                }
+            }
+            if (leader && it.i > 0) {                    // behind the load for the dot products, which is waited for earlier
+                ptx::tma_store_wait_read();
+                ptx::mbar_arrive(&sm.z_free[s ^ 1]);
+            }
+            SF_WAIT(&sm.staged[s], it.phase(), DEV_TIMEOUT_MMA);
+            if (leader) {
+                const unsigned char* slot = sm.tiles[s][2];
+#pragma unroll 1
+                for (int th = 0; th < it.len; ++th)
+                    if (tok + th * C < p.L) {
+                        ptx::tma_store_4d(m.out, slot + th * BOX, 0, h, tok + th * C, b);
+                        ptx::tma_store_4d(m.out, slot + FBOX + th * BOX, 64, h, tok + th * C, b);
                     }
-                    ptx::tc_fence_before_sync();
-                    ptx::mbar_arrive_warp(&sm.dk_free);
+                ptx::tma_store_commit();
+            }
+        }
+        if (leader) ptx::tma_store_wait();
+    } else if (warp == W_TAB) {
+        // four tokens per lane; the log-decays of the next tile are on their way while this one is worked on
+        const float* gh = g + (long long)b * p.bg + h;
+        float gv[4];
+        auto fetch = [&](const Tiles& t) {
+            const int base = t0 + t.c * C + 4 * lane, lim = min(p.L, t0 + (t.c + t.len) * C);
+            const float* src = gh + base * p.tg;
+#pragma unroll
+            for (int e = 0; e < 4; ++e, src += p.tg) gv[e] = base + e < lim ? __ldg(src) : 0.f;
+        };
+        fetch(it);
+        if (lane == 0) ptx::mbar_arrive(&sm.g_issued);
+        Tiles done = it;
+        while (true) {
+            const int s = it.stage();
+            // Below -128 a decay wipes the state in float32 all the same, and limited to it the sums beside a mask value keep their precision.
+#pragma unroll
+            for (int e = 0; e < 4; ++e) gv[e] = (gv[e] < -128.f ? -128.f : gv[e]) * LOG2E;
+            gv[1] += gv[0]; gv[2] += gv[1]; gv[3] += gv[2];
+            float pre = gv[3];
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const float up = __shfl_up_sync(0xffffffffu, pre, off);
+                if (lane >= off) pre += up;
+            }
+            const float total = __shfl_sync(0xffffffffu, pre, 31);
+            if (lane == 31) sm.total[s] = total;
+            pre -= gv[3];                                // tokens before this lane's
+#pragma unroll
+            for (int e = 0; e < 4; ++e) gv[e] = rev ? total - (gv[e] + pre) : gv[e] + pre;
+            *reinterpret_cast<float4*>(sm.b[s] + 4 * lane) = make_float4(gv[0], gv[1], gv[2], gv[3]);
+            const float ref = __shfl_sync(0xffffffffu, rev ? gv[0] : gv[3], rev ? lane & ~7 : lane | 7);
+            *reinterpret_cast<float4*>(sm.u[s] + 4 * lane) = make_float4(ptx::ex2(ref - gv[0]), ptx::ex2(ref - gv[1]), ptx::ex2(ref - gv[2]), ptx::ex2(ref - gv[3]));
+            ptx::mbar_arrive_warp(&sm.tab_full[s]);
+            const bool first = it.i == 0;
+            it.next();
+            if (it.more()) fetch(it);
+            if (first) {
+                grid_wait();
+                if (it.more()) continue;
+            }
+            // The tables of a tile have served once its output is staged; in their place come the halves of its row dot products.  At the end
+            // the last two tiles are left.
+            do {
+                const int sd = done.stage();
+                SF_WAIT(&sm.staged[sd], done.phase(), DEV_TIMEOUT_MMA);
+                if (dot) {
+                    const int tok = t0 + done.c * C + lane, lim = min(p.L, t0 + (done.c + done.len) * C);
+                    float* xo = xout + ((long long)b * p.H + h) * p.L + tok;
+#pragma unroll
+                    for (int e = 0; e < 4; ++e)
+                        if (tok + 32 * e < lim) xo[32 * e] = sm.u[sd][lane + 32 * e] + sm.b[sd][lane + 32 * e];
+                    __syncwarp();
                 }
+                done.next();
+            } while (!it.more() && done.more());
+            if (!it.more()) break;
+        }
+    } else {
+        const int wg = warp >> 2;
+        const long long bh = (long long)b * p.H + h;
+        // tables, first tiles, scores and mask need only the caller's inputs: they run while the scan finishes
+        if (wg >= 2) {
+            const int row = tid & 127, half = wg - 2;
+            for (; it.more(); it.next()) {
+                const int s = it.stage();
+                SF_WAIT(&sm.tab_full[s], it.phase(), DEV_TIMEOUT_MMA);
+                SF_WAIT(&sm.sc_done[s], it.phase(), DEV_TIMEOUT_MMA);
+                ptx::tc_fence_after_sync();
+                mask_tile(tmem + T_SC, sm.b[s], sm.u[s], rev, half);
+                const float a = ptx::ex2(sm.b[s][row]);
+                ptx::tc_fence_before_sync();
+                ptx::mbar_arrive_warp(&sm.p_ready[s]);
+                if (it.i == 0) grid_wait();
+                if (dot) SF_WAIT(&sm.e_full[s], it.phase(), DEV_TIMEOUT_TMA);
+                SF_WAIT(&sm.out_done[s], it.phase(), DEV_TIMEOUT_MMA);       // all of the tile's masks and row weights have been read
+                ptx::tc_fence_after_sync();
+                const float x = epilogue_tile(tmem + T_INTER, tmem + T_INTRA, sm.tiles[s][2], sm.tiles[s][0], a, half, dot, [&] {
+                    ptx::tc_fence_before_sync();
+                    ptx::mbar_arrive_warp(&sm.o_free[s]);
+                });
+                if (dot) (half ? sm.b : sm.u)[s][row] = x;
+                ptx::fence_proxy_async();
+                ptx::mbar_arrive_warp(&sm.staged[s]);
             }
         } else {
+            const float* S0 = p.single ? (s_init ? s_init + bh * (D * D) : nullptr) : states + (bh * p.NB + j) * (long long)(D * D);
             grid_wait();
-            for (int i = 0; i < nch; ++i) {
-                const int c = nch - 1 - i, s = i & 1;
-                const float* bch = sm.bloc + c * C;
-                SF_WAIT(&sm.full[s], (i >> 1) & 1, DEV_TIMEOUT_TMA);
-                // G, its bf16 copy and qw are rewritten below; the state update of the previous chunk is committed
-                // after every MMA that read them
-                if (i > 0) SF_WAIT(&sm.st_done[(i - 1) & 1], ((i - 1) >> 1) & 1, DEV_TIMEOUT_MMA);
+            state_init<4>(tmem + T_ST, S0, dot, 4 * wg);
+            int last_s = 0;
+            uint32_t last_ph = 0;
+            for (; it.more(); it.next()) {
+                const int s = it.stage();
+                SF_WAIT(&sm.tab_full[s], it.phase(), DEV_TIMEOUT_MMA);
+                float* dump = nullptr;                   // merged launches: the state entering a segment's first chunk goes out
+                if (!BWD && it.c == 0 && p.single && p.s_copy) dump = p.s_copy + bh * (D * D);
+                else if (!BWD && p.bslot) {
+                    const int slot = __ldg(p.bslot + c0 + it.c);
+                    if (slot >= 0) dump = p.bbase + slot * p.bstride + bh * (D * D);
+                }
+                if (it.i > 0) SF_WAIT(&sm.st_done[s ^ 1], (uint32_t)((it.i - 1) >> 1) & 1, DEV_TIMEOUT_MMA);
                 ptx::tc_fence_after_sync();
-                state_pass<4>(tmem + T_G, sm.gb, fast_exp(sm.ctot[c]), i == 0, G0, false, 4 * wg);
+                const float total = sm.total[s];
+                if (dump) state_out<4>(tmem + T_ST, dump, 4 * wg);
+                state_pass<4>(tmem + T_ST, sm.sb, ptx::ex2(total), 4 * wg);
                 ptx::fence_proxy_async();
                 ptx::tc_fence_before_sync();
-                ptx::mbar_arrive_warp(&sm.st_ready);
-                scale_box(sm.qw + wg * BOX, sm.tiles[s][0] + wg * BOX, t, [&](int row) { return fast_exp(bch[row]); });
+                ptx::mbar_arrive_warp(&sm.st_ready[s]);
+                SF_WAIT(&sm.full_xy[s], it.phase(), DEV_TIMEOUT_TMA);
+                SF_WAIT(&sm.sc_done[s], it.phase(), DEV_TIMEOUT_MMA);
+                scale_rows(sm.tiles[s][1], tid, [&](int row) { return ptx::ex2(total - sm.b[s][row]); });
                 ptx::fence_proxy_async();
-                ptx::mbar_arrive_warp(&sm.w_ready);
+                ptx::mbar_arrive_warp(&sm.y_ready[s]);
+                last_s = s; last_ph = it.phase();
             }
-            if (p.single) {                              // the gradient of the state entering the segment
-                SF_WAIT(&sm.st_done[(nch - 1) & 1], ((nch - 1) >> 1) & 1, DEV_TIMEOUT_MMA);
+            if ((!BWD || role == SWEEP_DV) && p.single) {       // the state (gradient) leaving the segment
+                SF_WAIT(&sm.st_done[last_s], last_ph, DEV_TIMEOUT_MMA);
                 ptx::tc_fence_after_sync();
-                state_out<4>(tmem + T_G, p.s_final + bh, 4 * wg);
+                state_out<4>(tmem + T_ST, p.s_final + bh * (D * D), 4 * wg);
             }
         }
     }
@@ -988,38 +869,34 @@ __device__ __forceinline__ void dkdv_body(const CUtensorMap* tmQ, const CUtensor
     if (warp == W_MMA) ptx::tmem_dealloc(tmem, 512);
 }
 
+// grid (H, NB, B): heads fastest, so that co-resident CTAs read neighbouring 256-byte pieces of the same tokens
 __global__ void __launch_bounds__(SW_THREADS, 1)
-tc_dkdv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
-               const __grid_constant__ CUtensorMap tmD, SegParams p, const float* __restrict__ g, const float* Gs,
-               const __nv_bfloat16* __restrict__ k_glob, __nv_bfloat16* __restrict__ dk, __nv_bfloat16* __restrict__ dv,
-               float* __restrict__ xk, int* status) {
-    dkdv_body(&tmQ, &tmK, &tmV, &tmD, p, g, Gs, k_glob, dk, dv, xk, status, blockIdx.x, blockIdx.y);
+tc_forward_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
+                  const __grid_constant__ CUtensorMap tmO, SegParams p, const float* __restrict__ g, const float* Hs) {
+    sweep_body<false>(SWEEP_O, {&tmQ, &tmK, &tmV, &tmQ, &tmO}, p, g, Hs, p.s_init, nullptr, blockIdx.x, blockIdx.y);
 }
 
-// Both sweeps of the backward in one launch, for launches that leave at least half of the device idle: they need nothing from
-// each other, so they then take the time of the longer one.  grid (H, 2 NB, B).
-struct PairArgs {
+// The backward's sweeps, any consecutive ones in one launch: grid (heads x sweeps, NB, B).  dk and dv of a block are neighbours:
+// they walk the same tokens at the same pace and read q and dO once from DRAM between them.
+struct BwdMaps { CUtensorMap q, k, v, dO, dq, dk, dv; };
+struct BwdArgs {
     const float *Hs, *Gs;
-    const __nv_bfloat16 *q, *k;
-    __nv_bfloat16 *dq, *dk, *dv;
+    const float *h_init, *g_init;                // one-block segments: the entering state, the gradient of the leaving state
     float *xq, *xk;
-    const float* g_init;                        // one-block segments: the gradient of the leaving state (SegParams::s_init is the entering state)
+    int first, count;                            // sweeps first .. first + count - 1
 };
 __global__ void __launch_bounds__(SW_THREADS, 1)
-tc_backward_pair_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
-                        const __grid_constant__ CUtensorMap tmD, SegParams p, const float* __restrict__ g, PairArgs a, int* status) {
-    const int j = blockIdx.y;
-    if (j < p.NB) {
-        sweep_body<true>(&tmD, &tmV, &tmK, p, g, a.Hs, a.dq, p.tqk, p.bqk, a.q, a.xq, status, blockIdx.x, j);
-    } else {
-        p.s_init = a.g_init;
-        dkdv_body(&tmQ, &tmK, &tmV, &tmD, p, g, a.Gs, a.k, a.dk, a.dv, a.xk, status, blockIdx.x, j - p.NB);
-    }
+tc_backward_kernel(const __grid_constant__ BwdMaps m, SegParams p, const float* __restrict__ g, BwdArgs a) {
+    const int h = blockIdx.x / a.count, role = a.first + blockIdx.x % a.count, j = blockIdx.y;
+    const bool dq = role == SWEEP_DQ, dk = role == SWEEP_DK;
+    const SweepMaps maps{dq ? &m.dO : dk ? &m.v : &m.k, dq ? &m.v : dk ? &m.dO : &m.q, dq ? &m.k : dk ? &m.q : &m.dO, dq ? &m.q : &m.k,
+                         dq ? &m.dq : dk ? &m.dk : &m.dv};
+    sweep_body<true>(role, maps, p, g, dq ? a.Hs : a.Gs, dq ? a.h_init : a.g_init, dq ? a.xq : a.xk, h, j);
 }
 
 // Self-test of the bounded wait: one warp waits on a barrier on which nothing ever arrives, with a short limit given by
 // the caller; the wait gives up, records DEV_TIMEOUT_SELFTEST in the status word and the kernel returns normally.
-__global__ void wait_selftest_kernel(long long limit_cycles, int* status) {
+__global__ void wait_selftest_kernel(long long limit_cycles) {
     __shared__ uint64_t bar;
     __shared__ int abort_flag;
     if (threadIdx.x == 0) {
@@ -1028,31 +905,22 @@ __global__ void wait_selftest_kernel(long long limit_cycles, int* status) {
         ptx::fence_mbar_init();
     }
     __syncthreads();
-    ptx::mbar_wait(&bar, 0, &abort_flag, status, DEV_TIMEOUT_SELFTEST, limit_cycles);
+    ptx::mbar_wait_limit<false>(ptx::smem_u32(&bar), 0, ptx::smem_u32(&abort_flag), DEV_TIMEOUT_SELFTEST, limit_cycles);
 }
 
 // ---- host launch -------------------------------------------------------------------------------------
-// Per-device host state: the address of the status word and whether the kernels' shared-memory attribute has been
-// set there (both belong to a device, not to the process).
+// Per-device host state: whether the kernels' shared-memory attribute has been set there (it belongs to a device, not to the
+// process).
 constexpr int MAX_DEVICES = 64;
-enum { K_AGG = 0, K_FWD, K_DQ, K_DKDV, K_PAIR, K_COUNT };
+enum { K_AGG = 0, K_FWD, K_BWD, K_COUNT };
 struct DeviceState {
-    int* status = nullptr;
     bool attr_done[K_COUNT] = {};
 };
 inline DeviceState* device_state() {
     static DeviceState table[MAX_DEVICES];
-    static std::mutex mu;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= MAX_DEVICES) { cudaGetLastError(); return nullptr; }
-    std::lock_guard<std::mutex> lk(mu);
-    DeviceState* d = &table[dev];
-    if (!d->status) {
-        void* sym = nullptr;
-        if (cudaGetSymbolAddress(&sym, g_dev_status) != cudaSuccess) { cudaGetLastError(); return nullptr; }
-        d->status = static_cast<int*>(sym);
-    }
-    return d;
+    return &table[dev];
 }
 template <typename K>
 inline bool opt_in_smem(DeviceState* d, int which, K kern, size_t bytes) {
@@ -1064,77 +932,52 @@ inline bool opt_in_smem(DeviceState* d, int which, K kern, size_t bytes) {
     return true;
 }
 
+inline bool map_qk(CUtensorMap* m, int rows, const SegParams& p, const void* base) { return make_tmap(m, rows, base, p.B, p.L, p.H, p.tqk, p.bqk); }
+inline bool map_v(CUtensorMap* m, int rows, const SegParams& p, const void* base) { return make_tmap(m, rows, base, p.B, p.L, p.H, p.tv, p.bv); }
+inline sf_status_t launched(bool ok) {
+    if (!ok) cudaGetLastError();
+    return ok ? SF_OK : SF_ERR_CUDA;
+}
+
 inline sf_status_t launch_wait_selftest(long long limit_cycles, cudaStream_t st) {
-    DeviceState* ds = device_state();
-    if (!ds) return SF_ERR_CUDA;
-    wait_selftest_kernel<<<1, 32, 0, st>>>(limit_cycles, ds->status);
+    wait_selftest_kernel<<<1, 32, 0, st>>>(limit_cycles);
     return cudaGetLastError() == cudaSuccess ? SF_OK : SF_ERR_CUDA;
 }
 
-// role: 0 aggregate, 1 forward output pass, 2 dq pass, 3 dk/dv pass (same order as the host's Role enum); early: launch_after()
-inline sf_status_t launch(int role, const sf_seg_desc_t* d, const SegParams& p, const void* q, const void* k, const void* v,
-                          const void* dO, const float* g, int mode, float* U, float* beta, const float* states, void* o,
-                          void* dq, void* dk, void* dv, float* xq, float* xk, bool early, cudaStream_t st, long long* n_launch) {
+// Block aggregates: mode 0 of (k, v), mode 1 of (q, dO); early: launch_after()
+inline sf_status_t launch_aggregate(const SegParams& p, const void* x, const void* y, const float* g, int mode, float* U, float* beta, bool early,
+                                    cudaStream_t st) {
     DeviceState* ds = device_state();
     if (!ds) return SF_ERR_CUDA;
-    int* status = ds->status;
     if (p.R > MAXR) return SF_ERR_UNSUPPORTED;
-    dim3 grid(p.H, p.NB, p.B);
-    bool ok = false;
-    auto map_qk = [&](CUtensorMap* m, const void* base) { return make_tmap(m, base, p.B, p.L, p.H, p.tqk, p.bqk); };
-    auto map_v = [&](CUtensorMap* m, const void* base) { return make_tmap(m, base, p.B, p.L, p.H, p.tv, p.bv); };
-    if (role == 0) {
-        CUtensorMap tmX, tmY;
-        if (!map_qk(&tmX, mode == 0 ? k : q) || !map_v(&tmY, mode == 0 ? v : dO)) return SF_ERR_CUDA;
-        constexpr size_t smem = sizeof(AggSmem) + 1024;
-        if (!opt_in_smem(ds, K_AGG, tc_aggregate_kernel, smem)) return SF_ERR_CUDA;
-        ok = launch_after(early, tc_aggregate_kernel, grid, AGG_THREADS, smem, st, tmX, tmY, p, g, mode, U, beta, status);
-    } else if (role == 1) {
-        CUtensorMap tq, tk, tv;
-        if (!map_qk(&tq, q) || !map_qk(&tk, k) || !map_v(&tv, v)) return SF_ERR_CUDA;
-        constexpr size_t smem = sizeof(SweepSmem) + 1024;
-        if (!opt_in_smem(ds, K_FWD, tc_sweep_kernel<false>, smem)) return SF_ERR_CUDA;
-        ok = launch_after(early, tc_sweep_kernel<false>, grid, SW_THREADS, smem, st, tq, tk, tv, p, g, states, static_cast<__nv_bfloat16*>(o), p.tv, p.bv,
-                          static_cast<const __nv_bfloat16*>(nullptr), static_cast<float*>(nullptr), status);
-    } else if (role == 2) {
-        CUtensorMap tk, tv, td;
-        if (!map_qk(&tk, k) || !map_v(&tv, v) || !map_v(&td, dO)) return SF_ERR_CUDA;
-        constexpr size_t smem = sizeof(SweepSmem) + 1024;
-        if (!opt_in_smem(ds, K_DQ, tc_sweep_kernel<true>, smem)) return SF_ERR_CUDA;
-        // roles: xq = dO, xk = v, xv = k; q is read from global memory for the row dot products
-        ok = launch_after(early, tc_sweep_kernel<true>, grid, SW_THREADS, smem, st, td, tv, tk, p, g, states, static_cast<__nv_bfloat16*>(dq), p.tqk, p.bqk,
-                          static_cast<const __nv_bfloat16*>(q), xq, status);
-    } else if (role == 3) {
-        CUtensorMap tq, tk, tv, td;
-        if (!map_qk(&tq, q) || !map_qk(&tk, k) || !map_v(&tv, v) || !map_v(&td, dO)) return SF_ERR_CUDA;
-        constexpr size_t smem = sizeof(DkdvSmem) + 1024;
-        if (!opt_in_smem(ds, K_DKDV, tc_dkdv_kernel, smem)) return SF_ERR_CUDA;
-        ok = launch_after(early, tc_dkdv_kernel, grid, SW_THREADS, smem, st, tq, tk, tv, td, p, g, states, static_cast<const __nv_bfloat16*>(k),
-                          static_cast<__nv_bfloat16*>(dk), static_cast<__nv_bfloat16*>(dv), xk, status);
-    } else {
-        return SF_ERR_UNSUPPORTED;
-    }
-    *n_launch += 1;
-    if (!ok) cudaGetLastError();
-    return ok ? SF_OK : SF_ERR_CUDA;
+    CUtensorMap tmX, tmY;
+    if (!map_qk(&tmX, C, p, x) || !map_v(&tmY, C, p, y)) return SF_ERR_CUDA;
+    constexpr size_t smem = sizeof(AggSmem) + 1024;
+    if (!opt_in_smem(ds, K_AGG, tc_aggregate_kernel, smem)) return SF_ERR_CUDA;
+    return launched(launch_after(early, tc_aggregate_kernel, dim3(p.H, p.NB, p.B), AGG_THREADS, smem, st, tmX, tmY, p, g, mode, U, beta));
 }
-
-// dq and dk/dv sweeps of a segment in one launch; `a` holds everything but the tensor maps' tensors.
-inline sf_status_t launch_pair(const SegParams& p, const void* q, const void* k, const void* v, const void* dO, const float* g, PairArgs a,
-                               bool early, cudaStream_t st, long long* n_launch) {
+inline sf_status_t launch_forward(const SegParams& p, const void* q, const void* k, const void* v, const float* g, const float* Hs, void* o, bool early,
+                                  cudaStream_t st) {
     DeviceState* ds = device_state();
     if (!ds) return SF_ERR_CUDA;
     if (p.R > MAXR) return SF_ERR_UNSUPPORTED;
-    CUtensorMap tq, tk, tv, td;
-    if (!make_tmap(&tq, q, p.B, p.L, p.H, p.tqk, p.bqk) || !make_tmap(&tk, k, p.B, p.L, p.H, p.tqk, p.bqk) ||
-        !make_tmap(&tv, v, p.B, p.L, p.H, p.tv, p.bv) || !make_tmap(&td, dO, p.B, p.L, p.H, p.tv, p.bv))
+    CUtensorMap tq, tk, tv, to;
+    if (!map_qk(&tq, TT, p, q) || !map_qk(&tk, TT, p, k) || !map_v(&tv, TT, p, v) || !map_v(&to, C, p, o)) return SF_ERR_CUDA;
+    if (!opt_in_smem(ds, K_FWD, tc_forward_kernel, sizeof(SweepSmem))) return SF_ERR_CUDA;
+    return launched(launch_after(early, tc_forward_kernel, dim3(p.H, p.NB, p.B), SW_THREADS, sizeof(SweepSmem), st, tq, tk, tv, to, p, g, Hs));
+}
+// a.first, a.count: which of the backward's sweeps; the output pointers of the others may be NULL
+inline sf_status_t launch_backward(const SegParams& p, const void* q, const void* k, const void* v, const void* dO, const float* g, void* dq, void* dk,
+                                   void* dv, const BwdArgs& a, bool early, cudaStream_t st) {
+    DeviceState* ds = device_state();
+    if (!ds) return SF_ERR_CUDA;
+    if (p.R > MAXR) return SF_ERR_UNSUPPORTED;
+    BwdMaps m;
+    if (!map_qk(&m.q, TT, p, q) || !map_qk(&m.k, TT, p, k) || !map_v(&m.v, TT, p, v) || !map_v(&m.dO, TT, p, dO) || !map_qk(&m.dq, C, p, dq ? dq : dk) ||
+        !map_qk(&m.dk, C, p, dk ? dk : dq) || !map_v(&m.dv, C, p, dv ? dv : dO))
         return SF_ERR_CUDA;
-    constexpr size_t smem = (sizeof(DkdvSmem) > sizeof(SweepSmem) ? sizeof(DkdvSmem) : sizeof(SweepSmem)) + 1024;
-    if (!opt_in_smem(ds, K_PAIR, tc_backward_pair_kernel, smem)) return SF_ERR_CUDA;
-    const bool ok = launch_after(early, tc_backward_pair_kernel, dim3(p.H, 2 * p.NB, p.B), SW_THREADS, smem, st, tq, tk, tv, td, p, g, a, ds->status);
-    *n_launch += 1;
-    if (!ok) cudaGetLastError();
-    return ok ? SF_OK : SF_ERR_CUDA;
+    if (!opt_in_smem(ds, K_BWD, tc_backward_kernel, sizeof(SweepSmem))) return SF_ERR_CUDA;
+    return launched(launch_after(early, tc_backward_kernel, dim3(p.H * a.count, p.NB, p.B), SW_THREADS, sizeof(SweepSmem), st, m, p, g, a));
 }
 
 }  // namespace tc

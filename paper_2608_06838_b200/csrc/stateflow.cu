@@ -341,11 +341,13 @@ sf_status_t launch_role(Path path, Role role, const sf_seg_desc_t* d, const SegP
     StageTimer timer(stage, st);
     early = early && !g_timing_on;                             // a timed kernel is bracketed by events
     if (path == Path::Tc) {
-        long long n = 0;
-        sf_status_t s = sf::tc::launch(static_cast<int>(role), d, p, a.q, a.k, a.v, a.dO, a.g, a.mode, a.U, a.beta, a.states,
-                                       a.o, a.dq, a.dk, a.dv, a.xq, a.xk, early, st, &n);
-        g_launches.fetch_add(n, std::memory_order_relaxed);
-        return s;
+        using namespace sf::tc;
+        g_launches.fetch_add(1, std::memory_order_relaxed);
+        if (role == Role::Aggregate) return launch_aggregate(p, a.mode == 0 ? a.k : a.q, a.mode == 0 ? a.v : a.dO, a.g, a.mode, a.U, a.beta, early, st);
+        if (role == Role::FwdOut) return launch_forward(p, a.q, a.k, a.v, a.g, a.states, a.o, early, st);
+        const bool dq = role == Role::BwdDq;
+        const BwdArgs b{a.states, a.states, p.s_init, p.s_init, a.xq, a.xk, dq ? SWEEP_DQ : SWEEP_DK, dq ? 1 : 2};
+        return launch_backward(p, a.q, a.k, a.v, a.dO, a.g, a.dq, a.dk, a.dv, b, early, st);
     }
     if (d->dtype == SF_F32) return launch_mma3_d(role, d, p, a, st);
     return launch_mma_d(role, d, p, a, st);
@@ -475,18 +477,16 @@ sf_status_t segment_fwd(Path path, const sf_seg_desc_t* d, const SegParams& p, c
     return fwd_out(path, d, p, x, w, st, true);
 }
 
-// dq and dk/dv sweeps, in one launch (tc_backward_pair_kernel) where both fit on the device at once.  `s` carries the one-block
+// dq and dk/dv sweeps, in one launch where both fit on the device at once.  `s` carries the one-block
 // settings for the dq sweep, g_init the gradient of the leaving state.  A timed run keeps the two launches apart.
 // 200 tokens x 16 heads, forward + backward: 76 us with eight launches, 44 with three (one block, this launch, early starts).
 sf_status_t bwd_sweeps(Path path, const sf_seg_desc_t* d, const SegParams& s, const BwdPtrs& x, const BwdWs& w, const float* Hs, const float* g_init,
                        cudaStream_t st) {
     if (path == Path::Tc && !g_timing_on && 2LL * s.B * s.H * s.NB <= sm_count()) {
-        long long n = 0;
-        sf::tc::PairArgs a{Hs, w.GU, static_cast<const __nv_bfloat16*>(x.q), static_cast<const __nv_bfloat16*>(x.k), static_cast<__nv_bfloat16*>(x.dq),
-                           static_cast<__nv_bfloat16*>(x.dk), static_cast<__nv_bfloat16*>(x.dv), w.xq, w.xk, g_init};
-        const sf_status_t r = sf::tc::launch_pair(s, x.q, x.k, x.v, x.dO, x.g, a, true, st, &n);
-        g_launches.fetch_add(n, std::memory_order_relaxed);
-        return r;
+        using namespace sf::tc;
+        g_launches.fetch_add(1, std::memory_order_relaxed);
+        const BwdArgs b{Hs, w.GU, s.s_init, g_init, w.xq, w.xk, SWEEP_DQ, 3};
+        return launch_backward(s, x.q, x.k, x.v, x.dO, x.g, x.dq, x.dk, x.dv, b, true, st);
     }
     SF_TRY(bwd_dq(path, d, s, x, w, Hs, st, true));
     SegParams t = s;
