@@ -278,6 +278,8 @@ __device__ __forceinline__ uint32_t mlo(uint32_t tile, uint32_t box_bytes) { ret
 // ==================================================================================================
 // Block aggregates on tensor cores: U = sum_s w_s x_s^T y_s over the block (M = N = 128, K = tokens).
 //   mode 0: (x, y) = (k, v), w_s = exp(beta - B_s);   mode 1: (x, y) = (q, dO), w_s = exp(B_s)
+// The chunks are visited against the order of the sweep that comes next (mode 0 from the last one on): it begins with what is still in
+// L2 (forward, 8192 tokens x 32 heads 84.5 -> 80.5 us, 16384 147.9 -> 144.8).
 // y is scaled by w in place in shared memory, then U += X^T (w*Y) with both operands MN-major.
 // 8 compute warps, one TMA warp, one MMA warp.
 constexpr int AGG_STAGES = 4;
@@ -305,6 +307,7 @@ tc_aggregate_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_consta
     const long long t0 = (long long)c0 * C;
     int* abort_flag = &sm.abort_flag;
     constexpr int WT = AGG_COMP / 32, WM = WT + 1;
+    auto at = [&](int c) { return mode == 0 ? nch - 1 - c : c; };
 
     if (tid == 0) {
         sm.abort_flag = 0;
@@ -330,8 +333,8 @@ tc_aggregate_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_consta
                 const int s = c % AGG_STAGES, it = c / AGG_STAGES;
                 if (it > 0) SF_WAIT(&sm.empty[s], (it - 1) & 1, DEV_TIMEOUT_MMA);
                 ptx::mbar_expect_tx(&sm.full[s], 2 * TILE);
-                tma_tile(sm.tiles[s][0], &tmX, &sm.full[s], h, (int)t0 + c * C, b);
-                tma_tile(sm.tiles[s][1], &tmY, &sm.full[s], h, (int)t0 + c * C, b);
+                tma_tile(sm.tiles[s][0], &tmX, &sm.full[s], h, (int)t0 + at(c) * C, b);
+                tma_tile(sm.tiles[s][1], &tmY, &sm.full[s], h, (int)t0 + at(c) * C, b);
             }
         }
     } else if (warp == WM) {
@@ -361,8 +364,9 @@ tc_aggregate_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_consta
         for (int c = 0; c < nch; ++c) {
             const int s = c % AGG_STAGES, it = c / AGG_STAGES;
             SF_WAIT(&sm.full[s], it & 1, DEV_TIMEOUT_TMA);
-            const float cof = sm.cofs[c], bC = sm.ctot[c];
-            const float* bch = sm.bloc + c * C;
+            const int cc = at(c);
+            const float cof = sm.cofs[cc], bC = sm.ctot[cc];
+            const float* bch = sm.bloc + cc * C;
             scale_tile<AGG_COMP>(sm.tiles[s][1], sm.tiles[s][1], tid,
                        [&](int row) { return fast_exp(mode == 0 ? (bC - bch[row]) + cof : bch[row] + cof); });
             ptx::fence_proxy_async();

@@ -108,7 +108,7 @@ int sm_count() {
 // kernel takes waves * (chunks per block + a fixed per-CTA cost of about six chunk times); more than one block adds the
 // aggregate and the scan, about two chunk times where their launches overlap (a segment of one block needs neither, see
 // one_block(); 16 heads x 500 tokens, forward: one block 24.5 us, two 20.7); so does
-// a launch too large for the backward's two sweeps to share the device (bwd_sweeps(); 64 heads x 500 tokens, forward + backward
+// a launch too large for two of the backward's sweeps to share the device (64 heads x 500 tokens, forward + backward
 // with replay: one block 84 us, two 96).  Pick the
 // length in [4, longest] that minimises this; ties go to the longer block (fewer block states in HBM).
 int auto_chunks_per_block(int NC, long long bh, int longest = 64) {
@@ -477,12 +477,12 @@ sf_status_t segment_fwd(Path path, const sf_seg_desc_t* d, const SegParams& p, c
     return fwd_out(path, d, p, x, w, st, true);
 }
 
-// dq and dk/dv sweeps, in one launch where both fit on the device at once.  `s` carries the one-block
-// settings for the dq sweep, g_init the gradient of the leaving state.  A timed run keeps the two launches apart.
-// 200 tokens x 16 heads, forward + backward: 76 us with eight launches, 44 with three (one block, this launch, early starts).
+// dq, dk and dv sweeps of a segment call.  On the tensor-core path they are one launch (a timed run keeps dq and dk/dv apart): the three of a
+// block run side by side and read its tokens while the others do, and there is one tail instead of two.  `s` carries the
+// one-block settings for the dq sweep, g_init the gradient of the leaving state.  Forward + backward of 8192 tokens x 32 heads 299 -> 288 us, 16384 545 -> 530.
 sf_status_t bwd_sweeps(Path path, const sf_seg_desc_t* d, const SegParams& s, const BwdPtrs& x, const BwdWs& w, const float* Hs, const float* g_init,
                        cudaStream_t st) {
-    if (path == Path::Tc && !g_timing_on && 2LL * s.B * s.H * s.NB <= sm_count()) {
+    if (path == Path::Tc && !g_timing_on) {
         using namespace sf::tc;
         g_launches.fetch_add(1, std::memory_order_relaxed);
         const BwdArgs b{Hs, w.GU, s.s_init, g_init, w.xq, w.xk, SWEEP_DQ, 3};
