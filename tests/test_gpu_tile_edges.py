@@ -183,3 +183,56 @@ def test_convolution_weight_gradient_with_infinite_last_inputs(C):
     assert torch.isnan(got[:2, 5]).all() and torch.isfinite(got[2:, 5]).all()
     rest = [c for c in range(C) if c not in (3, 5)]
     assert torch.equal(got[:, rest], ref[:, rest])
+
+
+@pytest.mark.parametrize("segs,cpb", [
+    ([64, 192, 64, 320], 0), ([64, 192, 64, 320], 3), ([64] * 7, 64), ([320, 64, 100], 5),        # segments that begin inside a tile, odd blocks
+    ([1], 0), ([65], 0), ([127], 0), ([128], 0), ([129], 1), ([191], 1), ([193], 2), ([449], 7),      # ragged ends of one- and two-chunk tiles
+])
+@pytest.mark.parametrize("merged", [0, 1])
+def test_tensor_core_tiles_of_one_and_two_chunks(segs, cpb, merged):
+    w = Workload("tc-tiles", 2, 3, 128, 128, segs, 64, g_scale=0.1, s_in_sigma=0.1, ds_out_sigma=0.1, seed=sum(segs))
+    x = inputs.make_inputs(w, DEV)
+    binding.sf_set_tuning(dict(merge_launches=merged))
+    try:
+        got, run = run_chain(w, x, chunks_per_block=cpb)
+        S = run.S_bounds.clone()
+    finally:
+        binding.sf_set_tuning(None)
+    compare(got, oracle_reference(x), tolerance(w), label="tc-tiles")
+    tok = 0
+    for i, n in enumerate(segs[:-1]):                       # the state entering each later segment
+        tok += n
+        part = {m: (t[:, :tok] if t is not None and t.dim() >= 3 and t.shape[1] == w.T else t) for m, t in x.items()}
+        ref = oracle_reference(part)["S_out"]
+        assert np.abs(inputs.to_f64(S[i + 1]) - ref).max() <= tolerance(w) * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("value", [float("inf"), float("nan")])
+def test_tensor_core_tiles_keep_values_that_are_not_finite_to_their_sixteen_tokens(value):
+    # what the masked products multiply by 0 reaches no row outside the value's own step of 16 tokens (96 .. 111)
+    w = Workload("tc-inf", 1, 2, 128, 128, [384], 64, g_scale=0.1, seed=3)
+    x = inputs.make_inputs(w, DEV)
+    x["v"][0, 100, 0, 5] = value
+    x["dO"][0, 100, 1, 7] = value
+    got, _ = run_chain(w, x)
+    assert torch.isfinite(got["o"][0, :96, 0].float()).all() and not torch.isfinite(got["o"][0, 100:, 0, 5].float()).any()
+    assert torch.isfinite(got["o"][0, :, 1].float()).all()
+    for n in ("dk", "dv"):
+        assert torch.isfinite(got[n][0, 112:, 1].float()).all(), n
+    assert not torch.isfinite(got["dv"][0, :101, 1, 7].float()).any()
+
+
+@pytest.mark.parametrize("mask", [-200.0, -1e4, -1e30])
+def test_tensor_core_tiles_with_log_decays_that_mask(mask):
+    w = Workload("tc-mask", 1, 2, 128, 128, [200], 64, g_scale=0.1, s_in_sigma=0.1, seed=4)
+    x = inputs.make_inputs(w, DEV)
+    x["g"][0, [30, 31, 90, 150]] = mask
+    d = binding.make_desc(x["q"], x["v"], x["g"], 64)
+    o, S = torch.empty_like(x["v"]), torch.empty(1, 2, 128, 128, device=DEV)
+    ws = torch.empty(max(binding.sf_workspace_bytes(d, 0), 256), dtype=torch.uint8, device=DEV)
+    binding.sf_segment_fwd(d, x["q"], x["k"], x["v"], x["g"], x["S_in"], o, S, ws)
+    torch.cuda.synchronize()
+    ref = oracle_reference(x)
+    for got, n in ((o, "o"), (S, "S_out")):
+        assert np.abs(inputs.to_f64(got) - ref[n]).max() <= tolerance(w) * np.abs(ref[n]).max(), n
