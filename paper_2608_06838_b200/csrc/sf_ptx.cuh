@@ -185,6 +185,15 @@ __device__ __forceinline__ void mul2(float& a, float& b, float f, float g) {
         "mul.rn.f32x2 x, x, y;\n\t"
         "mov.b64 {%0, %1}, x;\n\t}" : "+f"(a), "+f"(b) : "f"(f), "f"(g));
 }
+// two multiply-adds d += f g in one instruction
+__device__ __forceinline__ void fma2(float& d0, float& d1, float f0, float f1, float g0, float g1) {
+    asm("{\n\t.reg .b64 x, y, z;\n\t"
+        "mov.b64 x, {%0, %1};\n\t"
+        "mov.b64 y, {%2, %3};\n\t"
+        "mov.b64 z, {%4, %5};\n\t"
+        "fma.rn.f32x2 x, y, z, x;\n\t"
+        "mov.b64 {%0, %1}, x;\n\t}" : "+f"(d0), "+f"(d1) : "f"(f0), "f"(f1), "f"(g0), "f"(g1));
+}
 // 2^x with the single-instruction approximation (inputs here are <= 0 or moderate; flush-to-zero underflow is the wanted limit)
 __device__ __forceinline__ float ex2(float x) {
     float y;

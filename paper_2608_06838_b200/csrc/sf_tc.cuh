@@ -559,7 +559,7 @@ __device__ __forceinline__ float epilogue_tile(uint32_t inter, uint32_t intra, u
     const int q = (threadIdx.x >> 5) & 3, row = 32 * q + (threadIdx.x & 31);
     const uint32_t from = ((uint32_t)(q * 32) << 16) + 64 * half;
     unsigned char* box = slot + half * FBOX;
-    float dot = 0.f;
+    float dot0 = 0.f, dot1 = 0.f;                        // even and odd features
 #pragma unroll 1
     for (int cb = 0; cb < 2; ++cb) {
         float x[32], y[32];
@@ -568,7 +568,7 @@ __device__ __forceinline__ float epilogue_tile(uint32_t inter, uint32_t intra, u
         ptx::tmem_ld_wait();
         if (cb == 1) loaded();
 #pragma unroll
-        for (int i = 0; i < 32; ++i) y[i] = fmaf(a, x[i], y[i]);
+        for (int i = 0; i < 32; i += 2) ptx::fma2(y[i], y[i + 1], x[i], x[i + 1], a, a);
         if (with_dot) {
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
@@ -577,8 +577,7 @@ __device__ __forceinline__ float epilogue_tile(uint32_t inter, uint32_t intra, u
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&w[i]));
-                    dot = fmaf(y[8 * e + 2 * i], f.x, dot);
-                    dot = fmaf(y[8 * e + 2 * i + 1], f.y, dot);
+                    ptx::fma2(dot0, dot1, y[8 * e + 2 * i], y[8 * e + 2 * i + 1], f.x, f.y);
                 }
             }
         }
@@ -587,7 +586,7 @@ __device__ __forceinline__ float epilogue_tile(uint32_t inter, uint32_t intra, u
             st_unit(box, row, cb * 4 + e, make_uint4(pack2(y[8 * e], y[8 * e + 1]), pack2(y[8 * e + 2], y[8 * e + 3]),
                                                      pack2(y[8 * e + 4], y[8 * e + 5]), pack2(y[8 * e + 6], y[8 * e + 7])));
     }
-    return dot;
+    return dot0 + dot1;
 }
 
 // P z over K steps of 16 tokens: FROM .. TO - 1 of the eight, counted from the last one in the reverse sweeps, each for the lanes that have a
