@@ -110,7 +110,8 @@ int sm_count() {
 // one_block(); 16 heads x 500 tokens, forward: one block 24.5 us, two 20.7); so does
 // a launch too large for two of the backward's sweeps to share the device (64 heads x 500 tokens, forward + backward
 // with replay: one block 84 us, two 96).  Pick the
-// length in [4, longest] that minimises this; ties go to the longer block (fewer block states in HBM).
+// length in [4, longest] that minimises this; ties go to the longer block (fewer block states in HBM).  An odd block costs as
+// much as the next even one: the sweeps walk two chunks at a time (8 heads x 16384, forward + backward: blocks of 15 174.5 us, of 16 170.4).
 int auto_chunks_per_block(int NC, long long bh, int longest = 64) {
     const int sms = sm_count();
     int best = kDefaultChunksPerBlock;
@@ -119,7 +120,7 @@ int auto_chunks_per_block(int NC, long long bh, int longest = 64) {
         const int reff = r < NC ? r : NC;
         const long long nb = (NC + reff - 1) / reff;
         const long long waves = (nb * bh + sms - 1) / sms;
-        const long long cost = waves * (reff + 6) + (nb > 1 ? 2 : 0) + (nb > 1 && 2 * nb * bh > sms ? 2 : 0);
+        const long long cost = waves * (reff + (reff & 1) + 6) + (nb > 1 ? 2 : 0) + (nb > 1 && 2 * nb * bh > sms ? 2 : 0);
         if (best_cost < 0 || cost <= best_cost) { best_cost = cost; best = reff; }
         if (r >= NC) break;
     }
