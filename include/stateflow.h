@@ -32,7 +32,8 @@
  *    but an Inf may come out as NaN (the tensor cores take float32 operands as several
  *    terms).  Tokens that do not depend on it keep their values in the warp-level kernels.
  *    Log-decays below -1e4, -inf included, count as -1e4 in the kernels of float32 precision
- *    (warp-level, chunkwise delta rule): the state is wiped all the same.
+ *    (warp-level, chunkwise delta rule), those below -128 as -128 in the bf16 kernels of
+ *    128-wide heads: the state is wiped all the same.
  *  - Validation happens on the host before anything is launched.  A call that
  *    returns an error has enqueued nothing.  The library never throws, aborts,
  *    prints or traps the device.

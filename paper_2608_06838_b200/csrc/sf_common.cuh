@@ -68,6 +68,9 @@ enum : int { DEV_OK = 0, DEV_TIMEOUT_TMA = 1, DEV_TIMEOUT_MMA = 2, DEV_TIMEOUT_S
 // it, sums over a tile stay exact to 1e-10 in double precision also beside a mask value (-inf, the lowest float): differences of
 // the sums, taken for tokens behind it, are right.  NaN stays NaN.
 __device__ __forceinline__ double log_decay(float g) { return g < -1e4f ? -1e4 : (double)g; }
+// The same for the float32 tables of the tensor-core kernels (bf16): below -128 a decay wipes the state in float32 all the same, and 64
+// limited ones in a chunk leave the differences of its sums an error of 5e-4, an eighth of a bf16 rounding.
+__device__ __forceinline__ float log_decay_bf16(float g) { return g < -128.f ? -128.f : g; }
 
 __device__ __forceinline__ float to_f32(float x) { return x; }
 __device__ __forceinline__ float to_f32(__nv_bfloat16 x) { return __bfloat162float(x); }

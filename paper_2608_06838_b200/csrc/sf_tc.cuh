@@ -114,7 +114,8 @@ __device__ __forceinline__ void tma_tile(void* dst, const CUtensorMap* m, uint64
 // synchronise afterwards.
 //   bloc[t]  = inclusive cumulative log-decay of token t inside ITS chunk  (t = 0 .. nch*64-1)
 //   ctot[c]  = chunk totals
-// Tokens at or beyond `L` (a last chunk that is not full) get log-decay 0; TMA fills their tile rows with zeros.
+// of the log-decays as log_decay_bf16() limits them.  Tokens at or beyond `L` (a last chunk that is not full) get log-decay 0; TMA fills
+// their tile rows with zeros.
 // `issued`, if given, is an mbarrier (count = nwarps) on which every warp arrives once its loads are on their way: the
 // TMA warp waits for it, so that these small requests do not queue behind the first burst of tile loads that all CTAs
 // of the device send at the same moment.
@@ -132,14 +133,17 @@ __device__ __forceinline__ void prep_decay(const float* __restrict__ gh, long lo
             const int c = cbase + i * nwarps;
             const int r = c * C + 2 * lane;
             const bool on = c < nch;
-            g0[i] = on ? gh[(t0 + min(r, lim - 1)) * tg] * (r < lim ? 1.f : 0.f) : 0.f;
-            g1[i] = on ? gh[(t0 + min(r + 1, lim - 1)) * tg] * (r + 1 < lim ? 1.f : 0.f) : 0.f;
+            g0[i] = on ? gh[(t0 + min(r, lim - 1)) * tg] : 0.f;
+            g1[i] = on ? gh[(t0 + min(r + 1, lim - 1)) * tg] : 0.f;
         }
         if (issued && cbase == warp) { ptx::mbar_arrive_warp(issued); issued = nullptr; }
 #pragma unroll
         for (int i = 0; i < MAXC; ++i) {
             const int c = cbase + i * nwarps;
             if (c < nch) {
+                const int r = c * C + 2 * lane;             // selected, not multiplied by 0: the last token's value may be NaN
+                g0[i] = r < lim ? log_decay_bf16(g0[i]) : 0.f;
+                g1[i] = r + 1 < lim ? log_decay_bf16(g1[i]) : 0.f;
                 float incl = g0[i] + g1[i];
                 for (int off = 1; off < 32; off <<= 1) {
                     const float up = __shfl_up_sync(0xffffffffu, incl, off);
@@ -760,9 +764,8 @@ __device__ __forceinline__ void sweep_body(int role, const SweepMaps& m, const S
         Tiles done = it;
         while (true) {
             const int s = it.stage();
-            // Below -128 a decay wipes the state in float32 all the same, and limited to it the sums beside a mask value keep their precision.
 #pragma unroll
-            for (int e = 0; e < 4; ++e) gv[e] = (gv[e] < -128.f ? -128.f : gv[e]) * LOG2E;
+            for (int e = 0; e < 4; ++e) gv[e] = log_decay_bf16(gv[e]) * LOG2E;
             gv[1] += gv[0]; gv[2] += gv[1]; gv[3] += gv[2];
             float pre = gv[3];
 #pragma unroll

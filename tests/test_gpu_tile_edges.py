@@ -236,3 +236,25 @@ def test_tensor_core_tiles_with_log_decays_that_mask(mask):
     ref = oracle_reference(x)
     for got, n in ((o, "o"), (S, "S_out")):
         assert np.abs(inputs.to_f64(got) - ref[n]).max() <= tolerance(w) * np.abs(ref[n]).max(), n
+
+
+@pytest.mark.parametrize("cpb", [0, 1, 2, 3])
+@pytest.mark.parametrize("merged,save_states", [(0, True), (0, False), (1, True)])
+def test_tensor_core_blocks_with_log_decays_that_mask(cpb, merged, save_states):
+    # several blocks: their aggregates weigh the tokens too.  Masks on the first and the last token of a chunk, of a segment and of the
+    # ragged end, on odd and even tokens, on neighbours.
+    masks = MASKS + [-200.0]
+    w = Workload("tc-mask-blocks", 1, len(masks), 128, 128, [448, 321], 64, g_scale=0.1, s_in_sigma=0.3, ds_out_sigma=0.3, seed=70)
+    x = inputs.make_inputs(w, DEV)
+    for h, m in enumerate(masks):
+        for t in (0, 21, 22, 64, 127, 140 + h, 447, 500, 575, 700, 768):
+            x["g"][0, t, h] = m
+    binding.sf_set_tuning(dict(merge_launches=merged))
+    try:
+        got, run = run_chain(w, x, chunks_per_block=cpb, save_states=save_states)
+        S = inputs.to_f64(run.S_bounds[1])
+    finally:
+        binding.sf_set_tuning(None)
+    compare(got, oracle_reference(x), tolerance(w), label=w.name)
+    ref = oracle_reference({n: (t[:, :448] if n in ("q", "k", "v", "g", "dO") else t) for n, t in x.items()})["S_out"]
+    assert np.abs(S - ref).max() <= tolerance(w) * np.abs(ref).max()
