@@ -171,3 +171,50 @@ def test_two_host_threads_on_two_streams_give_the_bits_of_the_serial_run():
         for n in NAMES:
             assert torch.equal(out[i][n], serial[i][n]), (i, n)
     assert binding.sf_device_status() == 0
+
+
+FIRST_CALLS = """
+import sys, threading
+import torch
+sys.path.insert(0, sys.argv[1])
+from paper_2608_06838_b200 import binding, inputs
+from paper_2608_06838_b200.inputs import Workload
+
+N = 16
+w = Workload("first", 1, 2, 128, 128, [200], 64, seed=23)
+x = inputs.make_inputs(w, "cuda:0")
+d = binding.make_desc(x["q"], x["v"], x["g"], 64)
+mine = [(torch.empty_like(x["v"]), torch.empty(1, 2, 128, 128, device="cuda:0"), torch.empty(binding.sf_workspace_bytes(d, 0), dtype=torch.uint8, device="cuda:0"),
+         torch.cuda.Stream()) for _ in range(N)]
+torch.cuda.synchronize()
+gate, errors = threading.Barrier(N), []
+
+def work(i):
+    o, S, ws, st = mine[i]
+    with torch.cuda.stream(st):
+        torch.cuda.synchronize()
+        gate.wait()
+        try:
+            binding.sf_segment_fwd(d, x["q"], x["k"], x["v"], x["g"], None, o, S, ws)
+        except Exception as e:
+            errors.append(repr(e))
+
+threads = [threading.Thread(target=work, args=(i,)) for i in range(N)]
+for t in threads:
+    t.start()
+for t in threads:
+    t.join()
+torch.cuda.synchronize()
+assert not errors, errors
+assert all(torch.equal(m[0], mine[0][0]) for m in mine)
+"""
+
+
+def test_first_calls_of_many_host_threads():
+    # in a process of its own: nothing that the library looks up once has been looked up yet
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    for _ in range(3):
+        subprocess.run([sys.executable, "-c", FIRST_CALLS, root], check=True, timeout=300)
