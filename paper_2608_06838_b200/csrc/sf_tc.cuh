@@ -10,10 +10,12 @@
 // over tokens (ptx::desc_lo).
 #pragma once
 #include <cuda.h>
-#include <mutex>
+#include <memory>
+#include <new>
 
 #include "../../include/stateflow.h"
 #include "sf_common.cuh"
+#include "sf_map_cache.h"
 #include "sf_ptx.cuh"
 
 namespace sf {
@@ -59,23 +61,27 @@ inline EncodeTiledFn encode_fn() {
 }
 
 // Map of a [B, L, H, 128] bf16 view: dims (feature, head, token, batch), box = 64 features x 1 x `rows` tokens x 1.
-// A map is a pure function of (base, B, L, H, strides) and encoding one never reads device memory, so each host
-// thread keeps the last TMAP_CACHE maps it encoded: a chain that is launched again from the host (no graph) with the
-// same buffers re-encodes nothing.
-constexpr int TMAP_CACHE = 64;
+// A map is a pure function of (base, rows, B, L, H, strides) and encoding one never reads device memory, so each host
+// thread keeps the maps it encoded (up to MapCache::MAX_USED): a chain that is launched again from the host (no graph) with the
+// same buffers re-encodes nothing.  A segment's forward and backward take 12 (k, v, q, dO in boxes of 64 tokens for the aggregates and of 128
+// for the sweeps, o, dq, dk, dv in boxes of 64), so chains of up to 32 separately launched segments fit.
 struct TmapKey {
     const void* base; int rows, B, L, H; long long tok_stride, batch_stride;
     bool operator==(const TmapKey& o) const {
         return base == o.base && rows == o.rows && B == o.B && L == o.L && H == o.H && tok_stride == o.tok_stride && batch_stride == o.batch_stride;
     }
+    uint64_t hash() const {
+        uint64_t h = reinterpret_cast<uintptr_t>(base) >> 4;
+        for (uint64_t x : {(uint64_t)rows, (uint64_t)B, (uint64_t)L, (uint64_t)H, (uint64_t)tok_stride, (uint64_t)batch_stride}) h = h * 0x100000001B3ull + x;
+        return h;
+    }
 };
-struct TmapCache { TmapKey key[TMAP_CACHE]; CUtensorMap map[TMAP_CACHE]; int used = 0, next = 0; };
+using TmapCache = MapCache<TmapKey, CUtensorMap, 512>;
 
 inline bool make_tmap(CUtensorMap* m, int rows, const void* base, int B, int L, int H, long long tok_stride, long long batch_stride) {
-    thread_local TmapCache cache;
+    thread_local std::unique_ptr<TmapCache> cache(new (std::nothrow) TmapCache);
     const TmapKey key{base, rows, B, L, H, tok_stride, batch_stride};
-    for (int i = 0; i < cache.used; ++i)
-        if (cache.key[i] == key) { *m = cache.map[i]; return true; }
+    if (const CUtensorMap* kept = cache ? cache->find(key) : nullptr) { *m = *kept; return true; }
     EncodeTiledFn fn = encode_fn();
     if (!fn) return false;
     cuuint64_t dims[4] = {(cuuint64_t)D, (cuuint64_t)H, (cuuint64_t)L, (cuuint64_t)B};
@@ -94,11 +100,7 @@ inline bool make_tmap(CUtensorMap* m, int rows, const void* base, int B, int L, 
         cudaGetLastError();
         return false;
     }
-    const int slot = cache.next;
-    cache.key[slot] = key;
-    cache.map[slot] = *m;
-    cache.next = (slot + 1) % TMAP_CACHE;
-    if (cache.used < TMAP_CACHE) ++cache.used;
+    if (cache) cache->insert(key, *m);
     return true;
 }
 
@@ -978,15 +980,16 @@ inline sf_status_t launch_forward(const SegParams& p, const void* q, const void*
     if (!opt_in_smem(ds, K_FWD, tc_forward_kernel, sizeof(SweepSmem))) return SF_ERR_CUDA;
     return launched(launch_after(early, tc_forward_kernel, dim3(p.H, p.NB, p.B), SW_THREADS, sizeof(SweepSmem), st, tq, tk, tv, to, p, g, Hs));
 }
-// a.first, a.count: which of the backward's sweeps; the output pointers of the others may be NULL
+// a.first, a.count: which of the backward's sweeps; the output pointers of the others may be NULL, their maps are left blank
 inline sf_status_t launch_backward(const SegParams& p, const void* q, const void* k, const void* v, const void* dO, const float* g, void* dq, void* dk,
                                    void* dv, const BwdArgs& a, bool early, cudaStream_t st) {
     DeviceState* ds = device_state();
     if (!ds) return SF_ERR_CUDA;
     if (p.R > MAXR) return SF_ERR_UNSUPPORTED;
-    BwdMaps m;
-    if (!map_qk(&m.q, TT, p, q) || !map_qk(&m.k, TT, p, k) || !map_v(&m.v, TT, p, v) || !map_v(&m.dO, TT, p, dO) || !map_qk(&m.dq, C, p, dq ? dq : dk) ||
-        !map_qk(&m.dk, C, p, dk ? dk : dq) || !map_v(&m.dv, C, p, dv ? dv : dO))
+    auto runs = [&](int sweep) { return sweep >= a.first && sweep < a.first + a.count; };
+    BwdMaps m{};
+    if (!map_qk(&m.q, TT, p, q) || !map_qk(&m.k, TT, p, k) || !map_v(&m.v, TT, p, v) || !map_v(&m.dO, TT, p, dO) ||
+        (runs(SWEEP_DQ) && !map_qk(&m.dq, C, p, dq)) || (runs(SWEEP_DK) && !map_qk(&m.dk, C, p, dk)) || (runs(SWEEP_DV) && !map_v(&m.dv, C, p, dv)))
         return SF_ERR_CUDA;
     if (!opt_in_smem(ds, K_BWD, tc_backward_kernel, sizeof(SweepSmem))) return SF_ERR_CUDA;
     return launched(launch_after(early, tc_backward_kernel, dim3(p.H * a.count, p.NB, p.B), SW_THREADS, sizeof(SweepSmem), st, m, p, g, a));

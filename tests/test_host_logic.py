@@ -297,3 +297,53 @@ def test_host_wrapper_scratch_size_and_validation(lib):
     strided.tok_stride_qk = 2 * 2 * 128                            # the wrapper wants densely packed host tensors
     assert lib.sf_chain_fwd_bwd_host(ctypes.byref(strided), segs, 3, P, P, P, P, None, P, None, P, None, P, P, P, P, P,
                                      ctypes.c_void_p(0x40000), 1 << 40, None) == 1
+
+
+MAP_CACHE = r"""
+#include <initializer_list>
+#include "sf_map_cache.h"
+struct K { uintptr_t base; int rows; bool operator==(const K& o) const { return base == o.base && rows == o.rows; } uint64_t hash() const { return base * 31 + rows; } };
+struct V { uintptr_t base; int rows; char pad[100]; };
+using Cache = sf::MapCache<K, V, 512>;
+// keys as the launches of a chain ask for them: 12 per segment, forward then backward in reverse, `rounds` times; returns the lookups that found nothing
+static long run(Cache& c, int n_seg, uintptr_t stride, int rounds) {
+    long missed = 0;
+    for (int r = 0; r < rounds; ++r)
+        for (int pass = 0; pass < 2; ++pass)
+            for (int s = 0; s < n_seg; ++s)
+                for (int t = 0; t < (pass ? 11 : 6); ++t) {
+                    // forward: k, v at 64 rows, q, k, v at 128, o; backward: q, dO at 64, q, k, v, dO at 128, dq, dk, dv and k, v again
+                    static const int f[6][2] = {{1, 64}, {2, 64}, {0, 128}, {1, 128}, {2, 128}, {4, 64}};
+                    static const int b[11][2] = {{0, 64}, {3, 64}, {0, 128}, {1, 128}, {2, 128}, {3, 128}, {5, 64}, {6, 64}, {7, 64}, {1, 64}, {2, 64}};
+                    const int* x = pass ? b[t] : f[t];
+                    const K k{0x7f0000000000u + x[0] * stride * 64 + (pass ? n_seg - 1 - s : s) * stride, x[1]};
+                    const V* v = c.find(k);
+                    if (v) { if (v->base != k.base || v->rows != k.rows) return -1; }
+                    else { ++missed; V n{}; n.base = k.base; n.rows = k.rows; c.insert(k, n); }
+                }
+    return missed;
+}
+int main() {
+    for (uintptr_t stride : {(uintptr_t)256, (uintptr_t)4096, (uintptr_t)(134217728), (uintptr_t)(3 * 65536 + 1024)}) {
+        for (int n_seg : {1, 5, 6, 16, 32}) {
+            Cache* c = new Cache;
+            const long first = run(*c, n_seg, stride, 1), again = run(*c, n_seg, stride, 3);
+            if (first != 12L * n_seg || again != 0) return 1;
+            delete c;
+        }
+        Cache* c = new Cache;                            // more keys than it holds: still the right values
+        if (run(*c, 64, stride, 5) < 64) return 2;
+        delete c;
+    }
+    return 0;
+}
+"""
+
+
+def test_tensor_map_cache_holds_the_maps_of_a_chain(tmp_path):
+    import subprocess
+    src, exe = tmp_path / "cache.cpp", tmp_path / "cache"
+    src.write_text(MAP_CACHE)
+    csrc = os.path.join(ROOT, "paper_2608_06838_b200", "csrc")
+    subprocess.run(["g++", "-std=c++17", "-O1", "-fsanitize=address,undefined", "-I", csrc, "-o", str(exe), str(src)], check=True)
+    assert subprocess.run([str(exe)]).returncode == 0
