@@ -104,15 +104,16 @@ int sm_count() {
     return table[dev];
 }
 
-// Block length when the caller leaves it open: one CTA per (batch, head, block) and one CTA per SM, so a
-// kernel takes waves * (chunks per block + a fixed per-CTA cost of about six chunk times); more than one block adds the
-// aggregate and the scan, about two chunk times where their launches overlap (a segment of one block needs neither, see
-// one_block(); 16 heads x 500 tokens, forward: one block 24.5 us, two 20.7); so does
-// a launch too large for two of the backward's sweeps to share the device (64 heads x 500 tokens, forward + backward
-// with replay: one block 84 us, two 96).  Pick the
-// length in [4, longest] that minimises this; ties go to the longer block (fewer block states in HBM).  An odd block costs as
-// much as the next even one: the sweeps walk two chunks at a time (8 heads x 16384, forward + backward: blocks of 15 174.5 us, of 16 170.4).
-int auto_chunks_per_block(int NC, long long bh, int longest = 64) {
+// Block length when the caller leaves it open: one CTA per (batch, head, block) and one CTA per SM, so the forward sweep takes waves *
+// (chunks per block + a fixed per-CTA cost of about six chunk times); more than one block adds the aggregate and the scan, about two chunk
+// times where their launches overlap.  The backward has three CTAs per block and head.  Its time follows their waves less than that; two
+// chunk times more from half the device's SMs on keep blocks from getting too short for it (16 heads x 1152 tokens, backward: blocks of 4
+// chunks 38.4 us, of 6 32.9).  Pick the length in [4, longest] that minimises this; ties go to the longer block (fewer block states in HBM).
+// The sweeps walk two chunks at a time, so an odd block costs as much as the next even one (8 heads x 16384, forward + backward: blocks of 15
+// 174.5 us, of 16 170.4).  But where a launch has several waves, what counts is the bytes, and shorter blocks only add states and starts: so the length
+// is the longer of those with and without that rounding.  160 heads, forward + backward: 1472 tokens with it alone 349 us
+// (12 chunks), so 272 (23); 1856 tokens 436 (10) and 393 (15); 80 heads x 5120 519 (16) and 495 (27).
+int cheapest_block(int NC, long long bh, int longest, bool round_odd) {
     const int sms = sm_count();
     int best = kDefaultChunksPerBlock;
     long long best_cost = -1;
@@ -120,11 +121,14 @@ int auto_chunks_per_block(int NC, long long bh, int longest = 64) {
         const int reff = r < NC ? r : NC;
         const long long nb = (NC + reff - 1) / reff;
         const long long waves = (nb * bh + sms - 1) / sms;
-        const long long cost = waves * (reff + (reff & 1) + 6) + (nb > 1 ? 2 : 0) + (nb > 1 && 2 * nb * bh > sms ? 2 : 0);
+        const long long cost = waves * (reff + (round_odd ? reff & 1 : 0) + 6) + (nb > 1 ? 2 : 0) + (nb > 1 && 2 * nb * bh > sms ? 2 : 0);
         if (best_cost < 0 || cost <= best_cost) { best_cost = cost; best = reff; }
         if (r >= NC) break;
     }
     return best;
+}
+int auto_chunks_per_block(int NC, long long bh, int longest = 64) {
+    return std::max(cheapest_block(NC, bh, longest, false), cheapest_block(NC, bh, longest, true));
 }
 
 // The same choice for a segment that runs inside a chain of several.  There the sweeps of neighbouring segments

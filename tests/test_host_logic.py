@@ -106,6 +106,16 @@ def test_workspace_arithmetic(lib):
     assert binding.sf_chain_workspace_bytes(d, [0], 0) == 0 and binding.sf_chain_workspace_bytes(d, [100], 0) > 0
 
 
+@pytest.mark.parametrize("H,chunks,length", [
+    (8, 256, 16), (16, 18, 6), (32, 18, 6), (64, 10, 10),                     # an odd block counts as the next even one ...
+    (160, 23, 23), (160, 29, 15), (160, 46, 23), (160, 62, 21), (80, 80, 27), (80, 98, 33), (80, 116, 39),   # ... but leads to no shorter blocks
+    (32, 256, 64), (16, 64, 8), (1, 1, 1),
+])
+def test_block_lengths_that_the_library_chooses(lib, H, chunks, length):
+    # 148 SMs are assumed without a device
+    assert binding.sf_num_blocks(desc(H=H, seg_len=64 * chunks)) == -(-chunks // length)
+
+
 def test_status_strings(lib):
     assert binding.status_string(0) == "ok"
     assert "workspace" in binding.status_string(3)
