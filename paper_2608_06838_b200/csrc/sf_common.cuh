@@ -36,7 +36,8 @@ struct SegParams {
 
 // Programmatic dependent launch.  A kernel launched with launch_after() may start while the kernel before it in the stream
 // still runs, once every CTA of that one has called grid_launch_next(); what it does before grid_wait() may only touch its own
-// on-chip state and the caller's inputs.  grid_wait() returns when the kernel before has completed and its writes are visible;
+// on-chip state, the caller's inputs and, past L1, SegParams::bslot, whose writer (mark_bounds_kernel) has completed before any
+// of these can start: the kernel behind it, the merged chain's aggregate, is launched without the early start.  grid_wait() returns when the kernel before has completed and its writes are visible;
 // every CTA calls it, so completion carries over a sequence of such launches.  What a kernel of the same call wrote is read
 // through pointers without __restrict__: the data changes while this kernel is resident, so its loads must not count as
 // read-only ones, which may be moved ahead of the wait.

@@ -646,10 +646,11 @@ __device__ __forceinline__ void sweep_body(int role, const SweepMaps& m, const S
         ptx::fence_mbar_init();
     }
     if (warp == W_MMA) ptx::tmem_alloc(&sm.tmem_base, 512);
-    if (!BWD && warp == 1) {                             // where segments of a merged launch begin (a block has at most 64 chunks)
+    if (!BWD && warp == 1) {                             // where segments of a merged launch begin (a block has at most 64 chunks), ahead of
+                                                         // grid_wait(): see there
         unsigned long long cuts = 0;
         if (p.bslot) {
-            const bool lo = lane < nch && __ldg(p.bslot + c0 + lane) >= 0, hi = lane + 32 < nch && __ldg(p.bslot + c0 + lane + 32) >= 0;
+            const bool lo = lane < nch && __ldcg(p.bslot + c0 + lane) >= 0, hi = lane + 32 < nch && __ldcg(p.bslot + c0 + lane + 32) >= 0;
             cuts = __ballot_sync(0xffffffffu, lo) | ((unsigned long long)__ballot_sync(0xffffffffu, hi) << 32);
         }
         if (lane == 0) sm.cuts = cuts;
@@ -853,7 +854,7 @@ __device__ __forceinline__ void sweep_body(int role, const SweepMaps& m, const S
                 float* dump = nullptr;                   // merged launches: the state entering a segment's first chunk goes out
                 if (!BWD && it.c == 0 && p.single && p.s_copy) dump = p.s_copy + bh * (D * D);
                 else if (!BWD && p.bslot) {
-                    const int slot = __ldg(p.bslot + c0 + it.c);
+                    const int slot = __ldcg(p.bslot + c0 + it.c);
                     if (slot >= 0) dump = p.bbase + slot * p.bstride + bh * (D * D);
                 }
                 if (it.i > 0) SF_WAIT(&sm.st_done[s ^ 1], (uint32_t)((it.i - 1) >> 1) & 1, DEV_TIMEOUT_MMA);

@@ -748,7 +748,7 @@ sf_status_t chain_fwd_merged(const sf_seg_desc_t* vd, bool free_grid, const int3
         p.bbase = S_bounds;
         p.bstride = (long long)sN;
     }
-    SF_TRY(fwd_pre(path, vd, p, x, w, st));
+    SF_TRY(fwd_pre(path, vd, p, x, w, st, false));             // not early: the sweep reads `slot` ahead of its wait (see grid_wait())
     SF_TRY(fwd_scan(vd, p, x, w, st, true));
     if (!free_grid) {
         // S_bounds[i] = state entering the first block of segment i (a strided copy: one state per batch x head)
