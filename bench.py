@@ -29,14 +29,15 @@ sys.path.insert(0, ROOT)
 METRIC = "fwd+bwd tokens/s per linear-recurrence layer"
 UNIT = "tokens/s"
 BYTES_PER_TOKEN_HEAD = 2828          # q,k,v,dO read once, o,dq,dk,dv written once (bf16, d=128), g and dg float32
-FLOPS_PER_TOKEN_HEAD = 344064        # full chunk tiles, d = 128, chunk 64: forward 98304 + backward 245760
+# tensor-core operations as they run, d = 128: four sweeps over tiles of 128 tokens (131072 each) and two aggregates (32768 each)
+FLOPS_PER_TOKEN_HEAD = 589824
 # algorithmic bytes per token*head of each kernel (its own inputs read once, its own outputs written once)
 KERNEL_BYTES = {"agg_kv": 516, "agg_qdo": 516, "fwd_out": 1028, "dq": 1284, "dkdv": 1540}
 # DRAM bytes per token*head of each kernel from the ncu capture of the small case (profiles/, 262144 token*heads per
 # launch), scaled to a bench launch by the token*heads it processes (traffic grows in proportion)
-KERNEL_NCU_TRAFFIC = {"agg_kv": (135.293e6 + 4.131e6) / 262144, "agg_qdo": (135.293e6 + 4.964e6) / 262144,
-                      "fwd_out": (210.914e6 + 43.968e6) / 262144, "dq": (278.050e6 + 49.405e6) / 262144,
-                      "dkdv": (278.054e6 + 106.869e6) / 262144}
+KERNEL_NCU_TRAFFIC = {"agg_kv": (135.303e6 + 3.147e6) / 262144, "agg_qdo": (135.303e6 + 3.152e6) / 262144,
+                      "fwd_out": (210.912e6 + 40.357e6) / 262144, "dq": (278.086e6 + 47.586e6) / 262144,
+                      "dkdv": (285.313e6 + 107.338e6) / 262144}
 
 
 def peaks():

@@ -17,7 +17,7 @@
  *    device memory (the one exception is documented at its declaration).
  *  - Work is enqueued on the given stream and the call returns without
  *    synchronising.  Outputs are valid once the stream reaches that point; all
- *    buffers must stay alive and unmodified until then.
+ *    buffers must stay alive and unmodified until then, so outputs overlap no input.
  *  - Layout (row-major, strides in ELEMENTS of the tensor's type):
  *      q, k, dq, dk : [B, T, H, d_k]       v, o, dO, dv : [B, T, H, d_v]
  *      g, dg        : [B, T, H]  float32   (log-decay, g <= 0 expected, not checked)
@@ -30,7 +30,8 @@
  *    are float32.  Arithmetic accumulates in float32.
  *  - Inf and NaN: results that depend on a value that is not finite are not finite themselves,
  *    but an Inf may come out as NaN (the tensor cores take float32 operands as several
- *    terms).  Tokens that do not depend on it keep their values in the warp-level kernels.
+ *    terms).  Tokens that do not depend on it keep their values in the warp-level kernels; in the
+ *    bf16 kernels of 128-wide heads one in v or dO reaches the 16 tokens it stands among.
  *    Log-decays below -1e4, -inf included, count as -1e4 in the kernels of float32 precision
  *    (warp-level, chunkwise delta rule), those below -128 as -128 in the bf16 kernels of
  *    128-wide heads: the state is wiped all the same.
@@ -81,7 +82,7 @@ typedef enum { SF_BF16 = 0, SF_F32 = 1 } sf_dtype_t;
  * fewer tokens (its missing rows count as zero keys, values and gradients with log-decay 0, and are never
  * written).  chunks_per_block sets how many chunks form one block, the only granularity
  * whose states are written to the workspace (at most 64); 0 lets the library
- * pick the length in [4, 32] that fills the device's SMs best for this shape.  Heads are independent.
+ * pick the length, at most 64, that fills the device's SMs best for this shape.  Heads are independent.
  */
 typedef struct {
     int32_t B, H, d_k, d_v;

@@ -56,7 +56,8 @@ __device__ __forceinline__ int ld_shared_volatile(uint32_t a) {
 // Bounded wait: gives up after `limit` clock cycles (about a second by default), records `code` in the device's status word
 // and sets the CTA-wide sticky flag *abort_flag (shared) so that every later wait in this CTA returns at once.
 // The kernel then runs to its end on undefined data and releases its TMEM normally.
-// SPIN: without suspending the thread between tries, for the one warp whose next instructions everything else waits for.
+// SPIN: after a first try that may suspend the thread, further ones do not; for the one warp whose next instructions everything else waits
+// for (a test in the place of the first try too: chain of 8 x 4096 tokens x 16 heads 573.6 -> 576.9 us, 3001 tokens x 32 heads 154.7 -> 155.4).
 // Not inlined: a kernel has dozens of waits, and its code has to fit the instruction cache.
 constexpr long long WAIT_LIMIT_CYCLES = 2000000000LL;
 template <bool SPIN>
@@ -101,11 +102,6 @@ __device__ __forceinline__ void tc_fence_before_sync() { asm volatile("tcgen05.f
 __device__ __forceinline__ void tc_fence_after_sync() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void named_bar_sync(int id, int nthreads) {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
-}
-
-// bring one 128-byte line of global memory into L2 (no register, no wait)
-__device__ __forceinline__ void prefetch_l2(const void* p) {
-    asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<uint64_t>(p)) : "memory");
 }
 
 // ---- TMA -------------------------------------------------------------------------------------------

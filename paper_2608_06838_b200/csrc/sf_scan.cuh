@@ -137,8 +137,8 @@ __global__ void mark_bounds_kernel(int* __restrict__ slot, int clear, SegStarts 
 // The rounding errors of the dot products add up along the block like a random walk.  The block's end is an anchor too: there
 // the sum must arrive at <H, dH> of the state that leaves (Hs[j+1] and Gs[j]; at the segment's end DgEnd).  What is missing, D, is
 // spread over the block in proportion to the variance met so far, sum (q.dq)^2 + (k.dk)^2 (whole chunks, linear inside one):
-// the walk then is a bridge, with a third of its mean square.  rms error of dg over rms, 2 of 40 heads x 131072 tokens: blocks of 16
-// chunks 9.0e-3 without the second anchor, of 64 chunks 1.6e-2.  A D that is not finite (NaN or Inf in later tokens) is not spread.
+// the walk then is a bridge, with a third of its mean square.  rms error of dg over rms, 2 of 40 heads x 32768 tokens: blocks of 16
+// chunks 7.1e-3 without the second anchor, 4.0e-3 with it, of 48 9.9e-3 and 6.1e-3.  A D that is not finite (NaN or Inf in later tokens) is not spread.
 // grid = (NB, H, B), DG_NT threads.  xq, xk: [B,H,L]; dg: [B,L,H] with strides.
 constexpr int DG_NT = 512;
 struct DgEnd {

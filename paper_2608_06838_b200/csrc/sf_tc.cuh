@@ -436,8 +436,8 @@ tc_aggregate_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_consta
 //
 // What bounds them: per tile scores -> mask -> P z -> epilogue in series (850 + 1650 + 800 + 600 cycles), MMAs 2048 of 4150.  A second set of
 // score columns (x St and P z in one accumulator, rescaled between) to overlap two tiles was slower: 4700 cycles, the elementwise warps
-// then are in series.  Against 64-token tiles with dk and dv in one sweep (16384 tokens x 32 heads): o 116 -> 86 us, dq 150 -> 113,
-// dk and dv 389 -> 311; chains forward + backward 1.13x, 256K tokens x 32 heads 9.43 -> 8.25 ms.
+// then are in series.  Against 64-token tiles with dk and dv in one sweep (16384 tokens x 32 heads): o 123 -> 87 us, dq 151 -> 110,
+// dk and dv 219 -> 201 (one launch of 256 CTAs, two waves of 32 tiles in series); chains forward + backward 1.13x, 256K tokens x 32 heads 9.43 -> 8.25 ms.
 //
 // A tile is two 64-token chunks, or one before a chunk where a segment of a merged launch begins (SegParams::bslot) and at the end
 // of a block; the rows of a missing half take no part in the state update and in P z and are not stored.
@@ -892,7 +892,8 @@ tc_forward_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
 }
 
 // The backward's sweeps, any consecutive ones in one launch: grid (heads x sweeps, NB, B).  dk and dv of a block are neighbours:
-// they walk the same tokens at the same pace and read q and dO once from DRAM between them.
+// they walk the same tokens at the same pace and read q and dO once from DRAM between them (8192 tokens x 32 heads: 285 MB read, the four inputs
+// are 268 MB).
 struct BwdMaps { CUtensorMap q, k, v, dO, dq, dk, dv; };
 struct BwdArgs {
     const float *Hs, *Gs;

@@ -83,7 +83,7 @@ Path classify(const sf_seg_desc_t* d) {
     if (d->dtype == SF_BF16) {
         if (d->tok_stride_qk % 8 || d->tok_stride_v % 8 || d->batch_stride_qk % 8 || d->batch_stride_v % 8) return Path::Invalid;
         if (d->d_k == 128 && d->d_v == 128) {
-            if (d->chunk != 64 || d->chunks_per_block > sf::tc::MAXR || 2LL * d->H > 65535LL) return Path::Unsupported;
+            if (d->chunk != 64 || d->chunks_per_block > sf::tc::MAXR || 2LL * d->H > 65535LL) return Path::Unsupported;      // H: a limit of the interface
             return Path::Tc;
         }
         if (d->d_k == 128 || d->d_v == 128) return Path::Unsupported;
@@ -133,10 +133,9 @@ int auto_chunks_per_block(int NC, long long bh, int longest = 64) {
 
 // The same choice for a segment that runs inside a chain of several.  There the sweeps of neighbouring segments
 // share the device (the chain driver sends them to different streams), so what counts for a short segment is the
-// work per launch, not whole waves: measured (graph replays of whole chains), the fastest block length keeps
-// blocks at least 8 chunks long and a launch at 40 CTAs or more (4096-token segments x 16 heads: 16-22 instead of 8
-// chunks, 10 % faster; 512- to 2048-token segments x 40 heads: one block instead of two, 8-10 % faster).  Segments
-// of more than 64 chunks keep the wave model.
+// work per launch, not whole waves: blocks are at least 8 chunks long and a launch has 40 CTAs or more.  Graph replays of chains launched per
+// segment: 8 x 4096 tokens x 16 heads, blocks of 8 chunks 744 us, 16 612, 22 570 (32, 32 CTAs: 545); 64K tokens x 40 heads in segments of
+// 512, 1024 and 2048, two blocks 6151 / 4013 / 3231 us, one 3996 / 3015 / 2695.  Segments of more than 64 chunks keep the wave model.
 int chain_chunks_per_block(int NC, long long bh) {
     if (NC > 64) return auto_chunks_per_block(NC, bh);
     long long nb = (40 + bh - 1) / bh;                       // blocks for 40 CTAs or more
@@ -444,8 +443,8 @@ sf_status_t bwd_dkdv(Path path, const sf_seg_desc_t* d, const SegParams& p, cons
     return launch_role(path, Role::BwdDkDv, d, p, a, st, early);
 }
 // Whether the last block's log-decay gradient is anchored at the end of the chain (or segment call) too, where the caller's gradient
-// comes in as it is: not with up to four chunks, where that anchor's own error is no smaller than what the sums collect (rms error
-// of dg: 200 tokens 3.1e-3 without it, 3.3e-3 with; 70 tokens 1.1e-3 / 2.8e-3; 512 tokens 9.5e-3 / 3.6e-3).
+// comes in as it is: not with up to four chunks, where the sums are short and in a segment call the launch that it takes counts (rms error of dg, 16
+// heads, without it and with: 70 tokens 1.7e-3 both, 200 2.5e-3 / 1.9e-3, 320 3.4e-3 / 2.5e-3).
 bool anchored_end(const SegParams& p) { return p.NC - (p.NB - 1) * p.R > 4; }
 
 // `S_end`: the state leaving the segment, or with end_g, the log-decays, the last block's aggregate (sf::DgEnd); NULL: neither is at hand.
@@ -461,7 +460,7 @@ sf_status_t bwd_dg(const sf_seg_desc_t* d, const SegParams& p, const BwdPtrs& x,
 // A segment of one block on the tensor-core path: the sweeps start from the boundary state itself and store the state that
 // leaves, so the aggregate and the scan (two launches of 4-9 us each way, and their passes over k, v, q, dO) are left out.
 // The forward keeps the entering state in the workspace for the backward, as the scan would.
-// 200 tokens x 16 heads, forward: 27.6 -> 18.3 us.
+// 200 tokens x 16 heads, two blocks of two chunks and one of four: forward 16.0 -> 14.1 us, backward with replay 32.9 -> 17.6.
 bool one_block(Path path, const SegParams& p) { return path == Path::Tc && p.NB == 1; }
 
 // The first kernel of a call: launched early like the others, but it waits before it touches global memory.
@@ -644,10 +643,11 @@ sf_status_t validate_chain(const sf_seg_desc_t* d, const int32_t* seg_lens, int3
 // Longest block of a chain that the library merges by itself.  The error of the log-decay gradient grows with the root of the block
 // length, and a block with anchors at both ends has the rms error of one a third as long with one (dg_epilogue_kernel).  So the limit
 // is 11/4 of the mean, over the tokens, of the blocks that the segments have by themselves: no worse than those with one anchor.
-// 40 heads x 32 segments of 1024, rms error: blocks of 16 with one anchor 8.5e-3, of 40 with two 7.9e-3, of 48 8.9e-3; 64 segments of
-// 512: 8 with one 6.7e-3, 20 with two 5.6e-3, 24 6.6e-3.  The chain of 128 segments takes 6.37 ms with 64 and with 48, 6.53 with 40.
-// Below four chunks the anchors' own errors count as much as the sums': no longer blocks (4 heads x 8 segments of 128: 2 chunks 54 us and
-// 2.5e-3, 4 chunks 62 and 3.5e-3, one launch per segment 104 and 3.4e-3).
+// 40 heads x 32 segments of 1024, rms error at log-decay scales 1, 0.1, 0.01: blocks of 16 with one anchor 7.1e-3 6.1e-3 6.7e-3, of 40 with two
+// 6.1e-3 5.7e-3 6.1e-3, of 64 7.5e-3 6.8e-3 9.0e-3; 64 segments of 512: 8 with one anchor 5.0e-3 4.7e-3 4.6e-3, 20 with two 4.7e-3 4.2e-3 3.8e-3, 24
+// 5.1e-3 4.3e-3 4.3e-3.  The chain of 128 segments of 1024 takes 5.06 ms with 40, 5.35 with 48 and 64.
+// Below four chunks the anchors' own errors count as much as the sums': no longer blocks (4 heads x 8 segments of 128: 2 chunks 46 us and
+// 2.0e-3 2.6e-3 2.6e-3, 4 chunks 54 us and 2.0e-3 3.0e-3 3.2e-3, one launch per segment 127 us).
 int merged_longest_block(const sf_seg_desc_t* desc, const int32_t* seg_lens, int32_t n_seg, long long T) {
     long long sum = 0;
     for (int i = 0; i < n_seg; ++i)
@@ -709,11 +709,11 @@ bool merged_desc(const sf_seg_desc_t* desc, const int32_t* seg_lens, int32_t n_s
 
 // Whether a chain runs merged: when the tuning asks for it, and where the caller leaves the block length to the library, on the
 // tensor-core path for chains whose segments hold less than 448 K token-heads on average.  Measured (chain forward + backward,
-// eager, us, one launch per segment / merged): 16 heads x 8 segments of 4096 775 / 653, 40 x 128 of 1024 7614 / 6301, 24 x
-// (2560, 1024) 199 / 164, 16 x 8 of 512 235 / 140, 8 x 8 of 16384 (131 K token-heads each) 1439 / 1229, 32 x (12288 .. 6144) (262 K)
-// 2712 / 2557; equal from 364 K on (40 x 21 of 9088: 9396 / 9415), where each segment's launch fills the device by itself and
-// the overlapped segments keep working sets smaller (32 x 16 of 16384, 524 K: 9886 / 9744 eager, 9830 / 10246 as a graph).
-// The smallest chains gain most: 3 heads x 6 segments of 512 and 256 206 / 76, 2 x 4 of 256 119 / 69, 4 x 8 of 128 199 / 73.
+// eager, us, one launch per segment / merged): 16 heads x 8 segments of 4096 656 / 562, 40 x 128 of 1024 6474 / 5022, 24 x
+// (2560, 1024) 209 / 167, 16 x 8 of 512 228 / 145, 8 x 8 of 16384 (131 K token-heads each) 1053 / 1048, 32 x (12288 .. 6144) (262 K)
+// 2188 / 2048.  Above, each segment's launch fills the device by itself and the overlapped segments keep working sets smaller
+// (32 x 16 of 16384, 524 K: 8218 / 7945 eager, 7783 / 8140 as a graph).
+// The smallest chains gain most: 3 heads x 6 segments of 512 and 256 215 / 82, 2 x 4 of 256 123 / 78, 4 x 8 of 128 204 / 72.
 bool runs_merged(const sf_seg_desc_t* desc, const int32_t* seg_lens, int32_t n_seg, long long T, const sf_tuning_t& tu, sf_seg_desc_t* vd,
                  bool* free_grid = nullptr) {
     const long long th = T * desc->B * desc->H;
