@@ -29,8 +29,9 @@ sys.path.insert(0, ROOT)
 METRIC = "fwd+bwd tokens/s per linear-recurrence layer"
 UNIT = "tokens/s"
 BYTES_PER_TOKEN_HEAD = 2828          # q,k,v,dO read once, o,dq,dk,dv written once (bf16, d=128), g and dg float32
-# tensor-core operations as they run, d = 128: four sweeps over tiles of 128 tokens (131072 each) and two aggregates (32768 each)
-FLOPS_PER_TOKEN_HEAD = 589824
+# of the chunkwise form with full chunks, d = 128, chunk 64: forward 98304 + backward 245760 (the kernels run 589824: sweeps over tiles of 128
+# tokens, dk and dv apart, block aggregates)
+FLOPS_PER_TOKEN_HEAD = 344064
 # algorithmic bytes per token*head of each kernel (its own inputs read once, its own outputs written once)
 KERNEL_BYTES = {"agg_kv": 516, "agg_qdo": 516, "fwd_out": 1028, "dq": 1284, "dkdv": 1540}
 # DRAM bytes per token*head of each kernel from the ncu capture of the small case (profiles/, 262144 token*heads per
